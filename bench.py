@@ -130,7 +130,8 @@ def write_ncu_traffic(csv_path, precision, n, note, out_path=None):
         elif "kcolm_wr" in name:
             k = "col_level1"
         elif "kcol_wr" in name or "kcol_pipe" in name:
-            m = re.search(r"kcol_pipe<\s*\w+\s*,\s*(\w+)", name)   # the second template argument: MULTI
+            # (logs with a separate level-1 launch: the second of three template arguments)
+            m = re.search(r"kcol_pipe<\s*\w+\s*,\s*(\w+)\s*,", name)
             if m and m.group(1) not in ("false", "0"):
                 k = "col_level1"
             else:

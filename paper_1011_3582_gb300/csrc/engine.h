@@ -68,8 +68,8 @@ class Engine {
 // kernel kinds of one stage (index into the profile arrays)
 enum KernelKind {
     KK_ROW_FORWARD = 0,   // moments + forward row transforms
-    KK_COL_CONV = 1,      // column pass, convection
-    KK_COL_LEVEL1 = 2,    // column pass, level-1 derivatives
+    KK_COL_CONV = 1,      // column pass, convection and level-1 derivatives
+    KK_COL_LEVEL1 = 2,    // (level-1 derivatives by themselves: no launches)
     KK_ROW_LEVEL1 = 3,    // level-1 row inverse + Lambda/Phi + forward rows
     KK_COL_LEVEL2 = 4,    // column pass, level-2 divergences
     KK_ROW_FINAL = 5,     // row inverse + force + BGK + RK combination

@@ -2,7 +2,7 @@
 // and the per-precision plan.  Included by engine_f64.cu and engine_f32.cu
 // only (each instantiates one precision).
 //
-// One Runge-Kutta stage L(f) (Eq. 10) runs as six launches of the
+// One Runge-Kutta stage L(f) (Eq. 10) runs as five launches of the
 // pipelined kernels of kernels_pipe.cuh on the handle's stream (profile
 // names in parentheses):
 //   k1_pipe (row_forward_moments)  moments rho, u, T (Eqs. 7-9) of the stage
@@ -10,11 +10,11 @@
 //                           and g = M/T; forward row transforms of the 32
 //                           moving f_i and of rho, u_x, u_y, T, Pi, g
 //   kcol_pipe (col_convection)  column forward -> i (v_x k_m,x + v_y k_m,y)
-//                           -> column inverse for the 32 f_i (in place)
-//   kcol_pipe (col_level1)  the 8 level-1 derivative spectra that involve
-//                           k_y (d_y of rho, u, T, Pi, g; d_yy rho;
-//                           d_y div u)
-//   k3_pipe (row_level1)    the 7 derivatives in k_x alone, formed in the
+//                           -> column inverse for the f_i with v_y != 0 (in
+//                           place), and in the same launch the 8 level-1
+//                           column passes (d_y of rho, u, T, Pi, g; d_yy of
+//                           rho and u_y)
+//   k3_pipe (row_level1)    the derivatives with a factor k_x, formed in the
 //                           row spectrum (k3_form_x); row inverse of the
 //                           15; Lambda (Eq. 19), Phi = 2 q rho T grad T
 //                           (Eq. 23), the numerators of C (Eq. 22) and B
@@ -69,13 +69,20 @@ enum { D_RX, D_RY, D_LAP, D_UXX, D_UXY, D_UYX, D_UYY, D_DIVX, D_DIVY, D_TX, D_TY
 // that the Nyquist bins carry zero).  A derivative whose multiplier depends
 // on k_x alone needs no column transform: in the row-transformed slot it is
 // the pointwise product i k_x X / nx (the 1 / nx that the column pass would
-// leave).  So the level-1 column pass forms only the outputs that involve
-// k_y, 8 of the 15 (d_y of rho, u_x, u_y, T, Pi, g; d_yy rho;
-// d_xy u_x + d_yy u_y), and the row kernel K3 forms the other 7 from the
-// row spectra of rho, u_x, u_y, T, Pi, g before its inverse rows:
+// leave).  So the column pass forms only derivatives in k_y alone, each of
+// one input: d_y of rho, u_x, u_y, T, Pi, g and d_yy of rho, u_y; and the
+// row kernel K3 forms the rest from the row spectra of rho, u_x, u_y, T,
+// Pi, g and of those before its inverse rows:
 //   rho_x = i k_x rho^ / nx, lap rho = d_yy rho - k_x^2 rho^ / nx,
 //   u_xx = i k_x u_x^ / nx, u_yx = i k_x u_y^ / nx,
-//   d_x(div u) = i k_x (u_xx + u_yy), T_x, Pi_x, g_x = i k_x (.)^ / nx.
+//   d_x(div u) = i k_x (u_xx + u_yy), d_y(div u) = d_yy u_y + i k_x (d_y u_x),
+//   T_x, Pi_x, g_x = i k_x (.)^ / nx.
+// With one input and one output each, the level-1 passes are 8 more groups
+// of the convection launch.  A launch of their own for rho (two outputs) and
+// u (two inputs, two outputs) transformed two inputs fewer, but with three
+// tiles and 219 KB a block it left most SMs with one job's latency: 22.5 us
+// at 1024^2 in fp32, against the 9 us these jobs add to the convection
+// launch (69.8 -> 78.7 us); 48 and 15.9 us against none on 64^2 fp64 and fp32.
 // Level 2 in the same way: d_x Lambda_xx + d_y Lambda_xy is the column
 // pass of d_y Lambda_xy plus i k_x Lambda_xx^ / nx, formed by K3 (add_slot).
 // k3_src_slot(o): the slot K3 loads into its row o (-1: formed in K3).
@@ -794,7 +801,7 @@ class EngineT : public Engine {
 
     long steps() const override { return steps_; }
     void set_steps(long s) override { steps_ = s; }
-    int launches_per_step() const override { return 6 * (p_.integrator == 1 ? 1 : 3); }
+    int launches_per_step() const override { return 5 * (p_.integrator == 1 ? 1 : 3); }
     const fftlb_params &params() const override { return p_; }
 
   private:
@@ -824,9 +831,9 @@ class EngineT : public Engine {
     void *scratch_d_ = nullptr;
     std::vector<void *> allocs_;
     // group ranges in groups_
-    int conv_groups_ = 0, l1_groups_ = 0, l2_groups_ = 0, grad_groups_ = 0, inv_groups_ = 0;
+    int conv_groups_ = 0, l2_groups_ = 0, grad_groups_ = 0, inv_groups_ = 0;
     int nconv_ = NMOV;   // convection groups (velocities with v_y != 0)
-    int nconvl_ = NMOV;  // ... and the one-input level-1 groups after them
+    int nconvl_ = NMOV;  // ... and the level-1 groups after them
     // warp-resident fp32 row kernels (kernels_wr.cuh) for nx = 512, 1024:
     // their stage-1 twiddle table and launch shape
     static constexpr bool wr_ok_ = std::is_same<real, float>::value && !SPLIT;
@@ -835,10 +842,10 @@ class EngineT : public Engine {
     size_t smem5w_ = 0, smem1w_ = 0, smem3w_ = 0;
     int grid5w_ = 1, grid1w_ = 1, grid3w_ = 1;
     // warp-resident convection columns for ny = 256, 512, 1024
-    bool colwr_ = false, colmwr_ = false;
+    bool colwr_ = false;
     C *Twc_ = nullptr;
-    size_t smemcw_ = 0, smemcmw_ = 0;
-    int gridcw_ = 1, nbufcw_ = 1, gridcmw_ = 1, ntcw_ = 256;
+    size_t smemcw_ = 0;
+    int gridcw_ = 1, nbufcw_ = 1, ntcw_ = 256;
     CUtensorMap tmap_convw_{};
     // gradient kernels (k_grad_*): column tile width and shared memory
     int TWg_ = 0;
@@ -854,7 +861,7 @@ class EngineT : public Engine {
     int CH1_ = 8, SMAX1_ = 1, grid1_ = 1, NHB5_ = 1, WR3_ = 1, CH5_ = 8, grid5_ = 1, SMAX5_ = 1, BOXR_ = 1;
     int TWc_ = 1, TWl_ = 1, gridc_ = 1, gridl_ = 1, NBUFc_ = 2, NBUFl_ = 2, NBUF5_ = 2;
     size_t smem1_ = 0, smem3_ = 0, smem5_ = 0, smemc_ = 0, smeml_ = 0;
-    CUtensorMap tmap_conv_{}, tmap_l1_{};
+    CUtensorMap tmap_conv_{}, tmap_l2_{};
     // profiling
     bool prof_ = false;
     struct ProfEv {
@@ -920,8 +927,8 @@ class EngineT : public Engine {
         // write once (one-sided spectra count N reals per field)
         const double alg[KK_COUNT] = {
             (33 + 38 + 4) * NN * s,                   // f in; 38 spectra + rho, u, T out
-            2.0 * nconvl_ * NN * s,                   // the v_y != 0 spectra and T, Pi, g, u_y in; as many out
-            (3 + 4) * NN * s,                         // rho, u_x, u_y in; 4 out
+            2.0 * nconvl_ * NN * s,                   // the v_y != 0 spectra and the level-1 inputs in (rho, u_y twice); as many out
+            0,                                        // (level 1 runs in the convection launch)
             (14 + 2 + 3 + 6) * NN * s,                // 14 + rho, T in; 3 aux + 6 spectra out
             (3 + 3 + 3) * NN * s,                     // 3 in, 3 added, 3 out
             (32 + 3 + 4 + 3 + 33 + 33 * fbase + 33) * NN * s};
@@ -1250,7 +1257,7 @@ class EngineT : public Engine {
 
     Status build_groups() {
         static const double DX[5] = {1, 0, 0, 0, 0}, DY[5] = {0, 1, 0, 0, 0};
-        static const double DYY[5] = {0, 0, 0, -1, 0}, DXY[5] = {0, 0, 0, 0, -1};
+        static const double DYY[5] = {0, 0, 0, -1, 0};
         std::vector<GroupDesc> gs;
         // convection: i (v_x k_x + v_y k_y) f_i, in place, for the velocities
         // with v_y != 0 (the row kernel K1 writes i v_x k_x f_i^ / nx for the
@@ -1265,33 +1272,19 @@ class EngineT : public Engine {
             add_out(g, i - 1, 1, 0, c);
             gs.push_back(g);
         }
-        // level 1: the outputs that involve k_y (k3_src_slot: K3 forms the
-        // rest).  Four of one input and one output (d_y T, d_y Pi, d_y g,
-        // d_y u_y) run with the convection groups, in the same launch
-        // (nconvl_ groups from conv_groups_: they fill its last round of
-        // jobs); rho (d_y, d_yy) and u (d_y u_x, d_y div u) run as the
-        // level-1 launch.
+        // level 1: the derivatives in k_y alone (k3_src_slot: K3 forms the
+        // rest, and adds -k_x^2 rho^ / nx to d_yy rho, i k_x (d_y u_x) to
+        // d_yy u_y), in the convection launch (nconvl_ groups from
+        // conv_groups_)
         {
-            const int singles[4][2] = {{SLOT_T, D_TY}, {SLOT_PI, D_PIY}, {SLOT_G, D_GY}, {SLOT_UY, D_UYY}};
+            const int singles[8][2] = {{SLOT_RHO, D_RY}, {SLOT_RHO, D_LAP}, {SLOT_UX, D_UXY}, {SLOT_UY, D_UYY},
+                                       {SLOT_UY, D_DIVY}, {SLOT_T, D_TY}, {SLOT_PI, D_PIY}, {SLOT_G, D_GY}};
             for (auto &sgl : singles) {
                 GroupDesc g = group(1, sgl[0], 0);
-                add_out(g, SLOT_D1 + sgl[1], 1, 0, DY);
+                add_out(g, SLOT_D1 + sgl[1], 1, 0, sgl[1] == D_LAP || sgl[1] == D_DIVY ? DYY : DY);
                 gs.push_back(g);
             }
-            nconvl_ = nconv_ + 4;
-        }
-        l1_groups_ = (int)gs.size();
-        {
-            GroupDesc g = group(1, SLOT_RHO, 0);
-            add_out(g, SLOT_D1 + D_RY, 1, 0, DY);
-            add_out(g, SLOT_D1 + D_LAP, 1, 0, DYY);   // K3 adds -k_x^2 rho^ / nx
-            gs.push_back(g);
-        }
-        {
-            GroupDesc g = group(2, SLOT_UX, SLOT_UY);
-            add_out(g, SLOT_D1 + D_UXY, 1, 0, DY);
-            add_out(g, SLOT_D1 + D_DIVY, 2, 0, DXY, 1, DYY);   // D_y (D_x u_x + D_y u_y)
-            gs.push_back(g);
+            nconvl_ = nconv_ + 8;
         }
         // level 2: d_y of Lambda_xy, Lambda_yy, Phi_y plus the d_x terms K3
         // wrote (k3_mul_slot): outputs in 53, 55, 56
@@ -1426,16 +1419,13 @@ class EngineT : public Engine {
     static constexpr int NT1 = KCfg<real, KS_K1>::NT, NTC = KCfg<real, KS_COL>::NT, NT5 = KCfg<real, KS_K5>::NT;
     int ntrmax() const { return std::max(ntr_, ntr8_); }
     // shared memory of the column kernel: twiddles, pass tables, k tables,
-    // nbuf staged tiles of NIN inputs, NIN padded work tiles
-    size_t col_smem(bool multi, int tw, int nbuf) const {
+    // nbuf staged tiles, a padded work tile
+    size_t col_smem(int tw, int nbuf) const {
         const size_t cs = sizeof(C), rs = sizeof(real), pny = (size_t)padded_len(ny_);
         // staged input tiles are placed at 128-byte strides (tile_stride)
         const size_t tile = tile_stride<C>(tw, ny_) * cs, ptile = (size_t)tw * pny * cs, kt = (h_ + 1 + ny_) * rs;
-        const size_t nin = multi ? 2 : 1;
-        return nbuf > 1 ? (multi ? smem_bytes({ny_ * cs, ntc_ * cs, kt, nin * tile, nin * tile, ptile, ptile})
-                                 : smem_bytes({ny_ * cs, ntc_ * cs, kt, nin * tile, nin * tile, ptile}))
-                        : (multi ? smem_bytes({ny_ * cs, ntc_ * cs, kt, nin * tile, ptile, ptile})
-                                 : smem_bytes({ny_ * cs, ntc_ * cs, kt, nin * tile, ptile}));
+        return nbuf > 1 ? smem_bytes({ny_ * cs, ntc_ * cs, kt, tile, tile, ptile})
+                        : smem_bytes({ny_ * cs, ntc_ * cs, kt, tile, ptile});
     }
     // shared memory of the final row kernel for chunk size ch, nhb head
     // buffers and nbuf chunk buffers
@@ -1450,13 +1440,13 @@ class EngineT : public Engine {
     // (the input tiles themselves sit at 128-byte strides, tile_stride).
     bool boxes_aligned(int tw) const { return ny_ <= BOXR_ || ((size_t)BOXR_ * tw * sizeof(C)) % 128 == 0; }
     // buffers for a column tile width: two unless one gives more blocks per SM
-    Status col_nbuf(bool multi, int tw, int *nbuf, size_t *sm, int *grid) {
+    Status col_nbuf(int tw, int *nbuf, size_t *sm, int *grid) {
         int best = -1;
         for (int nb2 = 2; nb2 >= 1; --nb2) {
-            const size_t s = col_smem(multi, tw, nb2);
+            const size_t s = col_smem(tw, nb2);
             if (s > budget_) continue;
             int nb = 0;
-            Status st = multi ? occupancy(kcol_pipe<real, true, SPLIT>, NTC, s, &nb) : occupancy(kcol_pipe<real, false, SPLIT>, NTC, s, &nb);
+            Status st = occupancy(kcol_pipe<real, SPLIT>, NTC, s, &nb);
             if (!st.good()) return st;
             if (nb > best) {
                 best = nb;
@@ -1541,7 +1531,7 @@ class EngineT : public Engine {
                 break;
             }
         const size_t pny = (size_t)padded_len(ny_);
-        auto pick_tw = [&](bool multi, int *tw_out, int *nbuf_out, size_t *sm_out, int *grid_out) -> Status {
+        auto pick_tw = [&](int *tw_out, int *nbuf_out, size_t *sm_out, int *grid_out) -> Status {
             int bestscore = -1;
             *tw_out = 0;
             for (int tw = 8; tw >= 1; tw >>= 1) {
@@ -1550,10 +1540,9 @@ class EngineT : public Engine {
                 if (!boxes_aligned(tw)) continue;
                 for (int nbuf = 2; nbuf >= 1; --nbuf) {
                     int nb = 0;
-                    const size_t sm = col_smem(multi, tw, nbuf);
+                    const size_t sm = col_smem(tw, nbuf);
                     if (sm > budget) continue;
-                    Status s2 = multi ? occupancy(kcol_pipe<real, true, SPLIT>, NTC, sm, &nb)
-                                      : occupancy(kcol_pipe<real, false, SPLIT>, NTC, sm, &nb);
+                    Status s2 = occupancy(kcol_pipe<real, SPLIT>, NTC, sm, &nb);
                     if (!s2.good()) return s2;
                     // most blocks per SM, then the widest tile, then two buffers
                     const int score = nb * 1000 + tw * 10 + nbuf;
@@ -1569,10 +1558,10 @@ class EngineT : public Engine {
             if (!*tw_out) return Status::err(FFTLB_ERR_ARG, "grid too large for the column kernel");
             return Status::ok();
         };
-        if (!(st = pick_tw(false, &TWc_, &NBUFc_, &smemc_, &gridc_)).good()) return st;
-        if (!(st = pick_tw(true, &TWl_, &NBUFl_, &smeml_, &gridl_)).good()) return st;
+        if (!(st = pick_tw(&TWc_, &NBUFc_, &smemc_, &gridc_)).good()) return st;
+        if (!(st = pick_tw(&TWl_, &NBUFl_, &smeml_, &gridl_)).good()) return st;
         if (!(st = make_tmap(&tmap_conv_, TWc_)).good()) return st;
-        if (!(st = make_tmap(&tmap_l1_, TWl_)).good()) return st;
+        if (!(st = make_tmap(&tmap_l2_, TWl_)).good()) return st;
         // K3 (one row per block, not pipelined inside a block): most blocks
         // per SM first, so that one block's row loads overlap another's
         // transforms, then the most work rows
@@ -1692,20 +1681,6 @@ class EngineT : public Engine {
                     colwr_ = true;
                     ntcw_ = NTw;
                     gridcw_ = best * nsm_;
-                    const size_t sm = kcolm_wr_smem(ny_, h_);
-                    nb = 0;
-                    if (sm <= budget_) {
-                        st = ny_ == 1024 ? occupancy(kcolm_wr<1024>, NTw, sm, &nb)
-                           : ny_ == 512  ? occupancy(kcolm_wr<512>, NTw, sm, &nb)
-                           : ny_ == 256  ? occupancy(kcolm_wr<256>, NTw, sm, &nb)
-                                         : occupancy(kcolm_wr<128>, NTw, sm, &nb);
-                        if (!st.good()) return st;
-                    }
-                    if (nb > 0) {
-                        colmwr_ = true;
-                        smemcmw_ = sm;
-                        gridcmw_ = nb * nsm_;
-                    }
                 }
             }
         }
@@ -1787,8 +1762,8 @@ class EngineT : public Engine {
         if (!nbuf5) return Status::err(FFTLB_ERR_ARG, "tuning parameters exceed shared memory");
         if (sm1 > budget_ || sm5 > budget_) return Status::err(FFTLB_ERR_ARG, "tuning parameters exceed shared memory");
         Status st;
-        if (!(st = col_nbuf(false, twc, &nbc, &smc, &gc)).good()) return st;
-        if (!(st = col_nbuf(true, twl, &nbl, &sml, &gl)).good()) return st;
+        if (!(st = col_nbuf(twc, &nbc, &smc, &gc)).good()) return st;
+        if (!(st = col_nbuf(twl, &nbl, &sml, &gl)).good()) return st;
         int nb = 0;
         st = occ_k1(sm1, &nb);
         if (!st.good()) return st;
@@ -1816,7 +1791,7 @@ class EngineT : public Engine {
         gridl_ = gl;
         grid5_ = g5;
         tmap_conv_ = mc;
-        tmap_l1_ = ml;
+        tmap_l2_ = ml;
         return Status::ok();
     }
 
@@ -1929,9 +1904,11 @@ class EngineT : public Engine {
         return Status::ok();
     }
 
-    Status launch_col(int first, int count, bool level1) {
+    // column pass of one-input groups; level2: the level-2 launch (its own
+    // tile width on the pipelined kernels)
+    Status launch_col(int first, int count, bool level2) {
         if constexpr (wr_ok_) {
-            if (!level1 && colwr_) {
+            if (colwr_) {
                 if (count > kMaxColGroups) return Status::err(FFTLB_ERR_ARG, "too many column groups in one launch");
 #define FFTLB_KCOLWR(NYV)                                                                                     \
     launch_pdl("kcol_wr", kcol_wr<NYV>, gridcw_, ntcw_, smemcw_, specb_, (const GroupDesc *)(groups_ + first),     \
@@ -1943,25 +1920,13 @@ class EngineT : public Engine {
                                    : FFTLB_KCOLWR(128);
 #undef FFTLB_KCOLWR
             }
-            if (level1 && colmwr_) {
-                if (count > kMaxMGroups) return Status::err(FFTLB_ERR_ARG, "too many column groups in one launch");
-#define FFTLB_KCOLMWR(NYV)                                                                                    \
-    launch_pdl("kcolm_wr", kcolm_wr<NYV>, gridcmw_, ntcw_, smemcmw_, specb_, (const GroupDesc *)(groups_ + first), \
-               count, (const float *)kxt_, (const float *)kyt_, (const float2 *)Twc_, kp_, BOXR_, tmap_convw_, err_)
-                return ny_ == 1024 ? FFTLB_KCOLMWR(1024)
-                     : ny_ == 512  ? FFTLB_KCOLMWR(512)
-                     : ny_ == 256  ? FFTLB_KCOLMWR(256)
-                                   : FFTLB_KCOLMWR(128);
-#undef FFTLB_KCOLMWR
-            }
         }
-        if (level1)
-            kcol_pipe<real, true, SPLIT><<<gridl_, NTC, smeml_, stream_>>>(specb_, groups_ + first, count, kxt_,
-                                                                               kyt_, Wc_, Tc_, ntc_, kp_, TWl_, BOXR_,
-                                                                               NBUFl_, tmap_l1_, err_);
+        if (level2)
+            kcol_pipe<real, SPLIT><<<gridl_, NTC, smeml_, stream_>>>(specb_, groups_ + first, count, kxt_, kyt_, Wc_, Tc_,
+                                                                     ntc_, kp_, TWl_, BOXR_, NBUFl_, tmap_l2_, err_);
         else
-            kcol_pipe<real, false, SPLIT><<<gridc_, NTC, smemc_, stream_>>>(
-                specb_, groups_ + first, count, kxt_, kyt_, Wc_, Tc_, ntc_, kp_, TWc_, BOXR_, NBUFc_, tmap_conv_, err_);
+            kcol_pipe<real, SPLIT><<<gridc_, NTC, smemc_, stream_>>>(specb_, groups_ + first, count, kxt_, kyt_, Wc_, Tc_,
+                                                                     ntc_, kp_, TWc_, BOXR_, NBUFc_, tmap_conv_, err_);
         FFTLB_LAUNCHED("kcol_pipe");
         return Status::ok();
     }
@@ -2000,9 +1965,6 @@ class EngineT : public Engine {
         if (!(st = prof_begin(KK_COL_CONV)).good()) return st;
         if (!(st = launch_col(conv_groups_, nconvl_, false)).good()) return st;
         if (!(st = prof_end()).good()) return st;
-        if (!(st = prof_begin(KK_COL_LEVEL1)).good()) return st;
-        if (!(st = launch_col(l1_groups_, 2, true)).good()) return st;
-        if (!(st = prof_end()).good()) return st;
         if (!(st = prof_begin(KK_ROW_LEVEL1)).good()) return st;
         bool k3done = false;
         if constexpr (wr_ok_) {
@@ -2023,7 +1985,7 @@ class EngineT : public Engine {
         FFTLB_LAUNCHED("k3_pipe");
         if (!(st = prof_end()).good()) return st;
         if (!(st = prof_begin(KK_COL_LEVEL2)).good()) return st;
-        if (!(st = launch_col(l2_groups_, 3, false)).good()) return st;   // one input, one output each
+        if (!(st = launch_col(l2_groups_, 3, true)).good()) return st;
         if (!(st = prof_end()).good()) return st;
         if (!(st = prof_begin(KK_ROW_FINAL)).good()) return st;
         if constexpr (wr_ok_) {

@@ -400,23 +400,6 @@ template <typename real> struct ColMult {
     }
 };
 
-// output o of a derivative group: sum over its terms of M_term(k_x, k_y)
-// times input term_in, times the inverse normalisation (the per-element
-// form of col_multiply, for pp_out_fused_p2)
-template <typename real> struct GroupMult {
-    using C = typename cplx_of<real>::type;
-    real p[5], q[5], scale;
-    int two, in0, in1;
-    const real *kxs, *kys;
-    int kx0;
-    __device__ __forceinline__ C operator()(int b, int e, C x0, C x1) const {
-        const real ax = kxs[kx0 + b], ay = kys[e];
-        C acc = mult_apply<real>(p[0], p[1], p[2], p[3], p[4], ax, ay, in0 ? x1 : x0);
-        if (two) acc = cadd(acc, mult_apply<real>(q[0], q[1], q[2], q[3], q[4], ax, ay, in1 ? x1 : x0));
-        return cscale(acc, scale);
-    }
-};
-
 // Elements between consecutive staged input tiles of TW x ny values: the
 // tile size rounded up to 128 bytes, the alignment a tensor copy needs for
 // its shared-memory destination.
@@ -430,11 +413,12 @@ __host__ __device__ __forceinline__ size_t tile_stride(int TW, int ny) {
 // staged in shared memory once per launch by the warp-resident column
 // kernels (a per-job copy of the whole GroupDesc by one thread held every
 // other warp of the block at the next barrier).
+// The multiplier is i (c0 k_x + c1 k_y), or c3 k_y^2 where c3 is not zero.
 struct ColG {
     int nin, in_slot[2], out_slot, add_slot;
-    float c0, c1;
+    float c0, c1, c3;
 };
-constexpr int kMaxColGroups = 32;   // groups of one kcol_wr launch (32 convection groups)
+constexpr int kMaxColGroups = 40;   // groups of one kcol_wr launch (at most 32 convection + 8 level-1 groups)
 
 // (GD: GroupDesc in global memory, or ColG / GroupDesc staged in shared memory)
 template <typename C, typename GD>
@@ -472,9 +456,8 @@ __device__ __forceinline__ void kcol_prefetch(const GD *groups, int k, int ntile
     }
 }
 
-// MULTI = false: every group has one input and one output in place
-// (convection); MULTI = true: up to 2 inputs and several outputs.
-template <typename real, bool MULTI, bool TC = false>
+// Every group has one input and one output, which may be the same slot.
+template <typename real, bool TC = false>
 __global__ void __launch_bounds__(KCfg<real, KS_COL>::NT, KCfg<real, KS_COL>::MINB) kcol_pipe(typename cplx_of<real>::type *spec,
                                                                const GroupDesc *__restrict__ groups, int ngroups,
                                                                const real *__restrict__ kxt,
@@ -486,7 +469,6 @@ __global__ void __launch_bounds__(KCfg<real, KS_COL>::NT, KCfg<real, KS_COL>::MI
     const uint4 *tc = TC ? P.tc16 : nullptr;   // split-BF16 tensor-core first passes
     using C = typename cplx_of<real>::type;
     constexpr int NT = KCfg<real, KS_COL>::NT;
-    constexpr int NIN = MULTI ? 2 : 1;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar0, bar1;
     __shared__ GroupDesc gd;
@@ -501,13 +483,12 @@ __global__ void __launch_bounds__(KCfg<real, KS_COL>::NT, KCfg<real, KS_COL>::MI
     C *Tc = (C *)sc.take(ntc * sizeof(C));
     real *kxs = (real *)sc.take((size_t)(h + 1 + ny) * sizeof(real));   // k_x then k_y tables
     real *kys = kxs + h + 1;
-    const size_t tstr = tile_stride<C>(TW, ny);   // input s of a job at buf + s tstr
-    C *buf0 = (C *)sc.take((size_t)NIN * tstr * sizeof(C));
+    const size_t tstr = tile_stride<C>(TW, ny);
+    C *buf0 = (C *)sc.take(tstr * sizeof(C));
     // nbuf = 2: double-buffered (job k + 2 prefetched while job k + 1 runs);
     // nbuf = 1: one buffer (job k + 1 loaded after job k), for two blocks per SM
-    C *buf1 = nbuf > 1 ? (C *)sc.take((size_t)NIN * tstr * sizeof(C)) : buf0;
+    C *buf1 = nbuf > 1 ? (C *)sc.take(tstr * sizeof(C)) : buf0;
     C *wk0 = (C *)sc.take((size_t)ptile * sizeof(C));
-    C *wk1 = MULTI ? (C *)sc.take((size_t)ptile * sizeof(C)) : nullptr;
     const Lay lt{1, TW, 0}, lw{1, TW, 1};   // staged tile / padded work tile
     const int ntiles = h / TW;
     const int njobs_total = P.nrun * ngroups * ntiles;
@@ -557,129 +538,56 @@ __global__ void __launch_bounds__(KCfg<real, KS_COL>::NT, KCfg<real, KS_COL>::MI
             pend0 = false;
         }
         C *in0 = odd ? buf1 : buf0;
-        C *gout;
-        if (!MULTI) {
-            const C *R;
-            Lay lr;
-            if (pow2ny && kx0 != 0) {
-                // convection, power-of-two columns: forward passes, the last
-                // pass fused with the multiply and its adjoint, adjoint passes
-                // (splitting the tile's columns between two named-barrier
-                // halves measured slower: 228 -> 247 us at 1024^2, from the
-                // bank conflicts of half-width tiles)
-                const ColMult<real> m{(real)gd.c[0][0][0], (real)gd.c[0][0][1], (real)gd.c[0][0][2],
-                                      (real)gd.c[0][0][3], (real)gd.c[0][0][4], scale, kxs, kys, kx0};
-                const int w = pp_conv_p2<true>(in0, lt, wk0, lw, ny, TW, Tc, m, tid, NT, GroupSync{0, NT}, tc);
-                R = w ? wk0 : in0;
-                lr = w ? lw : lt;
-            } else {
-                // convection (the tile holding k_x = 0 pairs (k_y, -k_y) of the
-                // packed DC / row-Nyquist column; other lengths): forward,
-                // multiply in place, inverse
-                const int w1 = pp_fft_any<-1, true, 0, 1>(in0, lt, wk0, lw, ny, TW, Wc, Tc, tid, NT, 4, tc);
-                C *X = w1 ? wk0 : in0;
-                C *Y = w1 ? in0 : wk0;
-                const Lay lx = w1 ? lw : lt, ly = w1 ? lt : lw;
-                col_multiply<real>(X, lx, X, lx, X, lx, gd, 0, kxs, kys, kx0, TW, lgTW, ny, h, scale, NT);
-                __syncthreads();
-                const int w2 = w1 ? pp_fft_any<+1, true, 1, 0>(X, lx, Y, ly, ny, TW, Wc, Tc, tid, NT, 4, tc)
-                                  : pp_fft_any<+1, true, 0, 1>(X, lx, Y, ly, ny, TW, Wc, Tc, tid, NT, 4, tc);
-                R = w2 ? Y : X;
-                lr = w2 ? ly : lx;
-            }
-            gout = spec_r + (size_t)gd.out_slot[0] * slot + kx0;
-            if (gd.add_slot >= 0) {   // plus the term the row kernel formed
-                // (4 loads before their stores: gout may alias ad, so a load
-                // after a store could not be issued ahead of it)
-                const C *ad = spec_r + (size_t)gd.add_slot * slot + kx0;
-                for (int i0 = tid; i0 < tile; i0 += 4 * NT) {
-                    C a[4];
+        const C *R;
+        Lay lr;
+        if (pow2ny && kx0 != 0) {
+            // convection, power-of-two columns: forward passes, the last
+            // pass fused with the multiply and its adjoint, adjoint passes
+            // (splitting the tile's columns between two named-barrier
+            // halves measured slower: 228 -> 247 us at 1024^2, from the
+            // bank conflicts of half-width tiles)
+            const ColMult<real> m{(real)gd.c[0][0][0], (real)gd.c[0][0][1], (real)gd.c[0][0][2],
+                                  (real)gd.c[0][0][3], (real)gd.c[0][0][4], scale, kxs, kys, kx0};
+            const int w = pp_conv_p2<true>(in0, lt, wk0, lw, ny, TW, Tc, m, tid, NT, GroupSync{0, NT}, tc);
+            R = w ? wk0 : in0;
+            lr = w ? lw : lt;
+        } else {
+            // convection (the tile holding k_x = 0 pairs (k_y, -k_y) of the
+            // packed DC / row-Nyquist column; other lengths): forward,
+            // multiply in place, inverse
+            const int w1 = pp_fft_any<-1, true, 0, 1>(in0, lt, wk0, lw, ny, TW, Wc, Tc, tid, NT, 4, tc);
+            C *X = w1 ? wk0 : in0;
+            C *Y = w1 ? in0 : wk0;
+            const Lay lx = w1 ? lw : lt, ly = w1 ? lt : lw;
+            col_multiply<real>(X, lx, X, lx, X, lx, gd, 0, kxs, kys, kx0, TW, lgTW, ny, h, scale, NT);
+            __syncthreads();
+            const int w2 = w1 ? pp_fft_any<+1, true, 1, 0>(X, lx, Y, ly, ny, TW, Wc, Tc, tid, NT, 4, tc)
+                              : pp_fft_any<+1, true, 0, 1>(X, lx, Y, ly, ny, TW, Wc, Tc, tid, NT, 4, tc);
+            R = w2 ? Y : X;
+            lr = w2 ? ly : lx;
+        }
+        C *gout = spec_r + (size_t)gd.out_slot[0] * slot + kx0;
+        if (gd.add_slot >= 0) {   // plus the term the row kernel formed
+            // (4 loads before their stores: gout may alias ad, so a load
+            // after a store could not be issued ahead of it)
+            const C *ad = spec_r + (size_t)gd.add_slot * slot + kx0;
+            for (int i0 = tid; i0 < tile; i0 += 4 * NT) {
+                C a[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int idx = i0 + u * NT, e = idx >> lgTW, c = idx & (TW - 1);
-                        if (idx < tile) a[u] = ad[(size_t)e * h + c];
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int idx = i0 + u * NT, e = idx >> lgTW, c = idx & (TW - 1);
-                        if (idx < tile) gout[(size_t)e * h + c] = cadd(R[lr(c, e)], a[u]);
-                    }
+                for (int u = 0; u < 4; ++u) {
+                    const int idx = i0 + u * NT, e = idx >> lgTW, c = idx & (TW - 1);
+                    if (idx < tile) a[u] = ad[(size_t)e * h + c];
                 }
-            } else {
-                for (int idx = tid; idx < tile; idx += NT) {
-                    const int e = idx >> lgTW, c = idx & (TW - 1);
-                    gout[(size_t)e * h + c] = R[lr(c, e)];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int idx = i0 + u * NT, e = idx >> lgTW, c = idx & (TW - 1);
+                    if (idx < tile) gout[(size_t)e * h + c] = cadd(R[lr(c, e)], a[u]);
                 }
             }
         } else {
-            C *in1 = in0 + tstr;
-            if (pow2ny && kx0 != 0 && (ilog2(ny) & 3) != 0) {   // last pass radix <= 8
-                // inputs: forward passes 1 .. L-1 (X0 in {in0, wk0}, X1 in
-                // {in1, wk1}); each output: one fused pass into the free pair
-                // of buffers, then the adjoint passes L-1 .. 1
-                const GroupSync bs{0, NT};
-                const int wx = pp_fwd_head_p2<true>(in0, lt, wk0, lw, ny, TW, Tc, tid, NT, bs, tc);
-                if (gd.nin > 1) pp_fwd_head_p2<true>(in1, lt, wk1, lw, ny, TW, Tc, tid, NT, bs, tc);
-                const C *X0 = wx ? wk0 : in0, *X1 = wx ? wk1 : in1;
-                const Lay lx = wx ? lw : lt;
-                C *Q0 = wx ? in0 : wk0, *Q1 = wx ? in1 : wk1;
-                const Lay lq = wx ? lt : lw;
-                for (int o = 0; o < gd.nout; ++o) {
-                    GroupMult<real> m;
-                    for (int j = 0; j < 5; ++j) {
-                        m.p[j] = (real)gd.c[o][0][j];
-                        m.q[j] = (real)gd.c[o][1][j];
-                    }
-                    m.scale = scale;
-                    m.two = gd.nterm[o] > 1;
-                    m.in0 = gd.term_in[o][0];
-                    m.in1 = gd.term_in[o][1];
-                    m.kxs = kxs;
-                    m.kys = kys;
-                    m.kx0 = kx0;
-                    pp_out_fused_p2<true>(X0, X1, lx, gd.nin > 1, Q0, lq, ny, TW, Tc, m, tid, NT, bs);
-                    const int wq = pp_adj_tail_p2<true>(Q0, Q1, lq, ny, TW, Tc, tid, NT, bs, tc);
-                    const C *R = wq ? Q1 : Q0;
-                    gout = spec_r + (size_t)gd.out_slot[o] * slot + kx0;
-                    for (int idx = tid; idx < tile; idx += NT) {
-                        const int e = idx >> lgTW, c = idx & (TW - 1);
-                        gout[(size_t)e * h + c] = R[lq(c, e)];
-                    }
-                    __syncthreads();
-                }
-            } else {
-            // X0 in {in0, wk0}, X1 in {in1, wk1}; outputs ping-pong between
-            // the two buffers left free
-            const int w0 = pp_fft_any<-1, true, 0, 1>(in0, lt, wk0, lw, ny, TW, Wc, Tc, tid, NT, 4, tc);
-            C *X0 = w0 ? wk0 : in0;
-            C *F0 = w0 ? in0 : wk0;
-            const Lay lx0 = w0 ? lw : lt, lf0 = w0 ? lt : lw;
-            C *X1 = in1, *F1 = wk1;
-            Lay lx1 = lt, lf1 = lw;
-            if (gd.nin > 1) {
-                const int w1 = pp_fft_any<-1, true, 0, 1>(in1, lt, wk1, lw, ny, TW, Wc, Tc, tid, NT, 4, tc);
-                X1 = w1 ? wk1 : in1;
-                F1 = w1 ? in1 : wk1;
-                lx1 = w1 ? lw : lt;
-                lf1 = w1 ? lt : lw;
-            }
-            for (int o = 0; o < gd.nout; ++o) {
-                col_multiply<real>(F0, lf0, X0, lx0, X1, lx1, gd, o, kxs, kys, kx0, TW, lgTW, ny, h, scale, NT);
-                __syncthreads();
-                int w2;
-                if (lf0.pad) w2 = lf1.pad ? pp_fft_any<+1, true, 1, 1>(F0, lf0, F1, lf1, ny, TW, Wc, Tc, tid, NT, 4, tc)
-                                          : pp_fft_any<+1, true, 1, 0>(F0, lf0, F1, lf1, ny, TW, Wc, Tc, tid, NT, 4, tc);
-                else w2 = lf1.pad ? pp_fft_any<+1, true, 0, 1>(F0, lf0, F1, lf1, ny, TW, Wc, Tc, tid, NT, 4, tc)
-                                  : pp_fft_any<+1, true, 0, 0>(F0, lf0, F1, lf1, ny, TW, Wc, Tc, tid, NT, 4, tc);
-                const C *R = w2 ? F1 : F0;
-                const Lay lr = w2 ? lf1 : lf0;
-                gout = spec_r + (size_t)gd.out_slot[o] * slot + kx0;
-                for (int idx = tid; idx < tile; idx += NT) {
-                    const int e = idx >> lgTW, c = idx & (TW - 1);
-                    gout[(size_t)e * h + c] = R[lr(c, e)];
-                }
-                __syncthreads();
-            }
+            for (int idx = tid; idx < tile; idx += NT) {
+                const int e = idx >> lgTW, c = idx & (TW - 1);
+                gout[(size_t)e * h + c] = R[lr(c, e)];
             }
         }
         fence_proxy_async();
@@ -702,8 +610,8 @@ constexpr int NT3 = 256;
 // The level-1 derivatives K3 forms in the row spectrum (k3_src_slot), at
 // bin k of the one-sided rows of d (row o at d + o rs; bin 0 carries DC and
 // row-Nyquist, both with k_x = 0): row D_RX holds rho^, D_UXX u_x^, D_UYX
-// u_y^, D_TX T^, D_PIX Pi^, D_GX g^ as loaded; D_LAP holds d_yy rho and
-// D_UYY d_y u_y from the column pass.  ax = k_x of bin k, sx = 1 / nx.
+// u_y^, D_TX T^, D_PIX Pi^, D_GX g^ as loaded; D_LAP holds d_yy rho, D_UYY
+// d_y u_y, D_UXY d_y u_x and D_DIVY d_yy u_y from the column pass.  ax = k_x of bin k, sx = 1 / nx.
 template <typename real, typename C>
 __device__ __forceinline__ void k3_form_x(C *d, int rs, int k, real ax, real sx) {
     const real m = ax * sx;
@@ -717,6 +625,7 @@ __device__ __forceinline__ void k3_form_x(C *d, int rs, int k, real ax, real sx)
     d[D_UXX * rs + k] = uxx;                          // d_x u_x
     d[D_DIVX * rs + k] = imul(ax, cadd(uxx, d[D_UYY * rs + k]));   // d_x (d_x u_x + d_y u_y)
     d[D_UYX * rs + k] = imul(m, d[D_UYX * rs + k]);   // d_x u_y
+    d[D_DIVY * rs + k] = cadd(d[D_DIVY * rs + k], imul(ax, d[D_UXY * rs + k]));   // d_yy u_y + d_x (d_y u_x)
     d[D_TX * rs + k] = imul(m, d[D_TX * rs + k]);
     d[D_PIX * rs + k] = imul(m, d[D_PIX * rs + k]);
     d[D_GX * rs + k] = imul(m, d[D_GX * rs + k]);
