@@ -46,59 +46,15 @@
 #include <string>
 #include <vector>
 
+#include "col_kernels.h"
 #include "engine.h"
 #include "fft_device.cuh"
+#include "row_kernels.h"
+#include "stage_layout.cuh"
 
 namespace fftlb {
 
-constexpr int Q = 33;
-constexpr int NMOV = 32;
-constexpr int NT = 256;          // threads per block of every row / column kernel
-
-// spectrum slots
-constexpr int SLOT_RHO = 32, SLOT_UX = 33, SLOT_UY = 34, SLOT_T = 35, SLOT_PI = 36, SLOT_G = 37;
-constexpr int SLOT_D1 = 38;      // 15 level-1 derivative outputs
-constexpr int ND1 = 15;
-constexpr int SLOT_L2 = 53;      // Lxx, Lxy, Lyy, Phx, Phy; outputs in 53, 55, 56
-constexpr int NSLOT = 58;
-enum { D_RX, D_RY, D_LAP, D_UXX, D_UXY, D_UYX, D_UYY, D_DIVX, D_DIVY, D_TX, D_TY, D_PIX, D_PIY, D_GX, D_GY };
-
-// The windowed derivative multipliers are separable: D_x = i k_x (a
-// function of k_x alone), D_y = i k_y, and the second derivatives are their
-// products (Eqs. K1-K4 with the real part taken after each derivative, so
-// that the Nyquist bins carry zero).  A derivative whose multiplier depends
-// on k_x alone needs no column transform: in the row-transformed slot it is
-// the pointwise product i k_x X / nx (the 1 / nx that the column pass would
-// leave).  So the column pass forms only derivatives in k_y alone, each of
-// one input: d_y of rho, u_x, u_y, T, Pi, g and d_yy of rho, u_y; and the
-// row kernel K3 forms the rest from the row spectra of rho, u_x, u_y, T,
-// Pi, g and of those before its inverse rows:
-//   rho_x = i k_x rho^ / nx, lap rho = d_yy rho - k_x^2 rho^ / nx,
-//   u_xx = i k_x u_x^ / nx, u_yx = i k_x u_y^ / nx,
-//   d_x(div u) = i k_x (u_xx + u_yy), d_y(div u) = d_yy u_y + i k_x (d_y u_x),
-//   T_x, Pi_x, g_x = i k_x (.)^ / nx.
-// With one input and one output each, the level-1 passes are 8 more groups
-// of the convection launch.  A launch of their own for rho (two outputs) and
-// u (two inputs, two outputs) transformed two inputs fewer, but with three
-// tiles and 219 KB a block it left most SMs with one job's latency: 22.5 us
-// at 1024^2 in fp32, against the 9 us these jobs add to the convection
-// launch (69.8 -> 78.7 us); 48 and 15.9 us against none on 64^2 fp64 and fp32.
-// Level 2 in the same way: d_x Lambda_xx + d_y Lambda_xy is the column
-// pass of d_y Lambda_xy plus i k_x Lambda_xx^ / nx, formed by K3 (add_slot).
-// k3_src_slot(o): the slot K3 loads into its row o (-1: formed in K3).
-__host__ __device__ constexpr int k3_src_slot(int o) {
-    return o == D_RX ? SLOT_RHO : o == D_UXX ? SLOT_UX : o == D_UYX ? SLOT_UY : o == D_TX ? SLOT_T
-         : o == D_PIX ? SLOT_PI : o == D_GX ? SLOT_G : o == D_DIVX ? -1 : SLOT_D1 + o;
-}
-// K3's level-2 outputs: row r of Lambda_xx, Lambda_xy, Lambda_yy, Phi_x,
-// Phi_y goes to slot k3_raw_slot(r) as it is and to slot k3_mul_slot(r)
-// times i k_x / nx (-1: not written)
-__host__ __device__ constexpr int k3_raw_slot(int r) {
-    return r == 1 ? SLOT_L2 + 1 : r == 2 ? SLOT_L2 + 2 : r == 4 ? SLOT_L2 + 4 : -1;
-}
-__host__ __device__ constexpr int k3_mul_slot(int r) {
-    return r == 0 ? SLOT_L2 + 0 : r == 1 ? SLOT_D1 + D_DIVX : r == 3 ? SLOT_L2 + 3 : -1;
-}
+constexpr int NT = 256;          // threads per block of the auxiliary row / column kernels
 
 // velocity set (Eq. 1) and weight-polynomial coefficients (Eq. 4); each
 // translation unit holds its own copy, shared by all live engines of that
@@ -142,23 +98,6 @@ template <typename real> struct KP {
     real dx, dt, tau, a, b, K, H, q, zeta, scale;
     real scale_x;   // 1 / nx: the inverse normalisation a column pass leaves to the rows (scale * ny)
     const uint4 *tc16;
-};
-
-// One column-pass group: up to 2 input spectra and 6 outputs; every output
-// is a sum of up to 2 terms M(kx, ky) * input, with
-// M = i (c0 k_x + c1 k_y) + (c2 k_x^2 + c3 k_y^2 + c4 k_x k_y).
-// add_slot >= 0 (groups of one input and one output, the convection kernels
-// only): the column inverse of that output is added to slot add_slot's
-// values at the same positions (a term that needs no column transform,
-// formed by the row kernel that wrote add_slot).
-struct GroupDesc {
-    int nin, nout;
-    int in_slot[2];
-    int out_slot[6];
-    int nterm[6];
-    int term_in[6][2];
-    double c[6][2][5];
-    int add_slot;
 };
 
 // ---------------------------------------------------------------------------
@@ -847,6 +786,14 @@ class EngineT : public Engine {
     size_t smemcw_ = 0;
     int gridcw_ = 1, nbufcw_ = 1, ntcw_ = 256;
     CUtensorMap tmap_convw_{};
+    // row and column kernels of kernels_row.cuh / kernels_col.cuh, the
+    // argument blocks of their launches, and their tables
+    bool rowk_ = false, colk_ = false;
+    RowSet rs_;
+    ColSet cs_;
+    RowArgs<real> ra_{};
+    ColArgs<real> ca_conv_{}, ca_l2_{}, ca_inv_{};
+    C *Wh_ = nullptr, *Tcr_ = nullptr, *Wcp_ = nullptr;
     // gradient kernels (k_grad_*): column tile width and shared memory
     int TWg_ = 0;
     size_t smem_gr_ = 0, smem_gc_ = 0;
@@ -1032,6 +979,16 @@ class EngineT : public Engine {
         FFTLB_CU(cudaMemcpyToSymbol(c_Fkl, Fkl, sizeof Fkl));
         memcpy(vx_, vx, sizeof vx);
         memcpy(vy_, vy, sizeof vy);
+        for (int j = 0; j < Q; ++j) {
+            ra_.vx[j] = (real)vx[j];
+            ra_.vy[j] = (real)vy[j];
+            ra_.v2[j] = (real)v2[j];
+        }
+        for (int k = 0; k < 4; ++k)
+            for (int j = 0; j < 4; ++j) {
+                ra_.Fk[k][j] = (real)Fk[k][j];
+                ra_.Fkl[k][j] = (real)(Fk[k][j] - (double)(real)Fk[k][j]);
+            }
         return Status::ok();
     }
     double vx_[Q], vy_[Q];
@@ -1092,6 +1049,29 @@ class EngineT : public Engine {
         }
     }
 
+    // a[k1 P + l] = b[l E + k1] = exp(-2 pi i l k1 / n), n = E P
+    static void stage1_twiddles(std::vector<C> &a, std::vector<C> &b, int n, int P) {
+        const long double pi = 3.141592653589793238462643383279502884L;
+        const int E = n / P;
+        a.resize(n);
+        b.resize(n);
+        for (int k1 = 0; k1 < E; ++k1)
+            for (int l = 0; l < P; ++l) {
+                const long double t = 2.0L * pi * (long double)(l * k1) / (long double)n;
+                C w;
+                w.x = (real)cosl(t);
+                w.y = (real)(-sinl(t));
+                a[(size_t)k1 * P + l] = w;
+                b[(size_t)l * E + k1] = w;
+            }
+    }
+    Status upload_table(C **dst, const std::vector<C> &t) {
+        Status st = dalloc(dst, t.size());
+        if (!st.good()) return st;
+        FFTLB_CU(cudaMemcpy(*dst, t.data(), t.size() * sizeof(C), cudaMemcpyHostToDevice));
+        return Status::ok();
+    }
+
     // per-pass twiddle tables of the power-of-two passes (see
     // pass_twiddle_len): T[t Ns + k] = exp(-2 pi i t k / (Ns R))
     static void pass_twiddles(std::vector<C> &T, int n, int maxlr) {
@@ -1146,19 +1126,26 @@ class EngineT : public Engine {
         if (ntr_) FFTLB_CU(cudaMemcpy(Tr_, tr.data(), tr.size() * sizeof(C), cudaMemcpyHostToDevice));
         if (ntr8_) FFTLB_CU(cudaMemcpy(Tr8_, tr8.data(), tr8.size() * sizeof(C), cudaMemcpyHostToDevice));
         if (ntc_) FFTLB_CU(cudaMemcpy(Tc_, tc.data(), tc.size() * sizeof(C), cudaMemcpyHostToDevice));
-        if (wr_ok_ && (h_ == 512 || h_ == 256 || h_ == 128)) {
+        if (own_len(h_) && row_p(h_) > 0) {
             // tw[k1 P + l] = exp(-2 pi i l k1 / h) for the row configuration of h
-            const int P = h_ == 512 ? 32 : h_ == 256 ? 16 : 8, E = h_ / P;
-            std::vector<C> t1((size_t)h_);
-            const long double pi = 3.141592653589793238462643383279502884L;
-            for (int k1 = 0; k1 < E; ++k1)
-                for (int l = 0; l < P; ++l) {
-                    const long double a = 2.0L * pi * (long double)(l * k1) / (long double)h_;
-                    t1[(size_t)k1 * P + l].x = (real)cosl(a);
-                    t1[(size_t)k1 * P + l].y = (real)(-sinl(a));
-                }
-            if (!(st = dalloc(&Tw1_, t1.size())).good()) return st;
-            FFTLB_CU(cudaMemcpy(Tw1_, t1.data(), t1.size() * sizeof(C), cudaMemcpyHostToDevice));
+            std::vector<C> t1, t2;
+            stage1_twiddles(t1, t2, h_, row_p(h_));
+            if (!(st = upload_table(&Tw1_, t1)).good()) return st;
+            std::vector<C> wh(wp.begin(), wp.begin() + h_ / 2 + 1);
+            for (auto &w : wh) {
+                w.x *= real(0.5);
+                w.y *= real(0.5);
+            }
+            if (!(st = upload_table(&Wh_, wh)).good()) return st;
+        }
+        if (own_len(ny_) && col_p((int)sizeof(real), ny_) > 0) {
+            const int P = col_p((int)sizeof(real), ny_);
+            std::vector<C> t1, t2, w;
+            stage1_twiddles(t1, t2, ny_, P);
+            t1.insert(t1.end(), t2.begin(), t2.end());
+            if (!(st = upload_table(&Tcr_, t1)).good()) return st;
+            twiddles(w, P, P);
+            if (!(st = upload_table(&Wcp_, w)).good()) return st;
         }
         if (wr_ok_ && (ny_ == 1024 || ny_ == 512 || ny_ == 256 || ny_ == 128)) {
             // twc[k1 P + l] = exp(-2 pi i l k1 / ny) for the column configuration of
@@ -1255,6 +1242,23 @@ class EngineT : public Engine {
         }
     }
 
+    void col_args(ColArgs<real> &a, const std::vector<GroupDesc> &gs, int first, int count) {
+        a.h = h_;
+        a.ngroups = count;
+        a.spec = specb_;
+        a.kx = kxt_;
+        a.ky = kyt_;
+        a.tw = Tcr_;
+        a.twt = Tcr_ + ny_;
+        a.wp = Wcp_;
+        a.scale = (real)(1.0 / ((double)nx_ * (double)ny_));
+        for (int i = 0; i < count && i < kMaxColJobs; ++i) {
+            const GroupDesc &g = gs[first + i];
+            a.g[i] = ColGroup<real>{g.in_slot[0], g.out_slot[0], g.add_slot, (real)g.c[0][0][0], (real)g.c[0][0][1],
+                                    (real)g.c[0][0][3]};
+        }
+    }
+
     Status build_groups() {
         static const double DX[5] = {1, 0, 0, 0, 0}, DY[5] = {0, 1, 0, 0, 0};
         static const double DYY[5] = {0, 0, 0, -1, 0};
@@ -1317,6 +1321,9 @@ class EngineT : public Engine {
             add_out(g, 2, 1, 0, DY);
             gs.push_back(g);
         }
+        col_args(ca_conv_, gs, conv_groups_, nconvl_);
+        col_args(ca_l2_, gs, l2_groups_, 3);
+        col_args(ca_inv_, gs, inv_groups_, 1);
         Status st = dalloc(&groups_, gs.size());
         if (!st.good()) return st;
         FFTLB_CU(cudaMemcpy(groups_, gs.data(), gs.size() * sizeof(GroupDesc), cudaMemcpyHostToDevice));
@@ -1608,7 +1615,104 @@ class EngineT : public Engine {
         st = occ_k5(smem5_, &nb);
         if (!st.good()) return st;
         grid5_ = std::min(B_ * ny_, std::max(1, nb) * nsm_);
-        return configure_wr();
+        if (!(st = configure_wr()).good()) return st;
+        return configure_rowcol();
+    }
+
+    // whether transforms of n values may take the kernels of kernels_row.cuh /
+    // kernels_col.cuh: the split-BF16 mode keeps its own passes where they have
+    // a radix-16 first pass, and is the plain fp32 path elsewhere
+    static bool own_len(int n) { return !split_ || !is_pow2(n) || n < 16; }
+
+    // the kernels of kernels_row.cuh / kernels_col.cuh where they apply
+    Status configure_rowcol() {
+        if constexpr (sizeof(real) == 4) {
+            rs_ = row_set_f32_p2(h_);
+            if (!rs_.k1) rs_ = row_set_f32_r3(h_);
+            cs_ = col_set_f32(ny_);
+        } else {
+            rs_ = row_set_f64_p2(h_);
+            if (!rs_.k1) rs_ = row_set_f64_r3(h_);
+            cs_ = col_set_f64(ny_);
+        }
+        if (!own_len(h_)) rs_ = RowSet();
+        if (!own_len(ny_)) cs_ = ColSet();
+        if (rs_.k1 && Tw1_ && std::max({rs_.smem1, rs_.smem3, rs_.smem5}) <= budget_) {
+            const void *ks[3] = {rs_.k1, rs_.k3, rs_.k5};
+            for (const void *k : ks)
+                FFTLB_CU(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget_));
+            ra_.ny = ny_;
+            ra_.nrun = B_;
+            ra_.dt = kp_.dt;
+            ra_.itau = real(1) / kp_.tau;
+            ra_.a = kp_.a;
+            ra_.b = kp_.b;
+            ra_.K = kp_.K;
+            ra_.H = kp_.H;
+            ra_.q = kp_.q;
+            ra_.zeta = kp_.zeta;
+            ra_.scale_x = kp_.scale_x;
+            ra_.fields = fieldsb_;
+            ra_.aux = auxb_;
+            ra_.spec = specb_;
+            ra_.tw = Tw1_;
+            ra_.wp = Wp_;
+            ra_.wh = Wh_;
+            ra_.kx = kxt_;
+            ra_.err = err_;
+            // The persistent fp32 rows (k*_wr) keep their place where every
+            // SM has at least two rows: their prefetch then pays (1024^2:
+            // K1, K3, K5 72, 40, 123 us against 130, 102, 159), while with
+            // fewer rows most of the chip idles (1024x64: 19, 12, 25
+            // against 14, 12, 15; 512x4: 12, 10, 15 against 10, 10, 10).
+            // Everything else is faster here at every size: 64^2 fp32 31,
+            // 15, 27 -> 9, 10, 10; 384^2 fp32 74, 37, 83 -> 24, 25, 28; 64^2
+            // fp64 88, 35, 75 -> 31, 31, 30; 512^2 fp64 641, 263, 761 -> 488,
+            // 320, 614; 2048^2 fp32 716, 479, 1186 -> 590, 309, 620.
+            rowk_ = !(k1wr_ && k3wr_ && k5wr_ && (long)B_ * ny_ >= 2L * nsm_);
+        }
+        if (cs_.k && (cs_.tw == 0 || h_ % cs_.tw == 0) && cs_.smem <= budget_) {
+            if (cs_.tw) FFTLB_CU(cudaFuncSetAttribute(cs_.k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget_));
+            // kcol_wr keeps the lengths 512 and 1024, where its prefetch and
+            // (512) its wider tiles pay: convection and level 2 at 1024^2 79
+            // and 19 us against 90 and 28, at 512^2 25 and 12 against 25 and
+            // 21; at 256^2 12 and 10 against 10 and 8 here.
+            colk_ = !(colwr_ && ny_ >= 512);
+        }
+        return Status::ok();
+    }
+
+    // a row kernel over every row of every run, cs blocks (one cluster) a row
+    Status launch_row(const char *name, const void *k, size_t smem) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(B_ * ny_ * rs_.cs));
+        cfg.blockDim = dim3((unsigned)rs_.nt);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream_;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)rs_.cs;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        void *args[1] = {&ra_};
+        const cudaError_t e = cudaLaunchKernelExC(&cfg, k, args);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return Status::err(FFTLB_ERR_CUDA, std::string(name) + ": " + cudaGetErrorString(e));
+        }
+        return Status::ok();
+    }
+    // one launch of column jobs: every group, tile and run
+    Status launch_cols(ColArgs<real> &a, int nrun) {
+        const unsigned jobs = cs_.tw ? (unsigned)(a.ngroups * (h_ / cs_.tw)) : (unsigned)((a.ngroups * h_ + 127) / 128);
+        void *args[1] = {&a};
+        const cudaError_t e = cudaLaunchKernel(cs_.k, dim3(jobs, (unsigned)nrun), dim3((unsigned)cs_.nt), args, cs_.smem, stream_);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return Status::err(FFTLB_ERR_CUDA, std::string("column kernel: ") + cudaGetErrorString(e));
+        }
+        return Status::ok();
     }
 
     // the warp-resident final row kernel where it applies (fp32, nx = 512 or
@@ -1907,6 +2011,13 @@ class EngineT : public Engine {
     // column pass of one-input groups; level2: the level-2 launch (its own
     // tile width on the pipelined kernels)
     Status launch_col(int first, int count, bool level2) {
+        if (colk_) {
+            if (first == inv_groups_) {   // the selected run alone
+                ca_inv_.spec = spec_;
+                return launch_cols(ca_inv_, 1);
+            }
+            return launch_cols(level2 ? ca_l2_ : ca_conv_, B_);
+        }
         if constexpr (wr_ok_) {
             if (colwr_) {
                 if (count > kMaxColGroups) return Status::err(FFTLB_ERR_ARG, "too many column groups in one launch");
@@ -1939,8 +2050,18 @@ class EngineT : public Engine {
         }
         if (!(st = prof_begin(KK_ROW_FORWARD)).good()) return st;
         bool k1done = false;
+        if (rowk_) {
+            ra_.f = cur;
+            ra_.fcur = cur;
+            ra_.fbase = base;
+            ra_.fout = out;
+            ra_.alpha = alpha;
+            ra_.beta = beta;
+            if (!(st = launch_row("k1_row", rs_.k1, rs_.smem1)).good()) return st;
+            k1done = true;
+        }
         if constexpr (wr_ok_) {
-            if (k1wr_) {
+            if (!k1done && k1wr_) {
                 const int nt = nt_k1wr_host(h_);
                 auto *kern = h_ == 512 ? k1_wr<512> : h_ == 256 ? k1_wr<256> : k1_wr<128>;
                 if (!(st = launch_pdl("k1_wr", kern, grid1w_, nt, smem1w_, cur, specb_, fieldsb_,
@@ -1967,8 +2088,12 @@ class EngineT : public Engine {
         if (!(st = prof_end()).good()) return st;
         if (!(st = prof_begin(KK_ROW_LEVEL1)).good()) return st;
         bool k3done = false;
+        if (rowk_) {
+            if (!(st = launch_row("k3_row", rs_.k3, rs_.smem3)).good()) return st;
+            k3done = true;
+        }
         if constexpr (wr_ok_) {
-            if (k3wr_) {
+            if (!k3done && k3wr_) {
                 const int nt = nt_k3wr_host(h_);
                 auto *kern = h_ == 512 ? k3_wr<512> : h_ == 256 ? k3_wr<256> : k3_wr<128>;
                 if (!(st = launch_pdl("k3_wr", kern, grid3w_, nt, smem3w_, specb_, (const float *)fieldsb_, auxb_,
@@ -1988,6 +2113,10 @@ class EngineT : public Engine {
         if (!(st = launch_col(l2_groups_, 3, true)).good()) return st;
         if (!(st = prof_end()).good()) return st;
         if (!(st = prof_begin(KK_ROW_FINAL)).good()) return st;
+        if (rowk_) {
+            if (!(st = launch_row("k5_row", rs_.k5, rs_.smem5)).good()) return st;
+            return prof_end();
+        }
         if constexpr (wr_ok_) {
             if (k5wr_) {
                 const int nt = nt_k5wr_host(h_);

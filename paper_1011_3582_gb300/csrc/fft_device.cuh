@@ -15,11 +15,9 @@
 
 #include <type_traits>
 
-namespace fftlb {
+#include "fft_types.h"
 
-template <typename real> struct cplx_of;
-template <> struct cplx_of<double> { using type = double2; };
-template <> struct cplx_of<float> { using type = float2; };
+namespace fftlb {
 
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return C{a.x + b.x, a.y + b.y}; }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { return C{a.x - b.x, a.y - b.y}; }

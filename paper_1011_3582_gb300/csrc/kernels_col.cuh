@@ -1,0 +1,202 @@
+// Column passes without staged tiles, for the lengths, precisions and grid
+// sizes the persistent kernels (kcol_wr, kcol_pipe) do not serve well:
+//   kcol_reg   lengths 16 .. 2048 = 2^p and 24 .. 1536 = 3 2^p: one job (a
+//              tile of TW spectrum columns of one group) per block;
+//   kcol_line  lengths 4, 6, 8, 12: one column per thread, in registers.
+// Every group has one input and one output (which may be the same slot):
+// forward transform, multiplier i (c0 k_x + c1 k_y) or c3 k_y^2, inverse, plus
+// the values of the addend slot where the group has one.
+//
+// A column of NY = E P values is transformed by P threads as in kcol_wr, but
+// thread (c, l) loads its x[l + P t] straight from global memory into
+// registers: the tile passes through shared memory twice (the transpose and
+// its inverse) instead of three times, and a block needs one tile of shared
+// memory and no tables of its own, so that many small blocks fit an SM and
+// their loads overlap each other's transforms.  The packed column 0 of the
+// tile at k_x = 0 needs no pairing of (k_y, -k_y) (see kcol_wr).
+#pragma once
+
+#include "col_kernels.h"
+#include "fft_small.cuh"
+#include "stage_layout.cuh"
+
+namespace fftlb {
+
+namespace ck {
+
+template <typename real, int NY> struct Col {
+    using C = typename cplx_of<real>::type;
+    static constexpr int P = col_p(sizeof(real), NY), E = NY / P;
+    static constexpr bool PAIR = col_pair(sizeof(real), NY);   // stage 2: two threads per P-point DFT
+    static constexpr int PH = PAIR ? P / 2 : P;
+    static constexpr int TW = col_tw(sizeof(real), NY), NT = TW * P;
+    // rows of one memory phase (16 8-byte or 8 16-byte values) in different banks
+    static constexpr int PHASE = 128 / (int)sizeof(C), SW = TW < PHASE ? PHASE / TW - 1 : 0;
+};
+
+// position of stage-1 output (l, k1) of column c
+template <typename real, int NY> __device__ __forceinline__ int cp(int c, int l, int k1) {
+    using G = Col<real, NY>;
+    return (k1 * G::P + (l ^ (k1 & G::SW))) * G::TW + c;
+}
+
+template <typename real, int NY> constexpr int col_minb() {
+    using G = Col<real, NY>;
+    // 128 registers a thread where a thread holds up to 32 fp32 or 16 fp64
+    // complex values, 255 beyond
+    return sizeof(real) == 4 || (G::E <= 16 && G::PH <= 16) ? (512 / G::NT > 16 ? 16 : 512 / G::NT) : (256 / G::NT > 16 ? 16 : 256 / G::NT);
+}
+
+template <typename real, int NY>
+__global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_reg(const __grid_constant__ ColArgs<real> A) {
+    using G = Col<real, NY>;
+    using C = typename G::C;
+    constexpr int E = G::E, P = G::P, PH = G::PH, TW = G::TW;
+    extern __shared__ __align__(128) unsigned char col_smem_raw[];
+    C *T = reinterpret_cast<C *>(col_smem_raw);   // [NY][TW]
+    const int h = A.h, tid = threadIdx.x, c = tid % TW, jl = tid / TW;
+    const int ntiles = h / TW;
+    const int job = (int)blockIdx.x, g = job / ntiles, t = job - g * ntiles;   // (grid.y: run)
+    const size_t slot = (size_t)NY * h;
+    const ColGroup<real> &gr = A.g[g];
+    C *spec = A.spec + (size_t)blockIdx.y * NSLOT * slot + t * TW + c;
+    const C *__restrict__ in = spec + (size_t)gr.in * slot;
+    C v[E];
+#pragma unroll
+    for (int q = 0; q < E; ++q) v[q] = in[(size_t)(jl + P * q) * h];
+    SmallDFT<E, -1, C>::run(v);
+#pragma unroll
+    for (int k1 = 1; k1 < E; ++k1) v[k1] = cmul(v[k1], __ldg(A.tw + k1 * P + jl));
+#pragma unroll
+    for (int k1 = 0; k1 < E; ++k1) T[cp<real, NY>(c, jl, k1)] = v[k1];
+    __syncthreads();
+    // stage 2: forward, multiplier, inverse, conjugate twiddles
+    const real mx = gr.c0 * __ldg(A.kx + t * TW + c), c1 = gr.c1, c3 = gr.c3, scale = A.scale;
+    auto mult = [&](int k, C u) {
+        const real ay = __ldg(A.ky + k);
+        if (c3 != real(0)) return cscale(u, c3 * ay * ay * scale);   // uniform over the block
+        const real m = (mx + c1 * ay) * scale;
+        return C{-m * u.y, m * u.x};
+    };
+    if constexpr (!G::PAIR) {
+#pragma unroll
+        for (int q = 0; q < (E + P - 1) / P; ++q) {
+            const int k1 = jl + P * q;
+            if (E % P == 0 || k1 < E) {
+                C u[P];
+#pragma unroll
+                for (int l = 0; l < P; ++l) u[l] = T[cp<real, NY>(c, l, k1)];
+                SmallDFT<P, -1, C>::run(u);
+#pragma unroll
+                for (int k2 = 0; k2 < P; ++k2) u[k2] = mult(k1 + E * k2, u[k2]);
+                SmallDFT<P, +1, C>::run(u);
+#pragma unroll
+                for (int l = 0; l < P; ++l)
+                    T[cp<real, NY>(c, l, k1)] = l == 0 ? u[l] : cmul(u[l], cconj(__ldg(A.twt + l * E + k1)));
+            }
+        }
+    } else if (jl < 2 * E) {   // (whole warps)
+        // threads (k1, gg) = (jl / 2, jl % 2) hold the even (gg = 0) and the
+        // odd l; X[k2' + PH s] = V0[k2'] + (-1)^s W_P^k2' V1[k2']: thread gg
+        // takes k2' in [PH gg / 2, PH (gg + 1) / 2), exchanging the other
+        // half with its neighbour, and the inverse goes the same way back
+        constexpr int HH = PH / 2;
+        const int k1 = jl >> 1, gg = jl & 1;
+        C u[PH];
+#pragma unroll
+        for (int m = 0; m < PH; ++m) u[m] = T[cp<real, NY>(c, gg + 2 * m, k1)];
+        SmallDFT<PH, -1, C>::run(u);
+#pragma unroll
+        for (int i = 0; i < HH; ++i) {
+            const C send = gg ? u[i] : u[HH + i];
+            C recv;
+            recv.x = __shfl_xor_sync(0xffffffffu, send.x, TW);
+            recv.y = __shfl_xor_sync(0xffffffffu, send.y, TW);
+            const C a = gg ? recv : u[i], b = gg ? u[HH + i] : recv;
+            const int k2 = HH * gg + i;
+            const C w = __ldg(A.wp + k2);   // W_P^k2
+            const C tb = cmul(b, w);
+            const C x0 = mult(k1 + E * k2, cadd(a, tb)), x1 = mult(k1 + E * (k2 + PH), csub(a, tb));
+            const C ai = cadd(x0, x1), bi = cmul(csub(x0, x1), cconj(w));
+            const C back = gg ? ai : bi;   // thread 0 keeps the even half (ai), thread 1 the odd (bi)
+            C got;
+            got.x = __shfl_xor_sync(0xffffffffu, back.x, TW);
+            got.y = __shfl_xor_sync(0xffffffffu, back.y, TW);
+            u[i] = gg ? got : ai;
+            u[HH + i] = gg ? bi : got;
+        }
+        SmallDFT<PH, +1, C>::run(u);
+#pragma unroll
+        for (int m = 0; m < PH; ++m) {
+            const int l = gg + 2 * m;
+            T[cp<real, NY>(c, l, k1)] = cmul(u[m], cconj(__ldg(A.twt + l * E + k1)));
+        }
+    }
+    __syncthreads();
+    C *out = spec + (size_t)gr.out * slot;
+#pragma unroll
+    for (int k1 = 0; k1 < E; ++k1) v[k1] = T[cp<real, NY>(c, jl, k1)];
+    SmallDFT<E, +1, C>::run(v);
+    if (gr.add >= 0) {   // plus the term the row kernel formed (all loads first: out may be the addend's slot)
+        const C *ad = spec + (size_t)gr.add * slot;
+#pragma unroll
+        for (int q = 0; q < E; ++q) v[q] = cadd(v[q], ad[(size_t)(jl + P * q) * h]);
+    }
+#pragma unroll
+    for (int q = 0; q < E; ++q) out[(size_t)(jl + P * q) * h] = v[q];
+}
+
+// One column of a short grid per thread.
+template <typename real, int NY>
+__global__ void __launch_bounds__(128) kcol_line(const __grid_constant__ ColArgs<real> A) {
+    using C = typename cplx_of<real>::type;
+    const int h = A.h, ncol = A.ngroups * h;
+    const int i = (int)blockIdx.x * 128 + (int)threadIdx.x;
+    if (i >= ncol) return;
+    const int g = i / h, kx = i - g * h;
+    const size_t slot = (size_t)NY * h;
+    const ColGroup<real> &gr = A.g[g];
+    C *spec = A.spec + (size_t)blockIdx.y * NSLOT * slot + kx;
+    const C *in = spec + (size_t)gr.in * slot;
+    C v[NY], a[NY];
+#pragma unroll
+    for (int y = 0; y < NY; ++y) {
+        v[y] = in[(size_t)y * h];
+        a[y] = gr.add >= 0 ? spec[(size_t)gr.add * slot + (size_t)y * h] : C{0, 0};
+    }
+    SmallDFT<NY, -1, C>::run(v);
+    const real mx = gr.c0 * __ldg(A.kx + kx);
+#pragma unroll
+    for (int k = 0; k < NY; ++k) {
+        const real ay = __ldg(A.ky + k);
+        if (gr.c3 != real(0)) {
+            v[k] = cscale(v[k], gr.c3 * ay * ay * A.scale);
+        } else {
+            const real m = (mx + gr.c1 * ay) * A.scale;
+            v[k] = C{-m * v[k].y, m * v[k].x};
+        }
+    }
+    SmallDFT<NY, +1, C>::run(v);
+    C *out = spec + (size_t)gr.out * slot;
+#pragma unroll
+    for (int y = 0; y < NY; ++y) out[(size_t)y * h] = gr.add >= 0 ? cadd(v[y], a[y]) : v[y];
+}
+
+template <typename real, int NY> ColSet col_set() {
+    ColSet s;
+    if constexpr (NY <= 12) {
+        s.k = (const void *)&kcol_line<real, NY>;
+        s.nt = 128;
+        s.tw = 0;
+    } else {
+        s.k = (const void *)&kcol_reg<real, NY>;
+        s.nt = Col<real, NY>::NT;
+        s.tw = Col<real, NY>::TW;
+        s.smem = (size_t)NY * s.tw * 2 * sizeof(real);
+    }
+    return s;
+}
+
+}  // namespace ck
+
+}  // namespace fftlb

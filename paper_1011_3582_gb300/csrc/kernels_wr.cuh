@@ -21,55 +21,10 @@
 // layouts (the row groups of P = 8 share banks two ways).
 #pragma once
 
+#include "fft_small.cuh"
 #include "kernels_pipe.cuh"
 
 namespace fftlb {
-
-// cos(2 pi k / 32), k = 0..8 (the rest by symmetry)
-__device__ __forceinline__ constexpr double cos32(int k) {
-    return k == 0 ? 1.0
-         : k == 1 ? 0.98078528040323044913
-         : k == 2 ? 0.92387953251128675613
-         : k == 3 ? 0.83146961230254523708
-         : k == 4 ? 0.70710678118654752440
-         : k == 5 ? 0.55557023301960222474
-         : k == 6 ? 0.38268343236508977173
-         : k == 7 ? 0.19509032201612826785
-                  : 0.0;
-}
-
-// W_32^k = exp(DIR 2 pi i k / 32) for 0 <= k < 16, compile-time after unrolling
-template <int DIR, typename R>
-__device__ __forceinline__ void w32(int k, R &c, R &s) {
-    const double cc = k <= 8 ? cos32(k) : -cos32(16 - k);
-    const double ss = k <= 8 ? cos32(8 - k) : cos32(k - 8);
-    c = R(cc);
-    s = R(DIR < 0 ? -ss : ss);
-}
-
-// 32-point DFT as two 16-point DFTs of the even and odd inputs and one
-// radix-2 step with the constants W_32^k
-template <int DIR, typename C> struct SmallDFT<32, DIR, C> {
-    __device__ __forceinline__ static void run(C *v) {
-        using R = decltype(v[0].x);
-        C e[16], o[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            e[i] = v[2 * i];
-            o[i] = v[2 * i + 1];
-        }
-        SmallDFT<16, DIR, C>::run(e);
-        SmallDFT<16, DIR, C>::run(o);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            R c, s;
-            w32<DIR, R>(k, c, s);
-            const C t = k == 0 ? o[k] : C{o[k].x * c - o[k].y * s, o[k].x * s + o[k].y * c};
-            v[k] = cadd(e[k], t);
-            v[k + 16] = csub(e[k], t);
-        }
-    }
-};
 
 // Row configurations: H = E * P, P lanes per row, 32 / P rows per warp
 template <int H> struct RowCfg;

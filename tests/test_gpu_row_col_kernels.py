@@ -1,0 +1,69 @@
+"""Parity of the cluster-shared row kernels and the register-loaded column
+kernels (kernels_row.cuh, kernels_col.cuh) with the oracle: one SSP-RK3 step at
+every row length (with a short other axis) and every column length, the two
+precisions, zeta and H off zero so that every derivative row counts; odd
+partners (a length that only the general kernels take) on the other axis; and
+runs of one batch against single handles.
+
+Tolerances: fp64 1e-9 relative to the largest f (the stated bar); fp32
+gpu_common.fp32_force_bound, elementwise against max(|f|, mean |f|) as in the
+parity tests."""
+import numpy as np
+import pytest
+
+from gpu_common import fp32_force_bound, lib
+from oracle import fftlb_oracle as O
+from paper_1011_3582_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+ROWS = [32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1536, 2048]
+COLS = [4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1536, 2048]
+SHAPES = [(n, 6) for n in ROWS] + [(32, n) for n in COLS] + [(36, 64), (64, 54), (12, 96), (8, 16)]
+
+
+@pytest.fixture(scope="module")
+def fl():
+    return lib()
+
+
+def fields_of(nx, ny, seed):
+    return W.smooth_random(nx, ny, seed=seed, rho0=1.3, T0=0.9, amp=0.05, umax=0.02)
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("nx,ny", SHAPES)
+def test_one_step_matches_oracle(fl, nx, ny, precision):
+    if precision == 64 and max(nx, ny) > 1024:
+        pytest.skip("fp64 grids end at 1024")
+    f = fields_of(nx, ny, nx + ny)
+    kw = dict(nx=nx, ny=ny, zeta=1e-3, H=1e-6, K=1e-5)
+    p = O.Params(integrator=3, **kw)
+    ref = O.run(O.init_equilibrium(*f, p), p, 1)
+    with fl.Handle(fl.params(integrator=3, precision=precision, **kw)) as h:
+        h.set_fields(*f)
+        h.step(1)
+        out = h.get_f()
+    bound = 1e-9 if precision == 64 else fp32_force_bound((ny, nx), 1, f[0], f[3], K=1e-5 + 1e-6)
+    scale = np.maximum(np.abs(ref), np.abs(ref).mean())
+    assert (np.abs(out - ref) / scale).max() < bound
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+def test_batch_runs_equal_single_handles(fl, precision):
+    """Three runs of one shape in one launch give each run's own result."""
+    nx, ny = 96, 12
+    prm = fl.params(nx=nx, ny=ny, integrator=3, precision=precision)
+    starts = [fields_of(nx, ny, s) for s in (1, 2, 3)]
+    with fl.Batch([prm] * 3, autotune=False) as b:
+        for i, f in enumerate(starts):
+            b.set_fields(i, *f)
+        b.step(2)
+        got = [(b.get_f(i), b.invariants(i)) for i in range(3)]
+    for f, (g, inv) in zip(starts, got):
+        with fl.Handle(prm) as h:
+            h.set_fields(*f)
+            h.step(2)
+            assert np.array_equal(h.get_f(), g)
+            assert h.invariants() == inv
