@@ -27,21 +27,31 @@ __host__ __device__ constexpr bool col_pair(int size, int NY) {
 __host__ __device__ constexpr int col_tw(int size, int NY) {
     return size == 4 ? (NY >= 1536 ? 4 : 8) : 4;
 }
+// tables in shared memory (see kernels_col.cuh)
+__host__ __device__ constexpr bool col_tables(size_t size, int NY) { return size == 4 && NY < 1536; }
 
-// one group of a launch: slots and multiplier
+// one group of a launch: input slot (or distribution), output slot and
+// multiplier with the inverse normalisation folded in
 template <typename real> struct ColGroup {
-    int in, out, add;   // add < 0: no addend
+    int in, out, from_f;
     real c0, c1, c3;
 };
+
+// The tables of kcol_reg as one block: stage-1 twiddles exp(-2 pi i l k1 / NY) in
+// the orders [k1][l] and [l][k1], exp(-2 pi i k / P) (k < P), k_y of the NY bins
+template <typename real> __host__ __device__ constexpr unsigned col_table_bytes(int NY, int P) {
+    return (unsigned)((2 * NY + P) * 2 * sizeof(real) + NY * sizeof(real));
+}
 
 constexpr int kMaxColJobs = 40;   // groups of one launch
 
 template <typename real> struct ColArgs {
     using C = typename cplx_of<real>::type;
     C *spec;
+    const C *f;               // the stage state [run][33][ny][nx], as rows of nx / 2 complex values
     const real *kx, *ky;
-    const C *tw, *twt, *wp;   // [k1][l], [l][k1], exp(-2 pi i k / P)
-    real scale;
+    const C *tab;             // table block, see col_table_bytes
+    int *err;
     int h, ngroups;
     ColGroup<real> g[kMaxColJobs];
 };

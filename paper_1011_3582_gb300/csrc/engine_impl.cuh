@@ -2,30 +2,26 @@
 // and the per-precision plan.  Included by engine_f64.cu and engine_f32.cu
 // only (each instantiates one precision).
 //
-// One Runge-Kutta stage L(f) (Eq. 10) runs as five launches of the
-// pipelined kernels of kernels_pipe.cuh on the handle's stream (profile
-// names in parentheses):
-//   k1_pipe (row_forward_moments)  moments rho, u, T (Eqs. 7-9) of the stage
-//                           state, level-1 fields Pi = P^w - rho T (Eq. 18)
-//                           and g = M/T; forward row transforms of the 32
-//                           moving f_i and of rho, u_x, u_y, T, Pi, g
-//   kcol_pipe (col_convection)  column forward -> i (v_x k_m,x + v_y k_m,y)
-//                           -> column inverse for the f_i with v_y != 0 (in
-//                           place), and in the same launch the 8 level-1
-//                           column passes (d_y of rho, u, T, Pi, g; d_yy of
-//                           rho and u_y)
-//   k3_pipe (row_level1)    the derivatives with a factor k_x, formed in the
-//                           row spectrum (k3_form_x); row inverse of the
-//                           15; Lambda (Eq. 19), Phi = 2 q rho T grad T
-//                           (Eq. 23), the numerators of C (Eq. 22) and B
-//                           (Eq. 21); forward row transforms of Lambda_xx,
-//                           Lambda_xy, Lambda_yy, Phi_x, Phi_y, with the
-//                           d_x terms of level 2 formed in the row spectrum
-//   kcol_pipe (col_level2)  d_b Lambda_xb, d_b Lambda_yb, d_a Phi_a: the
-//                           column pass of the d_y terms plus the d_x terms
-//   k5_pipe (row_final)     row inverse of the convection terms and level-2
-//                           divergences; A, B, C, C_q (Eqs. 20-23), f^eq
-//                           (Eq. 3), I (Eq. 11), BGK and the RK combination.
+// One Runge-Kutta stage L(f) (Eq. 10) runs as five launches on the handle's
+// stream (profile names in parentheses):
+//   k1_* (row_forward_moments)  moments rho, u, T (Eqs. 7-9) of the stage state,
+//                           level-1 fields Pi = P^w - rho T (Eq. 18) and g =
+//                           M/T; forward row transforms of the f_i with v_x !=
+//                           0 and of rho, u_x, u_y, T, Pi, g
+//   kcol_* (col_convection) column passes: i (v_x k_m,x + v_y k_m,y) for the
+//                           f_i with v_y != 0, and the 8 level-1 derivatives
+//                           in k_y alone
+//   k3_* (row_level1)       inverse rows of the level-1 derivatives with a
+//                           factor k_x; Lambda (Eq. 19), Phi = 2 q rho T grad T
+//                           (Eq. 23), the numerators of C (Eq. 22) and B (Eq.
+//                           21) with the d_x terms of level 2
+//   kcol_* (col_level2)     d_y of Lambda_xy, Lambda_yy, Phi_y
+//   k5_* (row_final)        inverse rows of the convection terms; A, B, C, C_q
+//                           (Eqs. 20-23), f^eq (Eq. 3), I (Eq. 11), BGK and
+//                           the RK combination (Eq. 10).
+// stage_layout.cuh says which derivative takes which transforms.  The row
+// kernels come in three families, chosen per handle (configure_rowcol): *_wr
+// (kernels_wr.cuh), *_row (kernels_row.cuh), *_pipe (kernels_pipe.cuh).
 // This file holds the engine (plan, tables, launches) and the auxiliary
 // kernels of the per-run calls: equilibrium initialisation, moments,
 // conversions, and the gradient / invariant transforms.
@@ -753,9 +749,10 @@ class EngineT : public Engine {
     // device memory
     // batch bases (B_ runs back to back) and the views of the selected run
     int B_ = 1, run_ = 0;
-    real *f0b_ = nullptr, *f1b_ = nullptr, *fieldsb_ = nullptr, *auxb_ = nullptr;
+    real *f0b_ = nullptr, *f1b_ = nullptr;
+    real *fieldsb_ = nullptr, *auxb_ = nullptr;   // slots SLOT_F, SLOT_A of run 0
     C *specb_ = nullptr;
-    real *f0_ = nullptr, *f1_ = nullptr, *fields_ = nullptr, *aux_ = nullptr;
+    real *f0_ = nullptr, *f1_ = nullptr, *fields_ = nullptr;
     C *spec_ = nullptr;
     real *kxt_ = nullptr, *kyt_ = nullptr;
     C *Wr_ = nullptr, *Wp_ = nullptr, *Wc_ = nullptr;
@@ -785,7 +782,7 @@ class EngineT : public Engine {
     C *Twc_ = nullptr;
     size_t smemcw_ = 0;
     int gridcw_ = 1, nbufcw_ = 1, ntcw_ = 256;
-    CUtensorMap tmap_convw_{};
+    CUtensorMap tmap_convw_{}, fmap_convw_[2] = {};
     // row and column kernels of kernels_row.cuh / kernels_col.cuh, the
     // argument blocks of their launches, and their tables
     bool rowk_ = false, colk_ = false;
@@ -793,7 +790,7 @@ class EngineT : public Engine {
     ColSet cs_;
     RowArgs<real> ra_{};
     ColArgs<real> ca_conv_{}, ca_l2_{}, ca_inv_{};
-    C *Wh_ = nullptr, *Tcr_ = nullptr, *Wcp_ = nullptr;
+    C *Trow_ = nullptr, *Tcr_ = nullptr;
     // gradient kernels (k_grad_*): column tile width and shared memory
     int TWg_ = 0;
     size_t smem_gr_ = 0, smem_gc_ = 0;
@@ -808,7 +805,7 @@ class EngineT : public Engine {
     int CH1_ = 8, SMAX1_ = 1, grid1_ = 1, NHB5_ = 1, WR3_ = 1, CH5_ = 8, grid5_ = 1, SMAX5_ = 1, BOXR_ = 1;
     int TWc_ = 1, TWl_ = 1, gridc_ = 1, gridl_ = 1, NBUFc_ = 2, NBUFl_ = 2, NBUF5_ = 2;
     size_t smem1_ = 0, smem3_ = 0, smem5_ = 0, smemc_ = 0, smeml_ = 0;
-    CUtensorMap tmap_conv_{}, tmap_l2_{};
+    CUtensorMap tmap_conv_{}, tmap_l2_{}, fmap_conv_[2] = {};
     // profiling
     bool prof_ = false;
     struct ProfEv {
@@ -873,11 +870,11 @@ class EngineT : public Engine {
         // algorithmic bytes per launch: every value each kernel must read or
         // write once (one-sided spectra count N reals per field)
         const double alg[KK_COUNT] = {
-            (33 + 38 + 4) * NN * s,                   // f in; 38 spectra + rho, u, T out
-            2.0 * nconvl_ * NN * s,                   // the v_y != 0 spectra and the level-1 inputs in (rho, u_y twice); as many out
+            (33 + 24 + 6 + 6) * NN * s,               // f in; the v_x != 0 spectra, 6 field spectra, 6 fields out
+            (2.0 * nconvl_ - 1) * NN * s,             // spectra and real fields in (rho once), as many + 1 out
             0,                                        // (level 1 runs in the convection launch)
-            (14 + 2 + 3 + 6) * NN * s,                // 14 + rho, T in; 3 aux + 6 spectra out
-            (3 + 3 + 3) * NN * s,                     // 3 in, 3 added, 3 out
+            (16 + 3 + 3) * NN * s,                    // 8 spectra, 8 real rows in; 3 aux, 3 level-2 fields out
+            (3 + 3) * NN * s,                         // 3 in, 3 out
             (32 + 3 + 4 + 3 + 33 + 33 * fbase + 33) * NN * s};
         for (int k = 0; k < nkinds && k < KK_COUNT; ++k) {
             if (ms) ms[k] = prof_ms_[k];
@@ -895,8 +892,7 @@ class EngineT : public Engine {
         f0_ = f0b_ + r * Q * N_;
         f1_ = f1b_ ? f1b_ + r * Q * N_ : nullptr;
         spec_ = specb_ + r * NSLOT * ny_ * h_;
-        fields_ = fieldsb_ + r * 4 * N_;
-        aux_ = auxb_ + r * 3 * N_;
+        fields_ = fieldsb_ + r * NSLOT * N_;
     }
 
     unsigned grid1d() const {
@@ -999,8 +995,8 @@ class EngineT : public Engine {
         if (!(st = dalloc(&f0b_, B * Q * N_)).good()) return st;
         if (p_.integrator == 3 && !(st = dalloc(&f1b_, B * Q * N_)).good()) return st;
         if (!(st = dalloc(&specb_, B * NSLOT * ny_ * h_)).good()) return st;
-        if (!(st = dalloc(&fieldsb_, B * 4 * N_)).good()) return st;
-        if (!(st = dalloc(&auxb_, B * 3 * N_)).good()) return st;
+        fieldsb_ = reinterpret_cast<real *>(specb_) + (size_t)SLOT_F * N_;
+        auxb_ = reinterpret_cast<real *>(specb_) + (size_t)SLOT_A * N_;
         set_views(0);
         if (!(st = dalloc(&kxt_, (size_t)h_ + 1)).good()) return st;
         if (!(st = dalloc(&kyt_, (size_t)ny_)).good()) return st;
@@ -1126,26 +1122,36 @@ class EngineT : public Engine {
         if (ntr_) FFTLB_CU(cudaMemcpy(Tr_, tr.data(), tr.size() * sizeof(C), cudaMemcpyHostToDevice));
         if (ntr8_) FFTLB_CU(cudaMemcpy(Tr8_, tr8.data(), tr8.size() * sizeof(C), cudaMemcpyHostToDevice));
         if (ntc_) FFTLB_CU(cudaMemcpy(Tc_, tc.data(), tc.size() * sizeof(C), cudaMemcpyHostToDevice));
-        if (own_len(h_) && row_p(h_) > 0) {
-            // tw[k1 P + l] = exp(-2 pi i l k1 / h) for the row configuration of h
+        const int rp = row_p((int)sizeof(real), h_);
+        if (own_len(h_) && rp > 0) {
             std::vector<C> t1, t2;
-            stage1_twiddles(t1, t2, h_, row_p(h_));
-            if (!(st = upload_table(&Tw1_, t1)).good()) return st;
+            stage1_twiddles(t1, t2, h_, rp);
+            if (wr_ok_ && (h_ == 512 || h_ == 256 || h_ == 128) && !(st = upload_table(&Tw1_, t1)).good()) return st;
+            using L = RowTable<real>;
+            std::vector<C> blob((L::bytes(h_) + sizeof(C) - 1) / sizeof(C), C{0, 0});
+            unsigned char *b = reinterpret_cast<unsigned char *>(blob.data());
             std::vector<C> wh(wp.begin(), wp.begin() + h_ / 2 + 1);
+            memcpy(b + L::wp(h_), wh.data(), wh.size() * sizeof(C));
             for (auto &w : wh) {
                 w.x *= real(0.5);
                 w.y *= real(0.5);
             }
-            if (!(st = upload_table(&Wh_, wh)).good()) return st;
+            memcpy(b, wh.data(), wh.size() * sizeof(C));
+            memcpy(b + L::kx(h_), kx.data(), h_ * sizeof(real));
+            memcpy(b + L::tw(h_), t1.data(), t1.size() * sizeof(C));
+            if (!(st = upload_table(&Trow_, blob)).good()) return st;
         }
-        if (own_len(ny_) && col_p((int)sizeof(real), ny_) > 0) {
-            const int P = col_p((int)sizeof(real), ny_);
+        const int cp = col_p((int)sizeof(real), ny_);
+        if (own_len(ny_) && cp > 0) {
             std::vector<C> t1, t2, w;
-            stage1_twiddles(t1, t2, ny_, P);
+            stage1_twiddles(t1, t2, ny_, cp);
             t1.insert(t1.end(), t2.begin(), t2.end());
+            twiddles(w, cp, cp);
+            t1.insert(t1.end(), w.begin(), w.end());
+            const size_t n = t1.size();
+            t1.resize(n + ny_ / 2);   // ny reals
+            memcpy(t1.data() + n, ky.data(), ny_ * sizeof(real));
             if (!(st = upload_table(&Tcr_, t1)).good()) return st;
-            twiddles(w, P, P);
-            if (!(st = upload_table(&Wcp_, w)).good()) return st;
         }
         if (wr_ok_ && (ny_ == 1024 || ny_ == 512 || ny_ == 256 || ny_ == 128)) {
             // twc[k1 P + l] = exp(-2 pi i l k1 / ny) for the column configuration of
@@ -1219,13 +1225,13 @@ class EngineT : public Engine {
         }
     }
 
-    static GroupDesc group(int nin, int in0, int in1) {
+    static GroupDesc group(int nin, int in0, int in1, double scale) {
         GroupDesc g;
         memset(&g, 0, sizeof g);
         g.nin = nin;
         g.in_slot[0] = in0;
         g.in_slot[1] = in1;
-        g.add_slot = -1;
+        g.scale = scale;
         return g;
     }
     // add output: term list of (input index, c0..c4)
@@ -1248,14 +1254,12 @@ class EngineT : public Engine {
         a.spec = specb_;
         a.kx = kxt_;
         a.ky = kyt_;
-        a.tw = Tcr_;
-        a.twt = Tcr_ + ny_;
-        a.wp = Wcp_;
-        a.scale = (real)(1.0 / ((double)nx_ * (double)ny_));
+        a.tab = Tcr_;
+        a.err = err_;
         for (int i = 0; i < count && i < kMaxColJobs; ++i) {
             const GroupDesc &g = gs[first + i];
-            a.g[i] = ColGroup<real>{g.in_slot[0], g.out_slot[0], g.add_slot, (real)g.c[0][0][0], (real)g.c[0][0][1],
-                                    (real)g.c[0][0][3]};
+            a.g[i] = ColGroup<real>{g.in_slot[0], g.out_slot[0], g.from_f, (real)(g.c[0][0][0] * g.scale),
+                                    (real)(g.c[0][0][1] * g.scale), (real)(g.c[0][0][3] * g.scale)};
         }
     }
 
@@ -1263,51 +1267,45 @@ class EngineT : public Engine {
         static const double DX[5] = {1, 0, 0, 0, 0}, DY[5] = {0, 1, 0, 0, 0};
         static const double DYY[5] = {0, 0, 0, -1, 0};
         std::vector<GroupDesc> gs;
-        // convection: i (v_x k_x + v_y k_y) f_i, in place, for the velocities
-        // with v_y != 0 (the row kernel K1 writes i v_x k_x f_i^ / nx for the
-        // others)
+        const double sxy = 1.0 / ((double)nx_ * (double)ny_), sy = 1.0 / (double)ny_;
+        // convection: i (v_x k_x + v_y k_y) f_i for the velocities with v_y !=
+        // 0 (K1 writes i v_x k_x f_i^ / nx for the others), from the row spectrum
+        // in place or, with v_x = 0, from f_i itself
         conv_groups_ = (int)gs.size();
         nconv_ = 0;
         for (int i = 1; i < Q; ++i) {
             if (vy_[i] == 0.0) continue;
             ++nconv_;
-            GroupDesc g = group(1, i - 1, 0);
+            const bool real_rows = vx_[i] == 0.0;
+            GroupDesc g = group(1, real_rows ? i : i - 1, 0, real_rows ? sy : sxy);
+            g.from_f = real_rows ? 1 : 0;
             const double c[5] = {vx_[i], vy_[i], 0, 0, 0};
             add_out(g, i - 1, 1, 0, c);
             gs.push_back(g);
         }
-        // level 1: the derivatives in k_y alone (k3_src_slot: K3 forms the
-        // rest, and adds -k_x^2 rho^ / nx to d_yy rho, i k_x (d_y u_x) to
-        // d_yy u_y), in the convection launch (nconvl_ groups from
-        // conv_groups_)
+        // level 1: the derivatives in k_y alone, in the convection launch
+        // (nconvl_ groups from conv_groups_)
         {
-            const int singles[8][2] = {{SLOT_RHO, D_RY}, {SLOT_RHO, D_LAP}, {SLOT_UX, D_UXY}, {SLOT_UY, D_UYY},
-                                       {SLOT_UY, D_DIVY}, {SLOT_T, D_TY}, {SLOT_PI, D_PIY}, {SLOT_G, D_GY}};
-            for (auto &sgl : singles) {
-                GroupDesc g = group(1, sgl[0], 0);
-                add_out(g, SLOT_D1 + sgl[1], 1, 0, sgl[1] == D_LAP || sgl[1] == D_DIVY ? DYY : DY);
+            const int lv1[ND1][2] = {{SLOT_UX, D1_UXY}, {SLOT_UY, D1_UYY}, {SLOT_F + 0, D1_RY}, {SLOT_F + 0, D1_RYY},
+                                     {SLOT_F + 3, D1_TY}, {SLOT_F + 4, D1_PIY}, {SLOT_F + 5, D1_GY}, {SLOT_F + 2, D1_UYYY}};
+            for (auto &l : lv1) {
+                GroupDesc g = group(1, l[0], 0, l[0] < SLOT_F ? sxy : sy);
+                add_out(g, SLOT_D1 + l[1], 1, 0, l[1] == D1_RYY || l[1] == D1_UYYY ? DYY : DY);
                 gs.push_back(g);
             }
-            nconvl_ = nconv_ + 8;
+            nconvl_ = nconv_ + ND1;
         }
-        // level 2: d_y of Lambda_xy, Lambda_yy, Phi_y plus the d_x terms K3
-        // wrote (k3_mul_slot): outputs in 53, 55, 56
+        // level 2: d_y of Lambda_xy, Lambda_yy, Phi_y in place
         l2_groups_ = (int)gs.size();
-        {
-            const int l2[3][3] = {{SLOT_L2 + 1, SLOT_L2 + 0, SLOT_L2 + 0},          // in, out, add
-                                  {SLOT_L2 + 2, SLOT_L2 + 2, SLOT_D1 + D_DIVX},
-                                  {SLOT_L2 + 4, SLOT_L2 + 3, SLOT_L2 + 3}};
-            for (auto &e : l2) {
-                GroupDesc g = group(1, e[0], 0);
-                add_out(g, e[1], 1, 0, DY);
-                g.add_slot = e[2];
-                gs.push_back(g);
-            }
+        for (int r = 0; r < 3; ++r) {
+            GroupDesc g = group(1, SLOT_L2 + r, 0, sy);
+            add_out(g, SLOT_L2 + r, 1, 0, DY);
+            gs.push_back(g);
         }
         // gradient op: field i in slot i -> slots 20 + 2i, 21 + 2i
         grad_groups_ = (int)gs.size();
         for (int i = 0; i < 16; ++i) {
-            GroupDesc g = group(1, i, 0);
+            GroupDesc g = group(1, i, 0, sxy);
             add_out(g, 20 + 2 * i, 1, 0, DX);
             add_out(g, 21 + 2 * i, 1, 0, DY);
             gs.push_back(g);
@@ -1317,7 +1315,7 @@ class EngineT : public Engine {
         // spectrum by k_inv_rows)
         inv_groups_ = (int)gs.size();
         {
-            GroupDesc g = group(1, 0, 0);
+            GroupDesc g = group(1, 0, 0, sxy);
             add_out(g, 2, 1, 0, DY);
             gs.push_back(g);
         }
@@ -1389,17 +1387,17 @@ class EngineT : public Engine {
         return fn;
     }
 
-    // the spectrum arena as a 2-D tensor {2h reals, NSLOT ny rows}, boxes
-    // of {2 TW reals, BOXR rows}
-    Status make_tmap(CUtensorMap *m, int TW) {
+    // the spectrum arena (or the distributions at base, planes = Q) as a 2-D
+    // tensor {2h reals, B planes ny rows}, boxes of {2 TW reals, BOXR rows}
+    Status make_tmap(CUtensorMap *m, int TW, void *base = nullptr, int planes = NSLOT) {
         auto enc = tensor_map_encoder();
         if (!enc) return Status::err(FFTLB_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
-        cuuint64_t dims[2] = {(cuuint64_t)(2 * h_), (cuuint64_t)B_ * NSLOT * ny_};
+        cuuint64_t dims[2] = {(cuuint64_t)(2 * h_), (cuuint64_t)B_ * planes * ny_};
         cuuint64_t strides[1] = {(cuuint64_t)(2 * h_) * sizeof(real)};
         cuuint32_t box[2] = {(cuuint32_t)(2 * TW), (cuuint32_t)BOXR_};
         cuuint32_t es[2] = {1, 1};
         CUresult r = enc(m, sizeof(real) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                         (void *)specb_, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                         base ? base : (void *)specb_, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return Status::err(FFTLB_ERR_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
@@ -1420,6 +1418,12 @@ class EngineT : public Engine {
         FFTLB_CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim));
         FFTLB_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kernel, nthreads, smem));
         return Status::ok();
+    }
+
+    // maps of the two state buffers (f1b_ absent for Euler) for tile width TW
+    Status make_fmaps(CUtensorMap m[2], int TW) {
+        Status st = make_tmap(&m[0], TW, f0b_, Q);
+        return st.good() ? make_tmap(&m[1], TW, f1b_ ? f1b_ : f0b_, Q) : st;
     }
 
     size_t budget_ = 0, optin_ = 0;
@@ -1569,15 +1573,15 @@ class EngineT : public Engine {
         if (!(st = pick_tw(&TWl_, &NBUFl_, &smeml_, &gridl_)).good()) return st;
         if (!(st = make_tmap(&tmap_conv_, TWc_)).good()) return st;
         if (!(st = make_tmap(&tmap_l2_, TWl_)).good()) return st;
+        if (!(st = make_fmaps(fmap_conv_, TWc_)).good()) return st;
         // K3 (one row per block, not pipelined inside a block): most blocks
         // per SM first, so that one block's row loads overlap another's
         // transforms, then the most work rows
         {
             int bestnb = 0;
             WR3_ = 0;
-            for (int wr = ND1; wr >= 1; --wr) {
-                const size_t sm = smem_bytes({h_ * cs, h_ * cs, ntrmax() * cs, (size_t)ND1 * h_ * cs, (size_t)wr * ph * cs,
-                                              (size_t)2 * nx_ * rs});
+            for (int wr = NSP; wr >= 1; --wr) {
+                const size_t sm = smem_bytes({h_ * cs, h_ * cs, ntrmax() * cs, (size_t)NK3 * h_ * cs, (size_t)wr * ph * cs});
                 if (sm > budget) continue;
                 if (!(st = occupancy(k3_pipe<real, SPLIT>, NT3, sm, &nb)).good()) return st;
                 if (nb > bestnb) {
@@ -1637,7 +1641,7 @@ class EngineT : public Engine {
         }
         if (!own_len(h_)) rs_ = RowSet();
         if (!own_len(ny_)) cs_ = ColSet();
-        if (rs_.k1 && Tw1_ && std::max({rs_.smem1, rs_.smem3, rs_.smem5}) <= budget_) {
+        if (rs_.k1 && std::max({rs_.smem1, rs_.smem3, rs_.smem5}) <= budget_) {
             const void *ks[3] = {rs_.k1, rs_.k3, rs_.k5};
             for (const void *k : ks)
                 FFTLB_CU(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget_));
@@ -1652,13 +1656,8 @@ class EngineT : public Engine {
             ra_.q = kp_.q;
             ra_.zeta = kp_.zeta;
             ra_.scale_x = kp_.scale_x;
-            ra_.fields = fieldsb_;
-            ra_.aux = auxb_;
             ra_.spec = specb_;
-            ra_.tw = Tw1_;
-            ra_.wp = Wp_;
-            ra_.wh = Wh_;
-            ra_.kx = kxt_;
+            ra_.tab = Trow_;
             ra_.err = err_;
             // The persistent fp32 rows (k*_wr) keep their place where every
             // SM has at least two rows: their prefetch then pays (1024^2:
@@ -1683,15 +1682,15 @@ class EngineT : public Engine {
     }
 
     // a row kernel over every row of every run, cs blocks (one cluster) a row
-    Status launch_row(const char *name, const void *k, size_t smem) {
+    Status launch_row(const char *name, const void *k, int cs, size_t smem) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(B_ * ny_ * rs_.cs));
+        cfg.gridDim = dim3((unsigned)(B_ * ny_ * cs));
         cfg.blockDim = dim3((unsigned)rs_.nt);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = stream_;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)rs_.cs;
+        at[0].val.clusterDim.x = (unsigned)cs;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
@@ -1781,6 +1780,7 @@ class EngineT : public Engine {
                 }
                 if (best > 0) {
                     st = make_tmap(&tmap_convw_, TWw);
+                    if (st.good()) st = make_fmaps(fmap_convw_, TWw);
                     if (!st.good()) return st;
                     colwr_ = true;
                     ntcw_ = NTw;
@@ -1875,9 +1875,10 @@ class EngineT : public Engine {
         st = occ_k5(sm5, &nb);
         if (!st.good()) return st;
         const int g5 = std::min(B_ * ny_, std::max(1, nb) * nsm_);
-        CUtensorMap mc, ml;
+        CUtensorMap mc, ml, mf[2];
         if (!(st = make_tmap(&mc, twc)).good()) return st;
         if (!(st = make_tmap(&ml, twl)).good()) return st;
+        if (!(st = make_fmaps(mf, twc)).good()) return st;
         TWc_ = twc;
         TWl_ = twl;
         NBUFc_ = nbc;
@@ -1895,6 +1896,8 @@ class EngineT : public Engine {
         gridl_ = gl;
         grid5_ = g5;
         tmap_conv_ = mc;
+        fmap_conv_[0] = mf[0];
+        fmap_conv_[1] = mf[1];
         tmap_l2_ = ml;
         return Status::ok();
     }
@@ -2010,12 +2013,14 @@ class EngineT : public Engine {
 
     // column pass of one-input groups; level2: the level-2 launch (its own
     // tile width on the pipelined kernels)
-    Status launch_col(int first, int count, bool level2) {
+    Status launch_col(int first, int count, bool level2, const real *cur = nullptr) {
+        const int fm = cur && cur == f1b_ ? 1 : 0;   // the state buffer the groups with from_f read
         if (colk_) {
             if (first == inv_groups_) {   // the selected run alone
                 ca_inv_.spec = spec_;
                 return launch_cols(ca_inv_, 1);
             }
+            ca_conv_.f = reinterpret_cast<const C *>(cur);
             return launch_cols(level2 ? ca_l2_ : ca_conv_, B_);
         }
         if constexpr (wr_ok_) {
@@ -2024,7 +2029,7 @@ class EngineT : public Engine {
 #define FFTLB_KCOLWR(NYV)                                                                                     \
     launch_pdl("kcol_wr", kcol_wr<NYV>, gridcw_, ntcw_, smemcw_, specb_, (const GroupDesc *)(groups_ + first),     \
                count, (const float *)kxt_, (const float *)kyt_, (const float2 *)Twc_, kp_, BOXR_, nbufcw_,          \
-               tmap_convw_, err_)
+               tmap_convw_, fmap_convw_[fm], err_)
                 return ny_ == 1024 ? FFTLB_KCOLWR(1024)
                      : ny_ == 512  ? FFTLB_KCOLWR(512)
                      : ny_ == 256  ? FFTLB_KCOLWR(256)
@@ -2034,10 +2039,10 @@ class EngineT : public Engine {
         }
         if (level2)
             kcol_pipe<real, SPLIT><<<gridl_, NTC, smeml_, stream_>>>(specb_, groups_ + first, count, kxt_, kyt_, Wc_, Tc_,
-                                                                     ntc_, kp_, TWl_, BOXR_, NBUFl_, tmap_l2_, err_);
+                                                                     ntc_, kp_, TWl_, BOXR_, NBUFl_, tmap_l2_, tmap_l2_, err_);
         else
             kcol_pipe<real, SPLIT><<<gridc_, NTC, smemc_, stream_>>>(specb_, groups_ + first, count, kxt_, kyt_, Wc_, Tc_,
-                                                                     ntc_, kp_, TWc_, BOXR_, NBUFc_, tmap_conv_, err_);
+                                                                     ntc_, kp_, TWc_, BOXR_, NBUFc_, tmap_conv_, fmap_conv_[fm], err_);
         FFTLB_LAUNCHED("kcol_pipe");
         return Status::ok();
     }
@@ -2057,7 +2062,7 @@ class EngineT : public Engine {
             ra_.fout = out;
             ra_.alpha = alpha;
             ra_.beta = beta;
-            if (!(st = launch_row("k1_row", rs_.k1, rs_.smem1)).good()) return st;
+            if (!(st = launch_row("k1_row", rs_.k1, rs_.cs, rs_.smem1)).good()) return st;
             k1done = true;
         }
         if constexpr (wr_ok_) {
@@ -2084,19 +2089,19 @@ class EngineT : public Engine {
         FFTLB_LAUNCHED("k1_pipe");
         if (!(st = prof_end()).good()) return st;
         if (!(st = prof_begin(KK_COL_CONV)).good()) return st;
-        if (!(st = launch_col(conv_groups_, nconvl_, false)).good()) return st;
+        if (!(st = launch_col(conv_groups_, nconvl_, false, cur)).good()) return st;
         if (!(st = prof_end()).good()) return st;
         if (!(st = prof_begin(KK_ROW_LEVEL1)).good()) return st;
         bool k3done = false;
         if (rowk_) {
-            if (!(st = launch_row("k3_row", rs_.k3, rs_.smem3)).good()) return st;
+            if (!(st = launch_row("k3_row", rs_.k3, rs_.cs, rs_.smem3)).good()) return st;
             k3done = true;
         }
         if constexpr (wr_ok_) {
             if (!k3done && k3wr_) {
                 const int nt = nt_k3wr_host(h_);
                 auto *kern = h_ == 512 ? k3_wr<512> : h_ == 256 ? k3_wr<256> : k3_wr<128>;
-                if (!(st = launch_pdl("k3_wr", kern, grid3w_, nt, smem3w_, specb_, (const float *)fieldsb_, auxb_,
+                if (!(st = launch_pdl("k3_wr", kern, grid3w_, nt, smem3w_, specb_,
                                       (const float2 *)Tw1_, (const float2 *)Wp_, (const float *)kxt_, kp_, err_)).good())
                     return st;
                 k3done = true;
@@ -2104,7 +2109,7 @@ class EngineT : public Engine {
         }
         if (!k3done) {
             const int ml = row_maxlr(WR3_, NT3);
-            k3_pipe<real, SPLIT><<<B_ * ny_, NT3, smem3_, stream_>>>(specb_, fieldsb_, auxb_, Wr_, Wp_, ml == 3 ? Tr8_ : Tr_,
+            k3_pipe<real, SPLIT><<<B_ * ny_, NT3, smem3_, stream_>>>(specb_, Wr_, Wp_, ml == 3 ? Tr8_ : Tr_,
                                                               ml == 3 ? ntr8_ : ntr_, kxt_, kp_, WR3_, ml, err_);
         }
         FFTLB_LAUNCHED("k3_pipe");
@@ -2114,7 +2119,7 @@ class EngineT : public Engine {
         if (!(st = prof_end()).good()) return st;
         if (!(st = prof_begin(KK_ROW_FINAL)).good()) return st;
         if (rowk_) {
-            if (!(st = launch_row("k5_row", rs_.k5, rs_.smem5)).good()) return st;
+            if (!(st = launch_row("k5_row", rs_.k5, rs_.cs, rs_.smem5)).good()) return st;
             return prof_end();
         }
         if constexpr (wr_ok_) {

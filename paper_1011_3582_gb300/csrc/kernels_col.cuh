@@ -3,19 +3,24 @@
 //   kcol_reg   lengths 16 .. 2048 = 2^p and 24 .. 1536 = 3 2^p: one job (a
 //              tile of TW spectrum columns of one group) per block;
 //   kcol_line  lengths 4, 6, 8, 12: one column per thread, in registers.
-// Every group has one input and one output (which may be the same slot):
-// forward transform, multiplier i (c0 k_x + c1 k_y) or c3 k_y^2, inverse, plus
-// the values of the addend slot where the group has one.
+// Every group has one input (a slot or a distribution of the stage state) and
+// one output (which may be the same slot): forward transform, multiplier
+// i (c0 k_x + c1 k_y) or c3 k_y^2, inverse.
 //
 // A column of NY = E P values is transformed by P threads as in kcol_wr, but
 // thread (c, l) loads its x[l + P t] straight from global memory into
 // registers: the tile passes through shared memory twice (the transpose and
-// its inverse) instead of three times, and a block needs one tile of shared
-// memory and no tables of its own, so that many small blocks fit an SM and
-// their loads overlap each other's transforms.  The packed column 0 of the
+// its inverse) instead of three times, and a block holds one tile, so that
+// several blocks fit an SM and their loads overlap each other's transforms.
+// The tables of the 8-wide fp32 tiles come by one bulk copy that overlaps the
+// tile's loads: read through L1, they were cold in every launch, a latency per
+// handful of twiddles (one job's time on 384^2: 13.8 us, 10.2 with the copy).
+// 4-wide tiles are hardly larger than their tables (2048^2: convection 479 us
+// with the copy, 372 through L1), and fp64's arithmetic hides the latency.  The packed column 0 of the
 // tile at k_x = 0 needs no pairing of (k_y, -k_y) (see kcol_wr).
 #pragma once
 
+#include "async_copy.cuh"
 #include "col_kernels.h"
 #include "fft_small.cuh"
 #include "stage_layout.cuh"
@@ -31,8 +36,15 @@ template <typename real, int NY> struct Col {
     static constexpr int PH = PAIR ? P / 2 : P;
     static constexpr int TW = col_tw(sizeof(real), NY), NT = TW * P;
     // rows of one memory phase (16 8-byte or 8 16-byte values) in different banks
+    static constexpr bool TABS = col_tables(sizeof(real), NY);   // tables in shared memory
     static constexpr int PHASE = 128 / (int)sizeof(C), SW = TW < PHASE ? PHASE / TW - 1 : 0;
 };
+
+// a table value from shared or (read-only) global memory
+template <bool SH, typename T> __device__ __forceinline__ T tab(const T *p) {
+    if constexpr (SH) return *p;
+    else return __ldg(p);
+}
 
 // position of stage-1 output (l, k1) of column c
 template <typename real, int NY> __device__ __forceinline__ int cp(int c, int l, int k1) {
@@ -53,29 +65,46 @@ __global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_
     using C = typename G::C;
     constexpr int E = G::E, P = G::P, PH = G::PH, TW = G::TW;
     extern __shared__ __align__(128) unsigned char col_smem_raw[];
+    __shared__ __align__(8) uint64_t bar;
     C *T = reinterpret_cast<C *>(col_smem_raw);   // [NY][TW]
+    const C *tw = G::TABS ? T + (size_t)NY * TW : A.tab, *twt = tw + NY, *wp = twt + NY;   // the table block
+    const real *ky = reinterpret_cast<const real *>(wp + P);
     const int h = A.h, tid = threadIdx.x, c = tid % TW, jl = tid / TW;
     const int ntiles = h / TW;
     const int job = (int)blockIdx.x, g = job / ntiles, t = job - g * ntiles;   // (grid.y: run)
     const size_t slot = (size_t)NY * h;
     const ColGroup<real> &gr = A.g[g];
     C *spec = A.spec + (size_t)blockIdx.y * NSLOT * slot + t * TW + c;
-    const C *__restrict__ in = spec + (size_t)gr.in * slot;
+    // (no slot is both read and written by different columns of one launch)
+    const C *__restrict__ in = gr.from_f ? A.f + ((size_t)blockIdx.y * Q + gr.in) * slot + t * TW + c : spec + (size_t)gr.in * slot;
+    if (G::TABS && tid == 0) {
+        mbar_init(&bar, 1);
+        mbar_init_fence();
+        mbar_expect_tx(&bar, col_table_bytes<real>(NY, P));
+        bulk_g2s(T + (size_t)NY * TW, A.tab, col_table_bytes<real>(NY, P), &bar);
+    }
     C v[E];
 #pragma unroll
     for (int q = 0; q < E; ++q) v[q] = in[(size_t)(jl + P * q) * h];
     SmallDFT<E, -1, C>::run(v);
+    if constexpr (G::TABS) {
+        __syncthreads();   // the barrier is initialised before any thread polls it
+        if (!block_wait(&bar, 0, A.err)) {
+            mbar_wait_bounded(&bar, 0);
+            return;
+        }
+    }
 #pragma unroll
-    for (int k1 = 1; k1 < E; ++k1) v[k1] = cmul(v[k1], __ldg(A.tw + k1 * P + jl));
+    for (int k1 = 1; k1 < E; ++k1) v[k1] = cmul(v[k1], tab<G::TABS>(tw + k1 * P + jl));
 #pragma unroll
     for (int k1 = 0; k1 < E; ++k1) T[cp<real, NY>(c, jl, k1)] = v[k1];
     __syncthreads();
     // stage 2: forward, multiplier, inverse, conjugate twiddles
-    const real mx = gr.c0 * __ldg(A.kx + t * TW + c), c1 = gr.c1, c3 = gr.c3, scale = A.scale;
+    const real mx = gr.c0 * __ldg(A.kx + t * TW + c), c1 = gr.c1, c3 = gr.c3;
     auto mult = [&](int k, C u) {
-        const real ay = __ldg(A.ky + k);
-        if (c3 != real(0)) return cscale(u, c3 * ay * ay * scale);   // uniform over the block
-        const real m = (mx + c1 * ay) * scale;
+        const real ay = tab<G::TABS>(ky + k);
+        if (c3 != real(0)) return cscale(u, c3 * ay * ay);   // uniform over the block
+        const real m = mx + c1 * ay;
         return C{-m * u.y, m * u.x};
     };
     if constexpr (!G::PAIR) {
@@ -92,7 +121,7 @@ __global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_
                 SmallDFT<P, +1, C>::run(u);
 #pragma unroll
                 for (int l = 0; l < P; ++l)
-                    T[cp<real, NY>(c, l, k1)] = l == 0 ? u[l] : cmul(u[l], cconj(__ldg(A.twt + l * E + k1)));
+                    T[cp<real, NY>(c, l, k1)] = l == 0 ? u[l] : cmul(u[l], cconj(tab<G::TABS>(twt + l * E + k1)));
             }
         }
     } else if (jl < 2 * E) {   // (whole warps)
@@ -114,7 +143,7 @@ __global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_
             recv.y = __shfl_xor_sync(0xffffffffu, send.y, TW);
             const C a = gg ? recv : u[i], b = gg ? u[HH + i] : recv;
             const int k2 = HH * gg + i;
-            const C w = __ldg(A.wp + k2);   // W_P^k2
+            const C w = tab<G::TABS>(wp + k2);   // W_P^k2
             const C tb = cmul(b, w);
             const C x0 = mult(k1 + E * k2, cadd(a, tb)), x1 = mult(k1 + E * (k2 + PH), csub(a, tb));
             const C ai = cadd(x0, x1), bi = cmul(csub(x0, x1), cconj(w));
@@ -129,7 +158,7 @@ __global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_
 #pragma unroll
         for (int m = 0; m < PH; ++m) {
             const int l = gg + 2 * m;
-            T[cp<real, NY>(c, l, k1)] = cmul(u[m], cconj(__ldg(A.twt + l * E + k1)));
+            T[cp<real, NY>(c, l, k1)] = cmul(u[m], cconj(tab<G::TABS>(twt + l * E + k1)));
         }
     }
     __syncthreads();
@@ -137,11 +166,6 @@ __global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_
 #pragma unroll
     for (int k1 = 0; k1 < E; ++k1) v[k1] = T[cp<real, NY>(c, jl, k1)];
     SmallDFT<E, +1, C>::run(v);
-    if (gr.add >= 0) {   // plus the term the row kernel formed (all loads first: out may be the addend's slot)
-        const C *ad = spec + (size_t)gr.add * slot;
-#pragma unroll
-        for (int q = 0; q < E; ++q) v[q] = cadd(v[q], ad[(size_t)(jl + P * q) * h]);
-    }
 #pragma unroll
     for (int q = 0; q < E; ++q) out[(size_t)(jl + P * q) * h] = v[q];
 }
@@ -157,29 +181,26 @@ __global__ void __launch_bounds__(128) kcol_line(const __grid_constant__ ColArgs
     const size_t slot = (size_t)NY * h;
     const ColGroup<real> &gr = A.g[g];
     C *spec = A.spec + (size_t)blockIdx.y * NSLOT * slot + kx;
-    const C *in = spec + (size_t)gr.in * slot;
-    C v[NY], a[NY];
+    const C *in = gr.from_f ? A.f + ((size_t)blockIdx.y * Q + gr.in) * slot + kx : spec + (size_t)gr.in * slot;
+    C v[NY];
 #pragma unroll
-    for (int y = 0; y < NY; ++y) {
-        v[y] = in[(size_t)y * h];
-        a[y] = gr.add >= 0 ? spec[(size_t)gr.add * slot + (size_t)y * h] : C{0, 0};
-    }
+    for (int y = 0; y < NY; ++y) v[y] = in[(size_t)y * h];
     SmallDFT<NY, -1, C>::run(v);
     const real mx = gr.c0 * __ldg(A.kx + kx);
 #pragma unroll
     for (int k = 0; k < NY; ++k) {
         const real ay = __ldg(A.ky + k);
         if (gr.c3 != real(0)) {
-            v[k] = cscale(v[k], gr.c3 * ay * ay * A.scale);
+            v[k] = cscale(v[k], gr.c3 * ay * ay);
         } else {
-            const real m = (mx + gr.c1 * ay) * A.scale;
+            const real m = mx + gr.c1 * ay;
             v[k] = C{-m * v[k].y, m * v[k].x};
         }
     }
     SmallDFT<NY, +1, C>::run(v);
     C *out = spec + (size_t)gr.out * slot;
 #pragma unroll
-    for (int y = 0; y < NY; ++y) out[(size_t)y * h] = gr.add >= 0 ? cadd(v[y], a[y]) : v[y];
+    for (int y = 0; y < NY; ++y) out[(size_t)y * h] = v[y];
 }
 
 template <typename real, int NY> ColSet col_set() {
@@ -192,7 +213,7 @@ template <typename real, int NY> ColSet col_set() {
         s.k = (const void *)&kcol_reg<real, NY>;
         s.nt = Col<real, NY>::NT;
         s.tw = Col<real, NY>::TW;
-        s.smem = (size_t)NY * s.tw * 2 * sizeof(real);
+        s.smem = (size_t)NY * s.tw * 2 * sizeof(real) + (Col<real, NY>::TABS ? col_table_bytes<real>(NY, Col<real, NY>::P) : 0);
     }
     return s;
 }

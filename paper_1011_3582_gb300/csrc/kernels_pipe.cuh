@@ -20,6 +20,7 @@
 #pragma once
 
 #include "async_copy.cuh"
+#include "stage_site.cuh"
 
 // Threads per block (NT) and minimum resident blocks per SM (MINB) of the
 // persistent kernels, per precision and kernel kind.  fp32 defaults
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(KCfg<real, KS_K1>::NT, KCfg<real, KS_K1>::MINB
         const int yg = (int)blockIdx.x + ri * (int)gridDim.x;
         const int run = yg / ny, y = yg - run * ny;
         C *spec_r = spec + (size_t)run * NSLOT * slot;
-        real *fields_r = fields + (size_t)run * 4 * N;
+        real *fields_r = fields + (size_t)run * NSLOT * N;
         const int i0 = c * CH, nf = min(CH, Q - i0);
         if (!block_wait(bar, odd ? par1 : par0, err)) {
             if (pend0) mbar_wait_bounded(&bar0, par0);
@@ -255,7 +256,9 @@ __global__ void __launch_bounds__(KCfg<real, KS_K1>::NT, KCfg<real, KS_K1>::MINB
             for (int r = r0; r < nf; ++r) {
                 const int i = i0 + r;
                 C *dst = spec_r + (size_t)(i - 1) * slot + (size_t)y * h;
-                if (VY<real>(i) == real(0)) {
+                if (VX<real>(i) == real(0)) {
+                    // v_x = 0: the column pass takes f_i itself
+                } else if (VY<real>(i) == real(0)) {
                     // v_y = 0: the convection term needs no column pass; its
                     // row spectrum is i v_x k_x f^ / nx (the 1 / nx the column
                     // pass would leave)
@@ -284,8 +287,10 @@ __global__ void __launch_bounds__(KCfg<real, KS_K1>::NT, KCfg<real, KS_K1>::MINB
                     B[nx + x] = ux;
                     B[2 * nx + x] = uy;
                     B[3 * nx + x] = T;
-                    B[4 * nx + x] = rho * T / (real(1) - P.b * rho) - P.a * rho * rho - rho * T;   // Eq. 18
-                    B[5 * nx + x] = (P.K + P.H * T) / T;                                          // M / T
+                    const real Pi = rho * T / (real(1) - P.b * rho) - P.a * rho * rho - rho * T;   // Eq. 18
+                    const real g = (P.K + P.H * T) / T;                                          // M / T
+                    fields_r[4 * N + o] = B[4 * nx + x] = Pi;
+                    fields_r[5 * N + o] = B[5 * nx + x] = g;
                 }
                 a0[s] = a1[s] = a2[s] = a3[s] = real(0);
             }
@@ -409,51 +414,49 @@ __host__ __device__ __forceinline__ size_t tile_stride(int TW, int ny) {
     return bytes / sizeof(C);
 }
 
-// The fields of a group that the tile copies and a one-input job read,
-// staged in shared memory once per launch by the warp-resident column
-// kernels (a per-job copy of the whole GroupDesc by one thread held every
-// other warp of the block at the next barrier).
-// The multiplier is i (c0 k_x + c1 k_y), or c3 k_y^2 where c3 is not zero.
+// The fields of a group that the tile copies and a job read, staged in
+// shared memory once per launch by the warp-resident column kernels (a per-job
+// copy of the whole GroupDesc by one thread held every other warp of the block
+// at the next barrier).  The multiplier is i (c0 k_x + c1 k_y), or c3 k_y^2
+// where c3 is not zero, times the group's scale (folded into the constants).
 struct ColG {
-    int nin, in_slot[2], out_slot, add_slot;
+    int in_slot[1], out_slot, from_f;
     float c0, c1, c3;
 };
 constexpr int kMaxColGroups = 40;   // groups of one kcol_wr launch (at most 32 convection + 8 level-1 groups)
 
-// (GD: GroupDesc in global memory, or ColG / GroupDesc staged in shared memory)
-template <typename C, typename GD>
-__device__ __forceinline__ void kcol_issue(C *dst, uint64_t *bar, const GD *groups, int k, int ntiles,
-                                           int ngroups, int TW, int ny, int BOXR, const CUtensorMap *tmap) {
-    const int job = (int)blockIdx.x + k * (int)gridDim.x;
-    const int run = job / (ngroups * ntiles), jr = job - run * ngroups * ntiles;
-    const int g = jr / ntiles, t = jr - g * ntiles;
-    const GD *G = groups + g;
-    const int nin = G->nin;
-    const int tile = TW * ny;
-    mbar_expect_tx(bar, (uint32_t)(nin * tile * sizeof(C)));
-    for (int s = 0; s < nin; ++s) {
-        const int sl = run * NSLOT + G->in_slot[s];   // the tensor spans the arenas of all runs
-        for (int r0 = 0; r0 < ny; r0 += BOXR)
-            tma_load_2d(dst + (size_t)s * tile_stride<C>(TW, ny) + (size_t)r0 * TW, tmap, 2 * t * TW, sl * ny + r0, bar);
-    }
-    if (G->add_slot >= 0) {   // the addend tile, read at the job's store: into L2 now
-        const int sl = run * NSLOT + G->add_slot;
-        for (int r0 = 0; r0 < ny; r0 += BOXR) tma_prefetch_2d(tmap, 2 * t * TW, sl * ny + r0);
-    }
+// where a job's tile starts: the tensor map (spectrum arena or stage state)
+// and the first row
+struct ColSrc {
+    const CUtensorMap *map;
+    int row;
+};
+template <typename GD>
+__device__ __forceinline__ ColSrc col_src(const GD *G, int run, int ny, const CUtensorMap *tmap, const CUtensorMap *fmap) {
+    return G->from_f ? ColSrc{fmap, (run * Q + G->in_slot[0]) * ny} : ColSrc{tmap, (run * NSLOT + G->in_slot[0]) * ny};
 }
 
-// L2 prefetch of the tiles kcol_issue would load for job k
-template <typename GD>
-__device__ __forceinline__ void kcol_prefetch(const GD *groups, int k, int ntiles, int ngroups, int TW, int ny,
-                                              int BOXR, const CUtensorMap *tmap) {
+// (GD: GroupDesc in global memory, or ColG staged in shared memory)
+template <typename C, typename GD>
+__device__ __forceinline__ void kcol_issue(C *dst, uint64_t *bar, const GD *groups, int k, int ntiles, int ngroups, int TW,
+                                           int ny, int BOXR, const CUtensorMap *tmap, const CUtensorMap *fmap) {
     const int job = (int)blockIdx.x + k * (int)gridDim.x;
     const int run = job / (ngroups * ntiles), jr = job - run * ngroups * ntiles;
     const int g = jr / ntiles, t = jr - g * ntiles;
-    const GD *G = groups + g;
-    for (int s = 0; s < G->nin; ++s) {
-        const int sl = run * NSLOT + G->in_slot[s];
-        for (int r0 = 0; r0 < ny; r0 += BOXR) tma_prefetch_2d(tmap, 2 * t * TW, sl * ny + r0);
-    }
+    const ColSrc src = col_src(groups + g, run, ny, tmap, fmap);
+    mbar_expect_tx(bar, (uint32_t)(TW * ny * sizeof(C)));
+    for (int r0 = 0; r0 < ny; r0 += BOXR) tma_load_2d(dst + (size_t)r0 * TW, src.map, 2 * t * TW, src.row + r0, bar);
+}
+
+// L2 prefetch of the tile kcol_issue would load for job k
+template <typename GD>
+__device__ __forceinline__ void kcol_prefetch(const GD *groups, int k, int ntiles, int ngroups, int TW, int ny, int BOXR,
+                                              const CUtensorMap *tmap, const CUtensorMap *fmap) {
+    const int job = (int)blockIdx.x + k * (int)gridDim.x;
+    const int run = job / (ngroups * ntiles), jr = job - run * ngroups * ntiles;
+    const int g = jr / ntiles, t = jr - g * ntiles;
+    const ColSrc src = col_src(groups + g, run, ny, tmap, fmap);
+    for (int r0 = 0; r0 < ny; r0 += BOXR) tma_prefetch_2d(src.map, 2 * t * TW, src.row + r0);
 }
 
 // Every group has one input and one output, which may be the same slot.
@@ -465,7 +468,8 @@ __global__ void __launch_bounds__(KCfg<real, KS_COL>::NT, KCfg<real, KS_COL>::MI
                                                                const typename cplx_of<real>::type *__restrict__ Wc_g,
                                                                const typename cplx_of<real>::type *__restrict__ Tc_g,
                                                                int ntc, KP<real> P, int TW, int BOXR, int nbuf,
-                                                               const __grid_constant__ CUtensorMap tmap, int *err) {
+                                                               const __grid_constant__ CUtensorMap tmap,
+                                                               const __grid_constant__ CUtensorMap fmap, int *err) {
     const uint4 *tc = TC ? P.tc16 : nullptr;   // split-BF16 tensor-core first passes
     using C = typename cplx_of<real>::type;
     constexpr int NT = KCfg<real, KS_COL>::NT;
@@ -504,12 +508,11 @@ __global__ void __launch_bounds__(KCfg<real, KS_COL>::NT, KCfg<real, KS_COL>::MI
     load_tab(kys, kyt, ny, NT);
     __syncthreads();
     if (tid == 0) {
-        if (njobs > 0) kcol_issue(buf0, &bar0, groups, 0, ntiles, ngroups, TW, ny, BOXR, &tmap);
-        if (nbuf > 1 && njobs > 1) kcol_issue(buf1, &bar1, groups, 1, ntiles, ngroups, TW, ny, BOXR, &tmap);
+        if (njobs > 0) kcol_issue(buf0, &bar0, groups, 0, ntiles, ngroups, TW, ny, BOXR, &tmap, &fmap);
+        if (nbuf > 1 && njobs > 1) kcol_issue(buf1, &bar1, groups, 1, ntiles, ngroups, TW, ny, BOXR, &tmap, &fmap);
     }
     uint32_t par0 = 0, par1 = 0;
     bool pend0 = njobs > 0, pend1 = nbuf > 1 && njobs > 1;
-    const real scale = P.scale;
     for (int k = 0; k < njobs; ++k) {
         const bool odd = k & 1;
         uint64_t *bar = odd ? &bar1 : &bar0;
@@ -538,28 +541,32 @@ __global__ void __launch_bounds__(KCfg<real, KS_COL>::NT, KCfg<real, KS_COL>::MI
             pend0 = false;
         }
         C *in0 = odd ? buf1 : buf0;
+        // (the tile at k_x = 0 needs no pairing of (k_y, -k_y): the DC and
+        // row-Nyquist columns its column 0 packs both take the multiplier at
+        // k_x = 0, as the Nyquist bin of k_x is zero)
+        const ColMult<real> m{(real)gd.c[0][0][0], (real)gd.c[0][0][1], (real)gd.c[0][0][2], (real)gd.c[0][0][3],
+                              (real)gd.c[0][0][4], (real)gd.scale, kxs, kys, kx0};
         const C *R;
         Lay lr;
-        if (pow2ny && kx0 != 0) {
-            // convection, power-of-two columns: forward passes, the last
-            // pass fused with the multiply and its adjoint, adjoint passes
-            // (splitting the tile's columns between two named-barrier
-            // halves measured slower: 228 -> 247 us at 1024^2, from the
-            // bank conflicts of half-width tiles)
-            const ColMult<real> m{(real)gd.c[0][0][0], (real)gd.c[0][0][1], (real)gd.c[0][0][2],
-                                  (real)gd.c[0][0][3], (real)gd.c[0][0][4], scale, kxs, kys, kx0};
+        if (pow2ny) {
+            // power-of-two columns: forward passes, the last pass fused with
+            // the multiply and its adjoint, adjoint passes (splitting the
+            // tile's columns between two named-barrier halves measured slower:
+            // 228 -> 247 us at 1024^2, from the bank conflicts of half-width
+            // tiles)
             const int w = pp_conv_p2<true>(in0, lt, wk0, lw, ny, TW, Tc, m, tid, NT, GroupSync{0, NT}, tc);
             R = w ? wk0 : in0;
             lr = w ? lw : lt;
         } else {
-            // convection (the tile holding k_x = 0 pairs (k_y, -k_y) of the
-            // packed DC / row-Nyquist column; other lengths): forward,
-            // multiply in place, inverse
+            // other lengths: forward, multiply in place, inverse
             const int w1 = pp_fft_any<-1, true, 0, 1>(in0, lt, wk0, lw, ny, TW, Wc, Tc, tid, NT, 4, tc);
             C *X = w1 ? wk0 : in0;
             C *Y = w1 ? in0 : wk0;
             const Lay lx = w1 ? lw : lt, ly = w1 ? lt : lw;
-            col_multiply<real>(X, lx, X, lx, X, lx, gd, 0, kxs, kys, kx0, TW, lgTW, ny, h, scale, NT);
+            for (int idx = tid; idx < tile; idx += NT) {
+                const int e = idx >> lgTW, c = idx & (TW - 1), at = lx(c, e);
+                X[at] = m(c, e, X[at]);
+            }
             __syncthreads();
             const int w2 = w1 ? pp_fft_any<+1, true, 1, 0>(X, lx, Y, ly, ny, TW, Wc, Tc, tid, NT, 4, tc)
                               : pp_fft_any<+1, true, 0, 1>(X, lx, Y, ly, ny, TW, Wc, Tc, tid, NT, 4, tc);
@@ -567,34 +574,15 @@ __global__ void __launch_bounds__(KCfg<real, KS_COL>::NT, KCfg<real, KS_COL>::MI
             lr = w2 ? ly : lx;
         }
         C *gout = spec_r + (size_t)gd.out_slot[0] * slot + kx0;
-        if (gd.add_slot >= 0) {   // plus the term the row kernel formed
-            // (4 loads before their stores: gout may alias ad, so a load
-            // after a store could not be issued ahead of it)
-            const C *ad = spec_r + (size_t)gd.add_slot * slot + kx0;
-            for (int i0 = tid; i0 < tile; i0 += 4 * NT) {
-                C a[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int idx = i0 + u * NT, e = idx >> lgTW, c = idx & (TW - 1);
-                    if (idx < tile) a[u] = ad[(size_t)e * h + c];
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int idx = i0 + u * NT, e = idx >> lgTW, c = idx & (TW - 1);
-                    if (idx < tile) gout[(size_t)e * h + c] = cadd(R[lr(c, e)], a[u]);
-                }
-            }
-        } else {
-            for (int idx = tid; idx < tile; idx += NT) {
-                const int e = idx >> lgTW, c = idx & (TW - 1);
-                gout[(size_t)e * h + c] = R[lr(c, e)];
-            }
+        for (int idx = tid; idx < tile; idx += NT) {
+            const int e = idx >> lgTW, c = idx & (TW - 1);
+            gout[(size_t)e * h + c] = R[lr(c, e)];
         }
         fence_proxy_async();
         __syncthreads();
         if (tid == 0 && k + nbuf < njobs) {
             const bool nodd = (k + nbuf) & 1;   // the barrier of job k + nbuf
-            kcol_issue(in0, nodd ? &bar1 : &bar0, groups, k + nbuf, ntiles, ngroups, TW, ny, BOXR, &tmap);
+            kcol_issue(in0, nodd ? &bar1 : &bar0, groups, k + nbuf, ntiles, ngroups, TW, ny, BOXR, &tmap, &fmap);
             if (nodd) pend1 = true;
             else pend0 = true;
         }
@@ -609,31 +597,25 @@ constexpr int NT3 = 256;
 
 // The level-1 derivatives K3 forms in the row spectrum (k3_src_slot), at
 // bin k of the one-sided rows of d (row o at d + o rs; bin 0 carries DC and
-// row-Nyquist, both with k_x = 0): row D_RX holds rho^, D_UXX u_x^, D_UYX
-// u_y^, D_TX T^, D_PIX Pi^, D_GX g^ as loaded; D_LAP holds d_yy rho, D_UYY
-// d_y u_y, D_UXY d_y u_x and D_DIVY d_yy u_y from the column pass.  ax = k_x of bin k, sx = 1 / nx.
+// row-Nyquist, both with k_x = 0).  ax = k_x of bin k, sx = 1 / nx.
 template <typename real, typename C>
 __device__ __forceinline__ void k3_form_x(C *d, int rs, int k, real ax, real sx) {
     const real m = ax * sx;
     const C r = d[D_RX * rs + k];
-    C lap = d[D_LAP * rs + k];
-    lap.x -= ax * m * r.x;
-    lap.y -= ax * m * r.y;
-    d[D_LAP * rs + k] = lap;                          // (d_xx + d_yy) rho
-    d[D_RX * rs + k] = imul(m, r);                    // d_x rho
+    d[D_LAP * rs + k] = C{-ax * m * r.x, -ax * m * r.y};   // d_xx rho
+    d[D_RX * rs + k] = imul(m, r);                         // d_x rho
     const C uxx = imul(m, d[D_UXX * rs + k]);
-    d[D_UXX * rs + k] = uxx;                          // d_x u_x
+    d[D_UXX * rs + k] = uxx;                               // d_x u_x
     d[D_DIVX * rs + k] = imul(ax, cadd(uxx, d[D_UYY * rs + k]));   // d_x (d_x u_x + d_y u_y)
-    d[D_UYX * rs + k] = imul(m, d[D_UYX * rs + k]);   // d_x u_y
-    d[D_DIVY * rs + k] = cadd(d[D_DIVY * rs + k], imul(ax, d[D_UXY * rs + k]));   // d_yy u_y + d_x (d_y u_x)
+    d[D_DIVY * rs + k] = imul(ax, d[D_UXY * rs + k]);      // d_x (d_y u_x)
+    d[D_UYX * rs + k] = imul(m, d[D_UYX * rs + k]);        // d_x u_y
     d[D_TX * rs + k] = imul(m, d[D_TX * rs + k]);
     d[D_PIX * rs + k] = imul(m, d[D_PIX * rs + k]);
     d[D_GX * rs + k] = imul(m, d[D_GX * rs + k]);
 }
 
 template <typename real, bool TC = false>
-__global__ void __launch_bounds__(NT3) k3_pipe(typename cplx_of<real>::type *spec, const real *__restrict__ fields,
-                                               real *__restrict__ aux,
+__global__ void __launch_bounds__(NT3) k3_pipe(typename cplx_of<real>::type *spec,
                                                const typename cplx_of<real>::type *__restrict__ Wr_g,
                                                const typename cplx_of<real>::type *__restrict__ Wp_g,
                                                const typename cplx_of<real>::type *__restrict__ Tr_g, int ntr,
@@ -645,18 +627,15 @@ __global__ void __launch_bounds__(NT3) k3_pipe(typename cplx_of<real>::type *spe
     __shared__ __align__(8) uint64_t bar;
     const int nx = P.nx, ny = P.ny, h = P.h, tid = threadIdx.x;
     const int run = (int)blockIdx.x / ny, y = (int)blockIdx.x - run * ny;   // one row of one run per block
-    const size_t N = (size_t)nx * ny, slot = (size_t)ny * h;
-    spec += (size_t)run * NSLOT * slot;
-    fields += (size_t)run * 4 * N;
-    aux += (size_t)run * 3 * N;
+    const size_t slot = (size_t)ny * h;
+    spec += (size_t)run * NSLOT * slot + (size_t)y * h;
     const int ph = padded_len(h);
     SmemCursor sc{smem_raw, 0u};
     C *Wr = (C *)sc.take(h * sizeof(C));
     C *Wp = (C *)sc.take(h * sizeof(C));
     C *Tr = (C *)sc.take(ntr * sizeof(C));
-    C *d = (C *)sc.take((size_t)ND1 * h * sizeof(C));
+    C *d = (C *)sc.take((size_t)NK3 * h * sizeof(C));
     C *wk = (C *)sc.take((size_t)WR * ph * sizeof(C));
-    real *rT = (real *)sc.take((size_t)2 * nx * sizeof(real));
     const Lay la{h, 1, 0}, lb{ph, 1, 1};
     const uint32_t rowbytes = (uint32_t)(nx * sizeof(real));
     if (tid == 0) {
@@ -665,12 +644,9 @@ __global__ void __launch_bounds__(NT3) k3_pipe(typename cplx_of<real>::type *spe
     }
     __syncthreads();   // the barrier is initialised before any thread polls it
     if (tid == 0) {
-        mbar_expect_tx(&bar, (uint32_t)(ND1 + 1) * rowbytes);   // D_DIVX is formed here
-        for (int o = 0; o < ND1; ++o)
-            if (k3_src_slot(o) >= 0)
-                bulk_g2s(d + (size_t)o * h, spec + (size_t)k3_src_slot(o) * slot + (size_t)y * h, rowbytes, &bar);
-        bulk_g2s(rT, fields + (size_t)y * nx, rowbytes, &bar);
-        bulk_g2s(rT + nx, fields + 3 * N + (size_t)y * nx, rowbytes, &bar);
+        mbar_expect_tx(&bar, (uint32_t)(NK3 - 3) * rowbytes);   // D_LAP, D_DIVX, D_DIVY are formed here
+        for (int o = 0; o < NK3; ++o)
+            if (k3_src_slot(o) >= 0) bulk_g2s(d + (size_t)o * h, spec + (size_t)k3_src_slot(o) * slot, rowbytes, &bar);
     }
     load_tab(Wr, Wr_g, h, NT3);
     load_tab(Wp, Wp_g, h, NT3);
@@ -681,59 +657,39 @@ __global__ void __launch_bounds__(NT3) k3_pipe(typename cplx_of<real>::type *spe
     }
     for (int k = tid; k < h; k += NT3) k3_form_x<real>(d, h, k, kxt[k], P.scale_x);
     __syncthreads();
-    c2r_pre_l(d, la, h, ND1, Wp, tid, NT3);
+    c2r_pre_l(d, la, h, NSP, Wp, tid, NT3);
     __syncthreads();
-    rows_fft_to_A<+1>(d, la, wk, lb, h, ND1, WR, Wr, Tr, NT3, maxlr, tc);
-    const C *res = d;
-    const Lay lr = la;
+    rows_fft_to_A<+1>(d, la, wk, lb, h, NSP, WR, Wr, Tr, NT3, maxlr, tc);
     real *dw = reinterpret_cast<real *>(d);
+    auto out = [&](int s) { return reinterpret_cast<real *>(spec + (size_t)s * slot); };
     for (int x = tid; x < nx; x += NT3) {
-        const size_t s = (size_t)y * nx + x;
-        const real rho = rT[x], T = rT[nx + x];
-        const real rx = real_at<real>(res, lr, D_RX, x), ry = real_at<real>(res, lr, D_RY, x);
-        const real lap = real_at<real>(res, lr, D_LAP, x);
-        const real uxx = real_at<real>(res, lr, D_UXX, x), uxy = real_at<real>(res, lr, D_UXY, x);
-        const real uyx = real_at<real>(res, lr, D_UYX, x), uyy = real_at<real>(res, lr, D_UYY, x);
-        const real divx = real_at<real>(res, lr, D_DIVX, x), divy = real_at<real>(res, lr, D_DIVY, x);
-        const real Tx = real_at<real>(res, lr, D_TX, x), Ty = real_at<real>(res, lr, D_TY, x);
-        const real Pix = real_at<real>(res, lr, D_PIX, x), Piy = real_at<real>(res, lr, D_PIY, x);
-        const real gx = real_at<real>(res, lr, D_GX, x), gy = real_at<real>(res, lr, D_GY, x);
-        const real M = P.K + P.H * T;
-        const real Pi = rho * T / (real(1) - P.b * rho) - P.a * rho * rho - rho * T;
-        const real grad2 = rx * rx + ry * ry;
-        const real iso = -(rho * T * (rx * gx + ry * gy)) - M * (rho * lap + real(0.5) * grad2);   // Eq. 19
-        const real Lxx = M * rx * rx + iso, Lxy = M * rx * ry, Lyy = M * ry * ry + iso;
-        const real div = uxx + uyy;
-        const real Ldu = Lxx * uxx + Lxy * (uyx + uxy) + Lyy * uyy;
-        const real Cn = Pi * div + Ldu - P.zeta * div * div + P.a * rho * rho * div +
-                        P.K * (real(-0.5) * grad2 * div - rho * (rx * divx + ry * divy) -
-                               (rx * (uxx * rx + uyx * ry) + ry * (uxy * rx + uyy * ry)));   // Eq. 22
-        aux[s] = Cn;
-        aux[N + s] = Pix - P.zeta * divx;   // Eq. 21 without d_b Lambda_ab
-        aux[2 * N + s] = Piy - P.zeta * divy;
-        const real q2 = real(2) * P.q * rho * T;   // Eq. 23
-        // rows 0..4 of d (same site, same thread)
-        dw[0 * nx + x] = Lxx;
-        dw[1 * nx + x] = Lxy;
-        dw[2 * nx + x] = Lyy;
-        dw[3 * nx + x] = q2 * Tx;
-        dw[4 * nx + x] = q2 * Ty;
+        const Level2<real> l = level2_site<real>([&](int o) { return dw[(size_t)o * nx + x]; }, P);
+        out(SLOT_L2)[x] = l.Lxy;
+        out(SLOT_L2 + 1)[x] = l.Lyy;
+        out(SLOT_L2 + 2)[x] = l.Phy;
+        // rows 0..2: transformed next; 3..5: the numerators their d_x joins
+        // (same site, same thread)
+        dw[x] = l.Phx;
+        dw[nx + x] = l.Lxx;
+        dw[2 * nx + x] = l.Lxy;
+        dw[3 * nx + x] = l.Cn;
+        dw[4 * nx + x] = l.Bx;
+        dw[5 * nx + x] = l.By;
     }
     __syncthreads();
-    rows_fft_to_A<-1>(d, la, wk, lb, h, 5, WR, Wr, Tr, NT3, maxlr, tc);
-    C *res2 = d;
-    const Lay lr2 = la;
-    r2c_post_l(res2, lr2, h, 5, Wp, tid, NT3);
+    rows_fft_to_A<-1>(d, la, wk, lb, h, 3, WR, Wr, Tr, NT3, maxlr, tc);
+    r2c_post_l(d, la, h, 3, Wp, tid, NT3);
     __syncthreads();
-    for (int r = 0; r < 5; ++r) {
-        C *raw = k3_raw_slot(r) >= 0 ? spec + (size_t)k3_raw_slot(r) * slot + (size_t)y * h : nullptr;
-        C *mul = k3_mul_slot(r) >= 0 ? spec + (size_t)k3_mul_slot(r) * slot + (size_t)y * h : nullptr;
-        for (int k = tid; k < h; k += NT3) {
-            const C X = res2[lr2(r, k)];
-            if (raw) raw[k] = X;
-            if (mul) mul[k] = imul(kxt[k] * P.scale_x, X);   // the d_x term of level 2
-        }
+    for (int i = tid; i < 3 * h; i += NT3) {
+        const int r = i / h, k = i - r * h;
+        d[la(r, k)] = imul(kxt[k] * P.scale_x, d[la(r, k)]);
     }
+    __syncthreads();
+    c2r_pre_l(d, la, h, 3, Wp, tid, NT3);
+    __syncthreads();
+    rows_fft_to_A<+1>(d, la, wk, lb, h, 3, WR, Wr, Tr, NT3, maxlr, tc);
+    for (int x = tid; x < nx; x += NT3)
+        for (int r = 0; r < 3; ++r) out(SLOT_A + r)[x] = dw[(size_t)(3 + r) * nx + x] + dw[(size_t)r * nx + x];
 }
 
 // ---------------------------------------------------------------------------
@@ -741,7 +697,7 @@ __global__ void __launch_bounds__(NT3) k3_pipe(typename cplx_of<real>::type *spe
 // ---------------------------------------------------------------------------
 
 constexpr int CHMAX5 = 8;
-constexpr int NHEAD = 10;   // dLx, dLy, dPhi spectra; rho, ux, uy, T; Cn, Bnx, Bny
+constexpr int NHEAD = 10;   // the d_y parts of the three divergences; rho, ux, uy, T; Cn, Bnx, Bny
 
 template <typename real>
 __device__ __forceinline__ void k5_issue_chunk(const typename cplx_of<real>::type *spec, real *dst, uint64_t *bar,
@@ -764,13 +720,12 @@ __device__ __forceinline__ void k5_issue_head(const typename cplx_of<real>::type
     const int yg = (int)blockIdx.x + ri * (int)gridDim.x;
     const int run = yg / ny, y = yg - run * ny;
     spec += (size_t)run * NSLOT * slot;
-    fields += (size_t)run * 4 * N;
-    aux += (size_t)run * 3 * N;
+    fields += (size_t)run * NSLOT * N;
+    aux += (size_t)run * NSLOT * N;
     const uint32_t rowbytes = (uint32_t)(nx * sizeof(real));
     mbar_expect_tx(bar, (uint32_t)NHEAD * rowbytes);
-    bulk_g2s(dst, spec + (size_t)(SLOT_L2 + 0) * slot + (size_t)y * h, rowbytes, bar);
-    bulk_g2s(dst + nx, spec + (size_t)(SLOT_L2 + 2) * slot + (size_t)y * h, rowbytes, bar);
-    bulk_g2s(dst + 2 * (size_t)nx, spec + (size_t)(SLOT_L2 + 3) * slot + (size_t)y * h, rowbytes, bar);
+    for (int r = 0; r < 3; ++r)   // d_y Lambda_xy, d_y Lambda_yy, d_y Phi_y
+        bulk_g2s(dst + (size_t)r * nx, spec + (size_t)(SLOT_L2 + r) * slot + (size_t)y * h, rowbytes, bar);
     for (int r = 0; r < 4; ++r)
         bulk_g2s(dst + (size_t)(3 + r) * nx, fields + (size_t)r * N + (size_t)y * nx, rowbytes, bar);
     for (int r = 0; r < 3; ++r)
@@ -875,12 +830,6 @@ __global__ void __launch_bounds__(KCfg<real, KS_K5>::NT, KCfg<real, KS_K5>::MINB
                 hpar0 ^= 1;
                 hpend0 = false;
             }
-            C *l2 = reinterpret_cast<C *>(H);
-            c2r_pre_l(l2, la, h, 3, Wp, tid, NT);
-            __syncthreads();
-            const int w = pp_fft_any<+1, false, 0, 1>(l2, la, wk, lb, h, 3, Wr, Tr, tid, NT, maxlr, tc);
-            const C *lres = w ? wk : l2;
-            const Lay llr = w ? lb : la;
             // per-site coefficients, written over the head rows (same site,
             // same thread): row 0 <- e0, 1 <- e1x, 2 <- e1y, 7 <- C + C_q,
             // 8 <- 1 / T
@@ -889,8 +838,7 @@ __global__ void __launch_bounds__(KCfg<real, KS_K5>::NT, KCfg<real, KS_K5>::MINB
                 const int x = tid + s * NT;
                 if (x < nx) {
                     const real rho = H[3 * nx + x], ux = H[4 * nx + x], uy = H[5 * nx + x], T = H[6 * nx + x];
-                    const real dLx = real_at<real>(lres, llr, 0, x), dLy = real_at<real>(lres, llr, 1, x);
-                    const real dPh = real_at<real>(lres, llr, 2, x);
+                    const real dLx = H[x], dLy = H[nx + x], dPh = H[2 * nx + x];
                     const real rT = rho * T;
                     const real inv2 = real(1) / (real(2) * rho * T * T);
                     const real Bx = (H[8 * nx + x] + dLx) / rT;      // Eq. 21
@@ -940,6 +888,9 @@ __global__ void __launch_bounds__(KCfg<real, KS_K5>::NT, KCfg<real, KS_K5>::MINB
         const int w = pp_fft_any<+1, false, 0, 1>(Bc, la, wk, lb, h, nv, Wr, Tr, tid, NT, maxlr, tc);
         const C *cres = w ? wk : Bc;
         const Lay lcr = w ? lb : la;
+        // v_x = 0: the convection term is real in its slot (its row went
+        // through the transforms above unused)
+        const real *creal = reinterpret_cast<const real *>(spec + (size_t)run * NSLOT * slot + (size_t)y * h);
         if (CH == 8) {
             // the chunk is ring c + 1 (velocities 1 + 8c .. 8 + 8c, Eq. 1):
             // one speed, one weight F_k, and directions known at compile time
@@ -975,7 +926,7 @@ __global__ void __launch_bounds__(KCfg<real, KS_K5>::NT, KCfg<real, KS_K5>::MINB
                     const real br = p0 + vu * (p1 + vu * (p2 + vu * (p3 + vu * p4)));
                     const real fe = rF * br;                                                 // Eq. 3
                     const real I = -(g0 + dir_dot<real>(r, exk, eyk)) * fe;                   // Eq. 11
-                    const real conv = real_at<real>(cres, lcr, r, x);
+                    const real conv = (r & 3) == 2 ? creal[(size_t)(v0 + r) * N + x] : real_at<real>(cres, lcr, r, x);
                     const real rhs = -conv - (fc[r] - fe) * itau + I;                        // Eq. 10
                     real fn = beta * (fc[r] + dt * rhs);
                     if (with_base) fn += alpha * fb[r];
@@ -1020,7 +971,7 @@ __global__ void __launch_bounds__(KCfg<real, KS_K5>::NT, KCfg<real, KS_K5>::MINB
                         rF = (k == 4) ? F[4] : rF;
                         const real fe = rho * rF * br;                                          // Eq. 3
                         const real I = -(e0 + e1x * vx + e1y * vy + CC * v2) * fe;              // Eq. 11
-                        const real conv = real_at<real>(cres, lcr, r, x);
+                        const real conv = vx == real(0) ? creal[(size_t)(v0 + r) * N + x] : real_at<real>(cres, lcr, r, x);
                         const real rhs = -conv - (fc[r] - fe) * itau + I;                       // Eq. 10
                         real fn = beta * (fc[r] + dt * rhs);
                         if (with_base) fn += alpha * fb[r];

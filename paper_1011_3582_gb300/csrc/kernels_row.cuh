@@ -21,10 +21,9 @@
 // the row's own buffer, P-point DFTs), generalised: E need not be a multiple
 // of P (lane j takes the P-point DFTs k1 = j, j + P, ... < E), rows are padded
 // in shared memory so that the row groups of one memory phase use different
-// banks, and the tables come from global memory through L1 (a table of its
-// own in each short-lived block's shared memory would be a tenth of its
-// traffic).  Inverse rows form the packed half-length spectrum straight from
-// global memory, with no staging copy.
+// banks, and the tables come by one bulk copy that overlaps the first loads
+// (through L1 they are cold in every launch).  Inverse rows form the packed
+// half-length spectrum straight from global memory, with no staging copy.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -33,6 +32,7 @@
 #include "fft_small.cuh"
 #include "row_kernels.h"
 #include "stage_layout.cuh"
+#include "stage_site.cuh"
 
 namespace fftlb {
 
@@ -43,19 +43,30 @@ namespace cg = cooperative_groups;
 // row configuration (see row_p in row_kernels.h)
 template <typename real, int H> struct Row {
     using C = typename cplx_of<real>::type;
-    static constexpr int P = row_p(H), E = H / P;
-    static constexpr int NT = row_nt(sizeof(real), H), NG = NT / P;   // threads, row groups
-    static constexpr int CS = row_cs(sizeof(real), H);                // blocks per row
+    static constexpr int P = row_p((int)sizeof(real), H), E = H / P;
+    static constexpr int NT = row_nt((int)sizeof(real), H), NG = NT / P;   // threads, row groups
+    static constexpr int CS = row_cs((int)sizeof(real), H);           // blocks per row
     static constexpr int CHN = 32 / CS;                               // distribution rows per block
-    static constexpr int RC = row_stride(sizeof(real), H);            // complex values between rows
+    static constexpr int RC = row_stride((int)sizeof(real), H);            // complex values between rows
     static constexpr int NX = 2 * H;
     static constexpr int NXS = NX / CS;                               // sites per block in the pointwise parts
+    static constexpr int NRING = CHN / 8;                             // rings of velocities per block
+    // n rows shared by the blocks, in units of the rows of one warp (a warp
+    // with one row takes as long as a full one, which is what counts in fp64):
+    // row r belongs to block owner(r), as its row local(r) < share(n)
+    static constexpr int RPW = 32 / P;
+    static __host__ __device__ constexpr int owner(int r) { return (r / RPW) % CS; }
+    static __host__ __device__ constexpr int local(int r) { return r / (RPW * CS) * RPW + r % RPW; }
+    static __host__ __device__ constexpr int share(int n) { return (n + RPW * CS - 1) / (RPW * CS) * RPW; }
+    // the i-th row of block c
+    static __host__ __device__ constexpr int nth(int c, int i) { return (i / RPW * CS + c) * RPW + i % RPW; }
 };
 
 // resident blocks per SM the register allocation allows for: 128 registers a
-// thread, fp64 168 (255 for the 24-point first stage)
+// thread, 255 for the 24-point first stage in fp64 (168 for all of fp64 was one
+// wave more for K3 on 256^2: 128 us against 95)
 template <typename real, int H> constexpr int row_minb() {
-    return Row<real, H>::NT >= 256 ? 2 : sizeof(real) == 4 ? 4 : Row<real, H>::E >= 24 ? 2 : 3;
+    return Row<real, H>::NT >= 256 ? 2 : sizeof(real) == 4 ? 4 : Row<real, H>::E >= 24 ? 2 : 4;
 }
 
 template <int P> __device__ __forceinline__ unsigned lanes_of_row() {
@@ -65,13 +76,31 @@ template <int P> __device__ __forceinline__ unsigned lanes_of_row() {
 
 template <typename T> __device__ __forceinline__ T ldro(const T *p) { return __ldg(p); }
 
+// The table block [wh][kx][tw][wp] (row_table): K1 takes its first three
+// parts, K5 the last two, K3 all.
+template <typename real, int H> struct Tab {
+    using C = typename cplx_of<real>::type;
+    using L = RowTable<real>;
+    const C *wh, *tw, *wp;
+    const real *kx;
+    // in shared memory at p, holding the parts from byte `from` on
+    __device__ __forceinline__ Tab(const unsigned char *p, unsigned from)
+        : wh(reinterpret_cast<const C *>(p - from)), tw(reinterpret_cast<const C *>(p + L::tw(H) - from)),
+          wp(reinterpret_cast<const C *>(p + L::wp(H) - from)), kx(reinterpret_cast<const real *>(p + L::kx(H) - from)) {}
+};
+// thread 0: barrier, then the copy of bytes [from, to) of the block to dst
+template <typename C>
+__device__ __forceinline__ void table_issue(unsigned char *dst, const C *tab, unsigned from, unsigned to, uint64_t *bar) {
+    bulk_g2s(dst, reinterpret_cast<const unsigned char *>(tab) + from, to - from, bar);
+}
+
 // Position of stage-1 output (l, k1) in the row buffer.
 template <int P> __device__ __forceinline__ int tp(int l, int k1) { return k1 * P + (l ^ (k1 & (P - 1))); }
 
 // In-place DFT (DIR = -1) or unnormalised inverse (+1) of the H values at z
 // by lane j of the row's P lanes; tw[k1 P + l] = exp(-2 pi i l k1 / H).
 template <int H, int DIR, typename C>
-__device__ __forceinline__ void row_fft(C *z, const C *__restrict__ tw, int j) {
+__device__ __forceinline__ void row_fft(C *z, const C *tw, int j) {
     using real = decltype(z[0].x);
     constexpr int P = Row<real, H>::P, E = Row<real, H>::E;
     const unsigned gm = lanes_of_row<P>();
@@ -81,7 +110,7 @@ __device__ __forceinline__ void row_fft(C *z, const C *__restrict__ tw, int j) {
     SmallDFT<E, DIR, C>::run(v);
 #pragma unroll
     for (int k1 = 1; k1 < E; ++k1) {
-        C w = ldro(tw + k1 * P + j);
+        C w = tw[k1 * P + j];
         if (DIR > 0) w.y = -w.y;
         v[k1] = cmul(v[k1], w);
     }
@@ -150,7 +179,7 @@ __device__ __forceinline__ void row_fft(C *z, const C *__restrict__ tw, int j) {
 // Z[H-k]: X[k] = s/2 + w, X[H-k] = conj(s/2 - w), w = -i/2 exp(-2 pi i k / 2H)
 // d; wh[k] = exp(-2 pi i k / 2H) / 2.
 template <int H, typename C, typename Put>
-__device__ __forceinline__ void row_post(const C *z, const C *__restrict__ wh, int j, const Put &put) {
+__device__ __forceinline__ void row_post(const C *z, const C *wh, int j, const Put &put) {
     using R = decltype(z[0].x);
     constexpr int P = Row<R, H>::P;
 #pragma unroll
@@ -163,19 +192,21 @@ __device__ __forceinline__ void row_post(const C *z, const C *__restrict__ wh, i
         } else {
             const C p = z[k], q = z[H - k];
             const C s = cadd(p, cconj(q)), d = csub(p, cconj(q));
-            const C w = cmul(ldro(wh + k), cmul_mi(d));
+            const C w = cmul(wh[k], cmul_mi(d));
             put(k, C{R(0.5) * s.x + w.x, R(0.5) * s.y + w.y});
             if (H - k != k) put(H - k, C{R(0.5) * s.x - w.x, -(R(0.5) * s.y - w.y)});
         }
     }
 }
 
-// One-sided spectrum get(k), k < H -> the packed half-length spectrum Z in z
-// (Z[k] = a + i d conj(w), Z[H-k] = conj(a - i d conj(w)), a = X[k] + conj
-// X[H-k], d = X[k] - conj X[H-k], w = exp(-2 pi i k / 2H)); U pairs of loads in
-// flight.
-template <int H, typename C, typename Get>
-__device__ __forceinline__ void row_pre(C *z, const C *__restrict__ wp, int j, const Get &get) {
+// One-sided spectrum X[k] = form(k, a[k], b[k]), k < H, from the global rows a
+// (and b, NS = 2) -> the packed half-length spectrum Z in z (Z[k] = t + i d
+// conj(w), Z[H-k] = conj(t - i d conj(w)), t = X[k] + conj X[H-k], d = X[k] - conj
+// X[H-k], w = exp(-2 pi i k / 2H)); U pairs of loads in flight, ready() between
+// the first ones and their use.
+template <int H, int NS, typename C, typename Form, typename Ready>
+__device__ __forceinline__ void row_pre(C *z, const C *wp, int j, const C *__restrict__ a, const C *__restrict__ b,
+                                        const Form &form, const Ready &ready) {
     using R = decltype(z[0].x);
     constexpr int P = Row<R, H>::P, NK = H / (2 * P);   // k = j + P i, i < NK, and k = H / 2
     constexpr int UM = sizeof(R) == 8 ? 4 : 8;
@@ -183,26 +214,32 @@ __device__ __forceinline__ void row_pre(C *z, const C *__restrict__ wp, int j, c
     static_assert(H % (2 * P) == 0, "row configuration");
 #pragma unroll 1
     for (int i0 = 0; i0 < NK; i0 += U) {
-        C p[U], q[U];
+        C pa[U], qa[U], pb[NS > 1 ? U : 1], qb[NS > 1 ? U : 1];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int k = j + P * (i0 + u);
-            p[u] = get(k);
-            q[u] = get(k == 0 ? H / 2 : H - k);   // (lane 0's first pair: bins 0 and H / 2)
+            const int k = j + P * (i0 + u), kc = k == 0 ? H / 2 : H - k;   // (lane 0's first pair: bins 0 and H / 2)
+            pa[u] = ldro(a + k);
+            qa[u] = ldro(a + kc);
+            if constexpr (NS > 1) {
+                pb[u] = ldro(b + k);
+                qb[u] = ldro(b + kc);
+            }
         }
+        if (i0 == 0) ready();
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int k = j + P * (i0 + u);
+            const int k = j + P * (i0 + u), kc = k == 0 ? H / 2 : H - k;
+            const C p = form(k, pa[u], pb[NS > 1 ? u : 0]), q = form(kc, qa[u], qb[NS > 1 ? u : 0]);
             if (k == 0) {
-                z[0] = C{p[u].x + p[u].y, p[u].x - p[u].y};
-                // k = H / 2: a = 2 Re X, d = 2 i Im X, i d conj(w) = -2 i Im X
+                z[0] = C{p.x + p.y, p.x - p.y};
+                // k = H / 2: t = 2 Re X, d = 2 i Im X, i d conj(w) = -2 i Im X
                 // with w = -i: Z = 2 conj X
-                z[H / 2] = C{R(2) * q[u].x, R(-2) * q[u].y};
+                z[H / 2] = C{R(2) * q.x, R(-2) * q.y};
             } else {
-                const C a = cadd(p[u], cconj(q[u])), d = csub(p[u], cconj(q[u]));
-                const C t = cmul_i(cmul(d, cconj(ldro(wp + k))));
-                z[k] = cadd(a, t);
-                z[H - k] = cconj(csub(a, t));
+                const C t = cadd(p, cconj(q)), d = csub(p, cconj(q));
+                const C e = cmul_i(cmul(d, cconj(wp[k])));
+                z[k] = cadd(t, e);
+                z[H - k] = cconj(csub(t, e));
             }
         }
     }
@@ -226,6 +263,14 @@ __device__ __forceinline__ float wk(const RowArgs<float> &A, int k, float T) {
     return T * (s + c);
 }
 
+// this thread's bounded wait for the tables; running out is recorded
+__device__ __forceinline__ void table_wait(uint64_t *bar, int *err) {
+    if (!mbar_wait_bounded(bar, 0)) {
+        atomicOr(err, kErrWaitTimeout);
+        mbar_wait_bounded(bar, 0);
+    }
+}
+
 template <int CS> __device__ __forceinline__ int block_rank() {
     if constexpr (CS == 1) return 0;
     else return (int)cg::this_cluster().block_rank();
@@ -247,24 +292,36 @@ template <int CS, typename T> __device__ __forceinline__ T *in_block(T *p, int r
 
 // ---------------------------------------------------------------------------
 // K1: moments rho, u, T (Eqs. 7-9), Pi = P^w - rho T (Eq. 18), g = M/T, and the
-// forward rows of the 32 moving f_i and of rho, u_x, u_y, T, Pi, g.  Block c of
-// the row takes f_i, i = 1 + c CHN ..: it sums their share of the moments,
-// transforms them while the other blocks' sums arrive, forms the fields of
-// its slice of sites and sends each to the block that transforms it.
+// forward rows of the f_i with v_x != 0 and of rho, u_x, u_y, T, Pi, g.  Block c
+// of the row takes f_i, i = 1 + c CHN ..: it sums their share of the moments,
+// forms the fields of its slice of sites from everybody's sums, sends each
+// field to the block that transforms it, and then transforms its f_i and its
+// share of the fields together (the fields after the f_i, hiding the exchange,
+// took a second pass of the same length: 51 us against 37 on six 512x4 fp64
+// slabs).
 // ---------------------------------------------------------------------------
 
 template <typename real, int H>
 __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k1_row(const __grid_constant__ RowArgs<real> A) {
     using G = Row<real, H>;
     using C = typename G::C;
-    constexpr int CS = G::CS, CHN = G::CHN, RC = G::RC, NX = G::NX, NT = G::NT, P = G::P, NXS = G::NXS;
-    constexpr int NF = (6 + CS - 1) / CS;   // field rows per block
+    constexpr int CS = G::CS, CHN = G::CHN, RC = G::RC, NX = G::NX, NT = G::NT, P = G::P, NXS = G::NXS, NR = G::NRING;
     extern __shared__ __align__(128) unsigned char row_smem[];
     __shared__ __align__(8) uint64_t bar;
-    C *B = reinterpret_cast<C *>(row_smem);                       // [CHN + 1] rows
-    C *F = B + (CHN + 1) * RC;                                    // [NF] field rows
-    real *pm = reinterpret_cast<real *>(F + NF * RC);             // [4][NX] partial moments
-    const int tid = threadIdx.x, c = block_rank<CS>(), j = tid & (P - 1), grp = tid / P;
+    using LT = RowTable<real>;
+    C *B = reinterpret_cast<C *>(row_smem);     // [CHN + 1] rows
+    C *F = B + (CHN + 1) * RC;                  // [share(6)] field rows
+    C *S = F + G::share(6) * RC;                // [2 NR - 1] rows: partial moments, see pm
+    unsigned char *tb = reinterpret_cast<unsigned char *>(S + (2 * NR - 1) * RC);
+    const Tab<real, H> T(tb, 0);
+    // partial moment m of ring rr: two take the rows of the ring's directions 2
+    // and 6, which no transform needs (each site's values are read and replaced
+    // by one thread), one of all the rest velocity's row, the others rows of S
+    auto pm = [&](int rr, int m) -> real * {
+        C *p = m < 2 ? B + (rr * 8 + 2 + 4 * m) * RC : m == 2 && rr == 0 ? B + CHN * RC : S + (2 * rr + m - 3) * RC;
+        return reinterpret_cast<real *>(p);
+    };
+    const int c = block_rank<CS>(), tid = (int)threadIdx.x, j = tid & (P - 1), grp = tid / P;
     const int ny = A.ny, yg = (int)blockIdx.x / CS, run = yg / ny, y = yg - run * ny;
     const size_t N = (size_t)NX * ny, slot = (size_t)ny * H;
     const real *f = A.f + (size_t)run * Q * N + (size_t)y * NX;
@@ -276,94 +333,100 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k1_row(
     }
     __syncthreads();
     if (tid == 0) {
-        mbar_expect_tx(&bar, (uint32_t)(nrow * NX * sizeof(real)));
+        mbar_expect_tx(&bar, (uint32_t)(nrow * NX * sizeof(real)) + LT::wp(H));
         for (int r = 0; r < CHN; ++r)
             bulk_g2s(B + r * RC, f + (size_t)(1 + c * CHN + r) * N, NX * sizeof(real), &bar);
         if (c == 0) bulk_g2s(B + CHN * RC, f, NX * sizeof(real), &bar);
+        table_issue(tb, A.tab, 0, LT::wp(H), &bar);
     }
     // (a wait that runs out is recorded and the row carries on: leaving early
     // would pull this block's shared memory from under the others)
     if (!block_wait(&bar, 0, A.err)) mbar_wait_bounded(&bar, 0);
-    for (int x = tid; x < NX; x += NT) {
-        real m0 = 0, m1 = 0, m2 = 0, m3 = 0;
-        if (c == 0) m0 = reinterpret_cast<const real *>(B + CHN * RC)[x];
-#pragma unroll 8
-        for (int r = 0; r < CHN; ++r) {
-            const int i = 1 + c * CHN + r;
-            const real v = reinterpret_cast<const real *>(B + r * RC)[x];
-            m0 += v;
-            m1 += A.vx[i] * v;
-            m2 += A.vy[i] * v;
-            m3 += A.v2[i] * v;
-        }
-        pm[x] = m0;
-        pm[NX + x] = m1;
-        pm[2 * NX + x] = m2;
-        pm[3 * NX + x] = m3;
+    // one ring at one site: speed s, directions r pi / 4 (19 operations instead
+    // of 32 with the velocities one by one)
+    const real hh = real(0.70710678118654752440);
+    for (int it = tid; it < NR * NX; it += NT) {
+        const int rr = NR == 1 ? 0 : it / NX, x = NR == 1 ? it : it - rr * NX;
+        const int v0 = 1 + c * CHN + 8 * rr;
+        const real sk = A.vx[v0], sk2 = A.v2[v0];
+        real v[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = reinterpret_cast<const real *>(B + (rr * 8 + r) * RC)[x];
+        const real d04 = v[0] - v[4], d15 = v[1] - v[5], d26 = v[2] - v[6], d37 = v[3] - v[7];
+        const real sum = ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+        real m0 = sum;
+        if (c == 0 && rr == 0) m0 += reinterpret_cast<const real *>(B + CHN * RC)[x];
+        pm(rr, 0)[x] = m0;
+        pm(rr, 1)[x] = sk * (d04 + hh * (d15 - d37));
+        pm(rr, 2)[x] = sk * (d26 + hh * (d15 + d37));
+        pm(rr, 3)[x] = sk2 * sum;
     }
     row_arrive<CS>();
-    __syncthreads();
-#pragma unroll 1
-    for (int r = grp; r < CHN; r += G::NG) {
-        const int i = 1 + c * CHN + r;
-        C *z = B + r * RC;
-        row_fft<H, -1>(z, A.tw, j);
-        C *dst = spec + (size_t)(i - 1) * slot;
-        if (A.vy[i] == real(0)) {   // i v_x k_x f^ / nx, no column pass
-            const real sx = A.vx[i] * A.scale_x;
-            row_post<H>(z, A.wh, j, [&](int k, C X) {
-                const real m = ldro(A.kx + k) * sx;
-                dst[k] = C{-m * X.y, m * X.x};
-            });
-        } else {
-            row_post<H>(z, A.wh, j, [&](int k, C X) { dst[k] = X; });
-        }
-    }
     row_wait<CS>();
-    real *fields = A.fields + (size_t)run * 4 * N + (size_t)y * NX;
     for (int x = c * NXS + tid; x < (c + 1) * NXS; x += NT) {
         real m0 = 0, m1 = 0, m2 = 0, m3 = 0;
 #pragma unroll
         for (int b = 0; b < CS; ++b) {
-            const real *q = in_block<CS>(pm, b);
-            m0 += q[x];
-            m1 += q[NX + x];
-            m2 += q[2 * NX + x];
-            m3 += q[3 * NX + x];
+#pragma unroll
+            for (int rr = 0; rr < NR; ++rr) {
+                m0 += in_block<CS>(pm(rr, 0), b)[x];
+                m1 += in_block<CS>(pm(rr, 1), b)[x];
+                m2 += in_block<CS>(pm(rr, 2), b)[x];
+                m3 += in_block<CS>(pm(rr, 3), b)[x];
+            }
         }
         const real rho = m0, ux = m1 / m0, uy = m2 / m0;
-        const real T = real(0.5) * (m3 / m0 - (ux * ux + uy * uy));
-        fields[x] = rho;
-        fields[N + x] = ux;
-        fields[2 * N + x] = uy;
-        fields[3 * N + x] = T;
-        const real lv[6] = {rho, ux, uy, T, rho * T / (real(1) - A.b * rho) - A.a * rho * rho - rho * T,   // Eq. 18
-                            (A.K + A.H * T) / T};                                                          // M / T
+        const real Te = real(0.5) * (m3 / m0 - (ux * ux + uy * uy));
+        const real lv[6] = {rho, ux, uy, Te, rho * Te / (real(1) - A.b * rho) - A.a * rho * rho - rho * Te,   // Eq. 18
+                            (A.K + A.H * Te) / Te};                                                        // M / T
 #pragma unroll
-        for (int r = 0; r < 6; ++r) reinterpret_cast<real *>(in_block<CS>(F + (r / CS) * RC, r % CS))[x] = lv[r];
+        for (int r = 0; r < 6; ++r)
+            reinterpret_cast<real *>(in_block<CS>(F + G::local(r) * RC, G::owner(r)))[x] = lv[r];
     }
     row_arrive<CS>();
     row_wait<CS>();
-    for (int r = c + CS * grp; r < 6; r += CS * G::NG) {
-        C *z = F + (r / CS) * RC;
-        row_fft<H, -1>(z, A.tw, j);
-        C *dst = spec + (size_t)(SLOT_RHO + r) * slot;
-        row_post<H>(z, A.wh, j, [&](int k, C X) { dst[k] = X; });
+    // this block's distribution rows and its share of the field rows, one row
+    // group each: 6 of every 8 directions leave room for the fields
+    static_assert(6 * NR + G::share(6) <= G::NG, "one pass");
+    if (grp < 6 * NR) {
+        const int rr = NR == 1 ? 0 : grp / 6, r = rr * 8 + ring_dir(grp - 6 * rr), i = 1 + c * CHN + r;
+        C *z = B + r * RC;
+        row_fft<H, -1>(z, T.tw, j);
+        C *dst = spec + (size_t)(i - 1) * slot;
+        if (A.vy[i] == real(0)) {   // i v_x k_x f^ / nx, no column pass
+            const real sx = A.vx[i] * A.scale_x;
+            row_post<H>(z, T.wh, j, [&](int k, C X) {
+                const real m = T.kx[k] * sx;
+                dst[k] = C{-m * X.y, m * X.x};
+            });
+        } else {
+            row_post<H>(z, T.wh, j, [&](int k, C X) { dst[k] = X; });
+        }
+    } else {
+        const int q = grp - 6 * NR, r = G::nth(c, q);
+        if (q < G::share(6) && r < 6) {
+            C *z = F + q * RC;
+            C *real_row = spec + (size_t)(SLOT_F + r) * slot, *dst = spec + (size_t)(SLOT_RHO + r) * slot;
+#pragma unroll
+            for (int k = j; k < H; k += P) real_row[k] = z[k];
+            row_fft<H, -1>(z, T.tw, j);
+            row_post<H>(z, T.wh, j, [&](int k, C X) { dst[k] = X; });
+        }
     }
 }
 
 template <typename real, int H> size_t k1_row_smem() {
     using G = Row<real, H>;
-    return (size_t)(G::CHN + 1 + (6 + G::CS - 1) / G::CS) * G::RC * 2 * sizeof(real) + (size_t)4 * G::NX * sizeof(real);
+    return (size_t)(G::CHN + 1 + G::share(6) + 2 * G::NRING - 1) * G::RC * 2 * sizeof(real) + RowTable<real>::wp(H);
 }
 
 // ---------------------------------------------------------------------------
-// K3: inverse rows of the 15 level-1 derivatives (those with a factor k_x
-// formed here from the row spectra, stage_layout.cuh) -> Lambda (Eq. 19),
-// Phi = 2 q rho T grad T (Eq. 23), the numerators of C (Eq. 22) and B (Eq. 21)
-// -> forward rows of Lambda_xx, Lambda_xy, Lambda_yy, Phi_x, Phi_y.  Block c of
-// the row transforms the derivative rows o = c, c + CS, ..., takes its slice
-// of the sites, and transforms the output rows r = c, c + CS, ....
+// K3: inverse rows of the 11 level-1 derivatives that have a factor k_x or
+// start from a row spectrum (stage_layout.cuh) -> Lambda (Eq. 19), Phi (Eq. 23),
+// the numerators of C (Eq. 22) and B (Eq. 21) -> the row spectra of d_x of Phi_x,
+// Lambda_xx, Lambda_xy.  Their inverse rows are K5's, which has row groups to
+// spare for them; here they would be a third pass in a row (68 us against 52
+// on six 512x4 fp64 slabs).
 // ---------------------------------------------------------------------------
 
 template <typename real, int H>
@@ -371,110 +434,117 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k3_row(
     using G = Row<real, H>;
     using C = typename G::C;
     constexpr int CS = G::CS, RC = G::RC, NX = G::NX, NT = G::NT, P = G::P, NXS = G::NXS;
-    constexpr int ND = (ND1 + CS - 1) / CS, NL = (5 + CS - 1) / CS;
+    constexpr int ND = G::share(NSP), NL = G::share(3);
     extern __shared__ __align__(128) unsigned char row_smem[];
     C *D = reinterpret_cast<C *>(row_smem);   // [ND] derivative rows
-    C *L = D + ND * RC;                       // [NL] output rows
-    const int tid = threadIdx.x, c = block_rank<CS>(), j = tid & (P - 1), grp = tid / P;
+    C *L = D + ND * RC;                       // [NL] Phi_x, Lambda_xx, Lambda_xy
+    using LT = RowTable<real>;
+    unsigned char *tb = reinterpret_cast<unsigned char *>(L + NL * RC);
+    const Tab<real, H> T(tb, 0);
+    __shared__ __align__(8) uint64_t bar;
+    const int c = block_rank<CS>(), tid = (int)threadIdx.x, j = tid & (P - 1), grp = tid / P;
     const int ny = A.ny, yg = (int)blockIdx.x / CS, run = yg / ny, y = yg - run * ny;
-    const size_t N = (size_t)NX * ny, slot = (size_t)ny * H;
+    const size_t slot = (size_t)ny * H;
     C *spec = A.spec + (size_t)run * NSLOT * slot + (size_t)y * H;
     const real sx = A.scale_x;
-    const real *__restrict__ kx = A.kx;
+    const real *kx = T.kx;
+    if (tid == 0) {
+        mbar_init(&bar, 1);
+        mbar_init_fence();
+        mbar_expect_tx(&bar, LT::bytes(H));
+        table_issue(tb, A.tab, 0, LT::bytes(H), &bar);
+    }
+    __syncthreads();
+    bool first = true;
+    auto ready = [&]() {   // the tables are there (a wait that runs out is recorded; see k1_row)
+        if (first) table_wait(&bar, A.err);
+        first = false;
+    };
+    // the real rows of this block's slice of sites into L2 (if they are not
+    // there) ahead of the pointwise part
+    if (tid < NK3 - NSP)
+        bulk_prefetch_l2(reinterpret_cast<const real *>(spec + (size_t)k3_src_slot(NSP + tid) * slot) + c * NXS,
+                         NXS * sizeof(real));
 #pragma unroll 1
-    for (int o = c + CS * grp; o < ND1; o += CS * G::NG) {
-        C *z = D + (o / CS) * RC;
+    for (int q = grp; q < ND; q += G::NG) {
+        const int o = G::nth(c, q);
+        if (o >= NSP) continue;
+        C *z = D + q * RC;
         // (none of the slots read here is written by this launch)
-        const C *__restrict__ s0 = spec + (size_t)(o == D_DIVX ? SLOT_UX : k3_src_slot(o)) * slot;
-        if (o == D_LAP) {   // (d_xx + d_yy) rho
-            const C *__restrict__ s1 = spec + (size_t)SLOT_RHO * slot;
-            row_pre<H>(z, A.wp, j, [&](int k) {
-                const C a = ldro(s0 + k), b = ldro(s1 + k);
-                const real ax = ldro(kx + k), m = ax * sx;
-                return C{a.x - ax * m * b.x, a.y - ax * m * b.y};
-            });
+        const int s = o == D_LAP ? SLOT_RHO : o == D_DIVX ? SLOT_UX : o == D_DIVY ? SLOT_D1 + D1_UXY : k3_src_slot(o);
+        const C *__restrict__ s0 = spec + (size_t)s * slot;
+        if (o == D_LAP) {   // d_xx rho
+            row_pre<H, 1>(z, T.wp, j, s0, s0, [&](int k, C a, C) {
+                const real ax = kx[k], m = -ax * (ax * sx);
+                return C{m * a.x, m * a.y};
+            }, ready);
         } else if (o == D_DIVX) {   // d_x (d_x u_x + d_y u_y)
-            const C *__restrict__ s1 = spec + (size_t)(SLOT_D1 + D_UYY) * slot;
-            row_pre<H>(z, A.wp, j, [&](int k) {
-                const C a = ldro(s0 + k), b = ldro(s1 + k);
-                const real ax = ldro(kx + k), m = ax * sx;
+            row_pre<H, 2>(z, T.wp, j, s0, spec + (size_t)(SLOT_D1 + D1_UYY) * slot, [&](int k, C a, C b) {
+                const real ax = kx[k], m = ax * sx;
                 const C w = C{b.x - m * a.y, b.y + m * a.x};
                 return C{-ax * w.y, ax * w.x};
-            });
-        } else if (o == D_DIVY) {   // d_yy u_y + d_x (d_y u_x)
-            const C *__restrict__ s1 = spec + (size_t)(SLOT_D1 + D_UXY) * slot;
-            row_pre<H>(z, A.wp, j, [&](int k) {
-                const C a = ldro(s0 + k), b = ldro(s1 + k);
-                const real ax = ldro(kx + k);
-                return C{a.x - ax * b.y, a.y + ax * b.x};
-            });
-        } else if (o == D_RX || o == D_UXX || o == D_UYX || o == D_TX || o == D_PIX || o == D_GX) {   // d_x
-            row_pre<H>(z, A.wp, j, [&](int k) {
-                const C a = ldro(s0 + k);
-                const real m = ldro(kx + k) * sx;
+            }, ready);
+        } else if (o == D_UXY || o == D_UYY) {   // d_y, from the column pass
+            row_pre<H, 1>(z, T.wp, j, s0, s0, [](int, C a, C) { return a; }, ready);
+        } else {   // d_x (of d_y u_x, which carries its 1 / nx, for D_DIVY)
+            const real sm = o == D_DIVY ? real(1) : sx;
+            row_pre<H, 1>(z, T.wp, j, s0, s0, [&](int k, C a, C) {
+                const real m = kx[k] * sm;
                 return C{-m * a.y, m * a.x};
-            });
-        } else {   // d_y, from the column pass
-            row_pre<H>(z, A.wp, j, [&](int k) { return ldro(s0 + k); });
+            }, ready);
         }
         __syncwarp(lanes_of_row<P>());
-        row_fft<H, +1>(z, A.tw, j);
+        row_fft<H, +1>(z, T.tw, j);
     }
     row_arrive<CS>();
     row_wait<CS>();
-    const real *fields = A.fields + (size_t)run * 4 * N + (size_t)y * NX;
-    real *aux = A.aux + (size_t)run * 3 * N + (size_t)y * NX;
+    ready();   // (a group without a derivative row has not waited yet)
+    auto row = [&](int s) { return reinterpret_cast<real *>(spec + (size_t)s * slot); };
     for (int x = c * NXS + tid; x < (c + 1) * NXS; x += NT) {
-        const real rho = fields[x], T = fields[3 * N + x];
-        real d[ND1];
+        real d[NK3];
 #pragma unroll
-        for (int o = 0; o < ND1; ++o) d[o] = reinterpret_cast<const real *>(in_block<CS>(D + (o / CS) * RC, o % CS))[x];
-        const real rx = d[D_RX], ry = d[D_RY], div = d[D_UXX] + d[D_UYY];
-        const real M = A.K + A.H * T;
-        const real Pi = rho * T / (real(1) - A.b * rho) - A.a * rho * rho - rho * T;
-        const real grad2 = rx * rx + ry * ry;
-        const real iso = -(rho * T * (rx * d[D_GX] + ry * d[D_GY])) - M * (rho * d[D_LAP] + real(0.5) * grad2);   // Eq. 19
-        const real Lxx = M * rx * rx + iso, Lxy = M * rx * ry, Lyy = M * ry * ry + iso;
-        const real Ldu = Lxx * d[D_UXX] + Lxy * (d[D_UYX] + d[D_UXY]) + Lyy * d[D_UYY];
-        const real Cn = Pi * div + Ldu - A.zeta * div * div + A.a * rho * rho * div +
-                        A.K * (real(-0.5) * grad2 * div - rho * (rx * d[D_DIVX] + ry * d[D_DIVY]) -
-                               (rx * (d[D_UXX] * rx + d[D_UYX] * ry) + ry * (d[D_UXY] * rx + d[D_UYY] * ry)));   // Eq. 22
-        aux[x] = Cn;
-        aux[N + x] = d[D_PIX] - A.zeta * d[D_DIVX];   // Eq. 21 without d_b Lambda_ab
-        aux[2 * N + x] = d[D_PIY] - A.zeta * d[D_DIVY];
-        const real q2 = real(2) * A.q * rho * T;   // Eq. 23
-        const real lv[5] = {Lxx, Lxy, Lyy, q2 * d[D_TX], q2 * d[D_TY]};
+        for (int o = NSP; o < NK3; ++o) d[o] = row(k3_src_slot(o))[x];
 #pragma unroll
-        for (int r = 0; r < 5; ++r) reinterpret_cast<real *>(in_block<CS>(L + (r / CS) * RC, r % CS))[x] = lv[r];
+        for (int o = 0; o < NSP; ++o)
+            d[o] = reinterpret_cast<const real *>(in_block<CS>(D + G::local(o) * RC, G::owner(o)))[x];
+        const Level2<real> l = level2_site<real>([&](int o) { return d[o]; }, A);
+        const real lv[3] = {l.Phx, l.Lxx, l.Lxy};
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+            reinterpret_cast<real *>(in_block<CS>(L + G::local(r) * RC, G::owner(r)))[x] = lv[r];
+        row(SLOT_A)[x] = l.Cn;
+        row(SLOT_A + 1)[x] = l.Bx;
+        row(SLOT_A + 2)[x] = l.By;
+        row(SLOT_L2)[x] = l.Lxy;
+        row(SLOT_L2 + 1)[x] = l.Lyy;
+        row(SLOT_L2 + 2)[x] = l.Phy;
     }
     row_arrive<CS>();
     row_wait<CS>();
-    for (int r = c + CS * grp; r < 5; r += CS * G::NG) {
-        C *z = L + (r / CS) * RC;
-        row_fft<H, -1>(z, A.tw, j);
-        C *raw = k3_raw_slot(r) >= 0 ? spec + (size_t)k3_raw_slot(r) * slot : nullptr;
-        C *mul = k3_mul_slot(r) >= 0 ? spec + (size_t)k3_mul_slot(r) * slot : nullptr;
-        row_post<H>(z, A.wh, j, [&](int k, C X) {
-            if (raw) raw[k] = X;
-            if (mul) {   // the d_x term of level 2
-                const real m = ldro(kx + k) * sx;
-                mul[k] = C{-m * X.y, m * X.x};
-            }
+    for (int q = grp; q < NL; q += G::NG) {
+        const int r = G::nth(c, q);
+        if (r >= 3) continue;
+        C *z = L + q * RC;
+        row_fft<H, -1>(z, T.tw, j);
+        C *dst = spec + (size_t)(SLOT_X + r) * slot;
+        row_post<H>(z, T.wh, j, [&](int k, C X) {
+            const real m = kx[k] * sx;
+            dst[k] = C{-m * X.y, m * X.x};
         });
     }
 }
 
 template <typename real, int H> size_t k3_row_smem() {
     using G = Row<real, H>;
-    return (size_t)((ND1 + G::CS - 1) / G::CS + (5 + G::CS - 1) / G::CS) * G::RC * 2 * sizeof(real);
+    return (size_t)(G::share(NSP) + G::share(3)) * G::RC * 2 * sizeof(real) + RowTable<real>::bytes(H);
 }
 
 // ---------------------------------------------------------------------------
-// K5: inverse rows of the level-2 divergences and the 32 convection terms ->
-// A, B, C, C_q (Eqs. 20-23), f^eq (Eq. 3), I (Eq. 11), BGK and the RK
+// K5: inverse rows of the convection terms with v_x != 0 and of the d_x terms of
+// level 2, in one pass; A, B, C, C_q (Eqs. 20-23) from the latter, the numerators
+// and the column passes of level 2; f^eq (Eq. 3), I (Eq. 11), BGK and the RK
 // combination (Eq. 10).  Block c of the row takes the rings of velocities
-// 1 + c CHN .. and the level-2 row c (c < 3; with fewer than 3 blocks, rows
-// c, c + CS, ...); the coefficients of its slice of sites go to every block.
+// 1 + c CHN ..; the coefficients of its slice of sites go to every block.
 // ---------------------------------------------------------------------------
 
 constexpr int NCOEF = 5;   // e0, e1x, e1y, C + C_q, 1 / T
@@ -509,20 +579,23 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
     using G = Row<real, H>;
     using C = typename G::C;
     constexpr int CS = G::CS, CHN = G::CHN, RC = G::RC, NX = G::NX, NT = G::NT, P = G::P, NXS = G::NXS;
-    constexpr int N2 = (3 + CS - 1) / CS, NRING = CHN / 8;
+    constexpr int NRING = G::NRING;
     constexpr int V = sizeof(real) == 4 ? 2 : 1;   // sites per thread and pass of the epilogue
     static_assert(CHN % 8 == 0, "whole rings per block");
     extern __shared__ __align__(128) unsigned char row_smem[];
-    C *B = reinterpret_cast<C *>(row_smem);                 // [CHN] convection rows
-    C *S = B + CHN * RC;                                    // [N2] level-2 rows
-    real *co = reinterpret_cast<real *>(S + N2 * RC);       // [NCOEF][NX]
-    const int tid = threadIdx.x, c = block_rank<CS>(), j = tid & (P - 1), grp = tid / P;
+    C *B = reinterpret_cast<C *>(row_smem);                     // [6 NRING] convection rows
+    C *X = B + 6 * NRING * RC;                                  // [share(3)] d_x rows
+    real *co = reinterpret_cast<real *>(X + G::share(3) * RC);  // [NCOEF][NX]
+    using LT = RowTable<real>;
+    unsigned char *tb = reinterpret_cast<unsigned char *>(co + NCOEF * NX);
+    const Tab<real, H> TB(tb, LT::tw(H));
+    __shared__ __align__(8) uint64_t bar;
+    const int c = block_rank<CS>(), tid = (int)threadIdx.x, j = tid & (P - 1), grp = tid / P;
     const int ny = A.ny, yg = (int)blockIdx.x / CS, run = yg / ny, y = yg - run * ny;
     const size_t N = (size_t)NX * ny, slot = (size_t)ny * H;
     const C *__restrict__ spec = A.spec + (size_t)run * NSLOT * slot + (size_t)y * H;
     const size_t fo = (size_t)run * Q * N + (size_t)y * NX;
-    const real *fields = A.fields + (size_t)run * 4 * N + (size_t)y * NX;
-    const real *aux = A.aux + (size_t)run * 3 * N + (size_t)y * NX;
+    auto row = [&](int s) { return reinterpret_cast<const real *>(spec + (size_t)s * slot); };
     const real dt = A.dt, itau = A.itau, alpha = A.alpha, beta = A.beta;
     const bool with_base = alpha != real(0);
     if (tid < CHN) {   // this block's distribution rows into L2 ahead of the epilogue
@@ -530,35 +603,45 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
         bulk_prefetch_l2(A.fcur + o, NX * sizeof(real));
         if (with_base) bulk_prefetch_l2(A.fbase + o, NX * sizeof(real));
     }
-    // level-2 rows first: the others wait for them
-    for (int r = c + CS * grp; r < 3; r += CS * G::NG) {
-        C *z = S + (r / CS) * RC;
-        const C *__restrict__ src = spec + (size_t)(SLOT_L2 + (r == 0 ? 0 : r + 1)) * slot;
-        row_pre<H>(z, A.wp, j, [&](int k) { return ldro(src + k); });
-        __syncwarp(lanes_of_row<P>());
-        row_fft<H, +1>(z, A.tw, j);
+    if (tid == 0) {
+        mbar_init(&bar, 1);
+        mbar_init_fence();
+        mbar_expect_tx(&bar, LT::bytes(H) - LT::tw(H));
+        table_issue(tb, A.tab, LT::tw(H), LT::bytes(H), &bar);
     }
+    __syncthreads();
+    bool first = true;
+    auto ready = [&]() {   // the tables are there (a wait that runs out is recorded; see k1_row)
+        if (first) table_wait(&bar, A.err);
+        first = false;
+    };
+    static_assert(6 * NRING + G::share(3) <= G::NG, "one pass");
+    {
+        const int rr = NRING == 1 ? 0 : grp / 6, q = grp - 6 * NRING, r = G::nth(c, q < 0 ? 0 : q);
+        const bool conv = q < 0, dx = q >= 0 && q < G::share(3) && r < 3;
+        if (conv || dx) {
+            C *z = conv ? B + grp * RC : X + q * RC;
+            const C *__restrict__ src =
+                spec + (size_t)(conv ? c * CHN + rr * 8 + ring_dir(grp - 6 * rr) : SLOT_X + r) * slot;
+            row_pre<H, 1>(z, TB.wp, j, src, src, [](int, C a, C) { return a; }, ready);
+            __syncwarp(lanes_of_row<P>());
+            row_fft<H, +1>(z, TB.tw, j);
+        }
+    }
+    ready();   // (no copy is in flight when the block ends)
     row_arrive<CS>();
-#pragma unroll 1
-    for (int r = grp; r < CHN; r += G::NG) {
-        C *z = B + r * RC;
-        const C *__restrict__ src = spec + (size_t)(c * CHN + r) * slot;
-        row_pre<H>(z, A.wp, j, [&](int k) { return ldro(src + k); });
-        __syncwarp(lanes_of_row<P>());
-        row_fft<H, +1>(z, A.tw, j);
-    }
     row_wait<CS>();
     for (int x = c * NXS + tid; x < (c + 1) * NXS; x += NT) {
-        const real rho = fields[x], ux = fields[N + x], uy = fields[2 * N + x], T = fields[3 * N + x];
-        const real fc = A.fcur[fo + x], fb = with_base ? A.fbase[fo + x] : real(0);
-        const real a0 = aux[x], a1 = aux[N + x], a2 = aux[2 * N + x];
-        const real dLx = reinterpret_cast<const real *>(in_block<CS>(S, 0))[x];
-        const real dLy = reinterpret_cast<const real *>(in_block<CS>(S + (1 / CS) * RC, 1 % CS))[x];
-        const real dPh = reinterpret_cast<const real *>(in_block<CS>(S + (2 / CS) * RC, 2 % CS))[x];
+        real dx[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+            dx[r] = reinterpret_cast<const real *>(in_block<CS>(X + G::local(r) * RC, G::owner(r)))[x];
+        const real rho = row(SLOT_F)[x], ux = row(SLOT_F + 1)[x], uy = row(SLOT_F + 2)[x], T = row(SLOT_F + 3)[x];
         const real rT = rho * T, irT = real(1) / rT, iT = real(1) / T;
-        const real Bx = (a1 + dLx) * irT, By = (a2 + dLy) * irT;   // Eq. 21
-        const real CC = (a0 + dPh) * (real(0.5) * irT * iT);        // C + C_q, Eqs. 22-23
-        const real At = real(-2) * CC * T;                          // Eq. 20
+        const real Bx = (row(SLOT_A + 1)[x] + row(SLOT_L2)[x] + dx[1]) * irT;        // Eq. 21
+        const real By = (row(SLOT_A + 2)[x] + row(SLOT_L2 + 1)[x] + dx[2]) * irT;
+        const real CC = (row(SLOT_A)[x] + row(SLOT_L2 + 2)[x] + dx[0]) * (real(0.5) * irT * iT);   // C + C_q, Eqs. 22-23
+        const real At = real(-2) * CC * T;                                          // Eq. 20
         const real u2 = ux * ux + uy * uy;
         // I = -(A + B.(v-u) + CC |v-u|^2) f^eq = -(e0 + e1.v + CC |v|^2) f^eq
         const real e[NCOEF] = {At - (Bx * ux + By * uy) + CC * u2, Bx - real(2) * CC * ux, By - real(2) * CC * uy, CC, iT};
@@ -568,19 +651,23 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
 #pragma unroll
             for (int i = 0; i < NCOEF; ++i) q[i * NX + x] = e[i];
         }
-        // the rest velocity (no convection)
+    }
+    row_arrive<CS>();
+    row_wait<CS>();
+    // the rest velocity (no convection) at this block's slice
+    for (int x = c * NXS + tid; x < (c + 1) * NXS; x += NT) {
+        const real rho = row(SLOT_F)[x], ux = row(SLOT_F + 1)[x], uy = row(SLOT_F + 2)[x], T = row(SLOT_F + 3)[x];
+        const real fc = A.fcur[fo + x];
         real F0 = 0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) F0 += wk(A, k, T);
         F0 = real(1) - real(8) * F0;
-        const real qq = real(0.5) * u2 * iT, om = real(1) - qq;
+        const real qq = real(0.5) * (ux * ux + uy * uy) * co[4 * NX + x], om = real(1) - qq;
         const real fe = rho * F0 * (om + real(0.5) * qq * qq);
-        real fn = beta * (fc + dt * (-(fc - fe) * itau - e[0] * fe));
-        if (with_base) fn += alpha * fb;
+        real fn = beta * (fc + dt * (-(fc - fe) * itau - co[x] * fe));
+        if (with_base) fn += alpha * A.fbase[fo + x];
         A.fout[fo + x] = fn;
     }
-    row_arrive<CS>();
-    row_wait<CS>();
     // the rings of this block: velocities 1 + 8 k .. 8 + 8 k of Eq. 1, one
     // speed, one weight, the eight directions known at compile time
 #pragma unroll 1
@@ -591,17 +678,19 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
         const size_t o = fo + (size_t)(1 + v0) * N + x;
         const real *pc = A.fcur + o, *pb = A.fbase + o;
         real *po = A.fout + o;
-        real fc[8][V], fb[8][V];   // (all loads before any store: fout may be fcur or fbase)
+        real fc[8][V], fb[8][V], c2[V], c6[V];   // (all loads before any store: fout may be fcur or fbase)
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             ldv<real, V>(fc[r], pc + (size_t)r * N);
             if (with_base) ldv<real, V>(fb[r], pb + (size_t)r * N);
         }
+        ldv<real, V>(c2, row(v0 + 2) + x);   // v_x = 0: real from the column pass
+        ldv<real, V>(c6, row(v0 + 6) + x);
         real rho[V], ux[V], uy[V], T[V], e0[V], ex[V], ey[V], CC[V], iT[V];
-        ldv<real, V>(rho, fields + x);
-        ldv<real, V>(ux, fields + N + x);
-        ldv<real, V>(uy, fields + 2 * N + x);
-        ldv<real, V>(T, fields + 3 * N + x);
+        ldv<real, V>(rho, row(SLOT_F) + x);
+        ldv<real, V>(ux, row(SLOT_F + 1) + x);
+        ldv<real, V>(uy, row(SLOT_F + 2) + x);
+        ldv<real, V>(T, row(SLOT_F + 3) + x);
         ldv<real, V>(e0, co + x);
         ldv<real, V>(ex, co + NX + x);
         ldv<real, V>(ey, co + 2 * NX + x);
@@ -629,28 +718,46 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
             ep[q] = hh * (ex[q] + ey[q]);
             em[q] = hh * (ey[q] - ex[q]);
         }
-        const real *cr = reinterpret_cast<const real *>(B + rr * 8 * RC) + x;
+        const real *cr = reinterpret_cast<const real *>(B + rr * 6 * RC) + x;
+        // directions r and r + 4 together: f^eq = even +- odd in v.u
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            real cv[V], fn[V];
-            ldv<real, V>(cv, cr + (size_t)r * 2 * RC);
+        for (int r = 0; r < 4; ++r) {
+            real cv[2][V], fn[2][V];
+            if (r == 2) {
+#pragma unroll
+                for (int q = 0; q < V; ++q) {
+                    cv[0][q] = c2[q];
+                    cv[1][q] = c6[q];
+                }
+            } else {
+                ldv<real, V>(cv[0], cr + (size_t)ring_pos(r) * 2 * RC);
+                ldv<real, V>(cv[1], cr + (size_t)ring_pos(r + 4) * 2 * RC);
+            }
 #pragma unroll
             for (int q = 0; q < V; ++q) {
-                const real vu = ring_dot<real>(r, ux[q], uy[q], dp[q], dm[q]);
-                const real fe = p0[q] + vu * (p1[q] + vu * (p2[q] + vu * (p3[q] + vu * p4[q])));   // Eq. 3
-                const real g = g0[q] + ring_dot<real>(r, ex[q], ey[q], ep[q], em[q]);             // -I / f^eq, Eq. 11
-                const real rhs = -cv[q] - (fc[r][q] - fe) * itau - g * fe;                          // Eq. 10
-                fn[q] = beta * (fc[r][q] + dt * rhs);
-                if (with_base) fn[q] += alpha * fb[r][q];
+                const real vu = ring_dot<real>(r, ux[q], uy[q], dp[q], dm[q]), w2 = vu * vu;
+                const real ev = p0[q] + w2 * (p2[q] + w2 * p4[q]), od = vu * (p1[q] + w2 * p3[q]);   // Eq. 3
+                const real ed = ring_dot<real>(r, ex[q], ey[q], ep[q], em[q]);
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const real fe = s ? ev - od : ev + od;
+                    const real g = s ? g0[q] - ed : g0[q] + ed;   // -I / f^eq, Eq. 11
+                    const real f = fc[r + 4 * s][q];
+                    const real rhs = -cv[s][q] - (f - fe) * itau - g * fe;   // Eq. 10
+                    fn[s][q] = beta * (f + dt * rhs);
+                    if (with_base) fn[s][q] += alpha * fb[r + 4 * s][q];
+                }
             }
-            stv<real, V>(po + (size_t)r * N, fn);
+            stv<real, V>(po + (size_t)r * N, fn[0]);
+            stv<real, V>(po + (size_t)(r + 4) * N, fn[1]);
         }
     }
 }
 
 template <typename real, int H> size_t k5_row_smem() {
     using G = Row<real, H>;
-    return (size_t)(G::CHN + (3 + G::CS - 1) / G::CS) * G::RC * 2 * sizeof(real) + (size_t)NCOEF * G::NX * sizeof(real);
+    return (size_t)(6 * G::NRING + G::share(3)) * G::RC * 2 * sizeof(real) + (size_t)NCOEF * G::NX * sizeof(real) +
+           RowTable<real>::bytes(H) - RowTable<real>::tw(H);
 }
 
 template <typename real, int H> RowSet row_set() {

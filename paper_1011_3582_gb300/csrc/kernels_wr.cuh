@@ -201,37 +201,26 @@ __device__ __forceinline__ void r2c_post_wr(const C *z, C *out, const C *Wp, int
     }
 }
 
-// r2c_post_wr with two destinations: X to raw and i k_x X / nx (the d_x
-// term of a level-2 output) to mul; either may be null.  kxt[k] = k_x of
-// bin k, sx = 1 / nx; bin 0 (DC, row-Nyquist) has k_x = 0 for both.
+// r2c_post_wr times i k_x c: dst[k] = i kxt[k] sx X[k] (bin 0, DC and
+// row-Nyquist, has k_x = 0 for both).  dst may be z.
 template <int H, typename C>
-__device__ __forceinline__ void r2c_post_wr2(const C *z, C *raw, C *mul, const float *__restrict__ kxt, float sx,
-                                             const C *Wp, int j) {
+__device__ __forceinline__ void r2c_post_dx(const C *z, C *dst, const float *__restrict__ kxt, float sx, const C *Wp,
+                                            int j) {
     using R = decltype(z[0].x);
     constexpr int P = RowCfg<H>::P;
 #pragma unroll
     for (int k0 = 0; k0 <= H / 2; k0 += P) {
         const int k = k0 + j;
         if (k > H / 2) break;
-        C a, b;
         if (k == 0) {
-            const C z0 = z[0];
-            a = C{z0.x + z0.y, z0.x - z0.y};
+            dst[0] = C{0, 0};
         } else {
             const C p = z[k], q = z[H - k];
             const C ze = cscale(cadd(p, cconj(q)), R(0.5));
             const C zo = cscale(cmul_mi(csub(p, cconj(q))), R(0.5));
             const C wz = cmul(Wp[k], zo);
-            a = cadd(ze, wz);
-            b = cconj(csub(ze, wz));
-        }
-        if (raw) {
-            raw[k] = a;
-            if (k != 0 && H - k != k) raw[H - k] = b;
-        }
-        if (mul) {
-            mul[k] = imul(kxt[k] * sx, a);
-            if (k != 0 && H - k != k) mul[H - k] = imul(kxt[H - k] * sx, b);
+            dst[k] = imul(kxt[k] * sx, cadd(ze, wz));
+            if (H - k != k) dst[H - k] = imul(kxt[H - k] * sx, cconj(csub(ze, wz)));
         }
     }
 }
@@ -356,7 +345,7 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
         const int yg = (int)blockIdx.x + ri * (int)gridDim.x;
         const int run = yg / ny, y = yg - run * ny;
         C *spec_r = spec + (size_t)run * NSLOT * slot;
-        real *fields_r = fields + (size_t)run * 4 * N;
+        real *fields_r = fields + (size_t)run * NSLOT * N;
         const int i0 = k1w_first(c, NG), nf = k1w_count(c, NG);
         if (!block_wait(bar, odd ? par1 : par0, err)) {
             if (pend0) mbar_wait_bounded(&bar0, par0);
@@ -392,13 +381,14 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
         // velocity), i.e. f_i with i = i0 + that row, into slot i - 1
         {
             const int r = grp + (c == 0 ? 1 : 0);
-            if (r < nf) {
+            // (v_x = 0: the column pass takes f_i itself)
+            if (r < nf && VX<real>(i0 + r) != real(0)) {
                 const int i = i0 + r;
                 C *zr = reinterpret_cast<C *>(B) + (size_t)r * H;
                 C *dst = spec_r + (size_t)(i - 1) * slot + (size_t)y * H;
                 row_fft_wr<H, -1>(zr, tw, j, rsw);
                 if (VY<real>(i) == real(0))   // convection in k_x alone: i v_x k_x f^ / nx, no column pass
-                    r2c_post_wr2<H>(zr, (C *)nullptr, dst, kxs, VX<real>(i) * P.scale_x, Wp, j);
+                    r2c_post_dx<H>(zr, dst, kxs, VX<real>(i) * P.scale_x, Wp, j);
                 else
                     r2c_post_wr<H>(zr, dst, Wp, j);
             }
@@ -419,8 +409,12 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
                 fb[NX + x] = ux;
                 fb[2 * NX + x] = uy;
                 fb[3 * NX + x] = T;
-                fb[4 * NX + x] = rho * T / (real(1) - P.b * rho) - P.a * rho * rho - rho * T;   // Eq. 18
-                fb[5 * NX + x] = (P.K + P.H * T) / T;                                          // M / T
+                const real Pi = rho * T / (real(1) - P.b * rho) - P.a * rho * rho - rho * T;   // Eq. 18
+                const real g = (P.K + P.H * T) / T;                                          // M / T
+                fields_r[4 * N + o] = Pi;
+                fields_r[5 * N + o] = g;
+                fb[4 * NX + x] = Pi;
+                fb[5 * NX + x] = g;
                 a0[s] = a1[s] = a2[s] = a3[s] = real(0);
             }
             __syncthreads();
@@ -449,33 +443,27 @@ inline size_t k1_wr_smem(int H) {
 }
 
 // ---------------------------------------------------------------------------
-// K3 (fp32, nx = 2H): row inverse of the 15 level-1 derivative spectra ->
-// Lambda (Eq. 19), Phi = 2 q rho T grad T (Eq. 23), the numerators of C
-// (Eq. 22) and B (Eq. 21) -> forward row transforms of Lambda_xx,
-// Lambda_xy, Lambda_yy, Phi_x, Phi_y, as k3_pipe, with warp-resident row
-// transforms.  Persistent over the rows of all runs, one row per pass, two
-// buffers (15 spectrum rows + rho, T), the next-but-one row prefetched.
+// K3 (fp32, nx = 2H): inverse rows of the 11 level-1 derivatives that have a
+// factor k_x or start from a row spectrum (stage_layout.cuh) -> Lambda (Eq. 19),
+// Phi (Eq. 23), the numerators of C (Eq. 22) and B (Eq. 21) -> d_x of Lambda_xx,
+// Lambda_xy, Phi_x (a forward and an inverse row each) added to the numerators.
+// Persistent over the rows of all runs, one row per pass, one or two buffers
+// (11 transformed rows and 8 real ones).
 // ---------------------------------------------------------------------------
 
-template <typename real>
-__device__ __forceinline__ void k3_issue(const typename cplx_of<real>::type *spec, const real *fields, real *dst,
-                                         uint64_t *bar, int ri, int nx, int ny, size_t N, size_t slot, int h) {
+template <typename C>
+__device__ __forceinline__ void k3_issue(const C *spec, C *dst, uint64_t *bar, int ri, int ny, size_t slot, int h) {
     const int yg = (int)blockIdx.x + ri * (int)gridDim.x;
     const int run = yg / ny, y = yg - run * ny;
-    spec += (size_t)run * NSLOT * slot;
-    fields += (size_t)run * 4 * N;
-    const uint32_t rowbytes = (uint32_t)(nx * sizeof(real));
-    mbar_expect_tx(bar, (uint32_t)(ND1 + 1) * rowbytes);   // D_DIVX is formed in K3
-    for (int o = 0; o < ND1; ++o)
-        if (k3_src_slot(o) >= 0)
-            bulk_g2s(dst + (size_t)o * nx, spec + (size_t)k3_src_slot(o) * slot + (size_t)y * h, rowbytes, bar);
-    bulk_g2s(dst + (size_t)ND1 * nx, fields + (size_t)y * nx, rowbytes, bar);
-    bulk_g2s(dst + (size_t)(ND1 + 1) * nx, fields + 3 * N + (size_t)y * nx, rowbytes, bar);
+    spec += (size_t)run * NSLOT * slot + (size_t)y * h;
+    const uint32_t rowbytes = (uint32_t)(h * sizeof(C));
+    mbar_expect_tx(bar, (uint32_t)(NK3 - 3) * rowbytes);   // D_LAP, D_DIVX, D_DIVY are formed in K3
+    for (int o = 0; o < NK3; ++o)
+        if (k3_src_slot(o) >= 0) bulk_g2s(dst + (size_t)o * h, spec + (size_t)k3_src_slot(o) * slot, rowbytes, bar);
 }
 
 template <int H>
-__global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_wr(float2 *spec, const float *__restrict__ fields,
-                                                 float *__restrict__ aux, const float2 *__restrict__ tw_g,
+__global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_wr(float2 *spec, const float2 *__restrict__ tw_g,
                                                  const float2 *__restrict__ Wp_g, const float *__restrict__ kxt,
                                                  KP<float> P, int *err) {
     using C = float2;
@@ -483,19 +471,18 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
     constexpr int NX = 2 * H, NT = nt_k3wr<H>(), NB = nb_k3wr<H>();
     constexpr int PL = RowCfg<H>::P, RPW = 32 / PL, NG = (NT / 32) * RPW;   // row groups
     constexpr int SMAX = (NX + NT - 1) / NT;
-    constexpr int RB = ND1 + 2;   // rows per buffer
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar0, bar1;
-    const int nx = NX, ny = P.ny, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ny = P.ny, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int grp = warp * RPW + lane / PL, j = lane & (PL - 1);
     const int rsw = PL == 8 ? ((lane / PL) & 1) : 0;
-    const size_t N = (size_t)NX * ny, slot = (size_t)ny * H;
+    const size_t slot = (size_t)ny * H;
     SmemCursor sc{smem_raw, 0u};
     C *tw = (C *)sc.take(H * sizeof(C));
     C *Wp = (C *)sc.take((H / 2 + 1) * sizeof(C));
     real *kxs = (real *)sc.take(H * sizeof(real));   // k_x of the row bins
-    real *buf0 = (real *)sc.take((size_t)RB * NX * sizeof(real));
-    real *buf1 = NB > 1 ? (real *)sc.take((size_t)RB * NX * sizeof(real)) : buf0;
+    C *buf0 = (C *)sc.take((size_t)NK3 * H * sizeof(C));
+    C *buf1 = NB > 1 ? (C *)sc.take((size_t)NK3 * H * sizeof(C)) : buf0;
     const int NY = P.nrun * ny;
     const int nrows = (int)blockIdx.x < NY ? (NY - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     if (tid == 0) {   // (the first copies start before the tables load)
@@ -503,8 +490,8 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
         mbar_init(&bar1, 1);
         mbar_init_fence();
         grid_dep_wait();
-        if (nrows > 0) k3_issue<real>(spec, fields, buf0, &bar0, 0, nx, ny, N, slot, H);
-        if (NB > 1 && nrows > 1) k3_issue<real>(spec, fields, buf1, &bar1, 1, nx, ny, N, slot, H);
+        if (nrows > 0) k3_issue(spec, buf0, &bar0, 0, ny, slot, H);
+        if (NB > 1 && nrows > 1) k3_issue(spec, buf1, &bar1, 1, ny, slot, H);
     }
     load_tab4(tw, tw_g, H, NT);
     load_tab4(Wp, Wp_g, H / 2 + 1, NT);
@@ -519,8 +506,7 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
         uint64_t *bar = odd ? &bar1 : &bar0;
         const int yg = (int)blockIdx.x + ri * (int)gridDim.x;
         const int run = yg / ny, y = yg - run * ny;
-        C *spec_r = spec + (size_t)run * NSLOT * slot;
-        real *aux_r = aux + (size_t)run * 3 * N;
+        C *spec_r = spec + (size_t)run * NSLOT * slot + (size_t)y * H;
         if (!block_wait(bar, odd ? par1 : par0, err)) {
             if (pend0) mbar_wait_bounded(&bar0, par0);
             if (pend1) mbar_wait_bounded(&bar1, par1);
@@ -533,62 +519,54 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
             par0 ^= 1;
             pend0 = false;
         }
-        real *d = odd ? buf1 : buf0;
-        for (int k = tid; k < H; k += NT) k3_form_x<real>(reinterpret_cast<C *>(d), H, k, kxs[k], P.scale_x);
+        C *dc = odd ? buf1 : buf0;
+        real *d = reinterpret_cast<real *>(dc);
+        for (int k = tid; k < H; k += NT) k3_form_x<real>(dc, H, k, kxs[k], P.scale_x);
         __syncthreads();
-        for (int r = grp; r < ND1; r += NG) {   // (uniform over each row group)
-            C *zr = reinterpret_cast<C *>(d) + (size_t)r * H;
+        for (int r = grp; r < NSP; r += NG) {   // (uniform over each row group)
+            C *zr = dc + (size_t)r * H;
             c2r_pre_wr<H>(zr, Wp, j);
             __syncwarp(group_mask<PL>());
             row_fft_wr<H, +1>(zr, tw, j, rsw);
         }
         __syncthreads();
-        const real *rT = d + (size_t)ND1 * NX;
+        auto out = [&](int s) { return reinterpret_cast<real *>(spec_r + (size_t)s * slot); };
 #pragma unroll 1
         for (int s = 0; s < SMAX; ++s) {
             const int x = tid + s * NT;
-            const size_t o = (size_t)y * nx + x;
-            const real rho = rT[x], T = rT[NX + x];
-            const real rx = d[D_RX * NX + x], ry = d[D_RY * NX + x], lap = d[D_LAP * NX + x];
-            const real uxx = d[D_UXX * NX + x], uxy = d[D_UXY * NX + x];
-            const real uyx = d[D_UYX * NX + x], uyy = d[D_UYY * NX + x];
-            const real divx = d[D_DIVX * NX + x], divy = d[D_DIVY * NX + x];
-            const real Tx = d[D_TX * NX + x], Ty = d[D_TY * NX + x];
-            const real Pix = d[D_PIX * NX + x], Piy = d[D_PIY * NX + x];
-            const real gx = d[D_GX * NX + x], gy = d[D_GY * NX + x];
-            const real M = P.K + P.H * T;
-            const real Pi = rho * T / (real(1) - P.b * rho) - P.a * rho * rho - rho * T;
-            const real grad2 = rx * rx + ry * ry;
-            const real iso = -(rho * T * (rx * gx + ry * gy)) - M * (rho * lap + real(0.5) * grad2);   // Eq. 19
-            const real Lxx = M * rx * rx + iso, Lxy = M * rx * ry, Lyy = M * ry * ry + iso;
-            const real div = uxx + uyy;
-            const real Ldu = Lxx * uxx + Lxy * (uyx + uxy) + Lyy * uyy;
-            const real Cn = Pi * div + Ldu - P.zeta * div * div + P.a * rho * rho * div +
-                            P.K * (real(-0.5) * grad2 * div - rho * (rx * divx + ry * divy) -
-                                   (rx * (uxx * rx + uyx * ry) + ry * (uxy * rx + uyy * ry)));   // Eq. 22
-            aux_r[o] = Cn;
-            aux_r[N + o] = Pix - P.zeta * divx;   // Eq. 21 without d_b Lambda_ab
-            aux_r[2 * N + o] = Piy - P.zeta * divy;
-            const real q2 = real(2) * P.q * rho * T;   // Eq. 23
-            // rows 0..4 (same site, same thread)
-            d[0 * NX + x] = Lxx;
-            d[1 * NX + x] = Lxy;
-            d[2 * NX + x] = Lyy;
-            d[3 * NX + x] = q2 * Tx;
-            d[4 * NX + x] = q2 * Ty;
+            const Level2<real> l = level2_site<real>([&](int o) { return d[o * NX + x]; }, P);
+            out(SLOT_L2)[x] = l.Lxy;
+            out(SLOT_L2 + 1)[x] = l.Lyy;
+            out(SLOT_L2 + 2)[x] = l.Phy;
+            // rows 0..2: transformed next; 3..5: the numerators their d_x
+            // joins (same site, same thread)
+            d[x] = l.Phx;
+            d[NX + x] = l.Lxx;
+            d[2 * NX + x] = l.Lxy;
+            d[3 * NX + x] = l.Cn;
+            d[4 * NX + x] = l.Bx;
+            d[5 * NX + x] = l.By;
         }
         __syncthreads();
-        for (int r = grp; r < 5; r += NG) {
-            C *zr = reinterpret_cast<C *>(d) + (size_t)r * H;
+        for (int r = grp; r < 3; r += NG) {
+            C *zr = dc + (size_t)r * H;
             row_fft_wr<H, -1>(zr, tw, j, rsw);
-            C *raw = k3_raw_slot(r) >= 0 ? spec_r + (size_t)k3_raw_slot(r) * slot + (size_t)y * H : nullptr;
-            C *mul = k3_mul_slot(r) >= 0 ? spec_r + (size_t)k3_mul_slot(r) * slot + (size_t)y * H : nullptr;
-            r2c_post_wr2<H>(zr, raw, mul, kxs, P.scale_x, Wp, j);
+            r2c_post_dx<H>(zr, zr, kxs, P.scale_x, Wp, j);
+            __syncwarp(group_mask<PL>());
+            c2r_pre_wr<H>(zr, Wp, j);
+            __syncwarp(group_mask<PL>());
+            row_fft_wr<H, +1>(zr, tw, j, rsw);
+        }
+        __syncthreads();
+        for (int s = 0; s < SMAX; ++s) {
+            const int x = tid + s * NT;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) out(SLOT_A + r)[x] = d[(3 + r) * NX + x] + d[r * NX + x];
         }
         fence_proxy_async();
         __syncthreads();
         if (tid == 0 && ri + NB < nrows) {   // row ri + NB reuses this buffer
-            k3_issue<real>(spec, fields, d, bar, ri + NB, nx, ny, N, slot, H);
+            k3_issue(spec, dc, bar, ri + NB, ny, slot, H);
             if (odd) pend1 = true;
             else pend0 = true;
         }
@@ -597,8 +575,8 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
 
 // shared memory of k3_wr<H>
 inline size_t k3_wr_smem(int H) {
-    return smem_bytes({(size_t)H * 8, (size_t)(H / 2 + 1) * 8, (size_t)H * 4, (size_t)(ND1 + 2) * 2 * H * 4,
-                       nb_k3wr_host(H) > 1 ? (size_t)(ND1 + 2) * 2 * H * 4 : 0});
+    return smem_bytes({(size_t)H * 8, (size_t)(H / 2 + 1) * 8, (size_t)H * 4, (size_t)NK3 * 2 * H * 4,
+                       nb_k3wr_host(H) > 1 ? (size_t)NK3 * 2 * H * 4 : 0});
 }
 
 // ---------------------------------------------------------------------------
@@ -690,15 +668,16 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
             pend0 = false;
         }
         real *B = odd ? buf1 : buf0;
-        // inverse transforms: convection row grow of the chunk; with the
-        // first chunk, then (its copies complete) the 3 level-2 rows of the
-        // head (row groups 0..2)
+        // inverse transform of convection row grow of the chunk; with the
+        // first chunk, then the wait for the head
         {
-            const unsigned gm = group_mask<PL>();
-            C *zr = reinterpret_cast<C *>(B) + (size_t)grow * H;
-            c2r_pre_wr<H>(zr, Wp, j);
-            __syncwarp(gm);
-            row_fft_wr<H, +1>(zr, tw, j, rsw);
+            // (directions 2 and 6 of a ring, v_x = 0: real from the column pass)
+            if ((grow & 3) != 2) {
+                C *zr = reinterpret_cast<C *>(B) + (size_t)grow * H;
+                c2r_pre_wr<H>(zr, Wp, j);
+                __syncwarp(group_mask<PL>());
+                row_fft_wr<H, +1>(zr, tw, j, rsw);
+            }
             if (c == 0) {
                 if (!block_wait(hodd ? &hbar1 : &hbar0, hodd ? hpar1 : hpar0, err)) {
                     if (pend0) mbar_wait_bounded(&bar0, par0);
@@ -713,12 +692,6 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
                 } else {
                     hpar0 ^= 1;
                     hpend0 = false;
-                }
-                if (grow < 3) {   // uniform over each row group
-                    C *zh = reinterpret_cast<C *>(Hd) + (size_t)grow * H;
-                    c2r_pre_wr<H>(zh, Wp, j);
-                    __syncwarp(gm);
-                    row_fft_wr<H, +1>(zh, tw, j, rsw);
                 }
             }
         }
@@ -996,12 +969,13 @@ __global__ void __launch_bounds__(ColCfg<NY>::TW * ColCfg<NY>::P, ColCfg<NY>::TW
                                                                              const float2 *__restrict__ twc_g,
                                                                              KP<float> P, int BOXR, int nbuf,
                                                                              const __grid_constant__ CUtensorMap tmap,
+                                                                             const __grid_constant__ CUtensorMap fmap,
                                                                              int *err) {
     using C = float2;
     using real = float;
     constexpr int E = ColCfg<NY>::E, PP = ColCfg<NY>::P, TW = ColCfg<NY>::TW, NT = TW * PP;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bar0, bar1, abar;
+    __shared__ __align__(8) uint64_t bar0, bar1;
     __shared__ ColG gt[kMaxColGroups];   // ngroups <= kMaxColGroups (checked by the host)
     const int h = P.h, tid = threadIdx.x;
     const int c = tid % TW, jl = tid / TW;
@@ -1020,27 +994,25 @@ __global__ void __launch_bounds__(ColCfg<NY>::TW * ColCfg<NY>::P, ColCfg<NY>::TW
     if (tid == 0) {   // (the first copies start before the tables load)
         mbar_init(&bar0, 1);
         mbar_init(&bar1, 1);
-        mbar_init(&abar, 1);
         mbar_init_fence();
         grid_dep_wait();
-        if (njobs > 0) kcol_issue(buf0, &bar0, groups, 0, ntiles, ngroups, TW, NY, BOXR, &tmap);
-        if (nbuf > 1 && njobs > 1) kcol_issue(buf1, &bar1, groups, 1, ntiles, ngroups, TW, NY, BOXR, &tmap);
-        if (njobs > nbuf) kcol_prefetch(groups, nbuf, ntiles, ngroups, TW, NY, BOXR, &tmap);
+        if (njobs > 0) kcol_issue(buf0, &bar0, groups, 0, ntiles, ngroups, TW, NY, BOXR, &tmap, &fmap);
+        if (nbuf > 1 && njobs > 1) kcol_issue(buf1, &bar1, groups, 1, ntiles, ngroups, TW, NY, BOXR, &tmap, &fmap);
+        if (njobs > nbuf) kcol_prefetch(groups, nbuf, ntiles, ngroups, TW, NY, BOXR, &tmap, &fmap);
     }
     load_tab4(twc, twc_g, 2 * NY, NT);
     load_tab4(kxs, kxt, h + 1, NT);
     load_tab4(kys, kyt, NY, NT);
     for (int g = tid; g < ngroups; g += NT) {
         const GroupDesc &G = groups[g];
-        gt[g] = ColG{G.nin, {G.in_slot[0], G.in_slot[1]}, G.out_slot[0], G.add_slot, (float)G.c[0][0][0],
-                     (float)G.c[0][0][1], (float)G.c[0][0][3]};
+        gt[g] = ColG{{G.in_slot[0]}, G.out_slot[0], G.from_f, (float)(G.c[0][0][0] * G.scale),
+                     (float)(G.c[0][0][1] * G.scale), (float)(G.c[0][0][3] * G.scale)};
     }
     grid_dep_wait();
     grid_dep_launch();
     __syncthreads();
-    uint32_t par0 = 0, par1 = 0, apar = 0;
+    uint32_t par0 = 0, par1 = 0;
     bool pend0 = njobs > 0, pend1 = nbuf > 1 && njobs > 1;
-    const real scale = P.scale;
     for (int k = 0; k < njobs; ++k) {
         const bool odd = k & 1;
         uint64_t *bar = odd ? &bar1 : &bar0;
@@ -1061,7 +1033,7 @@ __global__ void __launch_bounds__(ColCfg<NY>::TW * ColCfg<NY>::P, ColCfg<NY>::TW
             pend0 = false;
         }
         C *T = odd ? buf1 : buf0;
-        const int oslot = gt[g].out_slot, aslot = gt[g].add_slot;
+        const int oslot = gt[g].out_slot;
         const real c0 = gt[g].c0, c1 = gt[g].c1, c3 = gt[g].c3;
         C v[E];
         // stage 1, forward
@@ -1088,9 +1060,9 @@ __global__ void __launch_bounds__(ColCfg<NY>::TW * ColCfg<NY>::P, ColCfg<NY>::TW
                 for (int k2 = 0; k2 < PP; ++k2) {
                     const real ay = kys[k1 + E * k2];
                     if (c3 != real(0)) {   // uniform over the block
-                        u[k2] = cscale(u[k2], c3 * ay * ay * scale);
+                        u[k2] = cscale(u[k2], c3 * ay * ay);
                     } else {
-                        const real m = (mx + c1 * ay) * scale;   // i m
+                        const real m = mx + c1 * ay;   // i m
                         u[k2] = C{-m * u[k2].y, m * u[k2].x};
                     }
                 }
@@ -1105,46 +1077,18 @@ __global__ void __launch_bounds__(ColCfg<NY>::TW * ColCfg<NY>::P, ColCfg<NY>::TW
         for (int k1 = 0; k1 < E; ++k1) v[k1] = T[cpos<NY>(c, jl, k1)];
         fence_proxy_async();
         __syncthreads();
-        // the tile buffer is free: with an addend, its tile comes into the
-        // buffer first (read after the inverse DFT), then the next job's
-        if (tid == 0 && aslot >= 0) {
-            const int sl = run * NSLOT + aslot;
-            mbar_expect_tx(&abar, (uint32_t)(tile * sizeof(C)));
-            for (int r0 = 0; r0 < NY; r0 += BOXR) tma_load_2d(T + (size_t)r0 * TW, &tmap, 2 * t * TW, sl * NY + r0, &abar);
-        }
-        if (tid == 0 && aslot < 0 && k + nbuf < njobs) {   // prefetch job k + nbuf into the buffer
+        if (tid == 0 && k + nbuf < njobs) {   // the tile buffer is free: job k + nbuf
             const bool nodd = (k + nbuf) & 1;
-            kcol_issue(T, nodd ? &bar1 : &bar0, gt, k + nbuf, ntiles, ngroups, TW, NY, BOXR, &tmap);
+            kcol_issue(T, nodd ? &bar1 : &bar0, gt, k + nbuf, ntiles, ngroups, TW, NY, BOXR, &tmap, &fmap);
             if (nodd) pend1 = true;
             else pend0 = true;
             // and the job after it into L2, so that its copy finds the tiles there
-            if (k + nbuf + 1 < njobs) kcol_prefetch(gt, k + nbuf + 1, ntiles, ngroups, TW, NY, BOXR, &tmap);
+            if (k + nbuf + 1 < njobs) kcol_prefetch(gt, k + nbuf + 1, ntiles, ngroups, TW, NY, BOXR, &tmap, &fmap);
         }
         SmallDFT<E, +1, C>::run(v);
         C *out = spec + (size_t)run * NSLOT * slot + (size_t)oslot * slot + kx0 + c;
-        if (aslot >= 0) {   // plus the term the row kernel formed
-            if (!block_wait(&abar, apar, err)) {
-                mbar_wait_bounded(&abar, apar);
-                if (pend0) mbar_wait_bounded(&bar0, par0);
-                if (pend1) mbar_wait_bounded(&bar1, par1);
-                return;
-            }
-            apar ^= 1;
 #pragma unroll
-            for (int q = 0; q < E; ++q) out[(size_t)(jl + PP * q) * h] = cadd(v[q], T[(jl + PP * q) * TW + c]);
-            fence_proxy_async();
-            __syncthreads();
-            if (tid == 0 && k + nbuf < njobs) {
-                const bool nodd = (k + nbuf) & 1;
-                kcol_issue(T, nodd ? &bar1 : &bar0, gt, k + nbuf, ntiles, ngroups, TW, NY, BOXR, &tmap);
-                if (nodd) pend1 = true;
-                else pend0 = true;
-                if (k + nbuf + 1 < njobs) kcol_prefetch(gt, k + nbuf + 1, ntiles, ngroups, TW, NY, BOXR, &tmap);
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < E; ++q) out[(size_t)(jl + PP * q) * h] = v[q];
-        }
+        for (int q = 0; q < E; ++q) out[(size_t)(jl + PP * q) * h] = v[q];
     }
 }
 

@@ -17,34 +17,45 @@ namespace fftlb {
 // Lanes per row of a half row of H = E P complex values (0: no
 // configuration).  E points of the first stage sit in each lane's registers:
 // up to 32 (fp32) or 24 (fp64) complex values.
-__host__ __device__ constexpr int row_p(int H) {
+__host__ __device__ constexpr int row_p(int size, int H) {
     return H == 1024 || H == 768 || H == 512 ? 32
          : H == 384 || H == 256 ? 16
-         : H == 192 || H == 128 || H == 96 || H == 64 ? 8
+         : H == 192 || H == 128 || H == 96 || H == 64 || (size == 8 && (H == 48 || H == 32)) ? 8
          : H == 48 || H == 32 || H == 24 || H == 16 ? 4 : 0;
 }
 // threads per block
-__host__ __device__ constexpr int row_nt(int, int H) { return row_p(H) == 32 ? 256 : 128; }
+__host__ __device__ constexpr int row_nt(int size, int H) { return row_p(size, H) == 32 ? 256 : 128; }
 // blocks per row (cluster size): as many as give every row group one
 // distribution row, at most 4
-__host__ __device__ constexpr int row_cs(int, int H) { return row_p(H) >= 16 ? 4 : row_p(H) == 8 ? 2 : 1; }
+__host__ __device__ constexpr int row_cs(int size, int H) { return row_p(size, H) >= 16 ? 4 : row_p(size, H) == 8 ? 2 : 1; }
 // complex values between rows in shared memory: rows of one memory phase
 // (half a warp of 8-byte, a quarter of 16-byte values) in different banks
 __host__ __device__ constexpr int row_stride(int size, int H) {
-    return H + (row_p(H) * 2 * size < 128 && row_p(H) < 16 ? row_p(H) : 0);
+    return H + (row_p(size, H) * 2 * size < 128 && row_p(size, H) < 16 ? row_p(size, H) : 0);
 }
+
+// The tables of the row kernels as one block of bytes: wh[k] = exp(-2 pi i k /
+// 2H) / 2 (k <= H / 2), kx[k] (k < H), the stage-1 twiddles tw[k1 P + l] = exp(-2
+// pi i l k1 / H), wp[k] = exp(-2 pi i k / 2H) (k <= H / 2); offsets of its parts,
+// each a multiple of 16 bytes
+template <typename real> struct RowTable {
+    static __host__ __device__ constexpr unsigned up(unsigned b) { return (b + 15u) & ~15u; }
+    static __host__ __device__ constexpr unsigned half(int H) { return up((H / 2 + 1) * 2 * sizeof(real)); }
+    static __host__ __device__ constexpr unsigned kx(int H) { return half(H); }
+    static __host__ __device__ constexpr unsigned tw(int H) { return kx(H) + up(H * sizeof(real)); }
+    static __host__ __device__ constexpr unsigned wp(int H) { return tw(H) + H * 2 * sizeof(real); }
+    static __host__ __device__ constexpr unsigned bytes(int H) { return wp(H) + half(H); }
+};
 
 template <typename real> struct RowArgs {
     using C = typename cplx_of<real>::type;
     int ny, nrun;
     real dt, itau, a, b, K, H, q, zeta, scale_x, alpha, beta;
     const real *f;      // K1: the stage state [run][33][ny][nx]
-    real *fields, *aux;
-    C *spec;
+    C *spec;            // the slots [run][NSLOT][ny][nx / 2]
     const real *fcur, *fbase;   // K5
     real *fout;
-    const C *tw, *wp, *wh;      // stage-1 twiddles; exp(-2 pi i k / nx), k <= H / 2, and half of it
-    const real *kx;
+    const C *tab;               // table block, see RowTable
     int *err;
     real vx[33], vy[33], v2[33];
     real Fk[4][4], Fkl[4][4];   // Eq. 4's polynomials (fp32: hi and lo parts)
