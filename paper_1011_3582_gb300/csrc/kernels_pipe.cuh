@@ -860,9 +860,7 @@ __global__ void __launch_bounds__(KCfg<real, KS_K5>::NT, KCfg<real, KS_K5>::MINB
                     const real fe = rho * F[0] * (om + real(0.5) * qq * qq);
                     const size_t o = fo + (size_t)y * nx + x;
                     const real fc = fcur[o];
-                    real fn = beta * (fc + dt * (-(fc - fe) * itau - e0 * fe));
-                    if (with_base) fn += alpha * fbase[o];
-                    fout[o] = fn;
+                    fout[o] = rk_combine(with_base, beta, dt, fc, with_base ? fbase[o] : real(0), -(fc - fe) * itau - e0 * fe);
                 }
             }
             __syncthreads();
@@ -928,9 +926,7 @@ __global__ void __launch_bounds__(KCfg<real, KS_K5>::NT, KCfg<real, KS_K5>::MINB
                     const real I = -(g0 + dir_dot<real>(r, exk, eyk)) * fe;                   // Eq. 11
                     const real conv = (r & 3) == 2 ? creal[(size_t)(v0 + r) * N + x] : real_at<real>(cres, lcr, r, x);
                     const real rhs = -conv - (fc[r] - fe) * itau + I;                        // Eq. 10
-                    real fn = beta * (fc[r] + dt * rhs);
-                    if (with_base) fn += alpha * fb[r];
-                    po[r * N] = fn;
+                    po[r * N] = rk_combine(with_base, beta, dt, fc[r], fb[r], rhs);
                 }
             }
         } else {
@@ -973,9 +969,7 @@ __global__ void __launch_bounds__(KCfg<real, KS_K5>::NT, KCfg<real, KS_K5>::MINB
                         const real I = -(e0 + e1x * vx + e1y * vy + CC * v2) * fe;              // Eq. 11
                         const real conv = vx == real(0) ? creal[(size_t)(v0 + r) * N + x] : real_at<real>(cres, lcr, r, x);
                         const real rhs = -conv - (fc[r] - fe) * itau + I;                       // Eq. 10
-                        real fn = beta * (fc[r] + dt * rhs);
-                        if (with_base) fn += alpha * fb[r];
-                        po[r * N] = fn;
+                        po[r * N] = rk_combine(with_base, beta, dt, fc[r], fb[r], rhs);
                     }
                 }
             }

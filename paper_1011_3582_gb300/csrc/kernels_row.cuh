@@ -596,8 +596,8 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
     const C *__restrict__ spec = A.spec + (size_t)run * NSLOT * slot + (size_t)y * H;
     const size_t fo = (size_t)run * Q * N + (size_t)y * NX;
     auto row = [&](int s) { return reinterpret_cast<const real *>(spec + (size_t)s * slot); };
-    const real dt = A.dt, itau = A.itau, alpha = A.alpha, beta = A.beta;
-    const bool with_base = alpha != real(0);
+    const real dt = A.dt, itau = A.itau, beta = A.beta;
+    const bool with_base = A.alpha != real(0);
     if (tid < CHN) {   // this block's distribution rows into L2 ahead of the epilogue
         const size_t o = fo + (size_t)(1 + c * CHN + tid) * N;
         bulk_prefetch_l2(A.fcur + o, NX * sizeof(real));
@@ -664,9 +664,8 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
         F0 = real(1) - real(8) * F0;
         const real qq = real(0.5) * (ux * ux + uy * uy) * co[4 * NX + x], om = real(1) - qq;
         const real fe = rho * F0 * (om + real(0.5) * qq * qq);
-        real fn = beta * (fc + dt * (-(fc - fe) * itau - co[x] * fe));
-        if (with_base) fn += alpha * A.fbase[fo + x];
-        A.fout[fo + x] = fn;
+        A.fout[fo + x] =
+            rk_combine(with_base, beta, dt, fc, with_base ? A.fbase[fo + x] : real(0), -(fc - fe) * itau - co[x] * fe);
     }
     // the rings of this block: velocities 1 + 8 k .. 8 + 8 k of Eq. 1, one
     // speed, one weight, the eight directions known at compile time
@@ -744,8 +743,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
                     const real g = s ? g0[q] - ed : g0[q] + ed;   // -I / f^eq, Eq. 11
                     const real f = fc[r + 4 * s][q];
                     const real rhs = -cv[s][q] - (f - fe) * itau - g * fe;   // Eq. 10
-                    fn[s][q] = beta * (f + dt * rhs);
-                    if (with_base) fn[s][q] += alpha * fb[r + 4 * s][q];
+                    fn[s][q] = rk_combine(with_base, beta, dt, f, fb[r + 4 * s][q], rhs);
                 }
             }
             stv<real, V>(po + (size_t)r * N, fn[0]);

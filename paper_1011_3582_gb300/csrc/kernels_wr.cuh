@@ -734,8 +734,7 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
                     weights_Fk<real>(T[q], F);
                     const real qq = real(0.5) * u2 / T[q], om = real(1) - qq;
                     const real fe = rho[q] * F[0] * (om + real(0.5) * qq * qq);
-                    fn[q] = beta * (fc[q] + dt * (-(fc[q] - fe) * itau - e0[q] * fe));
-                    if (with_base) fn[q] += alpha * fb[q];
+                    fn[q] = rk_combine(with_base, beta, dt, fc[q], fb[q], -(fc[q] - fe) * itau - e0[q] * fe);
                 }
                 st4(Hd + x0, e0);
                 st4(Hd + nx + x0, e1x);
@@ -769,9 +768,7 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
                     const real fe = rho * F[0] * (om + real(0.5) * qq * qq);
                     const size_t o = fo + (size_t)y * nx + x;
                     const real fc = fcur[o];
-                    real fn = beta * (fc + dt * (-(fc - fe) * itau - e0 * fe));
-                    if (with_base) fn += alpha * fbase[o];
-                    fout[o] = fn;
+                    fout[o] = rk_combine(with_base, beta, dt, fc, with_base ? fbase[o] : real(0), -(fc - fe) * itau - e0 * fe);
                 }
             }
             __syncthreads();
@@ -842,8 +839,7 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
                             const real fe = rF[q] * br;                                          // Eq. 3
                             const real I = -(g0[q] + dir_dot<real>(r0 + r, exk[q], eyk[q])) * fe;  // Eq. 11
                             const real rhs = -cv[q] - (fc[r][q] - fe) * itau + I;                // Eq. 10
-                            fn[q] = beta * (fc[r][q] + dt * rhs);
-                            if (with_base) fn[q] += alpha * fb[r][q];
+                            fn[q] = rk_combine(with_base, beta, dt, fc[r][q], fb[r][q], rhs);
                         }
                         st4(po + (size_t)(r0 + r) * N, fn);
                     }
@@ -881,9 +877,7 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
                     const real I = -(g0 + dir_dot<real>(r, exk, eyk)) * fe;                   // Eq. 11
                     const real conv = cres[(size_t)r * NX + x];
                     const real rhs = -conv - (fc[r] - fe) * itau + I;                        // Eq. 10
-                    real fn = beta * (fc[r] + dt * rhs);
-                    if (with_base) fn += alpha * fb[r];
-                    po[r * N] = fn;
+                    po[r * N] = rk_combine(with_base, beta, dt, fc[r], fb[r], rhs);
                 }
             }
             }

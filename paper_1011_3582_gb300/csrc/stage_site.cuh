@@ -38,4 +38,14 @@ __device__ __forceinline__ Level2<real> level2_site(const Row &d, const Par &P) 
     return o;
 }
 
+// One value's Runge-Kutta combination: f + dt rhs, or with a base state fb
+// (1 - beta) fb + beta (f + dt rhs) as fb + beta ((f - fb) + dt rhs).  In fp32
+// the weights 1/3 and 2/3 rounded add up to 1 + 3e-8, which scaled every f by
+// that each step (a mass drift of 2e-8 a step); here f and fb, which are close,
+// are subtracted without rounding and the small sum is rounded once.
+template <typename real>
+__device__ __forceinline__ real rk_combine(bool with_base, real beta, real dt, real f, real fb, real rhs) {
+    return with_base ? fb + beta * ((f - fb) + dt * rhs) : f + dt * rhs;
+}
+
 }  // namespace fftlb
