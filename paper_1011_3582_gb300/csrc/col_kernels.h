@@ -45,6 +45,28 @@ template <typename real> __host__ __device__ constexpr unsigned col_table_bytes(
 
 constexpr int kMaxColJobs = 40;   // groups of one launch
 
+// the gradient of caller fields (dx_row, dy_col): row and column tables
+template <typename real> struct GradArgs {
+    using C = typename cplx_of<real>::type;
+    const double2 *g;   // [fields][ny][nx / 2] pairs of fp64 values
+    double2 *out;       // [2 fields][ny][nx / 2]
+    const C *rtab, *ctab;
+    const real *ky;
+    int h, ny, nrows;   // nrows = fields ny
+    int *err;
+};
+
+// the gradient energy of a real field rho [ny][nx]
+template <typename real> struct EnergyArgs {
+    using C = typename cplx_of<real>::type;
+    const C *rho;
+    const C *rtab, *ctab;
+    const real *ky;
+    double *partial_x, *partial_y;   // one value per block of energy_row / energy_col
+    int h, ny;
+    int *err;
+};
+
 template <typename real> struct ColArgs {
     using C = typename cplx_of<real>::type;
     C *spec;
@@ -57,7 +79,7 @@ template <typename real> struct ColArgs {
 };
 
 struct ColSet {
-    const void *k = nullptr;
+    const void *k = nullptr, *dy = nullptr, *energy = nullptr;
     int nt = 0, tw = 0;   // tw = 0: a column per thread
     size_t smem = 0;
 };

@@ -290,29 +290,69 @@ __global__ void k_feq_init(const double *rho_g, const double *ux_g, const double
     }
 }
 
-template <typename real>
-__global__ void k_moments(const real *f, real *fields, size_t N) {
-    for (size_t s = blockIdx.x * (size_t)blockDim.x + threadIdx.x; s < N; s += (size_t)gridDim.x * blockDim.x) {
-        real m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+// Up to four fp64 output fields (null: not wanted)
+struct FieldPtrs {
+    double *p[4];
+};
+
+// Moments rho, u_x, u_y, T (Eqs. 7-9) of the state straight into fp64 fields, V
+// consecutive sites per thread (4 with 16-byte accesses, where the fields are so
+// aligned, or 1).  Bound by the 33 values a site it reads.
+template <typename real, int V>
+__global__ void __launch_bounds__(256) k_fields_out(const real *__restrict__ f, FieldPtrs out, size_t N) {
+    struct __align__(V == 4 ? 16 : sizeof(real)) VR {
+        real v[V];
+    };
+    struct __align__(V == 4 ? 16 : 8) VD {
+        double v[V];
+    };
+    for (size_t g = blockIdx.x * (size_t)256 + threadIdx.x; g < N / V; g += (size_t)gridDim.x * 256) {
+        real m0[V], m1[V], m2[V], m3[V];
+#pragma unroll
+        for (int s = 0; s < V; ++s) m0[s] = m1[s] = m2[s] = m3[s] = real(0);
+#pragma unroll 11
         for (int i = 0; i < Q; ++i) {
-            const real v = f[(size_t)i * N + s];
-            m0 += v;
-            m1 += VX<real>(i) * v;
-            m2 += VY<real>(i) * v;
-            m3 += V2<real>(i) * v;
+            const VR w = *reinterpret_cast<const VR *>(f + (size_t)i * N + V * g);
+#pragma unroll
+            for (int s = 0; s < V; ++s) {
+                m0[s] += w.v[s];
+                m1[s] += VX<real>(i) * w.v[s];
+                m2[s] += VY<real>(i) * w.v[s];
+                m3[s] += V2<real>(i) * w.v[s];
+            }
         }
-        const real ux = m1 / m0, uy = m2 / m0;
-        fields[s] = m0;
-        fields[N + s] = ux;
-        fields[2 * N + s] = uy;
-        fields[3 * N + s] = real(0.5) * (m3 / m0 - (ux * ux + uy * uy));
+        VD o[4];
+#pragma unroll
+        for (int s = 0; s < V; ++s) {
+            const real ux = m1[s] / m0[s], uy = m2[s] / m0[s];
+            o[0].v[s] = (double)m0[s];
+            o[1].v[s] = (double)ux;
+            o[2].v[s] = (double)uy;
+            o[3].v[s] = (double)(real(0.5) * (m3[s] / m0[s] - (ux * ux + uy * uy)));
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (out.p[q]) *reinterpret_cast<VD *>(out.p[q] + V * g) = o[q];
     }
 }
 
-template <typename real, typename TO>
-__global__ void k_convert(const real *src, TO *dst, size_t n) {
-    for (size_t s = blockIdx.x * (size_t)blockDim.x + threadIdx.x; s < n; s += (size_t)gridDim.x * blockDim.x)
-        dst[s] = (TO)src[s];
+// dst = src converted, V values per thread and pass (4 where both are 16-byte
+// aligned)
+template <typename TI, typename TO, int V>
+__global__ void __launch_bounds__(256) k_convert(const TI *__restrict__ src, TO *__restrict__ dst, size_t n) {
+    struct __align__(V == 4 ? 16 : sizeof(TI)) VI {
+        TI v[V];
+    };
+    struct __align__(V == 4 ? 16 : sizeof(TO)) VO {
+        TO v[V];
+    };
+    for (size_t g = blockIdx.x * (size_t)256 + threadIdx.x; g < n / V; g += (size_t)gridDim.x * 256) {
+        const VI a = reinterpret_cast<const VI *>(src)[g];
+        VO b;
+#pragma unroll
+        for (int s = 0; s < V; ++s) b.v[s] = (TO)a.v[s];
+        reinterpret_cast<VO *>(dst)[g] = b;
+    }
 }
 
 // Forward row transforms of nf real fields (row-major [nf][ny][nx]) into
@@ -368,8 +408,9 @@ __global__ void __launch_bounds__(NT) k_rows_inverse(const typename cplx_of<real
 // x-gradient energy sum_x (D_x rho)^2 by Parseval's relation: slot 0 holds
 // Z = DFT_x rho, D_x rho has spectrum i k_x Z (k_x is zero at DC and at the
 // row Nyquist bin), and over the two-sided spectrum sum_x d^2 =
-// (1 / nx) sum_k |DFT d|^2.  partial[8 y + 0..7] = mass, px, py, e_T
-// part, max |u|, count, x-gradient energy, 0 (k_inv_grad_y fills 7).
+// (1 / nx) sum_k |DFT d|^2.  partial[6 y + 0..5] = mass, px, py, e_T part,
+// max |u|, count; partial[6 ny + y] = x-gradient energy (k_inv_grad_y:
+// partial[7 ny + y]).
 // Per-site values in the working precision (no fp64 square roots or
 // products for fp32 fields), sums in fp64.
 template <typename real>
@@ -452,7 +493,8 @@ __global__ void __launch_bounds__(NT) k_inv_rows(const real *__restrict__ f, rea
             acc = red[tid][0];
             for (int w = 1; w < NT / 32; ++w) acc = tid == 4 ? fmax(acc, red[tid][w]) : acc + red[tid][w];
         }
-        partial[(size_t)y * 8 + tid] = acc;
+        if (tid < 6) partial[(size_t)y * 6 + tid] = acc;
+        else if (tid == 6 && with_grad) partial[(size_t)6 * ny + y] = acc;
     }
 }
 
@@ -460,7 +502,7 @@ __global__ void __launch_bounds__(NT) k_inv_rows(const real *__restrict__ f, rea
 // sum_x (D_y rho)^2 by Parseval's relation from Y = DFT_x(D_y rho) / nx in
 // spectrum slot 2 (the column pass's output; bin 0 packs the real DC and
 // Nyquist values): nx (Y_0.x^2 + Y_0.y^2 + sum_{0<k<h} 2 |Y_k|^2), into
-// partial[8 y + 7].
+// partial[7 ny + y].
 template <typename real>
 __global__ void __launch_bounds__(NT) k_inv_grad_y(const typename cplx_of<real>::type *spec, double *partial,
                                                    KP<real> P) {
@@ -480,32 +522,104 @@ __global__ void __launch_bounds__(NT) k_inv_grad_y(const typename cplx_of<real>:
     if (tid == 0) {
         double acc = 0;
         for (int w = 0; w < NT / 32; ++w) acc += red[w];
-        partial[(size_t)y * 8 + 7] = acc * nx;
+        partial[(size_t)7 * ny + y] = acc * nx;
     }
 }
 
-// The invariants from the per-row partials of k_inv_rows / k_inv_grad_y:
-// out[0..5] = mass, px, py, e_T (with K / 2 times the gradient energy),
-// max |u|, count.
-static __global__ void k_reduce_partials(const double *partial, int ny, double K, double *out) {
-    __shared__ double red[8][NT];
+// Invariant sums without transforms: the moments (Eqs. 7-9) into fields and per
+// block mass, px, py, e_T of Eq. 17 without its gradient part, max |u| and the
+// count of non-finite or unphysical sites, partial[6 block + ..].  Four
+// consecutive sites per thread (N is a multiple of 4: both axes are even), 16
+// bytes a load; bound by the 33 values a site it reads.  Per-site values in
+// the working precision, sums in fp64.
+template <typename real>
+__global__ void __launch_bounds__(256) k_inv_sites(const real *__restrict__ f, real *__restrict__ fields, double *partial,
+                                                   size_t N, real pa, real pb) {
+    __shared__ double red[6][8];
+    struct __align__(16) V4 {
+        real v[4];
+    };
+    double m = 0, px = 0, py = 0, e = 0, bad = 0;
+    real um = 0;
+    for (size_t g = blockIdx.x * (size_t)256 + threadIdx.x; g < N / 4; g += (size_t)gridDim.x * 256) {
+        real m0[4] = {0, 0, 0, 0}, m1[4] = {0, 0, 0, 0}, m2[4] = {0, 0, 0, 0}, m3[4] = {0, 0, 0, 0};
+#pragma unroll 11
+        for (int i = 0; i < Q; ++i) {
+            const V4 w = *reinterpret_cast<const V4 *>(f + (size_t)i * N + 4 * g);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                m0[s] += w.v[s];
+                m1[s] += VX<real>(i) * w.v[s];
+                m2[s] += VY<real>(i) * w.v[s];
+                m3[s] += V2<real>(i) * w.v[s];
+            }
+        }
+        V4 o[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const real rho = m0[s], ux = m1[s] / rho, uy = m2[s] / rho, u2 = ux * ux + uy * uy;
+            const real T = real(0.5) * (m3[s] / rho - u2);
+            o[0].v[s] = rho;
+            o[1].v[s] = ux;
+            o[2].v[s] = uy;
+            o[3].v[s] = T;
+            m += (double)rho;
+            px += (double)(rho * ux);
+            py += (double)(rho * uy);
+            e += (double)(rho * T - pa * rho * rho + rho * u2 * real(0.5));
+            um = um > sqrt(u2) ? um : sqrt(u2);
+            const bool ok = isfinite(rho) && isfinite(ux) && isfinite(uy) && isfinite(T) && rho > real(0) && T > real(0) &&
+                            pb * rho < real(1);
+            bad += ok ? 0.0 : 1.0;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) *reinterpret_cast<V4 *>(fields + (size_t)q * N + 4 * g) = o[q];
+    }
+    double v[6] = {m, px, py, e, (double)um, bad};
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+        for (int w = 16; w > 0; w >>= 1) {
+            const double o = __shfl_down_sync(0xffffffffu, v[q], w);
+            v[q] = q == 4 ? fmax(v[q], o) : v[q] + o;
+        }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane == 0)
+        for (int q = 0; q < 6; ++q) red[q][warp] = v[q];
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        double acc = red[threadIdx.x][0];
+        for (int w = 1; w < 8; ++w) acc = threadIdx.x == 4 ? fmax(acc, red[threadIdx.x][w]) : acc + red[threadIdx.x][w];
+        partial[(size_t)blockIdx.x * 6 + threadIdx.x] = acc;
+    }
+}
+
+// The invariants from n blocks' six partial sums and the ng gradient-energy
+// partials after them: out[0..5] = mass, px, py, e_T (with K / 2 times the
+// gradient energy), max |u|, count; out[6] = the device error word.
+static __global__ void k_reduce_partials(const double *partial, int n, int ng, double K, double *out, const int *err) {
+    __shared__ double red[7][NT / 32];
     const int tid = threadIdx.x;
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int y = tid; y < ny; y += NT) {
-        for (int q = 0; q < 8; ++q) {
-            const double v = partial[(size_t)y * 8 + q];
+    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
+    for (int b = tid; b < n; b += NT)
+        for (int q = 0; q < 6; ++q) {
+            const double v = partial[(size_t)b * 6 + q];
             acc[q] = (q == 4) ? fmax(acc[q], v) : acc[q] + v;
         }
-    }
-    for (int q = 0; q < 8; ++q) red[q][tid] = acc[q];
+    for (int b = tid; b < ng; b += NT) acc[6] += partial[(size_t)6 * n + b];
+    for (int q = 0; q < 7; ++q)
+        for (int w = 16; w > 0; w >>= 1) {
+            const double o = __shfl_down_sync(0xffffffffu, acc[q], w);
+            acc[q] = q == 4 ? fmax(acc[q], o) : acc[q] + o;
+        }
+    if ((tid & 31) == 0)
+        for (int q = 0; q < 7; ++q) red[q][tid >> 5] = acc[q];
     __syncthreads();
-    for (int w = NT / 2; w > 0; w >>= 1) {
-        if (tid < w)
-            for (int q = 0; q < 8; ++q)
-                red[q][tid] = (q == 4) ? fmax(red[q][tid], red[q][tid + w]) : red[q][tid] + red[q][tid + w];
-        __syncthreads();
+    if (tid == 0) {
+        for (int q = 0; q < 7; ++q)
+            for (int w = 1; w < NT / 32; ++w) red[q][0] = q == 4 ? fmax(red[q][0], red[q][w]) : red[q][0] + red[q][w];
+        for (int q = 0; q < 6; ++q) out[q] = q == 3 ? red[3][0] + 0.5 * K * red[6][0] : red[q][0];
+        out[6] = (double)*err;
     }
-    if (tid < 6) out[tid] = tid == 3 ? red[3][0] + 0.5 * K * (red[6][0] + red[7][0]) : red[tid][0];
 }
 
 }  // namespace fftlb
@@ -603,11 +717,14 @@ class EngineT : public Engine {
         const double *src[4] = {rho, ux, uy, T};
         for (int i = 0; i < 4; ++i)
             if (!src[i]) return Status::err(FFTLB_ERR_ARG, "set_fields: NULL field");
-        double *tmp = reinterpret_cast<double *>(scratch_d_);
-        for (int i = 0; i < 4; ++i)
-            FFTLB_CU(cudaMemcpyAsync(tmp + i * N_, src[i], N_ * sizeof(double),
-                                     on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, stream_));
-        k_feq_init<real><<<grid1d(), 256, 0, stream_>>>(tmp, tmp + N_, tmp + 2 * N_, tmp + 3 * N_, f0_, N_);
+        if (!on_device) {
+            double *tmp = reinterpret_cast<double *>(scratch_d_);
+            for (int i = 0; i < 4; ++i) {
+                FFTLB_CU(cudaMemcpyAsync(tmp + i * N_, src[i], N_ * sizeof(double), cudaMemcpyHostToDevice, stream_));
+                src[i] = tmp + i * N_;
+            }
+        }
+        k_feq_init<real><<<grid1d(), 256, 0, stream_>>>(src[0], src[1], src[2], src[3], f0_, N_);
         FFTLB_LAUNCHED("k_feq_init");
         FFTLB_CU(cudaStreamSynchronize(stream_));
         steps_ = 0;
@@ -646,18 +763,19 @@ class EngineT : public Engine {
             Status st = check_err();
             if (!st.good()) return st;
         }
-        k_moments<real><<<grid1d(), 256, 0, stream_>>>(f0_, fields_, N_);
-        FFTLB_LAUNCHED("k_moments");
-        double *tmp = reinterpret_cast<double *>(scratch_d_);
-        k_convert<real, double><<<grid1d(), 256, 0, stream_>>>(fields_, tmp, 4 * N_);
-        FFTLB_LAUNCHED("k_convert");
         double *dst[4] = {rho, ux, uy, T};
-        for (int i = 0; i < 4; ++i) {
-            if (!dst[i]) continue;
-            FFTLB_CU(cudaMemcpyAsync(dst[i], tmp + i * N_, N_ * sizeof(double),
-                                     on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, stream_));
-        }
-        if (!on_device) FFTLB_CU(cudaStreamSynchronize(stream_));
+        double *tmp = reinterpret_cast<double *>(scratch_d_);
+        FieldPtrs o;
+        for (int i = 0; i < 4; ++i) o.p[i] = on_device ? dst[i] : dst[i] ? tmp + i * N_ : nullptr;
+        if (aligned16(o.p[0]) && aligned16(o.p[1]) && aligned16(o.p[2]) && aligned16(o.p[3]))
+            k_fields_out<real, 4><<<grid1d(4), 256, 0, stream_>>>(f0_, o, N_);
+        else
+            k_fields_out<real, 1><<<grid1d(), 256, 0, stream_>>>(f0_, o, N_);
+        FFTLB_LAUNCHED("k_fields_out");
+        if (on_device) return Status::ok();
+        for (int i = 0; i < 4; ++i)
+            if (dst[i]) FFTLB_CU(cudaMemcpyAsync(dst[i], o.p[i], N_ * sizeof(double), cudaMemcpyDeviceToHost, stream_));
+        FFTLB_CU(cudaStreamSynchronize(stream_));
         return Status::ok();
     }
 
@@ -667,22 +785,34 @@ class EngineT : public Engine {
             FFTLB_CU(cudaMemcpyAsync(f, f0_, Q * N_ * sizeof(double), cudaMemcpyDeviceToDevice, stream_));
             return Status::ok();
         }
-        double *tmp = reinterpret_cast<double *>(scratch_d_);   // scratch holds >= 33 N doubles
-        k_convert<real, double><<<grid1d(), 256, 0, stream_>>>(f0_, tmp, Q * N_);
-        FFTLB_LAUNCHED("k_convert");
-        FFTLB_CU(cudaMemcpyAsync(f, tmp, Q * N_ * sizeof(double),
-                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, stream_));
-        if (!on_device) FFTLB_CU(cudaStreamSynchronize(stream_));
+        if (on_device) return convert<real, double>(f0_, f);
+        const double *src = reinterpret_cast<const double *>(f0_);
+        if (sizeof(real) == 4) {
+            double *tmp = reinterpret_cast<double *>(scratch_d_);   // scratch holds >= 33 N doubles
+            Status st = convert<real, double>(f0_, tmp);
+            if (!st.good()) return st;
+            src = tmp;
+        }
+        FFTLB_CU(cudaMemcpyAsync(f, src, Q * N_ * sizeof(double), cudaMemcpyDeviceToHost, stream_));
+        FFTLB_CU(cudaStreamSynchronize(stream_));
         return Status::ok();
     }
 
     Status set_f(const double *f, bool on_device) override {
         if (!f) return Status::err(FFTLB_ERR_ARG, "set_f: NULL");
-        double *tmp = reinterpret_cast<double *>(scratch_d_);
-        FFTLB_CU(cudaMemcpyAsync(tmp, f, Q * N_ * sizeof(double),
-                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, stream_));
-        k_convert<double, real><<<grid1d(), 256, 0, stream_>>>(tmp, f0_, Q * N_);
-        FFTLB_LAUNCHED("k_convert");
+        if (sizeof(real) == 8) {
+            FFTLB_CU(cudaMemcpyAsync(f0_, f, Q * N_ * sizeof(double),
+                                     on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, stream_));
+        } else {
+            const double *src = f;
+            if (!on_device) {
+                double *tmp = reinterpret_cast<double *>(scratch_d_);
+                FFTLB_CU(cudaMemcpyAsync(tmp, f, Q * N_ * sizeof(double), cudaMemcpyHostToDevice, stream_));
+                src = tmp;
+            }
+            Status st = convert<double, real>(src, f0_);
+            if (!st.good()) return st;
+        }
         FFTLB_CU(cudaStreamSynchronize(stream_));
         return Status::ok();
     }
@@ -704,6 +834,22 @@ class EngineT : public Engine {
     Status gradient(const double *g, double *out, int nfields) override {
         if (!g || !out || nfields < 1 || nfields > 16)
             return Status::err(FFTLB_ERR_ARG, "gradient: need device pointers and 1 <= nfields <= 16");
+        if (rowcol_) {   // D_x by rows, D_y by columns, straight between the caller's buffers
+            GradArgs<real> a{};
+            a.g = reinterpret_cast<const double2 *>(g);
+            a.out = reinterpret_cast<double2 *>(out);
+            a.rtab = Trow_;
+            a.ctab = Tcr_;
+            a.ky = kyt_;
+            a.h = h_;
+            a.ny = ny_;
+            a.nrows = ny_ * nfields;
+            a.err = err_;
+            void *args[1] = {&a};
+            FFTLB_CU(cudaLaunchKernel(rs_.dx, dim3((a.nrows + rs_.ng - 1) / rs_.ng), dim3(rs_.nt), args, rs_.smem_rows, stream_));
+            FFTLB_CU(cudaLaunchKernel(cs_.dy, dim3(col_tiles(), nfields), dim3(cs_.nt), args, cs_.smem, stream_));
+            return Status::ok();
+        }
         // the stage's transform code (and, for split handles, its split-BF16
         // first passes); field i in slot i -> D_x, D_y in slots 20 + 2i, 21 + 2i
         Status st = grad_config();
@@ -763,7 +909,7 @@ class EngineT : public Engine {
     uint4 *tc16_ = nullptr;             // their A fragments (dft16_fragments)
     int ntr_ = 0, ntc_ = 0, ntr8_ = 0;
     GroupDesc *groups_ = nullptr;
-    double *partial_ = nullptr, *red_ = nullptr;
+    double *partial_ = nullptr, *red_ = nullptr, *host_red_ = nullptr;   // host_red_: pinned
     void *scratch_d_ = nullptr;
     std::vector<void *> allocs_;
     // group ranges in groups_
@@ -785,7 +931,8 @@ class EngineT : public Engine {
     CUtensorMap tmap_convw_{}, fmap_convw_[2] = {};
     // row and column kernels of kernels_row.cuh / kernels_col.cuh, the
     // argument blocks of their launches, and their tables
-    bool rowk_ = false, colk_ = false;
+    bool rowk_ = false, colk_ = false;   // taken by the stage
+    bool rowcol_ = false;                // both exist for this grid (gradient, invariants)
     RowSet rs_;
     ColSet cs_;
     RowArgs<real> ra_{};
@@ -895,9 +1042,19 @@ class EngineT : public Engine {
         fields_ = fieldsb_ + r * NSLOT * N_;
     }
 
-    unsigned grid1d() const {
-        size_t b = (N_ + 255) / 256;
+    unsigned grid1d(int per = 1) const {   // per: sites per thread
+        size_t b = (N_ / per + 255) / 256;
         return (unsigned)(b > 4096 ? 4096 : b);
+    }
+    static bool aligned16(const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
+    // 33 N values from src to dst
+    template <typename TI, typename TO> Status convert(const TI *src, TO *dst) {
+        if (aligned16(src) && aligned16(dst))
+            k_convert<TI, TO, 4><<<8 * nsm_, 256, 0, stream_>>>(src, dst, Q * N_);
+        else
+            k_convert<TI, TO, 1><<<8 * nsm_, 256, 0, stream_>>>(src, dst, Q * N_);
+        FFTLB_LAUNCHED("k_convert");
+        return Status::ok();
     }
 
     template <typename T> Status dalloc(T **ptr, size_t count) {
@@ -914,6 +1071,8 @@ class EngineT : public Engine {
 
     void release() {
         for (void *p : allocs_) cudaFree(p);
+        if (host_red_) cudaFreeHost(host_red_);
+        host_red_ = nullptr;
         allocs_.clear();
     }
 
@@ -1003,7 +1162,12 @@ class EngineT : public Engine {
         if (!(st = dalloc(&Wr_, (size_t)h_)).good()) return st;
         if (!(st = dalloc(&Wp_, (size_t)h_)).good()) return st;
         if (!(st = dalloc(&Wc_, (size_t)ny_)).good()) return st;
-        if (!(st = dalloc(&partial_, (size_t)ny_ * 8)).good()) return st;
+        // partial sums: 6 per block of k_inv_sites (or row of k_inv_rows), one per block of the energies
+        if (!(st = dalloc(&partial_, (size_t)6 * std::max<size_t>(ny_, 4096) + 2 * (size_t)ny_ + h_)).good()) return st;
+        if (cudaMallocHost((void **)&host_red_, 8 * sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
+            return Status::err(FFTLB_ERR_OOM, "cudaMallocHost failed");
+        }
         if (!(st = dalloc(&red_, 8)).good()) return st;
         if (!(st = dalloc(&err_, 4)).good()) return st;
         FFTLB_CU(cudaMemset(err_, 0, 4 * sizeof(int)));
@@ -1630,6 +1794,7 @@ class EngineT : public Engine {
 
     // the kernels of kernels_row.cuh / kernels_col.cuh where they apply
     Status configure_rowcol() {
+        bool rows_ok = false;
         if constexpr (sizeof(real) == 4) {
             rs_ = row_set_f32_p2(h_);
             if (!rs_.k1) rs_ = row_set_f32_r3(h_);
@@ -1642,9 +1807,10 @@ class EngineT : public Engine {
         if (!own_len(h_)) rs_ = RowSet();
         if (!own_len(ny_)) cs_ = ColSet();
         if (rs_.k1 && std::max({rs_.smem1, rs_.smem3, rs_.smem5}) <= budget_) {
-            const void *ks[3] = {rs_.k1, rs_.k3, rs_.k5};
+            const void *ks[5] = {rs_.k1, rs_.k3, rs_.k5, rs_.dx, rs_.energy};
             for (const void *k : ks)
                 FFTLB_CU(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget_));
+            rows_ok = rs_.smem_rows <= budget_;
             ra_.ny = ny_;
             ra_.nrun = B_;
             ra_.dt = kp_.dt;
@@ -1671,7 +1837,10 @@ class EngineT : public Engine {
             rowk_ = !(k1wr_ && k3wr_ && k5wr_ && (long)B_ * ny_ >= 2L * nsm_);
         }
         if (cs_.k && (cs_.tw == 0 || h_ % cs_.tw == 0) && cs_.smem <= budget_) {
-            if (cs_.tw) FFTLB_CU(cudaFuncSetAttribute(cs_.k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget_));
+            rowcol_ = rows_ok;
+            const void *ks[3] = {cs_.k, cs_.dy, cs_.energy};
+            for (const void *k : ks)
+                if (cs_.tw) FFTLB_CU(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget_));
             // kcol_wr keeps the lengths 512 and 1024, where its prefetch and
             // (512) its wider tiles pay: convection and level 2 at 1024^2 79
             // and 19 us against 90 and 28, at 512^2 25 and 12 against 25 and
@@ -1702,6 +1871,7 @@ class EngineT : public Engine {
         }
         return Status::ok();
     }
+    unsigned col_tiles() const { return cs_.tw ? (unsigned)(h_ / cs_.tw) : (unsigned)((h_ + 127) / 128); }
     // one launch of column jobs: every group, tile and run
     Status launch_cols(ColArgs<real> &a, int nrun) {
         const unsigned jobs = cs_.tw ? (unsigned)(a.ngroups * (h_ / cs_.tw)) : (unsigned)((a.ngroups * h_ + 127) / 128);
@@ -2149,34 +2319,62 @@ class EngineT : public Engine {
 
     // device error word (bounded waits that ran out)
     Status check_err() {
-        int e = 0;
-        FFTLB_CU(cudaMemcpyAsync(&e, err_, sizeof(int), cudaMemcpyDeviceToHost, stream_));
+        int *e = reinterpret_cast<int *>(host_red_);
+        FFTLB_CU(cudaMemcpyAsync(e, err_, sizeof(int), cudaMemcpyDeviceToHost, stream_));
         FFTLB_CU(cudaStreamSynchronize(stream_));
-        if (e) return Status::err(FFTLB_ERR_TIMEOUT, "a bounded device wait ran out (error word " + std::to_string(e) + ")");
+        if (*e) return Status::err(FFTLB_ERR_TIMEOUT, "a bounded device wait ran out (error word " + std::to_string(*e) + ")");
         return Status::ok();
     }
 
     // (one synchronisation: the sums and the device error word of the steps
     // before them come back together)
     Status sums(bool with_grad, double out[6]) {
-        k_inv_rows<real><<<ny_, NT, with_grad ? smem_rows1_ : 0, stream_>>>(f0_, fields_, spec_, partial_, Wr_, Wp_,
-                                                                          kxt_, kp_, with_grad ? 1 : 0);
-        FFTLB_LAUNCHED("k_inv_rows");
-        if (with_grad) {
-            Status st = launch_col(inv_groups_, 1, false);
-            if (!st.good()) return st;
-            k_inv_grad_y<real><<<ny_, NT, 0, stream_>>>(spec_, partial_, kp_);
-            FFTLB_LAUNCHED("k_inv_grad_y");
+        int n0 = 0, nx0 = 0, ny0 = 0;   // blocks of the site sums and of the two energies
+        if (rowcol_) {
+            n0 = inv_blocks();
+            k_inv_sites<real><<<n0, 256, 0, stream_>>>(f0_, fields_, partial_, N_, kp_.a, kp_.b);
+            FFTLB_LAUNCHED("k_inv_sites");
+            if (with_grad) {
+                EnergyArgs<real> a{};
+                a.rho = reinterpret_cast<const C *>(fields_);
+                a.rtab = Trow_;
+                a.ctab = Tcr_;
+                a.ky = kyt_;
+                a.h = h_;
+                a.ny = ny_;
+                a.err = err_;
+                nx0 = (ny_ + rs_.ng - 1) / rs_.ng;
+                ny0 = (int)col_tiles();
+                a.partial_x = partial_ + (size_t)n0 * 6;
+                a.partial_y = a.partial_x + nx0;
+                void *args[1] = {&a};
+                FFTLB_CU(cudaLaunchKernel(rs_.energy, dim3(nx0), dim3(rs_.nt), args, rs_.smem_rows, stream_));
+                FFTLB_CU(cudaLaunchKernel(cs_.energy, dim3(ny0), dim3(cs_.nt), args, cs_.smem, stream_));
+            }
+        } else {
+            n0 = ny_;
+            k_inv_rows<real><<<ny_, NT, with_grad ? smem_rows1_ : 0, stream_>>>(f0_, fields_, spec_, partial_, Wr_, Wp_,
+                                                                              kxt_, kp_, with_grad ? 1 : 0);
+            FFTLB_LAUNCHED("k_inv_rows");
+            if (with_grad) {
+                Status st = launch_col(inv_groups_, 1, false);
+                if (!st.good()) return st;
+                k_inv_grad_y<real><<<ny_, NT, 0, stream_>>>(spec_, partial_, kp_);
+                FFTLB_LAUNCHED("k_inv_grad_y");
+                nx0 = ny0 = ny_;
+            }
         }
-        k_reduce_partials<<<1, NT, 0, stream_>>>(partial_, ny_, (double)p_.K, red_);
+        k_reduce_partials<<<1, NT, 0, stream_>>>(partial_, n0, nx0 + ny0, (double)p_.K, red_, err_);
         FFTLB_LAUNCHED("k_reduce_partials");
-        int e = 0;
-        FFTLB_CU(cudaMemcpyAsync(out, red_, 6 * sizeof(double), cudaMemcpyDeviceToHost, stream_));
-        FFTLB_CU(cudaMemcpyAsync(&e, err_, sizeof(int), cudaMemcpyDeviceToHost, stream_));
+        FFTLB_CU(cudaMemcpyAsync(host_red_, red_, 8 * sizeof(double), cudaMemcpyDeviceToHost, stream_));
         FFTLB_CU(cudaStreamSynchronize(stream_));
+        for (int q = 0; q < 6; ++q) out[q] = host_red_[q];
+        const int e = (int)host_red_[6];
         if (e) return Status::err(FFTLB_ERR_TIMEOUT, "a bounded device wait ran out (error word " + std::to_string(e) + ")");
         return Status::ok();
     }
+    // blocks of k_inv_sites: enough for every SM, each with whole vectors of sites
+    int inv_blocks() const { return (int)std::min<size_t>((N_ / 4 + 255) / 256, (size_t)4 * nsm_); }
 };
 
 }  // namespace fftlb

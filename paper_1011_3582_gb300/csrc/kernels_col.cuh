@@ -22,6 +22,7 @@
 
 #include "async_copy.cuh"
 #include "col_kernels.h"
+#include "block_sum.cuh"
 #include "fft_small.cuh"
 #include "stage_layout.cuh"
 
@@ -59,54 +60,58 @@ template <typename real, int NY> constexpr int col_minb() {
     return sizeof(real) == 4 || (G::E <= 16 && G::PH <= 16) ? (512 / G::NT > 16 ? 16 : 512 / G::NT) : (256 / G::NT > 16 ? 16 : 256 / G::NT);
 }
 
-template <typename real, int NY>
-__global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_reg(const __grid_constant__ ColArgs<real> A) {
+// The tables of kcol_reg's length in shared memory behind the tile (copied by
+// thread 0 while the tile loads) or in global memory.
+template <typename real, int NY> struct ColTab {
+    using G = Col<real, NY>;
+    using C = typename G::C;
+    const C *tw, *twt, *wp;
+    const real *ky;
+    __device__ __forceinline__ ColTab(C *tile, const C *g) {
+        tw = G::TABS ? tile + (size_t)NY * G::TW : g;
+        twt = tw + NY;
+        wp = twt + NY;
+        ky = reinterpret_cast<const real *>(wp + G::P);
+    }
+    static __device__ __forceinline__ void issue(C *tile, const C *g, uint64_t *bar) {
+        if (G::TABS && threadIdx.x == 0) {
+            mbar_init(bar, 1);
+            mbar_init_fence();
+            mbar_expect_tx(bar, col_table_bytes<real>(NY, G::P));
+            bulk_g2s(tile + (size_t)NY * G::TW, g, col_table_bytes<real>(NY, G::P), bar);
+        }
+    }
+    // the block's wait; false if it ran out (the copy is no longer in flight)
+    static __device__ __forceinline__ bool wait(uint64_t *bar, int *err) {
+        if constexpr (G::TABS) {
+            __syncthreads();   // the barrier is initialised before any thread polls it
+            if (!block_wait(bar, 0, err)) {
+                mbar_wait_bounded(bar, 0);
+                return false;
+            }
+        }
+        return true;
+    }
+};
+
+// The passes of thread (c, jl) over a tile: v = x[jl + P t] of column c in; with
+// INV, v = the inverse transform of mult(k, X[k]) out, otherwise mult sees
+// every X[k] once and v is undefined.  Returns false if the tables never came.
+template <typename real, int NY, bool INV, typename Mult>
+__device__ __forceinline__ bool col_pass(typename Col<real, NY>::C (&v)[Col<real, NY>::E], typename Col<real, NY>::C *T,
+                                         const ColTab<real, NY> &tb, uint64_t *bar, int *err, int c, int jl,
+                                         const Mult &mult) {
     using G = Col<real, NY>;
     using C = typename G::C;
     constexpr int E = G::E, P = G::P, PH = G::PH, TW = G::TW;
-    extern __shared__ __align__(128) unsigned char col_smem_raw[];
-    __shared__ __align__(8) uint64_t bar;
-    C *T = reinterpret_cast<C *>(col_smem_raw);   // [NY][TW]
-    const C *tw = G::TABS ? T + (size_t)NY * TW : A.tab, *twt = tw + NY, *wp = twt + NY;   // the table block
-    const real *ky = reinterpret_cast<const real *>(wp + P);
-    const int h = A.h, tid = threadIdx.x, c = tid % TW, jl = tid / TW;
-    const int ntiles = h / TW;
-    const int job = (int)blockIdx.x, g = job / ntiles, t = job - g * ntiles;   // (grid.y: run)
-    const size_t slot = (size_t)NY * h;
-    const ColGroup<real> &gr = A.g[g];
-    C *spec = A.spec + (size_t)blockIdx.y * NSLOT * slot + t * TW + c;
-    // (no slot is both read and written by different columns of one launch)
-    const C *__restrict__ in = gr.from_f ? A.f + ((size_t)blockIdx.y * Q + gr.in) * slot + t * TW + c : spec + (size_t)gr.in * slot;
-    if (G::TABS && tid == 0) {
-        mbar_init(&bar, 1);
-        mbar_init_fence();
-        mbar_expect_tx(&bar, col_table_bytes<real>(NY, P));
-        bulk_g2s(T + (size_t)NY * TW, A.tab, col_table_bytes<real>(NY, P), &bar);
-    }
-    C v[E];
-#pragma unroll
-    for (int q = 0; q < E; ++q) v[q] = in[(size_t)(jl + P * q) * h];
     SmallDFT<E, -1, C>::run(v);
-    if constexpr (G::TABS) {
-        __syncthreads();   // the barrier is initialised before any thread polls it
-        if (!block_wait(&bar, 0, A.err)) {
-            mbar_wait_bounded(&bar, 0);
-            return;
-        }
-    }
+    if (!ColTab<real, NY>::wait(bar, err)) return false;
 #pragma unroll
-    for (int k1 = 1; k1 < E; ++k1) v[k1] = cmul(v[k1], tab<G::TABS>(tw + k1 * P + jl));
+    for (int k1 = 1; k1 < E; ++k1) v[k1] = cmul(v[k1], tab<G::TABS>(tb.tw + k1 * P + jl));
 #pragma unroll
     for (int k1 = 0; k1 < E; ++k1) T[cp<real, NY>(c, jl, k1)] = v[k1];
     __syncthreads();
     // stage 2: forward, multiplier, inverse, conjugate twiddles
-    const real mx = gr.c0 * __ldg(A.kx + t * TW + c), c1 = gr.c1, c3 = gr.c3;
-    auto mult = [&](int k, C u) {
-        const real ay = tab<G::TABS>(ky + k);
-        if (c3 != real(0)) return cscale(u, c3 * ay * ay);   // uniform over the block
-        const real m = mx + c1 * ay;
-        return C{-m * u.y, m * u.x};
-    };
     if constexpr (!G::PAIR) {
 #pragma unroll
         for (int q = 0; q < (E + P - 1) / P; ++q) {
@@ -118,10 +123,12 @@ __global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_
                 SmallDFT<P, -1, C>::run(u);
 #pragma unroll
                 for (int k2 = 0; k2 < P; ++k2) u[k2] = mult(k1 + E * k2, u[k2]);
-                SmallDFT<P, +1, C>::run(u);
+                if constexpr (INV) {
+                    SmallDFT<P, +1, C>::run(u);
 #pragma unroll
-                for (int l = 0; l < P; ++l)
-                    T[cp<real, NY>(c, l, k1)] = l == 0 ? u[l] : cmul(u[l], cconj(tab<G::TABS>(twt + l * E + k1)));
+                    for (int l = 0; l < P; ++l)
+                        T[cp<real, NY>(c, l, k1)] = l == 0 ? u[l] : cmul(u[l], cconj(tab<G::TABS>(tb.twt + l * E + k1)));
+                }
             }
         }
     } else if (jl < 2 * E) {   // (whole warps)
@@ -143,31 +150,174 @@ __global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_
             recv.y = __shfl_xor_sync(0xffffffffu, send.y, TW);
             const C a = gg ? recv : u[i], b = gg ? u[HH + i] : recv;
             const int k2 = HH * gg + i;
-            const C w = tab<G::TABS>(wp + k2);   // W_P^k2
-            const C tb = cmul(b, w);
-            const C x0 = mult(k1 + E * k2, cadd(a, tb)), x1 = mult(k1 + E * (k2 + PH), csub(a, tb));
-            const C ai = cadd(x0, x1), bi = cmul(csub(x0, x1), cconj(w));
-            const C back = gg ? ai : bi;   // thread 0 keeps the even half (ai), thread 1 the odd (bi)
-            C got;
-            got.x = __shfl_xor_sync(0xffffffffu, back.x, TW);
-            got.y = __shfl_xor_sync(0xffffffffu, back.y, TW);
-            u[i] = gg ? got : ai;
-            u[HH + i] = gg ? bi : got;
+            const C w = tab<G::TABS>(tb.wp + k2);   // W_P^k2
+            const C t = cmul(b, w);
+            const C x0 = mult(k1 + E * k2, cadd(a, t)), x1 = mult(k1 + E * (k2 + PH), csub(a, t));
+            if constexpr (INV) {
+                const C ai = cadd(x0, x1), bi = cmul(csub(x0, x1), cconj(w));
+                const C back = gg ? ai : bi;   // thread 0 keeps the even half (ai), thread 1 the odd (bi)
+                C got;
+                got.x = __shfl_xor_sync(0xffffffffu, back.x, TW);
+                got.y = __shfl_xor_sync(0xffffffffu, back.y, TW);
+                u[i] = gg ? got : ai;
+                u[HH + i] = gg ? bi : got;
+            }
         }
-        SmallDFT<PH, +1, C>::run(u);
+        if constexpr (INV) {
+            SmallDFT<PH, +1, C>::run(u);
 #pragma unroll
-        for (int m = 0; m < PH; ++m) {
-            const int l = gg + 2 * m;
-            T[cp<real, NY>(c, l, k1)] = cmul(u[m], cconj(tab<G::TABS>(twt + l * E + k1)));
+            for (int m = 0; m < PH; ++m) {
+                const int l = gg + 2 * m;
+                T[cp<real, NY>(c, l, k1)] = cmul(u[m], cconj(tab<G::TABS>(tb.twt + l * E + k1)));
+            }
         }
     }
-    __syncthreads();
+    if constexpr (INV) {
+        __syncthreads();
+#pragma unroll
+        for (int k1 = 0; k1 < E; ++k1) v[k1] = T[cp<real, NY>(c, jl, k1)];
+        SmallDFT<E, +1, C>::run(v);
+    }
+    return true;
+}
+
+template <typename real, int NY>
+__global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_reg(const __grid_constant__ ColArgs<real> A) {
+    using G = Col<real, NY>;
+    using C = typename G::C;
+    constexpr int E = G::E, P = G::P, TW = G::TW;
+    extern __shared__ __align__(128) unsigned char col_smem_raw[];
+    __shared__ __align__(8) uint64_t bar;
+    C *T = reinterpret_cast<C *>(col_smem_raw);   // [NY][TW]
+    const ColTab<real, NY> tb(T, A.tab);
+    const int h = A.h, tid = threadIdx.x, c = tid % TW, jl = tid / TW;
+    const int ntiles = h / TW;
+    const int job = (int)blockIdx.x, g = job / ntiles, t = job - g * ntiles;   // (grid.y: run)
+    const size_t slot = (size_t)NY * h;
+    const ColGroup<real> &gr = A.g[g];
+    C *spec = A.spec + (size_t)blockIdx.y * NSLOT * slot + t * TW + c;
+    // (no slot is both read and written by different columns of one launch)
+    const C *__restrict__ in =
+        gr.from_f ? A.f + ((size_t)blockIdx.y * Q + gr.in) * slot + t * TW + c : spec + (size_t)gr.in * slot;
+    ColTab<real, NY>::issue(T, A.tab, &bar);
+    C v[E];
+#pragma unroll
+    for (int q = 0; q < E; ++q) v[q] = in[(size_t)(jl + P * q) * h];
+    const real mx = gr.c0 * __ldg(A.kx + t * TW + c), c1 = gr.c1, c3 = gr.c3;
+    const bool ok = col_pass<real, NY, true>(v, T, tb, &bar, A.err, c, jl, [&](int k, C u) {
+        const real ay = tab<G::TABS>(tb.ky + k);
+        if (c3 != real(0)) return cscale(u, c3 * ay * ay);   // uniform over the block
+        const real m = mx + c1 * ay;
+        return C{-m * u.y, m * u.x};
+    });
+    if (!ok) return;
     C *out = spec + (size_t)gr.out * slot;
 #pragma unroll
-    for (int k1 = 0; k1 < E; ++k1) v[k1] = T[cp<real, NY>(c, jl, k1)];
-    SmallDFT<E, +1, C>::run(v);
-#pragma unroll
     for (int q = 0; q < E; ++q) out[(size_t)(jl + P * q) * h] = v[q];
+}
+
+// D_y of caller fields g[field][ny][nx] (fp64) into out[2 field + 1] (see
+// dx_row; grid: (tiles, fields)), the columns taken two real ones at a time as
+// in the stage.
+template <typename real, int NY>
+__global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) dy_col(const __grid_constant__ GradArgs<real> A) {
+    using G = Col<real, NY>;
+    using C = typename G::C;
+    constexpr int E = G::E, P = G::P, TW = G::TW;
+    extern __shared__ __align__(128) unsigned char col_smem_raw[];
+    __shared__ __align__(8) uint64_t bar;
+    C *T = reinterpret_cast<C *>(col_smem_raw);
+    const ColTab<real, NY> tb(T, A.ctab);
+    const int h = A.h, c = threadIdx.x % TW, jl = threadIdx.x / TW;
+    const size_t slot = (size_t)NY * h, at = (size_t)blockIdx.x * TW + c;
+    const double2 *__restrict__ in = A.g + (size_t)blockIdx.y * slot + at;
+    ColTab<real, NY>::issue(T, A.ctab, &bar);
+    C v[E];
+#pragma unroll
+    for (int q = 0; q < E; ++q) {
+        const double2 x = in[(size_t)(jl + P * q) * h];
+        v[q] = C{(real)x.x, (real)x.y};
+    }
+    const real s = real(1.0 / NY);
+    const bool ok = col_pass<real, NY, true>(v, T, tb, &bar, A.err, c, jl, [&](int k, C u) {
+        const real m = tab<G::TABS>(tb.ky + k) * s;
+        return C{-m * u.y, m * u.x};
+    });
+    if (!ok) return;
+    double2 *out = A.out + (2 * (size_t)blockIdx.y + 1) * slot + at;
+#pragma unroll
+    for (int q = 0; q < E; ++q) out[(size_t)(jl + P * q) * h] = make_double2((double)v[q].x, (double)v[q].y);
+}
+template <typename real, int NY>
+__global__ void __launch_bounds__(128) dy_line(const __grid_constant__ GradArgs<real> A) {
+    using C = typename cplx_of<real>::type;
+    const int h = A.h, kx = (int)blockIdx.x * 128 + (int)threadIdx.x;
+    if (kx >= h) return;
+    const size_t slot = (size_t)NY * h;
+    const double2 *in = A.g + (size_t)blockIdx.y * slot + kx;
+    C v[NY];
+#pragma unroll
+    for (int y = 0; y < NY; ++y) {
+        const double2 x = in[(size_t)y * h];
+        v[y] = C{(real)x.x, (real)x.y};
+    }
+    SmallDFT<NY, -1, C>::run(v);
+#pragma unroll
+    for (int k = 0; k < NY; ++k) {
+        const real m = __ldg(A.ky + k) * real(1.0 / NY);
+        v[k] = C{-m * v[k].y, m * v[k].x};
+    }
+    SmallDFT<NY, +1, C>::run(v);
+    double2 *out = A.out + (2 * (size_t)blockIdx.y + 1) * slot + kx;
+#pragma unroll
+    for (int y = 0; y < NY; ++y) out[(size_t)y * h] = make_double2((double)v[y].x, (double)v[y].y);
+}
+
+// Sum over the tile's columns of (D_y rho)^2 by Parseval's relation, from the
+// real field rho two columns at a time: with Z the transform of f + i f',
+// sum_y (D_y f)^2 + (D_y f')^2 = (1 / ny) sum_k k_y^2 |Z_k|^2 (no inverse).
+// partial[block]: fp64.
+template <typename real, int NY>
+__global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) energy_col(const __grid_constant__ EnergyArgs<real> A) {
+    using G = Col<real, NY>;
+    using C = typename G::C;
+    constexpr int E = G::E, P = G::P, TW = G::TW;
+    extern __shared__ __align__(128) unsigned char col_smem_raw[];
+    __shared__ __align__(8) uint64_t bar;
+    C *T = reinterpret_cast<C *>(col_smem_raw);
+    const ColTab<real, NY> tb(T, A.ctab);
+    const int h = A.h, c = threadIdx.x % TW, jl = threadIdx.x / TW;
+    const C *__restrict__ in = A.rho + (size_t)blockIdx.x * TW + c;
+    ColTab<real, NY>::issue(T, A.ctab, &bar);
+    C v[E];
+#pragma unroll
+    for (int q = 0; q < E; ++q) v[q] = in[(size_t)(jl + P * q) * h];
+    double e = 0;
+    const bool ok = col_pass<real, NY, false>(v, T, tb, &bar, A.err, c, jl, [&](int k, C u) {
+        const real m = tab<G::TABS>(tb.ky + k);
+        e += (double)(m * m * (u.x * u.x + u.y * u.y));
+        return u;
+    });
+    if (!ok) return;
+    block_sum_store(e * (1.0 / NY), A.partial_y + blockIdx.x);
+}
+template <typename real, int NY>
+__global__ void __launch_bounds__(128) energy_line(const __grid_constant__ EnergyArgs<real> A) {
+    using C = typename cplx_of<real>::type;
+    const int h = A.h, kx = (int)blockIdx.x * 128 + (int)threadIdx.x;
+    double e = 0;
+    if (kx < h) {
+        C v[NY];
+#pragma unroll
+        for (int y = 0; y < NY; ++y) v[y] = A.rho[(size_t)y * h + kx];
+        SmallDFT<NY, -1, C>::run(v);
+#pragma unroll
+        for (int k = 0; k < NY; ++k) {
+            const real m = __ldg(A.ky + k);
+            e += (double)(m * m * (v[k].x * v[k].x + v[k].y * v[k].y));
+        }
+    }
+    block_sum_store(e * (1.0 / NY), A.partial_y + blockIdx.x);
 }
 
 // One column of a short grid per thread.
@@ -207,10 +357,14 @@ template <typename real, int NY> ColSet col_set() {
     ColSet s;
     if constexpr (NY <= 12) {
         s.k = (const void *)&kcol_line<real, NY>;
+        s.dy = (const void *)&dy_line<real, NY>;
+        s.energy = (const void *)&energy_line<real, NY>;
         s.nt = 128;
         s.tw = 0;
     } else {
         s.k = (const void *)&kcol_reg<real, NY>;
+        s.dy = (const void *)&dy_col<real, NY>;
+        s.energy = (const void *)&energy_col<real, NY>;
         s.nt = Col<real, NY>::NT;
         s.tw = Col<real, NY>::TW;
         s.smem = (size_t)NY * s.tw * 2 * sizeof(real) + (Col<real, NY>::TABS ? col_table_bytes<real>(NY, Col<real, NY>::P) : 0);

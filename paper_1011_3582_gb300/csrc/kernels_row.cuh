@@ -29,6 +29,8 @@
 #include <cooperative_groups.h>
 
 #include "async_copy.cuh"
+#include "block_sum.cuh"
+#include "col_kernels.h"
 #include "fft_small.cuh"
 #include "row_kernels.h"
 #include "stage_layout.cuh"
@@ -758,12 +760,137 @@ template <typename real, int H> size_t k5_row_smem() {
            RowTable<real>::bytes(H) - RowTable<real>::tw(H);
 }
 
+// ---------------------------------------------------------------------------
+// Single rows: one row per row group, NG rows per block, no cluster.
+// ---------------------------------------------------------------------------
+
+// Half-length transform Z of a real row -> the packed half-length spectrum of
+// its d_x (i k_x X / nx), in place: row_post, the product and row_pre pair by
+// pair.
+template <int H, typename C>
+__device__ __forceinline__ void row_dx(C *z, const C *wh, const C *wp, const decltype(C::x) *kx, int j) {
+    using R = decltype(z[0].x);
+    constexpr int P = Row<R, H>::P;
+    const R sx = R(1.0 / (2 * H));
+#pragma unroll
+    for (int k0 = 0; k0 <= H / 2; k0 += P) {
+        const int k = k0 + j;
+        if (k > H / 2) break;
+        if (k == 0) {
+            z[0] = C{0, 0};
+        } else {
+            const C p = z[k], q = z[H - k];
+            const C s = cadd(p, cconj(q)), d = csub(p, cconj(q));
+            const C w = cmul(wh[k], cmul_mi(d));
+            const R m = kx[k] * sx, mh = kx[H - k] * sx;
+            // X[k] = s/2 + w, X[H-k] = conj(s/2 - w); Y = i m X
+            const C yk = C{-m * (R(0.5) * s.y + w.y), m * (R(0.5) * s.x + w.x)};
+            const C yc = C{mh * (R(0.5) * s.y - w.y), -mh * (R(0.5) * s.x - w.x)};   // conj Y[H-k]
+            const C a = cadd(yk, yc), e = csub(yk, yc);
+            const C t = cmul_i(cmul(e, cconj(wp[k])));
+            z[k] = cadd(a, t);
+            if (H - k != k) z[H - k] = cconj(csub(a, t));
+        }
+    }
+}
+
+// tables [0, bytes) behind the NG rows of a single-row kernel
+template <typename real, int H>
+__device__ __forceinline__ bool single_tables(unsigned char *tb, const typename Row<real, H>::C *tab, uint64_t *bar, int *err) {
+    if (threadIdx.x == 0) {
+        mbar_init(bar, 1);
+        mbar_init_fence();
+        mbar_expect_tx(bar, RowTable<real>::bytes(H));
+        table_issue(tb, tab, 0, RowTable<real>::bytes(H), bar);
+    }
+    __syncthreads();
+    if (block_wait(bar, 0, err)) return true;
+    mbar_wait_bounded(bar, 0);
+    return false;
+}
+
+// D_x of caller fields g (fp64 rows) into out[2 field]: a derivative along x
+// needs the row's own transforms and nothing else.
+template <typename real, int H>
+__global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) dx_row(const __grid_constant__ GradArgs<real> A) {
+    using G = Row<real, H>;
+    using C = typename G::C;
+    constexpr int P = G::P;
+    extern __shared__ __align__(128) unsigned char row_smem[];
+    __shared__ __align__(8) uint64_t bar;
+    C *B = reinterpret_cast<C *>(row_smem);
+    unsigned char *tb = reinterpret_cast<unsigned char *>(B + G::NG * G::RC);
+    const Tab<real, H> T(tb, 0);
+    const int tid = threadIdx.x, j = tid & (P - 1), grp = tid / P, r = (int)blockIdx.x * G::NG + grp;
+    const bool mine = r < A.nrows;
+    C *z = B + grp * G::RC;
+    if (mine) {
+        const double2 *__restrict__ in = A.g + (size_t)r * H;
+        double2 x[G::E];
+#pragma unroll
+        for (int t = 0; t < G::E; ++t) x[t] = in[j + P * t];
+#pragma unroll
+        for (int t = 0; t < G::E; ++t) z[j + P * t] = C{(real)x[t].x, (real)x[t].y};
+    }
+    if (!single_tables<real, H>(tb, A.rtab, &bar, A.err)) return;
+    if (!mine) return;
+    row_fft<H, -1>(z, T.tw, j);
+    row_dx<H>(z, T.wh, T.wp, T.kx, j);
+    __syncwarp(lanes_of_row<P>());
+    row_fft<H, +1>(z, T.tw, j);
+    const int field = r / A.ny, y = r - field * A.ny;
+    double2 *out = A.out + ((size_t)2 * field * A.ny + y) * H;
+#pragma unroll
+    for (int t = 0; t < G::E; ++t) {
+        const C w = z[j + P * t];
+        out[j + P * t] = make_double2((double)w.x, (double)w.y);
+    }
+}
+
+// Sum over the block's rows of (D_x rho)^2 by Parseval's relation: over the
+// two-sided spectrum sum_x d^2 = (1 / nx) sum_k |i k_x X_k|^2.
+template <typename real, int H>
+__global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) energy_row(const __grid_constant__ EnergyArgs<real> A) {
+    using G = Row<real, H>;
+    using C = typename G::C;
+    constexpr int P = G::P;
+    extern __shared__ __align__(128) unsigned char row_smem[];
+    __shared__ __align__(8) uint64_t bar;
+    C *B = reinterpret_cast<C *>(row_smem);
+    unsigned char *tb = reinterpret_cast<unsigned char *>(B + G::NG * G::RC);
+    const Tab<real, H> T(tb, 0);
+    const int tid = threadIdx.x, j = tid & (P - 1), grp = tid / P, y = (int)blockIdx.x * G::NG + grp;
+    const bool mine = y < A.ny;
+    C *z = B + grp * G::RC;
+    if (mine) {
+        const C *__restrict__ in = A.rho + (size_t)y * H;
+#pragma unroll
+        for (int t = 0; t < G::E; ++t) z[j + P * t] = in[j + P * t];
+    }
+    if (!single_tables<real, H>(tb, A.rtab, &bar, A.err)) return;
+    double e = 0;
+    if (mine) {
+        row_fft<H, -1>(z, T.tw, j);
+        row_post<H>(z, T.wh, j, [&](int k, C X) {
+            if (k > 0) {
+                const real m = T.kx[k];
+                e += 2.0 * (double)(m * m * (X.x * X.x + X.y * X.y));
+            }
+        });
+    }
+    block_sum_store(e * (1.0 / (2 * H)), A.partial_x + blockIdx.x);
+}
+
 template <typename real, int H> RowSet row_set() {
     using G = Row<real, H>;
     RowSet s;
     s.k1 = (const void *)&k1_row<real, H>;
     s.k3 = (const void *)&k3_row<real, H>;
     s.k5 = (const void *)&k5_row<real, H>;
+    s.dx = (const void *)&dx_row<real, H>;
+    s.energy = (const void *)&energy_row<real, H>;
+    s.ng = G::NG;
+    s.smem_rows = (size_t)G::NG * G::RC * 2 * sizeof(real) + RowTable<real>::bytes(H);
     s.nt = G::NT;
     s.cs = G::CS;
     s.smem1 = k1_row_smem<real, H>();

@@ -63,6 +63,9 @@ template <typename real> struct RowArgs {
 
 struct RowSet {
     const void *k1 = nullptr, *k3 = nullptr, *k5 = nullptr;
+    const void *dx = nullptr, *energy = nullptr;   // single-row kernels: ng rows a block, smem_rows bytes
+    int ng = 1;
+    size_t smem_rows = 0;
     int nt = 0, cs = 1;
     size_t smem1 = 0, smem3 = 0, smem5 = 0;
 };

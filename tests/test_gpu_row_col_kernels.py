@@ -84,3 +84,68 @@ def test_uniform_state_is_a_bitwise_fixed_point_in_fp32(fl, nx, ny):
         f0 = h.get_f()
         h.step(20)
         assert np.array_equal(h.get_f(), f0)
+
+
+GRAD = [(n, 6) for n in ROWS] + [(32, n) for n in COLS]
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("nx,ny", GRAD)
+def test_gradient_and_invariants_match_oracle(fl, nx, ny, precision):
+    """fftlb_gradient of three fields (bounds of test_gpu_spectral.py: 1e-12 and
+    2e-5 of the largest derivative) and the conservation sums of a state: every
+    per-site value carries at most 16 roundings (2e-15, 1e-6 relative), summed
+    in fp64, measured against the sums of the parts' absolute values."""
+    if precision == 64 and max(nx, ny) > 1024:
+        pytest.skip("fp64 grids end at 1024")
+    rng = np.random.default_rng(nx * 7 + ny)
+    g = rng.standard_normal((3, ny, nx))
+    f = fields_of(nx, ny, nx + 2 * ny)
+    p = O.Params(nx=nx, ny=ny)
+    with fl.Handle(fl.params(nx=nx, ny=ny, precision=precision)) as h:
+        gd = torch.from_numpy(g).cuda()
+        out = torch.empty((6, ny, nx), dtype=torch.float64, device="cuda")
+        h.gradient(gd, out, 3)
+        torch.cuda.synchronize()
+        h.set_fields(*f)
+        inv = h.invariants()
+    out = out.cpu().numpy()
+    tol = 1e-12 if precision == 64 else 2e-5
+    for i in range(3):
+        for q, ax in ((0, "x"), (1, "y")):
+            d = O.D(g[i], ax, 1 / 256, 4)
+            assert np.abs(out[2 * i + q] - d).max() <= tol * np.abs(d).max()
+    f0 = O.init_equilibrium(*f, p)
+    ref = O.invariants(f0, p)
+    rho, ux, uy, T = O.moments(f0)
+    area = p.dx ** 2
+    grad2 = O.D(rho, "x", p.dx, 4) ** 2 + O.D(rho, "y", p.dx, 4) ** 2
+    scale = dict(mass=rho.sum() * area, px=(4.3 * rho).sum() * area, py=(4.3 * rho).sum() * area, umax=4.3,
+                 eT=(rho * T + p.a * rho ** 2 + p.K * grad2 / 2 + rho).sum() * area)
+    for k, s in scale.items():
+        assert abs(inv[k] - ref[k]) <= (1e-13 if precision == 64 else 2e-6) * s
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+def test_device_reads_into_unaligned_buffers(fl, precision):
+    """Device buffers one value off 16-byte alignment take the scalar accesses
+    and give the same values, in and out."""
+    nx, ny = 36, 18
+    n = nx * ny
+    f = fields_of(nx, ny, 5)
+    with fl.Handle(fl.params(nx=nx, ny=ny, precision=precision)) as h:
+        h.set_fields(*f)
+        buf = torch.empty(33 * n + 1, dtype=torch.float64, device="cuda")
+        off = buf[1:].view(33, ny, nx)
+        h.get_f(off, on_device=True)
+        ref = torch.empty((33, ny, nx), dtype=torch.float64, device="cuda")
+        h.get_f(ref, on_device=True)
+        fo = [torch.empty(n + 1, dtype=torch.float64, device="cuda")[1:].view(ny, nx) for _ in range(4)]
+        h.fields(*fo, on_device=True)
+        host = h.fields()
+        torch.cuda.synchronize()
+        assert torch.equal(off, ref)
+        for a, b in zip(fo, host):
+            assert np.array_equal(a.cpu().numpy(), b)
+        h.set_f(off, on_device=True)
+        assert np.array_equal(h.get_f(), ref.cpu().numpy())
