@@ -38,13 +38,11 @@ __device__ __forceinline__ void mbar_init_fence() {
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // Programmatic dependent launch: a kernel launched with programmatic stream
-// serialization may start while the kernel before it on the stream is
-// still running.  grid_dep_wait() returns once that kernel has completed
-// and its memory operations are visible; every read or write of memory the
-// previous kernels touch comes after it.  grid_dep_launch() lets the next
-// such kernel's blocks start (their prologue) as this grid's blocks exit.
+// serialization may start before the kernel before it on the stream has been
+// retired.  grid_dep_wait() returns once that kernel has completed and its
+// memory operations are visible; every read or write of memory the previous
+// kernels touch comes after it.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
@@ -115,12 +113,6 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
 // memory: no destination, no barrier, nothing to wait for
 __device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
-
-// L2 prefetch of one box of a 2-D tensor map at (x, y) (x as for tma_load_2d)
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *map, int x, int y) {
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y)
-                 : "memory");
 }
 
 }  // namespace fftlb

@@ -923,12 +923,6 @@ class EngineT : public Engine {
     C *Tw1_ = nullptr;
     size_t smem5w_ = 0, smem1w_ = 0, smem3w_ = 0;
     int grid5w_ = 1, grid1w_ = 1, grid3w_ = 1;
-    // warp-resident convection columns for ny = 256, 512, 1024
-    bool colwr_ = false;
-    C *Twc_ = nullptr;
-    size_t smemcw_ = 0;
-    int gridcw_ = 1, nbufcw_ = 1, ntcw_ = 256;
-    CUtensorMap tmap_convw_{}, fmap_convw_[2] = {};
     // row and column kernels of kernels_row.cuh / kernels_col.cuh, the
     // argument blocks of their launches, and their tables
     bool rowk_ = false, colk_ = false;   // taken by the stage
@@ -1316,24 +1310,6 @@ class EngineT : public Engine {
             t1.resize(n + ny_ / 2);   // ny reals
             memcpy(t1.data() + n, ky.data(), ny_ * sizeof(real));
             if (!(st = upload_table(&Tcr_, t1)).good()) return st;
-        }
-        if (wr_ok_ && (ny_ == 1024 || ny_ == 512 || ny_ == 256 || ny_ == 128)) {
-            // twc[k1 P + l] = exp(-2 pi i l k1 / ny) for the column configuration of
-            // ny, followed by the same values ordered [l][k1] (twc[ny + l E + k1])
-            const int P = col_p_host(ny_), E = ny_ / P;
-            std::vector<C> t1((size_t)2 * ny_);
-            const long double pi = 3.141592653589793238462643383279502884L;
-            for (int k1 = 0; k1 < E; ++k1)
-                for (int l = 0; l < P; ++l) {
-                    const long double a = 2.0L * pi * (long double)(l * k1) / (long double)ny_;
-                    C w;
-                    w.x = (real)cosl(a);
-                    w.y = (real)(-sinl(a));
-                    t1[(size_t)k1 * P + l] = w;
-                    t1[(size_t)ny_ + (size_t)l * E + k1] = w;
-                }
-            if (!(st = dalloc(&Twc_, t1.size())).good()) return st;
-            FFTLB_CU(cudaMemcpy(Twc_, t1.data(), t1.size() * sizeof(C), cudaMemcpyHostToDevice));
         }
         if (split_) {
             std::vector<uint4> fr;
@@ -1841,28 +1817,26 @@ class EngineT : public Engine {
             const void *ks[3] = {cs_.k, cs_.dy, cs_.energy};
             for (const void *k : ks)
                 if (cs_.tw) FFTLB_CU(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget_));
-            // kcol_wr keeps the lengths 512 and 1024, where its prefetch and
-            // (512) its wider tiles pay: convection and level 2 at 1024^2 79
-            // and 19 us against 90 and 28, at 512^2 25 and 12 against 25 and
-            // 21; at 256^2 12 and 10 against 10 and 8 here.
-            colk_ = !(colwr_ && ny_ >= 512);
+            colk_ = true;
         }
         return Status::ok();
     }
 
     // a row kernel over every row of every run, cs blocks (one cluster) a row
-    Status launch_row(const char *name, const void *k, int cs, size_t smem) {
+    Status launch_row(const char *name, const void *k, int nt, int cs, size_t smem) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(B_ * ny_ * cs));
-        cfg.blockDim = dim3((unsigned)rs_.nt);
+        cfg.blockDim = dim3((unsigned)nt);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = stream_;
-        cudaLaunchAttribute at[1];
+        cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = (unsigned)cs;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = 2;
         void *args[1] = {&ra_};
         const cudaError_t e = cudaLaunchKernelExC(&cfg, k, args);
         if (e != cudaSuccess) {
@@ -1876,7 +1850,17 @@ class EngineT : public Engine {
     Status launch_cols(ColArgs<real> &a, int nrun) {
         const unsigned jobs = cs_.tw ? (unsigned)(a.ngroups * (h_ / cs_.tw)) : (unsigned)((a.ngroups * h_ + 127) / 128);
         void *args[1] = {&a};
-        const cudaError_t e = cudaLaunchKernel(cs_.k, dim3(jobs, (unsigned)nrun), dim3((unsigned)cs_.nt), args, cs_.smem, stream_);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(jobs, (unsigned)nrun);
+        cfg.blockDim = dim3((unsigned)cs_.nt);
+        cfg.dynamicSmemBytes = cs_.smem;
+        cfg.stream = stream_;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelExC(&cfg, cs_.k, args);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return Status::err(FFTLB_ERR_CUDA, std::string("column kernel: ") + cudaGetErrorString(e));
@@ -1923,38 +1907,6 @@ class EngineT : public Engine {
                 if (nb >= 1) {
                     k1wr_ = true;
                     grid1w_ = std::min(B_ * ny_, nb * nsm_);
-                }
-            }
-            const int TWw = Twc_ ? col_tw_host(ny_) : 1, NTw = TWw * (Twc_ ? col_p_host(ny_) : 1);
-            if (Twc_ && h_ % TWw == 0) {
-                // one or two tile buffers: the most blocks per SM, then two
-                // (FFTLB_COLWR_NBUF fixes the count at build time)
-                int best = 0;
-#ifdef FFTLB_COLWR_NBUF
-                for (int nb2 = FFTLB_COLWR_NBUF; nb2 == FFTLB_COLWR_NBUF; --nb2) {
-#else
-                for (int nb2 = 2; nb2 >= 1; --nb2) {
-#endif
-                    const size_t sm = kcol_wr_smem(ny_, h_, nb2);
-                    if (sm > budget_) continue;
-                    st = ny_ == 1024 ? occupancy(kcol_wr<1024>, NTw, sm, &nb)
-                       : ny_ == 512  ? occupancy(kcol_wr<512>, NTw, sm, &nb)
-                       : ny_ == 256  ? occupancy(kcol_wr<256>, NTw, sm, &nb)
-                                     : occupancy(kcol_wr<128>, NTw, sm, &nb);
-                    if (!st.good()) return st;
-                    if (nb > best) {
-                        best = nb;
-                        nbufcw_ = nb2;
-                        smemcw_ = sm;
-                    }
-                }
-                if (best > 0) {
-                    st = make_tmap(&tmap_convw_, TWw);
-                    if (st.good()) st = make_fmaps(fmap_convw_, TWw);
-                    if (!st.good()) return st;
-                    colwr_ = true;
-                    ntcw_ = NTw;
-                    gridcw_ = best * nsm_;
                 }
             }
         }
@@ -2140,29 +2092,12 @@ class EngineT : public Engine {
     }
 
   private:
-    // Launch of a warp-resident kernel, with programmatic stream
-    // serialization when built with FFTLB_PDL=1: its blocks may then start
-    // their prologue while the kernel before it finishes (each of these
-    // kernels calls grid_dep_wait before it touches memory that earlier
-    // kernels wrote or read).  Off by default: measured at 1024^2, the step
-    // took 1.230 ms with it against 1.077 ms without.
-#ifndef FFTLB_PDL
-#define FFTLB_PDL 0
-#endif
-    // The final row kernel alone (FFTLB_PDL_K5): it overlaps the level-2
-    // launch's tail with its first convection chunk, and only its head copies
-    // wait for that launch.
-#ifndef FFTLB_PDL_K5
-#define FFTLB_PDL_K5 0
-#endif
+    // Launch of a warp-resident kernel with programmatic stream serialization
+    // (kernels_row.cuh says what it gives; each kernel calls grid_dep_wait
+    // before it touches memory that earlier kernels wrote or read)
     template <typename... KArgs, typename... Args>
     Status launch_pdl(const char *name, void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
                       Args &&...args) {
-        return launch_ex(name, FFTLB_PDL, kernel, grid, block, smem, std::forward<Args>(args)...);
-    }
-    template <typename... KArgs, typename... Args>
-    Status launch_ex(const char *name, int pdl, void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
-                     Args &&...args) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(grid);
         cfg.blockDim = dim3(block);
@@ -2170,7 +2105,7 @@ class EngineT : public Engine {
         cfg.stream = stream_;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[0].val.programmaticStreamSerializationAllowed = pdl;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
         const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
@@ -2192,20 +2127,6 @@ class EngineT : public Engine {
             }
             ca_conv_.f = reinterpret_cast<const C *>(cur);
             return launch_cols(level2 ? ca_l2_ : ca_conv_, B_);
-        }
-        if constexpr (wr_ok_) {
-            if (colwr_) {
-                if (count > kMaxColGroups) return Status::err(FFTLB_ERR_ARG, "too many column groups in one launch");
-#define FFTLB_KCOLWR(NYV)                                                                                     \
-    launch_pdl("kcol_wr", kcol_wr<NYV>, gridcw_, ntcw_, smemcw_, specb_, (const GroupDesc *)(groups_ + first),     \
-               count, (const float *)kxt_, (const float *)kyt_, (const float2 *)Twc_, kp_, BOXR_, nbufcw_,          \
-               tmap_convw_, fmap_convw_[fm], err_)
-                return ny_ == 1024 ? FFTLB_KCOLWR(1024)
-                     : ny_ == 512  ? FFTLB_KCOLWR(512)
-                     : ny_ == 256  ? FFTLB_KCOLWR(256)
-                                   : FFTLB_KCOLWR(128);
-#undef FFTLB_KCOLWR
-            }
         }
         if (level2)
             kcol_pipe<real, SPLIT><<<gridl_, NTC, smeml_, stream_>>>(specb_, groups_ + first, count, kxt_, kyt_, Wc_, Tc_,
@@ -2232,7 +2153,7 @@ class EngineT : public Engine {
             ra_.fout = out;
             ra_.alpha = alpha;
             ra_.beta = beta;
-            if (!(st = launch_row("k1_row", rs_.k1, rs_.cs, rs_.smem1)).good()) return st;
+            if (!(st = launch_row("k1_row", rs_.k1, rs_.nt, rs_.cs, rs_.smem1)).good()) return st;
             k1done = true;
         }
         if constexpr (wr_ok_) {
@@ -2264,7 +2185,7 @@ class EngineT : public Engine {
         if (!(st = prof_begin(KK_ROW_LEVEL1)).good()) return st;
         bool k3done = false;
         if (rowk_) {
-            if (!(st = launch_row("k3_row", rs_.k3, rs_.cs, rs_.smem3)).good()) return st;
+            if (!(st = launch_row("k3_row", rs_.k3, rs_.nt3, rs_.cs, rs_.smem3)).good()) return st;
             k3done = true;
         }
         if constexpr (wr_ok_) {
@@ -2289,14 +2210,14 @@ class EngineT : public Engine {
         if (!(st = prof_end()).good()) return st;
         if (!(st = prof_begin(KK_ROW_FINAL)).good()) return st;
         if (rowk_) {
-            if (!(st = launch_row("k5_row", rs_.k5, rs_.cs, rs_.smem5)).good()) return st;
+            if (!(st = launch_row("k5_row", rs_.k5, rs_.nt, rs_.cs, rs_.smem5)).good()) return st;
             return prof_end();
         }
         if constexpr (wr_ok_) {
             if (k5wr_) {
                 const int nt = nt_k5wr_host(h_);
                 auto *kern = h_ == 512 ? k5_wr<512> : h_ == 256 ? k5_wr<256> : k5_wr<128>;
-                if (!(st = launch_ex("k5_wr", FFTLB_PDL || FFTLB_PDL_K5, kern, grid5w_, nt, smem5w_, (const float2 *)specb_,
+                if (!(st = launch_pdl("k5_wr", kern, grid5w_, nt, smem5w_, (const float2 *)specb_,
                                       (const float *)fieldsb_, (const float *)auxb_, cur, base, out, alpha, beta,
                                       (const float2 *)Tw1_, (const float2 *)Wp_, kp_, err_)).good())
                     return st;

@@ -1,5 +1,4 @@
-// Column passes without staged tiles, for the lengths, precisions and grid
-// sizes the persistent kernels (kcol_wr, kcol_pipe) do not serve well:
+// Column passes without staged tiles, in fp32 and fp64:
 //   kcol_reg   lengths 16 .. 2048 = 2^p and 24 .. 1536 = 3 2^p: one job (a
 //              tile of TW spectrum columns of one group) per block;
 //   kcol_line  lengths 4, 6, 8, 12: one column per thread, in registers.
@@ -7,17 +6,27 @@
 // one output (which may be the same slot): forward transform, multiplier
 // i (c0 k_x + c1 k_y) or c3 k_y^2, inverse.
 //
-// A column of NY = E P values is transformed by P threads as in kcol_wr, but
-// thread (c, l) loads its x[l + P t] straight from global memory into
-// registers: the tile passes through shared memory twice (the transpose and
-// its inverse) instead of three times, and a block holds one tile, so that
-// several blocks fit an SM and their loads overlap each other's transforms.
+// A column of NY = E P values is transformed by P threads in two register
+// stages: thread (c, l) takes the E-point DFT of x[l + P t], times W_NY^(l k1),
+// and stores it transposed in shared memory; thread (c, k1) takes the P-point
+// DFTs over l, applies the multiplier to X[k1 + E k2], and goes back the same
+// way (P points by two threads, with one shuffle each way, where they do not
+// fit one thread's registers).  The values come straight from global memory
+// into registers, so the tile passes through shared memory twice, a block holds
+// one tile, and several blocks on an SM overlap loads and transforms.  A
+// persistent kernel that staged tiles by tensor copies (two buffers, L2
+// prefetch) took 77.7 us for the convection launch of 1024^2 fp32 and 17.9 for
+// level 2 (one job's latency), 24.5 and 11.8 at 512^2; this one 79.2 and 14.6,
+// 20.9 and 10.2.  Both are held by the FMA pipe and the loads' latency at 16
+// warps per SM (44% of the issue slots, 3.4 TB/s).
+// The packed column 0 of the tile at k_x = 0 (DC real, row-Nyquist imaginary)
+// needs no pairing of (k_y, -k_y): both columns it carries take the multiplier
+// at k_x = 0, because the Nyquist bin of k_x is zero.
 // The tables of the 8-wide fp32 tiles come by one bulk copy that overlaps the
 // tile's loads: read through L1, they were cold in every launch, a latency per
 // handful of twiddles (one job's time on 384^2: 13.8 us, 10.2 with the copy).
 // 4-wide tiles are hardly larger than their tables (2048^2: convection 479 us
-// with the copy, 372 through L1), and fp64's arithmetic hides the latency.  The packed column 0 of the
-// tile at k_x = 0 needs no pairing of (k_y, -k_y) (see kcol_wr).
+// with the copy, 372 through L1), and fp64's arithmetic hides the latency.
 #pragma once
 
 #include "async_copy.cuh"
@@ -200,6 +209,7 @@ __global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) kcol_
     const C *__restrict__ in =
         gr.from_f ? A.f + ((size_t)blockIdx.y * Q + gr.in) * slot + t * TW + c : spec + (size_t)gr.in * slot;
     ColTab<real, NY>::issue(T, A.tab, &bar);
+    grid_dep_wait();   // (see kernels_row.cuh)
     C v[E];
 #pragma unroll
     for (int q = 0; q < E; ++q) v[q] = in[(size_t)(jl + P * q) * h];
@@ -324,6 +334,7 @@ __global__ void __launch_bounds__(128) energy_line(const __grid_constant__ Energ
 template <typename real, int NY>
 __global__ void __launch_bounds__(128) kcol_line(const __grid_constant__ ColArgs<real> A) {
     using C = typename cplx_of<real>::type;
+    grid_dep_wait();
     const int h = A.h, ncol = A.ngroups * h;
     const int i = (int)blockIdx.x * 128 + (int)threadIdx.x;
     if (i >= ncol) return;

@@ -414,31 +414,18 @@ __host__ __device__ __forceinline__ size_t tile_stride(int TW, int ny) {
     return bytes / sizeof(C);
 }
 
-// The fields of a group that the tile copies and a job read, staged in
-// shared memory once per launch by the warp-resident column kernels (a per-job
-// copy of the whole GroupDesc by one thread held every other warp of the block
-// at the next barrier).  The multiplier is i (c0 k_x + c1 k_y), or c3 k_y^2
-// where c3 is not zero, times the group's scale (folded into the constants).
-struct ColG {
-    int in_slot[1], out_slot, from_f;
-    float c0, c1, c3;
-};
-constexpr int kMaxColGroups = 40;   // groups of one kcol_wr launch (at most 32 convection + 8 level-1 groups)
-
 // where a job's tile starts: the tensor map (spectrum arena or stage state)
 // and the first row
 struct ColSrc {
     const CUtensorMap *map;
     int row;
 };
-template <typename GD>
-__device__ __forceinline__ ColSrc col_src(const GD *G, int run, int ny, const CUtensorMap *tmap, const CUtensorMap *fmap) {
+__device__ __forceinline__ ColSrc col_src(const GroupDesc *G, int run, int ny, const CUtensorMap *tmap, const CUtensorMap *fmap) {
     return G->from_f ? ColSrc{fmap, (run * Q + G->in_slot[0]) * ny} : ColSrc{tmap, (run * NSLOT + G->in_slot[0]) * ny};
 }
 
-// (GD: GroupDesc in global memory, or ColG staged in shared memory)
-template <typename C, typename GD>
-__device__ __forceinline__ void kcol_issue(C *dst, uint64_t *bar, const GD *groups, int k, int ntiles, int ngroups, int TW,
+template <typename C>
+__device__ __forceinline__ void kcol_issue(C *dst, uint64_t *bar, const GroupDesc *groups, int k, int ntiles, int ngroups, int TW,
                                            int ny, int BOXR, const CUtensorMap *tmap, const CUtensorMap *fmap) {
     const int job = (int)blockIdx.x + k * (int)gridDim.x;
     const int run = job / (ngroups * ntiles), jr = job - run * ngroups * ntiles;
@@ -446,17 +433,6 @@ __device__ __forceinline__ void kcol_issue(C *dst, uint64_t *bar, const GD *grou
     const ColSrc src = col_src(groups + g, run, ny, tmap, fmap);
     mbar_expect_tx(bar, (uint32_t)(TW * ny * sizeof(C)));
     for (int r0 = 0; r0 < ny; r0 += BOXR) tma_load_2d(dst + (size_t)r0 * TW, src.map, 2 * t * TW, src.row + r0, bar);
-}
-
-// L2 prefetch of the tile kcol_issue would load for job k
-template <typename GD>
-__device__ __forceinline__ void kcol_prefetch(const GD *groups, int k, int ntiles, int ngroups, int TW, int ny, int BOXR,
-                                              const CUtensorMap *tmap, const CUtensorMap *fmap) {
-    const int job = (int)blockIdx.x + k * (int)gridDim.x;
-    const int run = job / (ngroups * ntiles), jr = job - run * ngroups * ntiles;
-    const int g = jr / ntiles, t = jr - g * ntiles;
-    const ColSrc src = col_src(groups + g, run, ny, tmap, fmap);
-    for (int r0 = 0; r0 < ny; r0 += BOXR) tma_prefetch_2d(src.map, 2 * t * TW, src.row + r0);
 }
 
 // Every group has one input and one output, which may be the same slot.

@@ -24,6 +24,14 @@
 // banks, and the tables come by one bulk copy that overlaps the first loads
 // (through L1 they are cold in every launch).  Inverse rows form the packed
 // half-length spectrum straight from global memory, with no staging copy.
+//
+// The stage's kernels are launched with programmatic stream serialization and
+// no explicit trigger: a launch's blocks start as the one before ends, without
+// the full hand-over between grids, and wait for its memory (grid_dep_wait) once
+// their barriers and tables are under way and before they touch anything the
+// stage writes.  A step on 64^2 fp32 83 -> 50 us, on 64^2 fp64 241 -> 204, on
+// 2048^2 fp32 4618 -> 4547.  Triggered early instead, the waiting blocks fill the
+// SMs that are idle first and then run crowded there (64^2 fp64 389 us).
 #pragma once
 
 #include <cooperative_groups.h>
@@ -43,10 +51,10 @@ namespace rk {
 namespace cg = cooperative_groups;
 
 // row configuration (see row_p in row_kernels.h)
-template <typename real, int H> struct Row {
+template <typename real, int H, int NT_ = row_nt((int)sizeof(real), H)> struct Row {
     using C = typename cplx_of<real>::type;
     static constexpr int P = row_p((int)sizeof(real), H), E = H / P;
-    static constexpr int NT = row_nt((int)sizeof(real), H), NG = NT / P;   // threads, row groups
+    static constexpr int NT = NT_, NG = NT / P;                       // threads, row groups
     static constexpr int CS = row_cs((int)sizeof(real), H);           // blocks per row
     static constexpr int CHN = 32 / CS;                               // distribution rows per block
     static constexpr int RC = row_stride((int)sizeof(real), H);            // complex values between rows
@@ -69,6 +77,10 @@ template <typename real, int H> struct Row {
 // wave more for K3 on 256^2: 128 us against 95)
 template <typename real, int H> constexpr int row_minb() {
     return Row<real, H>::NT >= 256 ? 2 : sizeof(real) == 4 ? 4 : Row<real, H>::E >= 24 ? 2 : 4;
+}
+
+template <typename real, int H> constexpr int row_minb3() {
+    return row_minb<real, H>() * (Row<real, H>::NT / row_nt3((int)sizeof(real), H));
 }
 
 template <int P> __device__ __forceinline__ unsigned lanes_of_row() {
@@ -334,6 +346,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k1_row(
         mbar_init_fence();
     }
     __syncthreads();
+    grid_dep_wait();
     if (tid == 0) {
         mbar_expect_tx(&bar, (uint32_t)(nrow * NX * sizeof(real)) + LT::wp(H));
         for (int r = 0; r < CHN; ++r)
@@ -432,8 +445,8 @@ template <typename real, int H> size_t k1_row_smem() {
 // ---------------------------------------------------------------------------
 
 template <typename real, int H>
-__global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k3_row(const __grid_constant__ RowArgs<real> A) {
-    using G = Row<real, H>;
+__global__ void __launch_bounds__(row_nt3((int)sizeof(real), H), row_minb3<real, H>()) k3_row(const __grid_constant__ RowArgs<real> A) {
+    using G = Row<real, H, row_nt3((int)sizeof(real), H)>;
     using C = typename G::C;
     constexpr int CS = G::CS, RC = G::RC, NX = G::NX, NT = G::NT, P = G::P, NXS = G::NXS;
     constexpr int ND = G::share(NSP), NL = G::share(3);
@@ -457,6 +470,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k3_row(
         table_issue(tb, A.tab, 0, LT::bytes(H), &bar);
     }
     __syncthreads();
+    grid_dep_wait();
     bool first = true;
     auto ready = [&]() {   // the tables are there (a wait that runs out is recorded; see k1_row)
         if (first) table_wait(&bar, A.err);
@@ -537,7 +551,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k3_row(
 }
 
 template <typename real, int H> size_t k3_row_smem() {
-    using G = Row<real, H>;
+    using G = Row<real, H, row_nt3((int)sizeof(real), H)>;
     return (size_t)(G::share(NSP) + G::share(3)) * G::RC * 2 * sizeof(real) + RowTable<real>::bytes(H);
 }
 
@@ -568,6 +582,7 @@ template <typename real> __device__ __forceinline__ real ring_dot(int r, real a,
 
 template <typename real, int V> struct Vec;
 template <> struct Vec<float, 2> { using T = float2; };
+template <> struct Vec<float, 4> { using T = float4; };
 template <> struct Vec<double, 1> { using T = double; };
 template <typename real, int V> __device__ __forceinline__ void ldv(real (&a)[V], const real *p) {
     *reinterpret_cast<typename Vec<real, V>::T *>(a) = *reinterpret_cast<const typename Vec<real, V>::T *>(p);
@@ -582,7 +597,13 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
     using C = typename G::C;
     constexpr int CS = G::CS, CHN = G::CHN, RC = G::RC, NX = G::NX, NT = G::NT, P = G::P, NXS = G::NXS;
     constexpr int NRING = G::NRING;
-    constexpr int V = sizeof(real) == 4 ? 2 : 1;   // sites per thread and pass of the epilogue
+    // sites per thread and pass of the epilogue, and ring pairs (r, r + 4) loaded
+    // before any of their stores: 16-byte accesses on long rows (two halves of a
+    // ring, for the registers), all 8 directions at once on short ones
+#ifndef K5V
+#define K5V 4
+#endif
+    constexpr int V = sizeof(real) == 8 ? 1 : H >= 256 ? K5V : 2, RP = V == 4 ? 2 : 4;
     static_assert(CHN % 8 == 0, "whole rings per block");
     extern __shared__ __align__(128) unsigned char row_smem[];
     C *B = reinterpret_cast<C *>(row_smem);                     // [6 NRING] convection rows
@@ -600,11 +621,6 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
     auto row = [&](int s) { return reinterpret_cast<const real *>(spec + (size_t)s * slot); };
     const real dt = A.dt, itau = A.itau, beta = A.beta;
     const bool with_base = A.alpha != real(0);
-    if (tid < CHN) {   // this block's distribution rows into L2 ahead of the epilogue
-        const size_t o = fo + (size_t)(1 + c * CHN + tid) * N;
-        bulk_prefetch_l2(A.fcur + o, NX * sizeof(real));
-        if (with_base) bulk_prefetch_l2(A.fbase + o, NX * sizeof(real));
-    }
     if (tid == 0) {
         mbar_init(&bar, 1);
         mbar_init_fence();
@@ -612,6 +628,12 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
         table_issue(tb, A.tab, LT::tw(H), LT::bytes(H), &bar);
     }
     __syncthreads();
+    grid_dep_wait();
+    if (tid < CHN) {   // this block's distribution rows into L2 ahead of the epilogue
+        const size_t o = fo + (size_t)(1 + c * CHN + tid) * N;
+        bulk_prefetch_l2(A.fcur + o, NX * sizeof(real));
+        if (with_base) bulk_prefetch_l2(A.fbase + o, NX * sizeof(real));
+    }
     bool first = true;
     auto ready = [&]() {   // the tables are there (a wait that runs out is recorded; see k1_row)
         if (first) table_wait(&bar, A.err);
@@ -679,14 +701,6 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
         const size_t o = fo + (size_t)(1 + v0) * N + x;
         const real *pc = A.fcur + o, *pb = A.fbase + o;
         real *po = A.fout + o;
-        real fc[8][V], fb[8][V], c2[V], c6[V];   // (all loads before any store: fout may be fcur or fbase)
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            ldv<real, V>(fc[r], pc + (size_t)r * N);
-            if (with_base) ldv<real, V>(fb[r], pb + (size_t)r * N);
-        }
-        ldv<real, V>(c2, row(v0 + 2) + x);   // v_x = 0: real from the column pass
-        ldv<real, V>(c6, row(v0 + 6) + x);
         real rho[V], ux[V], uy[V], T[V], e0[V], ex[V], ey[V], CC[V], iT[V];
         ldv<real, V>(rho, row(SLOT_F) + x);
         ldv<real, V>(ux, row(SLOT_F + 1) + x);
@@ -722,34 +736,39 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
         const real *cr = reinterpret_cast<const real *>(B + rr * 6 * RC) + x;
         // directions r and r + 4 together: f^eq = even +- odd in v.u
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            real cv[2][V], fn[2][V];
-            if (r == 2) {
+        for (int r0 = 0; r0 < 4; r0 += RP) {
+            real fc[2 * RP][V], fb[2 * RP][V], cv[2 * RP][V];
+            // (a direction's loads come before its stores: fout may be fcur or
+            // fbase, at the same site)
+#pragma unroll
+            for (int q = 0; q < 2 * RP; ++q) {
+                const int r = r0 + (q >> 1) + 4 * (q & 1);
+                ldv<real, V>(fc[q], pc + (size_t)r * N);
+                if (with_base) ldv<real, V>(fb[q], pb + (size_t)r * N);
+                if ((r & 3) == 2) ldv<real, V>(cv[q], row(v0 + r) + x);   // v_x = 0: real from the column pass
+                else ldv<real, V>(cv[q], cr + (size_t)ring_pos(r) * 2 * RC);
+            }
+#pragma unroll
+            for (int h = 0; h < RP; ++h) {
+                const int r = r0 + h;
+                real fn[2][V];
 #pragma unroll
                 for (int q = 0; q < V; ++q) {
-                    cv[0][q] = c2[q];
-                    cv[1][q] = c6[q];
-                }
-            } else {
-                ldv<real, V>(cv[0], cr + (size_t)ring_pos(r) * 2 * RC);
-                ldv<real, V>(cv[1], cr + (size_t)ring_pos(r + 4) * 2 * RC);
-            }
+                    const real vu = ring_dot<real>(r, ux[q], uy[q], dp[q], dm[q]), w2 = vu * vu;
+                    const real ev = p0[q] + w2 * (p2[q] + w2 * p4[q]), od = vu * (p1[q] + w2 * p3[q]);   // Eq. 3
+                    const real ed = ring_dot<real>(r, ex[q], ey[q], ep[q], em[q]);
 #pragma unroll
-            for (int q = 0; q < V; ++q) {
-                const real vu = ring_dot<real>(r, ux[q], uy[q], dp[q], dm[q]), w2 = vu * vu;
-                const real ev = p0[q] + w2 * (p2[q] + w2 * p4[q]), od = vu * (p1[q] + w2 * p3[q]);   // Eq. 3
-                const real ed = ring_dot<real>(r, ex[q], ey[q], ep[q], em[q]);
-#pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    const real fe = s ? ev - od : ev + od;
-                    const real g = s ? g0[q] - ed : g0[q] + ed;   // -I / f^eq, Eq. 11
-                    const real f = fc[r + 4 * s][q];
-                    const real rhs = -cv[s][q] - (f - fe) * itau - g * fe;   // Eq. 10
-                    fn[s][q] = rk_combine(with_base, beta, dt, f, fb[r + 4 * s][q], rhs);
+                    for (int s = 0; s < 2; ++s) {
+                        const real fe = s ? ev - od : ev + od;
+                        const real g = s ? g0[q] - ed : g0[q] + ed;   // -I / f^eq, Eq. 11
+                        const real f = fc[2 * h + s][q];
+                        const real rhs = -cv[2 * h + s][q] - (f - fe) * itau - g * fe;   // Eq. 10
+                        fn[s][q] = rk_combine(with_base, beta, dt, f, fb[2 * h + s][q], rhs);
+                    }
                 }
+                stv<real, V>(po + (size_t)r * N, fn[0]);
+                stv<real, V>(po + (size_t)(r + 4) * N, fn[1]);
             }
-            stv<real, V>(po + (size_t)r * N, fn[0]);
-            stv<real, V>(po + (size_t)(r + 4) * N, fn[1]);
         }
     }
 }
@@ -892,6 +911,7 @@ template <typename real, int H> RowSet row_set() {
     s.ng = G::NG;
     s.smem_rows = (size_t)G::NG * G::RC * 2 * sizeof(real) + RowTable<real>::bytes(H);
     s.nt = G::NT;
+    s.nt3 = row_nt3((int)sizeof(real), H);
     s.cs = G::CS;
     s.smem1 = k1_row_smem<real, H>();
     s.smem3 = k3_row_smem<real, H>();

@@ -331,7 +331,6 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
     load_tab4(Wp, Wp_g, H / 2 + 1, NT);
     load_tab4(kxs, kxt, H, NT);
     grid_dep_wait();
-    grid_dep_launch();
     __syncthreads();
     uint32_t par0 = 0, par1 = 0;
     bool pend0 = njobs > 0, pend1 = njobs > 1;
@@ -497,7 +496,6 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
     load_tab4(Wp, Wp_g, H / 2 + 1, NT);
     load_tab4(kxs, kxt, H, NT);
     grid_dep_wait();
-    grid_dep_launch();
     __syncthreads();
     uint32_t par0 = 0, par1 = 0;
     bool pend0 = nrows > 0, pend1 = NB > 1 && nrows > 1;
@@ -639,7 +637,6 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
     }
     load_tab4(tw, tw_g, H, NT);
     load_tab4(Wp, Wp_g, H / 2 + 1, NT);
-    grid_dep_launch();
     __syncthreads();
     uint32_t par0 = 0, par1 = 0, hpar0 = 0, hpar1 = 0;
     bool pend0 = njobs > 0, pend1 = njobs > 1, hpend0 = nrows > 0, hpend1 = NHB > 1 && nrows > 1;
@@ -910,187 +907,6 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
             }
         }
     }
-}
-
-// ---------------------------------------------------------------------------
-// Column transforms of a tile of TW spectrum columns of length NY = E * P
-// (the tile [NY][TW] complex as the tensor copy lands it): thread (c, l)
-// (c < TW fastest, l < P) holds column c's x[l + P t], t < E:
-//   stage 1: E-point DFT over t, times W_NY^(l k1), stored in place at row
-//            k1 P + (l ^ (k1 & SW)) of the tile (SW = 16 / TW - 1: the row
-//            swizzle that keeps stage 2's reads conflict-free; the rows it
-//            exchanges belong to threads of the same warp, so __syncwarp
-//            orders the in-place store);
-//   __syncthreads;
-//   stage 2: thread (c, j) takes k1 = j + P q (q < E / P) and the P-point
-//            DFT over l: the spectrum X[k1 + E k2] of column c in registers;
-//            the multiplier (convection: i (v_x k_x + v_y k_y) / (nx ny)),
-//            the inverse P-point DFT and the conjugate twiddles follow in
-//            registers and the values go back where they were read;
-//   __syncthreads;
-//   stage 1 inverse: the inverse E-point DFT over k1, stored to global.
-// The packed column 0 of the tile at k_x = 0 (DC real, row-Nyquist
-// imaginary) needs no pairing of (k_y, -k_y): both columns it carries take
-// the multiplier at k_x = 0, because the Nyquist bin of k_x is zero.
-// ---------------------------------------------------------------------------
-
-// (FFTLB_COL1024_TW: the 1024-point tile width, 8 by default; 4 halves the
-// blocks and doubles their number per SM, measured slower: convection 102 ->
-// 112 us, level 1 62 -> 96 us at 1024^2)
-#ifndef FFTLB_COL1024_TW
-#define FFTLB_COL1024_TW 8
-#endif
-template <int NY> struct ColCfg;
-template <> struct ColCfg<1024> { static constexpr int E = 32, P = 32, TW = FFTLB_COL1024_TW; };
-template <> struct ColCfg<512> { static constexpr int E = 32, P = 16, TW = 16; };
-template <> struct ColCfg<256> { static constexpr int E = 16, P = 16, TW = 16; };
-template <> struct ColCfg<128> { static constexpr int E = 16, P = 8, TW = 32; };
-inline int col_tw_host(int NY) { return NY == 1024 ? FFTLB_COL1024_TW : NY == 128 ? 32 : 16; }
-inline int col_p_host(int NY) { return NY == 1024 ? 32 : NY == 128 ? 8 : 16; }
-
-template <int NY>
-__device__ __forceinline__ int cpos(int c, int l, int k1) {
-    constexpr int P = ColCfg<NY>::P, TW = ColCfg<NY>::TW, SW = TW < 16 ? 16 / TW - 1 : 0;
-    return (k1 * P + (l ^ (k1 & SW))) * TW + c;
-}
-
-template <int NY>
-__global__ void __launch_bounds__(ColCfg<NY>::TW * ColCfg<NY>::P, ColCfg<NY>::TW * ColCfg<NY>::P >= 256 ? 2 : 4) kcol_wr(float2 *spec,
-                                                                             const GroupDesc *__restrict__ groups,
-                                                                             int ngroups,
-                                                                             const float *__restrict__ kxt,
-                                                                             const float *__restrict__ kyt,
-                                                                             const float2 *__restrict__ twc_g,
-                                                                             KP<float> P, int BOXR, int nbuf,
-                                                                             const __grid_constant__ CUtensorMap tmap,
-                                                                             const __grid_constant__ CUtensorMap fmap,
-                                                                             int *err) {
-    using C = float2;
-    using real = float;
-    constexpr int E = ColCfg<NY>::E, PP = ColCfg<NY>::P, TW = ColCfg<NY>::TW, NT = TW * PP;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bar0, bar1;
-    __shared__ ColG gt[kMaxColGroups];   // ngroups <= kMaxColGroups (checked by the host)
-    const int h = P.h, tid = threadIdx.x;
-    const int c = tid % TW, jl = tid / TW;
-    const size_t slot = (size_t)NY * h;
-    constexpr int tile = TW * NY;
-    SmemCursor sc{smem_raw, 0u};
-    C *twc = (C *)sc.take((size_t)2 * NY * sizeof(C));   // [k1][l] (stage 1), then [l][k1] (stage 2)
-    const C *twt = twc + NY;
-    real *kxs = (real *)sc.take((size_t)(h + 1) * sizeof(real));
-    real *kys = (real *)sc.take(NY * sizeof(real));
-    C *buf0 = (C *)sc.take((size_t)tile * sizeof(C));
-    C *buf1 = nbuf > 1 ? (C *)sc.take((size_t)tile * sizeof(C)) : buf0;
-    const int ntiles = h / TW;
-    const int njobs_total = P.nrun * ngroups * ntiles;
-    const int njobs = (int)blockIdx.x < njobs_total ? (njobs_total - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    if (tid == 0) {   // (the first copies start before the tables load)
-        mbar_init(&bar0, 1);
-        mbar_init(&bar1, 1);
-        mbar_init_fence();
-        grid_dep_wait();
-        if (njobs > 0) kcol_issue(buf0, &bar0, groups, 0, ntiles, ngroups, TW, NY, BOXR, &tmap, &fmap);
-        if (nbuf > 1 && njobs > 1) kcol_issue(buf1, &bar1, groups, 1, ntiles, ngroups, TW, NY, BOXR, &tmap, &fmap);
-        if (njobs > nbuf) kcol_prefetch(groups, nbuf, ntiles, ngroups, TW, NY, BOXR, &tmap, &fmap);
-    }
-    load_tab4(twc, twc_g, 2 * NY, NT);
-    load_tab4(kxs, kxt, h + 1, NT);
-    load_tab4(kys, kyt, NY, NT);
-    for (int g = tid; g < ngroups; g += NT) {
-        const GroupDesc &G = groups[g];
-        gt[g] = ColG{{G.in_slot[0]}, G.out_slot[0], G.from_f, (float)(G.c[0][0][0] * G.scale),
-                     (float)(G.c[0][0][1] * G.scale), (float)(G.c[0][0][3] * G.scale)};
-    }
-    grid_dep_wait();
-    grid_dep_launch();
-    __syncthreads();
-    uint32_t par0 = 0, par1 = 0;
-    bool pend0 = njobs > 0, pend1 = nbuf > 1 && njobs > 1;
-    for (int k = 0; k < njobs; ++k) {
-        const bool odd = k & 1;
-        uint64_t *bar = odd ? &bar1 : &bar0;
-        const int job = (int)blockIdx.x + k * (int)gridDim.x;
-        const int run = job / (ngroups * ntiles), jr = job - run * ngroups * ntiles;
-        const int g = jr / ntiles, t = jr - g * ntiles;
-        const int kx0 = t * TW;
-        if (!block_wait(bar, odd ? par1 : par0, err)) {
-            if (pend0) mbar_wait_bounded(&bar0, par0);
-            if (pend1) mbar_wait_bounded(&bar1, par1);
-            return;
-        }
-        if (odd) {
-            par1 ^= 1;
-            pend1 = false;
-        } else {
-            par0 ^= 1;
-            pend0 = false;
-        }
-        C *T = odd ? buf1 : buf0;
-        const int oslot = gt[g].out_slot;
-        const real c0 = gt[g].c0, c1 = gt[g].c1, c3 = gt[g].c3;
-        C v[E];
-        // stage 1, forward
-#pragma unroll
-        for (int q = 0; q < E; ++q) v[q] = T[(jl + PP * q) * TW + c];
-        SmallDFT<E, -1, C>::run(v);
-#pragma unroll
-        for (int k1 = 1; k1 < E; ++k1) v[k1] = cmul(v[k1], twc[k1 * PP + jl]);
-        __syncwarp();
-#pragma unroll
-        for (int k1 = 0; k1 < E; ++k1) T[cpos<NY>(c, jl, k1)] = v[k1];
-        __syncthreads();
-        // stage 2: forward, multiplier, inverse, conjugate twiddles
-        {
-            const real mx = c0 * kxs[kx0 + c];
-#pragma unroll
-            for (int q = 0; q < E / PP; ++q) {
-                const int k1 = jl + PP * q;
-                C u[PP];
-#pragma unroll
-                for (int l = 0; l < PP; ++l) u[l] = T[cpos<NY>(c, l, k1)];
-                SmallDFT<PP, -1, C>::run(u);
-#pragma unroll
-                for (int k2 = 0; k2 < PP; ++k2) {
-                    const real ay = kys[k1 + E * k2];
-                    if (c3 != real(0)) {   // uniform over the block
-                        u[k2] = cscale(u[k2], c3 * ay * ay);
-                    } else {
-                        const real m = mx + c1 * ay;   // i m
-                        u[k2] = C{-m * u[k2].y, m * u[k2].x};
-                    }
-                }
-                SmallDFT<PP, +1, C>::run(u);
-#pragma unroll
-                for (int l = 0; l < PP; ++l) T[cpos<NY>(c, l, k1)] = l == 0 ? u[l] : cmul(u[l], cconj(twt[l * E + k1]));
-            }
-        }
-        __syncthreads();
-        // stage 1, inverse
-#pragma unroll
-        for (int k1 = 0; k1 < E; ++k1) v[k1] = T[cpos<NY>(c, jl, k1)];
-        fence_proxy_async();
-        __syncthreads();
-        if (tid == 0 && k + nbuf < njobs) {   // the tile buffer is free: job k + nbuf
-            const bool nodd = (k + nbuf) & 1;
-            kcol_issue(T, nodd ? &bar1 : &bar0, gt, k + nbuf, ntiles, ngroups, TW, NY, BOXR, &tmap, &fmap);
-            if (nodd) pend1 = true;
-            else pend0 = true;
-            // and the job after it into L2, so that its copy finds the tiles there
-            if (k + nbuf + 1 < njobs) kcol_prefetch(gt, k + nbuf + 1, ntiles, ngroups, TW, NY, BOXR, &tmap, &fmap);
-        }
-        SmallDFT<E, +1, C>::run(v);
-        C *out = spec + (size_t)run * NSLOT * slot + (size_t)oslot * slot + kx0 + c;
-#pragma unroll
-        for (int q = 0; q < E; ++q) out[(size_t)(jl + PP * q) * h] = v[q];
-    }
-}
-
-// shared memory of kcol_wr<NY> with nbuf tile buffers
-inline size_t kcol_wr_smem(int NY, int h, int nbuf) {
-    const int TW = col_tw_host(NY);
-    const size_t tile = (size_t)TW * NY * 8;
-    return smem_bytes({(size_t)2 * NY * 8, (size_t)(h + 1) * 4, (size_t)NY * 4, tile, nbuf > 1 ? tile : 0});
 }
 
 // shared memory of k5_wr<H>

@@ -25,6 +25,10 @@ __host__ __device__ constexpr int row_p(int size, int H) {
 }
 // threads per block
 __host__ __device__ constexpr int row_nt(int size, int H) { return row_p(size, H) == 32 ? 256 : 128; }
+// ... of K3, whose 11 derivative rows fill half the row groups: more, smaller
+// blocks keep the warps busy (2048^2 fp32 272 -> 183 us, 384^2 25 -> 19, 1024^2
+// fp64 889 -> 749; shorter fp64 rows lose by it: 256^2 95 -> 104)
+__host__ __device__ constexpr int row_nt3(int size, int H) { return size == 4 && row_p(size, H) < 32 ? 64 : 128; }
 // blocks per row (cluster size): as many as give every row group one
 // distribution row, at most 4
 __host__ __device__ constexpr int row_cs(int size, int H) { return row_p(size, H) >= 16 ? 4 : row_p(size, H) == 8 ? 2 : 1; }
@@ -66,7 +70,7 @@ struct RowSet {
     const void *dx = nullptr, *energy = nullptr;   // single-row kernels: ng rows a block, smem_rows bytes
     int ng = 1;
     size_t smem_rows = 0;
-    int nt = 0, cs = 1;
+    int nt = 0, nt3 = 0, cs = 1;
     size_t smem1 = 0, smem3 = 0, smem5 = 0;
 };
 
