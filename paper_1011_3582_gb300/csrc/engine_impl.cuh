@@ -2161,7 +2161,7 @@ class EngineT : public Engine {
                 const int nt = nt_k1wr_host(h_);
                 auto *kern = h_ == 512 ? k1_wr<512> : h_ == 256 ? k1_wr<256> : k1_wr<128>;
                 if (!(st = launch_pdl("k1_wr", kern, grid1w_, nt, smem1w_, cur, specb_, fieldsb_,
-                                      (const float2 *)Tw1_, (const float2 *)Wp_, (const float *)kxt_, kp_, err_)).good())
+                                      (const float2 *)Tw1_, (const float2 *)Trow_, (const float *)kxt_, kp_, err_)).good())
                     return st;
                 k1done = true;
             }
@@ -2193,7 +2193,7 @@ class EngineT : public Engine {
                 const int nt = nt_k3wr_host(h_);
                 auto *kern = h_ == 512 ? k3_wr<512> : h_ == 256 ? k3_wr<256> : k3_wr<128>;
                 if (!(st = launch_pdl("k3_wr", kern, grid3w_, nt, smem3w_, specb_,
-                                      (const float2 *)Tw1_, (const float2 *)Wp_, (const float *)kxt_, kp_, err_)).good())
+                                      (const float2 *)Tw1_, (const float2 *)Wp_, (const float2 *)Trow_, (const float *)kxt_, kp_, err_)).good())
                     return st;
                 k3done = true;
             }

@@ -587,8 +587,15 @@ template <> struct Vec<double, 1> { using T = double; };
 template <typename real, int V> __device__ __forceinline__ void ldv(real (&a)[V], const real *p) {
     *reinterpret_cast<typename Vec<real, V>::T *>(a) = *reinterpret_cast<const typename Vec<real, V>::T *>(p);
 }
-template <typename real, int V> __device__ __forceinline__ void stv(real *p, const real (&a)[V]) {
-    *reinterpret_cast<typename Vec<real, V>::T *>(p) = *reinterpret_cast<const typename Vec<real, V>::T *>(a);
+// f^n of the later Runge-Kutta stages and the new f leave the L2 first: they are
+// not read again before the spectra are (2048^2 fp32 592 -> 562 us, 768^2 103.6 ->
+// 101.8; the same for K1's reads of f cost 2048^2 326 -> 333, and for the stage
+// state gave nothing)
+template <typename real, int V> __device__ __forceinline__ void ldv_once(real (&a)[V], const real *p) {
+    *reinterpret_cast<typename Vec<real, V>::T *>(a) = __ldcs(reinterpret_cast<const typename Vec<real, V>::T *>(p));
+}
+template <typename real, int V> __device__ __forceinline__ void stv_once(real *p, const real (&a)[V]) {
+    __stcs(reinterpret_cast<typename Vec<real, V>::T *>(p), *reinterpret_cast<const typename Vec<real, V>::T *>(a));
 }
 
 template <typename real, int H>
@@ -600,10 +607,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
     // sites per thread and pass of the epilogue, and ring pairs (r, r + 4) loaded
     // before any of their stores: 16-byte accesses on long rows (two halves of a
     // ring, for the registers), all 8 directions at once on short ones
-#ifndef K5V
-#define K5V 4
-#endif
-    constexpr int V = sizeof(real) == 8 ? 1 : H >= 256 ? K5V : 2, RP = V == 4 ? 2 : 4;
+    constexpr int V = sizeof(real) == 8 ? 1 : H >= 256 ? 4 : 2, RP = V == 4 ? 2 : 4;
     static_assert(CHN % 8 == 0, "whole rings per block");
     extern __shared__ __align__(128) unsigned char row_smem[];
     C *B = reinterpret_cast<C *>(row_smem);                     // [6 NRING] convection rows
@@ -712,7 +716,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
         ldv<real, V>(CC, co + 3 * NX + x);
         ldv<real, V>(iT, co + 4 * NX + x);
         const real hh = real(0.70710678118654752440);
-        real p0[V], p1[V], p2[V], p3[V], p4[V], g0[V], dp[V], dm[V], ep[V], em[V];
+        real p0[V], p1[V], p2[V], p3[V], p4[V], h0[V], dp[V], dm[V], ep[V], em[V];
 #pragma unroll
         for (int q = 0; q < V; ++q) {
             const real qq = real(0.5) * (ux[q] * ux[q] + uy[q] * uy[q]) * iT[q], om = real(1) - qq;
@@ -723,7 +727,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
             p2[q] = real(0.5) * r2 * om;
             p3[q] = r3 * (real(1) / real(6));
             p4[q] = r3 * iT[q] * (real(1) / real(24));
-            g0[q] = e0[q] + CC[q] * sk2;
+            h0[q] = itau - (e0[q] + CC[q] * sk2);
             ux[q] *= sk;
             uy[q] *= sk;
             ex[q] *= sk;
@@ -744,7 +748,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
             for (int q = 0; q < 2 * RP; ++q) {
                 const int r = r0 + (q >> 1) + 4 * (q & 1);
                 ldv<real, V>(fc[q], pc + (size_t)r * N);
-                if (with_base) ldv<real, V>(fb[q], pb + (size_t)r * N);
+                if (with_base) ldv_once<real, V>(fb[q], pb + (size_t)r * N);
                 if ((r & 3) == 2) ldv<real, V>(cv[q], row(v0 + r) + x);   // v_x = 0: real from the column pass
                 else ldv<real, V>(cv[q], cr + (size_t)ring_pos(r) * 2 * RC);
             }
@@ -760,14 +764,15 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
 #pragma unroll
                     for (int s = 0; s < 2; ++s) {
                         const real fe = s ? ev - od : ev + od;
-                        const real g = s ? g0[q] - ed : g0[q] + ed;   // -I / f^eq, Eq. 11
+                        // (1 / tau - g) f^eq - f / tau - convection, g = -I / f^eq (Eqs. 10, 11)
+                        const real hd = s ? h0[q] + ed : h0[q] - ed;
                         const real f = fc[2 * h + s][q];
-                        const real rhs = -cv[2 * h + s][q] - (f - fe) * itau - g * fe;   // Eq. 10
+                        const real rhs = hd * fe - cv[2 * h + s][q] - f * itau;
                         fn[s][q] = rk_combine(with_base, beta, dt, f, fb[2 * h + s][q], rhs);
                     }
                 }
-                stv<real, V>(po + (size_t)r * N, fn[0]);
-                stv<real, V>(po + (size_t)(r + 4) * N, fn[1]);
+                stv_once<real, V>(po + (size_t)r * N, fn[0]);
+                stv_once<real, V>(po + (size_t)(r + 4) * N, fn[1]);
             }
         }
     }

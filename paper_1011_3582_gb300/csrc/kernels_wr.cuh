@@ -178,9 +178,9 @@ __device__ __forceinline__ void row_fft_wr(C *z, const C *tw, int j, int rsw) {
 // half-length transform of the packed row) -> one-sided spectrum X[0 .. H-1]
 // with the real Nyquist value in the imaginary part of X[0], written to
 // out (global memory, coalesced: lanes take consecutive k and H - k).
-// Wp[k] = exp(-2 pi i k / 2H), k <= H / 2.
+// Wh[k] = exp(-2 pi i k / 2H) / 2, k <= H / 2.
 template <int H, typename C>
-__device__ __forceinline__ void r2c_post_wr(const C *z, C *out, const C *Wp, int j) {
+__device__ __forceinline__ void r2c_post_wr(const C *z, C *out, const C *Wh, int j) {
     using R = decltype(z[0].x);
     constexpr int P = RowCfg<H>::P;
 #pragma unroll
@@ -192,11 +192,9 @@ __device__ __forceinline__ void r2c_post_wr(const C *z, C *out, const C *Wp, int
             out[0] = C{z0.x + z0.y, z0.x - z0.y};
         } else {
             const C p = z[k], q = z[H - k];
-            const C ze = cscale(cadd(p, cconj(q)), R(0.5));
-            const C zo = cscale(cmul_mi(csub(p, cconj(q))), R(0.5));
-            const C wz = cmul(Wp[k], zo);
-            out[k] = cadd(ze, wz);
-            if (H - k != k) out[H - k] = cconj(csub(ze, wz));
+            const C s = cadd(p, cconj(q)), w = cmul(Wh[k], cmul_mi(csub(p, cconj(q))));
+            out[k] = C{R(0.5) * s.x + w.x, R(0.5) * s.y + w.y};
+            if (H - k != k) out[H - k] = C{R(0.5) * s.x - w.x, w.y - R(0.5) * s.y};
         }
     }
 }
@@ -204,7 +202,7 @@ __device__ __forceinline__ void r2c_post_wr(const C *z, C *out, const C *Wp, int
 // r2c_post_wr times i k_x c: dst[k] = i kxt[k] sx X[k] (bin 0, DC and
 // row-Nyquist, has k_x = 0 for both).  dst may be z.
 template <int H, typename C>
-__device__ __forceinline__ void r2c_post_dx(const C *z, C *dst, const float *__restrict__ kxt, float sx, const C *Wp,
+__device__ __forceinline__ void r2c_post_dx(const C *z, C *dst, const float *__restrict__ kxt, float sx, const C *Wh,
                                             int j) {
     using R = decltype(z[0].x);
     constexpr int P = RowCfg<H>::P;
@@ -216,11 +214,9 @@ __device__ __forceinline__ void r2c_post_dx(const C *z, C *dst, const float *__r
             dst[0] = C{0, 0};
         } else {
             const C p = z[k], q = z[H - k];
-            const C ze = cscale(cadd(p, cconj(q)), R(0.5));
-            const C zo = cscale(cmul_mi(csub(p, cconj(q))), R(0.5));
-            const C wz = cmul(Wp[k], zo);
-            dst[k] = imul(kxt[k] * sx, cadd(ze, wz));
-            if (H - k != k) dst[H - k] = imul(kxt[H - k] * sx, cconj(csub(ze, wz)));
+            const C s = cadd(p, cconj(q)), w = cmul(Wh[k], cmul_mi(csub(p, cconj(q))));
+            dst[k] = imul(kxt[k] * sx, C{R(0.5) * s.x + w.x, R(0.5) * s.y + w.y});
+            if (H - k != k) dst[H - k] = imul(kxt[H - k] * sx, C{R(0.5) * s.x - w.x, w.y - R(0.5) * s.y});
         }
     }
 }
@@ -239,14 +235,12 @@ __device__ __forceinline__ void c2r_pre_wr(C *z, const C *Wp, int j) {
             const C x0 = z[0];
             z[0] = C{x0.x + x0.y, x0.x - x0.y};
         } else {
+            // with a = p + conj q, e = i (p - conj q) conj w: Z[k] = a + e,
+            // Z[H - k] = conj(a - e)
             const C p = z[k], q = z[H - k];
-            const C w = Wp[k];
-            const C wc = cconj(w);
-            z[k] = cadd(cadd(p, cconj(q)), cmul_i(cmul(csub(p, cconj(q)), wc)));
-            if (H - k != k) {
-                const C mw = C{-w.x, -w.y};
-                z[H - k] = cadd(cadd(q, cconj(p)), cmul_i(cmul(csub(q, cconj(p)), mw)));
-            }
+            const C a = cadd(p, cconj(q)), e = cmul_i(cmul(csub(p, cconj(q)), cconj(Wp[k])));
+            z[k] = cadd(a, e);
+            if (H - k != k) z[H - k] = cconj(csub(a, e));
         }
     }
 }
@@ -261,6 +255,18 @@ __device__ __forceinline__ void ld4(float (&a)[4], const float *p) {
 }
 __device__ __forceinline__ void st4(float *p, const float (&a)[4]) {
     *reinterpret_cast<float4 *>(p) = make_float4(a[0], a[1], a[2], a[3]);
+}
+// ... of values that leave the L2 first: f^n and the new f are not read again
+// before the spectra are (1024^2: K5 107.6 -> 106.2 us)
+__device__ __forceinline__ void ld4_once(float (&a)[4], const float *p) {
+    const float4 v = __ldcs(reinterpret_cast<const float4 *>(p));
+    a[0] = v.x;
+    a[1] = v.y;
+    a[2] = v.z;
+    a[3] = v.w;
+}
+__device__ __forceinline__ void st4_once(float *p, const float (&a)[4]) {
+    __stcs(reinterpret_cast<float4 *>(p), make_float4(a[0], a[1], a[2], a[3]));
 }
 
 // ---------------------------------------------------------------------------
@@ -293,7 +299,7 @@ __device__ __forceinline__ void k1w_issue(const float *f, float *dst, uint64_t *
 
 template <int H>
 __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_wr(const float *__restrict__ f, float2 *spec, float *__restrict__ fields,
-                                                 const float2 *__restrict__ tw_g, const float2 *__restrict__ Wp_g,
+                                                 const float2 *__restrict__ tw_g, const float2 *__restrict__ Wh_g,
                                                  const float *__restrict__ kxt, KP<float> P, int *err) {
     using C = float2;
     using real = float;
@@ -302,7 +308,7 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
     constexpr int NG = NWARP * RPW;                // row groups per block
     constexpr int CH = NG + 1, NCH = NMOV / NG;    // rows per chunk buffer, chunks per row
     constexpr int SMAX = (NX + NT - 1) / NT;
-    static_assert(NMOV % NG == 0 && NG >= 6, "chunking");
+    static_assert(NMOV % NG == 0 && NG % 8 == 0, "chunking");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar0, bar1;
     const int nx = NX, ny = P.ny, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -311,7 +317,7 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
     const size_t N = (size_t)NX * ny, slot = (size_t)ny * H;
     SmemCursor sc{smem_raw, 0u};
     C *tw = (C *)sc.take(H * sizeof(C));
-    C *Wp = (C *)sc.take((H / 2 + 1) * sizeof(C));
+    C *Wh = (C *)sc.take((H / 2 + 1) * sizeof(C));
     real *kxs = (real *)sc.take(H * sizeof(real));   // k_x of the row bins
     real *buf0 = (real *)sc.take((size_t)CH * NX * sizeof(real));
     real *buf1 = (real *)sc.take((size_t)CH * NX * sizeof(real));
@@ -328,7 +334,7 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
         if (njobs > 1) k1w_issue(f, buf1, &bar1, 1, NCH, NG, nx, ny, N);
     }
     load_tab4(tw, tw_g, H, NT);
-    load_tab4(Wp, Wp_g, H / 2 + 1, NT);
+    load_tab4(Wh, Wh_g, H / 2 + 1, NT);
     load_tab4(kxs, kxt, H, NT);
     grid_dep_wait();
     __syncthreads();
@@ -359,19 +365,26 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
             pend0 = false;
         }
         real *B = odd ? buf1 : buf0;
-        // moments (Eqs. 7-9): sums over this chunk's rows
-#pragma unroll 1
-        for (int r = 0; r < nf; ++r) {
-            const int i = i0 + r;
-            const real vx = VX<real>(i), vy = VY<real>(i), v2 = V2<real>(i);
+        // moments (Eqs. 7-9): sums over this chunk's rows, ring by ring (speed
+        // s_k, directions r pi / 4), 19 operations a ring and site
+        const int q0 = c == 0 ? 1 : 0;   // chunk row of the first ring's direction 0
 #pragma unroll
-            for (int s = 0; s < SMAX; ++s) {
-                const int x = tid + s * NT;
-                const real v = B[(size_t)r * NX + x];
-                a0[s] += v;
-                a1[s] += vx * v;
-                a2[s] += vy * v;
-                a3[s] += v2 * v;
+        for (int s = 0; s < SMAX; ++s) {
+            const int x = tid + s * NT;
+            if (c == 0) a0[s] += B[x];   // the rest velocity
+#pragma unroll 1
+            for (int rr = 0; rr < NG / 8; ++rr) {
+                const real *q = B + (size_t)(q0 + 8 * rr) * NX + x;
+                const int v0 = 1 + c * NG + 8 * rr;
+                real v[8];
+#pragma unroll
+                for (int r = 0; r < 8; ++r) v[r] = q[(size_t)r * NX];
+                const real sum = ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+                const real d15 = v[1] - v[5], d37 = v[3] - v[7], hh = real(0.70710678118654752440);
+                a0[s] += sum;
+                a1[s] += VX<real>(v0) * ((v[0] - v[4]) + hh * (d15 - d37));
+                a2[s] += VX<real>(v0) * ((v[2] - v[6]) + hh * (d15 + d37));
+                a3[s] += V2<real>(v0) * sum;
             }
         }
         __syncthreads();
@@ -387,9 +400,9 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
                 C *dst = spec_r + (size_t)(i - 1) * slot + (size_t)y * H;
                 row_fft_wr<H, -1>(zr, tw, j, rsw);
                 if (VY<real>(i) == real(0))   // convection in k_x alone: i v_x k_x f^ / nx, no column pass
-                    r2c_post_dx<H>(zr, dst, kxs, VX<real>(i) * P.scale_x, Wp, j);
+                    r2c_post_dx<H>(zr, dst, kxs, VX<real>(i) * P.scale_x, Wh, j);
                 else
-                    r2c_post_wr<H>(zr, dst, Wp, j);
+                    r2c_post_wr<H>(zr, dst, Wh, j);
             }
         }
         if (c == NCH - 1) {
@@ -420,7 +433,7 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
             if (grp < 6) {
                 C *zr = reinterpret_cast<C *>(fb) + (size_t)grp * H;
                 row_fft_wr<H, -1>(zr, tw, j, rsw);
-                r2c_post_wr<H>(zr, spec_r + (size_t)(SLOT_RHO + grp) * slot + (size_t)y * H, Wp, j);
+                r2c_post_wr<H>(zr, spec_r + (size_t)(SLOT_RHO + grp) * slot + (size_t)y * H, Wh, j);
             }
         }
         fence_proxy_async();
@@ -463,7 +476,8 @@ __device__ __forceinline__ void k3_issue(const C *spec, C *dst, uint64_t *bar, i
 
 template <int H>
 __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_wr(float2 *spec, const float2 *__restrict__ tw_g,
-                                                 const float2 *__restrict__ Wp_g, const float *__restrict__ kxt,
+                                                 const float2 *__restrict__ Wp_g, const float2 *__restrict__ Wh_g,
+                                                 const float *__restrict__ kxt,
                                                  KP<float> P, int *err) {
     using C = float2;
     using real = float;
@@ -479,6 +493,7 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
     SmemCursor sc{smem_raw, 0u};
     C *tw = (C *)sc.take(H * sizeof(C));
     C *Wp = (C *)sc.take((H / 2 + 1) * sizeof(C));
+    C *Wh = (C *)sc.take((H / 2 + 1) * sizeof(C));
     real *kxs = (real *)sc.take(H * sizeof(real));   // k_x of the row bins
     C *buf0 = (C *)sc.take((size_t)NK3 * H * sizeof(C));
     C *buf1 = NB > 1 ? (C *)sc.take((size_t)NK3 * H * sizeof(C)) : buf0;
@@ -494,6 +509,7 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
     }
     load_tab4(tw, tw_g, H, NT);
     load_tab4(Wp, Wp_g, H / 2 + 1, NT);
+    load_tab4(Wh, Wh_g, H / 2 + 1, NT);
     load_tab4(kxs, kxt, H, NT);
     grid_dep_wait();
     __syncthreads();
@@ -549,7 +565,7 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
         for (int r = grp; r < 3; r += NG) {
             C *zr = dc + (size_t)r * H;
             row_fft_wr<H, -1>(zr, tw, j, rsw);
-            r2c_post_dx<H>(zr, zr, kxs, P.scale_x, Wp, j);
+            r2c_post_dx<H>(zr, zr, kxs, P.scale_x, Wh, j);
             __syncwarp(group_mask<PL>());
             c2r_pre_wr<H>(zr, Wp, j);
             __syncwarp(group_mask<PL>());
@@ -573,7 +589,7 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
 
 // shared memory of k3_wr<H>
 inline size_t k3_wr_smem(int H) {
-    return smem_bytes({(size_t)H * 8, (size_t)(H / 2 + 1) * 8, (size_t)H * 4, (size_t)NK3 * 2 * H * 4,
+    return smem_bytes({(size_t)H * 8, (size_t)(H / 2 + 1) * 8, (size_t)(H / 2 + 1) * 8, (size_t)H * 4, (size_t)NK3 * 2 * H * 4,
                        nb_k3wr_host(H) > 1 ? (size_t)NK3 * 2 * H * 4 : 0});
 }
 
@@ -793,52 +809,60 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
                 ld4(e1x, Hd + nx + x0);
                 ld4(e1y, Hd + 2 * nx + x0);
                 ld4(CC, Hd + 7 * nx + x0);
-                real rF[4], p0[4], p1[4], p2[4], p3[4], p4[4], g0[4], uxk[4], uyk[4], exk[4], eyk[4];
+                real p0[4], p1[4], p2[4], p3[4], p4[4], h0[4], uxk[4], uyk[4], exk[4], eyk[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const real qq = real(0.5) * (ux[q] * ux[q] + uy[q] * uy[q]) * iT[q], om = real(1) - qq;
-                    p0[q] = om + real(0.5) * qq * qq;
-                    p1[q] = om * iT[q];
-                    p2[q] = real(0.5) * om * iT[q] * iT[q];
-                    p3[q] = iT[q] * iT[q] * iT[q] * (real(1) / real(6));
-                    p4[q] = iT[q] * iT[q] * iT[q] * iT[q] * (real(1) / real(24));
-                    rF[q] = rho[q] * weight_Fk<real>(k, T[q]);   // Eq. 4
-                    g0[q] = e0[q] + CC[q] * sk2;
+                    const real rF = rho[q] * weight_Fk<real>(k, T[q]);   // Eq. 4
+                    const real r1 = rF * iT[q], r2 = r1 * iT[q], r3 = r2 * iT[q];
+                    p0[q] = rF * (om + real(0.5) * qq * qq);   // rho F_k times the factors of Eq. 3
+                    p1[q] = r1 * om;
+                    p2[q] = real(0.5) * r2 * om;
+                    p3[q] = r3 * (real(1) / real(6));
+                    p4[q] = r3 * iT[q] * (real(1) / real(24));
+                    h0[q] = itau - (e0[q] + CC[q] * sk2);
                     uxk[q] = sk * ux[q];
                     uyk[q] = sk * uy[q];
                     exk[q] = sk * e1x[q];
                     eyk[q] = sk * e1y[q];
                 }
-                // (FFTLB_K5_VEC = 1: the distributions of four directions are
+                // directions r and r + 4 together: f^eq = even +- odd in v.u;
+                // rhs = (1 / tau - g) f^eq - f / tau - convection with g = -I /
+                // f^eq (Eqs. 10, 11).  The distributions of two such pairs are
                 // loaded before any of their stores, as fout may alias fcur or
-                // fbase; 2: all eight, through restrict-qualified pointers, as
-                // each element is read before the same thread writes it)
+                // fbase.
                 const real *__restrict__ pc = fcur + o0;
                 const real *__restrict__ pb = fbase + o0;
                 real *__restrict__ po = fout + o0;
-                constexpr int RH = FFTLB_K5_VEC == 1 ? 4 : 8;
 #pragma unroll
-                for (int r0 = 0; r0 < 8; r0 += RH) {
-                    real fc[RH][4], fb[RH][4];
+                for (int r0 = 0; r0 < 4; r0 += 2) {
+                    real fc[4][4], fb[4][4];
 #pragma unroll
-                    for (int r = 0; r < RH; ++r) {
-                        ld4(fc[r], pc + (size_t)(r0 + r) * N);
-                        if (with_base) ld4(fb[r], pb + (size_t)(r0 + r) * N);
+                    for (int r = 0; r < 4; ++r) {
+                        const int d = r0 + (r >> 1) + 4 * (r & 1);
+                        ld4(fc[r], pc + (size_t)d * N);
+                        if (with_base) ld4_once(fb[r], pb + (size_t)d * N);
                     }
 #pragma unroll
-                    for (int r = 0; r < RH; ++r) {
-                        real cv[4], fn[4];
-                        ld4(cv, cres + (size_t)(r0 + r) * NX + x0);
+                    for (int r = 0; r < 2; ++r) {
+                        real cv[2][4], fn[2][4];
+                        ld4(cv[0], cres + (size_t)(r0 + r) * NX + x0);
+                        ld4(cv[1], cres + (size_t)(r0 + r + 4) * NX + x0);
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
-                            const real vu = dir_dot<real>(r0 + r, uxk[q], uyk[q]);
-                            const real br = p0[q] + vu * (p1[q] + vu * (p2[q] + vu * (p3[q] + vu * p4[q])));
-                            const real fe = rF[q] * br;                                          // Eq. 3
-                            const real I = -(g0[q] + dir_dot<real>(r0 + r, exk[q], eyk[q])) * fe;  // Eq. 11
-                            const real rhs = -cv[q] - (fc[r][q] - fe) * itau + I;                // Eq. 10
-                            fn[q] = rk_combine(with_base, beta, dt, fc[r][q], fb[r][q], rhs);
+                            const real vu = dir_dot<real>(r0 + r, uxk[q], uyk[q]), w2 = vu * vu;
+                            const real ev = p0[q] + w2 * (p2[q] + w2 * p4[q]), od = vu * (p1[q] + w2 * p3[q]);   // Eq. 3
+                            const real ed = dir_dot<real>(r0 + r, exk[q], eyk[q]);
+#pragma unroll
+                            for (int s = 0; s < 2; ++s) {
+                                const real fe = s ? ev - od : ev + od, hd = s ? h0[q] + ed : h0[q] - ed;
+                                const real f = fc[2 * r + s][q];
+                                const real rhs = hd * fe - cv[s][q] - f * itau;
+                                fn[s][q] = rk_combine(with_base, beta, dt, f, fb[2 * r + s][q], rhs);
+                            }
                         }
-                        st4(po + (size_t)(r0 + r) * N, fn);
+                        st4_once(po + (size_t)(r0 + r) * N, fn[0]);
+                        st4_once(po + (size_t)(r0 + r + 4) * N, fn[1]);
                     }
                 }
             } else {
