@@ -49,9 +49,18 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
                  : "memory");
 }
 
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
+// PEER: the phase also orders what other blocks of the cluster wrote
+template <bool PEER = false> __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     uint32_t ok;
-    asm volatile(
+    if constexpr (PEER)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+    else asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
@@ -69,12 +78,13 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 // bounded wait by this thread; false if the phase did not complete within
 // limit_ns of %globaltimer time (or kWaitPolls polls)
+template <bool PEER = false>
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity,
                                                   unsigned long long limit_ns = kWaitNs) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<PEER>(bar, parity)) return true;
     const unsigned long long t0 = global_ns();
     for (unsigned i = 1; i < kWaitPolls; ++i) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait<PEER>(bar, parity)) return true;
         if ((i & 63u) == 0 && global_ns() - t0 > limit_ns) return false;
     }
     return false;

@@ -68,6 +68,12 @@ template <typename real, int H, int NT_ = row_nt((int)sizeof(real), H)> struct R
     static __host__ __device__ constexpr int owner(int r) { return (r / RPW) % CS; }
     static __host__ __device__ constexpr int local(int r) { return r / (RPW * CS) * RPW + r % RPW; }
     static __host__ __device__ constexpr int share(int n) { return (n + RPW * CS - 1) / (RPW * CS) * RPW; }
+    // block c's rows among n
+    static __host__ __device__ constexpr int nrows(int c, int n) {
+        int m = 0;
+        for (int r = 0; r < n; ++r) m += owner(r) == c;
+        return m;
+    }
     // the i-th row of block c
     static __host__ __device__ constexpr int nth(int c, int i) { return (i / RPW * CS + c) * RPW + i % RPW; }
 };
@@ -277,11 +283,12 @@ __device__ __forceinline__ float wk(const RowArgs<float> &A, int k, float T) {
     return T * (s + c);
 }
 
-// this thread's bounded wait for the tables; running out is recorded
-__device__ __forceinline__ void table_wait(uint64_t *bar, int *err) {
-    if (!mbar_wait_bounded(bar, 0)) {
+// this thread's bounded wait for the tables or (PEER) for what the row's other
+// blocks push; running out is recorded
+template <bool PEER = false> __device__ __forceinline__ void table_wait(uint64_t *bar, int *err) {
+    if (!mbar_wait_bounded<PEER>(bar, 0)) {
         atomicOr(err, kErrWaitTimeout);
-        mbar_wait_bounded(bar, 0);
+        mbar_wait_bounded<PEER>(bar, 0);
     }
 }
 
@@ -298,6 +305,49 @@ template <int CS> __device__ __forceinline__ void row_wait() {
     if constexpr (CS > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     else __syncthreads();
 }
+// The row's blocks push what each other needs instead of reading it behind a
+// barrier: copies and stores into another block's shared memory that complete on
+// that block's mbarrier need no fence, while a cluster barrier's release holds
+// every warp until all its accesses have been performed.  A block stays until
+// the others are done with its memory: row_leave() where it needs nothing more
+// from them, row_gone() at its end (no data is handed over by these two).
+// Against a cluster barrier for every hand-over: 384^2 fp32 215 -> 196 us a step,
+// 768^2 699 -> 650, 2048^2 4480 -> 4288 (K5 562 -> 521), 128^2 64.2 -> 60.4, 64^2
+// fp64 204 -> 198.  The first hand-over of K1 and K3 keeps the barrier: pushed,
+// it needs room for three more rows, a resident block less on the long ones, and
+// one release a block on the others' mbarriers took as long (384^2: 198).
+template <int CS> __device__ __forceinline__ void row_leave() {
+    if constexpr (CS > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+}
+template <int CS> __device__ __forceinline__ void row_gone() {
+    if constexpr (CS > 1) asm volatile("barrier.cluster.wait;" ::: "memory");
+}
+// p's address in block r's part of the cluster's shared memory
+__device__ __forceinline__ uint32_t peer_u32(const void *p, int r) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(r));
+    return a;
+}
+// v to p in block r, completing on bar in block r
+__device__ __forceinline__ void push(float *p, float v, uint64_t *bar, int r) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(peer_u32(p, r)),
+                 "r"(__float_as_uint(v)), "r"(peer_u32(bar, r))
+                 : "memory");
+}
+__device__ __forceinline__ void push(double *p, double v, uint64_t *bar, int r) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(peer_u32(p, r)),
+                 "l"(__double_as_longlong(v)), "r"(peer_u32(bar, r))
+                 : "memory");
+}
+// `bytes` (a multiple of 16, both addresses 16-byte aligned) from src of this
+// block to dst in block r, completing on bar in block r
+__device__ __forceinline__ void push_bulk(void *dst, const void *src, uint32_t bytes, uint64_t *bar, int r) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     peer_u32(dst, r)),
+                 "r"(smem_u32(src)), "r"(bytes), "r"(peer_u32(bar, r))
+                 : "memory");
+}
+
 // p's counterpart in block r of the cluster
 template <int CS, typename T> __device__ __forceinline__ T *in_block(T *p, int r) {
     if constexpr (CS == 1) return p;
@@ -308,7 +358,7 @@ template <int CS, typename T> __device__ __forceinline__ T *in_block(T *p, int r
 // K1: moments rho, u, T (Eqs. 7-9), Pi = P^w - rho T (Eq. 18), g = M/T, and the
 // forward rows of the f_i with v_x != 0 and of rho, u_x, u_y, T, Pi, g.  Block c
 // of the row takes f_i, i = 1 + c CHN ..: it sums their share of the moments,
-// forms the fields of its slice of sites from everybody's sums, sends each
+// forms the fields of its slice of sites from everybody's sums, pushes each
 // field to the block that transforms it, and then transforms its f_i and its
 // share of the fields together (the fields after the f_i, hiding the exchange,
 // took a second pass of the same length: 51 us against 37 on six 512x4 fp64
@@ -321,7 +371,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k1_row(
     using C = typename G::C;
     constexpr int CS = G::CS, CHN = G::CHN, RC = G::RC, NX = G::NX, NT = G::NT, P = G::P, NXS = G::NXS, NR = G::NRING;
     extern __shared__ __align__(128) unsigned char row_smem[];
-    __shared__ __align__(8) uint64_t bar;
+    __shared__ __align__(8) uint64_t bar, fbar;
     using LT = RowTable<real>;
     C *B = reinterpret_cast<C *>(row_smem);     // [CHN + 1] rows
     C *F = B + (CHN + 1) * RC;                  // [share(6)] field rows
@@ -343,7 +393,9 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k1_row(
     const int nrow = c == 0 ? CHN + 1 : CHN;                      // block 0 also sums the rest velocity
     if (tid == 0) {
         mbar_init(&bar, 1);
+        mbar_init(&fbar, 1);
         mbar_init_fence();
+        mbar_expect_tx(&fbar, G::nrows(c, 6) * NX * sizeof(real));   // its field rows, from every block
     }
     __syncthreads();
     grid_dep_wait();
@@ -395,11 +447,14 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k1_row(
         const real lv[6] = {rho, ux, uy, Te, rho * Te / (real(1) - A.b * rho) - A.a * rho * rho - rho * Te,   // Eq. 18
                             (A.K + A.H * Te) / Te};                                                        // M / T
 #pragma unroll
-        for (int r = 0; r < 6; ++r)
-            reinterpret_cast<real *>(in_block<CS>(F + G::local(r) * RC, G::owner(r)))[x] = lv[r];
+        for (int r = 0; r < 6; ++r) {
+            real *q = reinterpret_cast<real *>(F + G::local(r) * RC) + x;
+            if constexpr (CS == 1) *q = lv[r];
+            else push(q, lv[r], &fbar, G::owner(r));
+        }
     }
-    row_arrive<CS>();
-    row_wait<CS>();
+    if constexpr (CS == 1) __syncthreads();
+    row_leave<CS>();   // (has read the others' sums; its field rows come by fbar)
     // this block's distribution rows and its share of the field rows, one row
     // group each: 6 of every 8 directions leave room for the fields
     static_assert(6 * NR + G::share(6) <= G::NG, "one pass");
@@ -420,6 +475,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k1_row(
     } else {
         const int q = grp - 6 * NR, r = G::nth(c, q);
         if (q < G::share(6) && r < 6) {
+            if constexpr (CS > 1) table_wait<true>(&fbar, A.err);
             C *z = F + q * RC;
             C *real_row = spec + (size_t)(SLOT_F + r) * slot, *dst = spec + (size_t)(SLOT_RHO + r) * slot;
 #pragma unroll
@@ -428,6 +484,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k1_row(
             row_post<H>(z, T.wh, j, [&](int k, C X) { dst[k] = X; });
         }
     }
+    row_gone<CS>();
 }
 
 template <typename real, int H> size_t k1_row_smem() {
@@ -456,7 +513,7 @@ __global__ void __launch_bounds__(row_nt3((int)sizeof(real), H), row_minb3<real,
     using LT = RowTable<real>;
     unsigned char *tb = reinterpret_cast<unsigned char *>(L + NL * RC);
     const Tab<real, H> T(tb, 0);
-    __shared__ __align__(8) uint64_t bar;
+    __shared__ __align__(8) uint64_t bar, lbar;
     const int c = block_rank<CS>(), tid = (int)threadIdx.x, j = tid & (P - 1), grp = tid / P;
     const int ny = A.ny, yg = (int)blockIdx.x / CS, run = yg / ny, y = yg - run * ny;
     const size_t slot = (size_t)ny * H;
@@ -465,7 +522,9 @@ __global__ void __launch_bounds__(row_nt3((int)sizeof(real), H), row_minb3<real,
     const real *kx = T.kx;
     if (tid == 0) {
         mbar_init(&bar, 1);
+        mbar_init(&lbar, 1);
         mbar_init_fence();
+        mbar_expect_tx(&lbar, G::nrows(c, 3) * NX * sizeof(real));   // its rows of L, from every block
         mbar_expect_tx(&bar, LT::bytes(H));
         table_issue(tb, A.tab, 0, LT::bytes(H), &bar);
     }
@@ -526,8 +585,11 @@ __global__ void __launch_bounds__(row_nt3((int)sizeof(real), H), row_minb3<real,
         const Level2<real> l = level2_site<real>([&](int o) { return d[o]; }, A);
         const real lv[3] = {l.Phx, l.Lxx, l.Lxy};
 #pragma unroll
-        for (int r = 0; r < 3; ++r)
-            reinterpret_cast<real *>(in_block<CS>(L + G::local(r) * RC, G::owner(r)))[x] = lv[r];
+        for (int r = 0; r < 3; ++r) {
+            real *q = reinterpret_cast<real *>(L + G::local(r) * RC) + x;
+            if constexpr (CS == 1) *q = lv[r];
+            else push(q, lv[r], &lbar, G::owner(r));
+        }
         row(SLOT_A)[x] = l.Cn;
         row(SLOT_A + 1)[x] = l.Bx;
         row(SLOT_A + 2)[x] = l.By;
@@ -535,11 +597,12 @@ __global__ void __launch_bounds__(row_nt3((int)sizeof(real), H), row_minb3<real,
         row(SLOT_L2 + 1)[x] = l.Lyy;
         row(SLOT_L2 + 2)[x] = l.Phy;
     }
-    row_arrive<CS>();
-    row_wait<CS>();
+    if constexpr (CS == 1) __syncthreads();
+    row_leave<CS>();   // (has read the others' rows; its rows of L come by lbar)
     for (int q = grp; q < NL; q += G::NG) {
         const int r = G::nth(c, q);
         if (r >= 3) continue;
+        if constexpr (CS > 1) table_wait<true>(&lbar, A.err);
         C *z = L + q * RC;
         row_fft<H, -1>(z, T.tw, j);
         C *dst = spec + (size_t)(SLOT_X + r) * slot;
@@ -548,6 +611,7 @@ __global__ void __launch_bounds__(row_nt3((int)sizeof(real), H), row_minb3<real,
             dst[k] = C{-m * X.y, m * X.x};
         });
     }
+    row_gone<CS>();
 }
 
 template <typename real, int H> size_t k3_row_smem() {
@@ -616,7 +680,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
     using LT = RowTable<real>;
     unsigned char *tb = reinterpret_cast<unsigned char *>(co + NCOEF * NX);
     const Tab<real, H> TB(tb, LT::tw(H));
-    __shared__ __align__(8) uint64_t bar;
+    __shared__ __align__(8) uint64_t bar, xbar, cbar;
     const int c = block_rank<CS>(), tid = (int)threadIdx.x, j = tid & (P - 1), grp = tid / P;
     const int ny = A.ny, yg = (int)blockIdx.x / CS, run = yg / ny, y = yg - run * ny;
     const size_t N = (size_t)NX * ny, slot = (size_t)ny * H;
@@ -627,11 +691,16 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
     const bool with_base = A.alpha != real(0);
     if (tid == 0) {
         mbar_init(&bar, 1);
+        mbar_init(&xbar, 1);
+        mbar_init(&cbar, 1);
         mbar_init_fence();
+        mbar_expect_tx(&xbar, 3 * NXS * sizeof(real));                  // d_x at this block's slice
+        mbar_expect_tx(&cbar, (CS - 1) * NCOEF * NXS * sizeof(real));   // the other slices' coefficients
         mbar_expect_tx(&bar, LT::bytes(H) - LT::tw(H));
         table_issue(tb, A.tab, LT::tw(H), LT::bytes(H), &bar);
     }
     __syncthreads();
+    row_leave<CS>();   // (the barriers are initialised)
     grid_dep_wait();
     if (tid < CHN) {   // this block's distribution rows into L2 ahead of the epilogue
         const size_t o = fo + (size_t)(1 + c * CHN + tid) * N;
@@ -654,16 +723,25 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
             row_pre<H, 1>(z, TB.wp, j, src, src, [](int, C a, C) { return a; }, ready);
             __syncwarp(lanes_of_row<P>());
             row_fft<H, +1>(z, TB.tw, j);
+            if constexpr (CS > 1) {
+                fence_proxy_async();
+                __syncwarp(lanes_of_row<P>());
+            }
         }
+        ready();   // (no copy is in flight when the block ends)
+        row_gone<CS>();
+        // the d_x rows' slices into the first three rows of co, each to the
+        // block that replaces them by coefficients
+        if (CS > 1 && dx && j < CS)
+            push_bulk(co + r * NX + j * NXS, reinterpret_cast<const real *>(X + q * RC) + j * NXS, NXS * sizeof(real), &xbar, j);
     }
-    ready();   // (no copy is in flight when the block ends)
-    row_arrive<CS>();
-    row_wait<CS>();
+    if constexpr (CS == 1) __syncthreads();
+    else table_wait<true>(&xbar, A.err);
     for (int x = c * NXS + tid; x < (c + 1) * NXS; x += NT) {
         real dx[3];
 #pragma unroll
         for (int r = 0; r < 3; ++r)
-            dx[r] = reinterpret_cast<const real *>(in_block<CS>(X + G::local(r) * RC, G::owner(r)))[x];
+            dx[r] = CS == 1 ? reinterpret_cast<const real *>(X + G::local(r) * RC)[x] : co[r * NX + x];
         const real rho = row(SLOT_F)[x], ux = row(SLOT_F + 1)[x], uy = row(SLOT_F + 2)[x], T = row(SLOT_F + 3)[x];
         const real rT = rho * T, irT = real(1) / rT, iT = real(1) / T;
         const real Bx = (row(SLOT_A + 1)[x] + row(SLOT_L2)[x] + dx[1]) * irT;        // Eq. 21
@@ -674,14 +752,15 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
         // I = -(A + B.(v-u) + CC |v-u|^2) f^eq = -(e0 + e1.v + CC |v|^2) f^eq
         const real e[NCOEF] = {At - (Bx * ux + By * uy) + CC * u2, Bx - real(2) * CC * ux, By - real(2) * CC * uy, CC, iT};
 #pragma unroll
-        for (int b = 0; b < CS; ++b) {
-            real *q = in_block<CS>(co, b);
-#pragma unroll
-            for (int i = 0; i < NCOEF; ++i) q[i * NX + x] = e[i];
-        }
+        for (int i = 0; i < NCOEF; ++i) co[i * NX + x] = e[i];
     }
-    row_arrive<CS>();
-    row_wait<CS>();
+    if constexpr (CS > 1) fence_proxy_async();
+    __syncthreads();
+    if (CS > 1 && tid < (CS - 1) * NCOEF) {
+        const int i = tid / (CS - 1), b = tid - i * (CS - 1);
+        real *q = co + i * NX + c * NXS;
+        push_bulk(q, q, NXS * sizeof(real), &cbar, b < c ? b : b + 1);
+    }
     // the rest velocity (no convection) at this block's slice
     for (int x = c * NXS + tid; x < (c + 1) * NXS; x += NT) {
         const real rho = row(SLOT_F)[x], ux = row(SLOT_F + 1)[x], uy = row(SLOT_F + 2)[x], T = row(SLOT_F + 3)[x];
@@ -695,6 +774,8 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
         A.fout[fo + x] =
             rk_combine(with_base, beta, dt, fc, with_base ? A.fbase[fo + x] : real(0), -(fc - fe) * itau - co[x] * fe);
     }
+    if constexpr (CS > 1) table_wait<true>(&cbar, A.err);
+    row_leave<CS>();   // (nothing more comes; its own slices may still be on their way)
     // the rings of this block: velocities 1 + 8 k .. 8 + 8 k of Eq. 1, one
     // speed, one weight, the eight directions known at compile time
 #pragma unroll 1
@@ -776,6 +857,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
             }
         }
     }
+    row_gone<CS>();
 }
 
 template <typename real, int H> size_t k5_row_smem() {
