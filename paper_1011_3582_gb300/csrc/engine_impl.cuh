@@ -1284,11 +1284,15 @@ class EngineT : public Engine {
         if (own_len(h_) && rp > 0) {
             std::vector<C> t1, t2;
             stage1_twiddles(t1, t2, h_, rp);
-            if (wr_ok_ && (h_ == 512 || h_ == 256 || h_ == 128) && !(st = upload_table(&Tw1_, t1)).good()) return st;
+            if (wr_ok_ && (h_ == 512 || h_ == 256 || h_ == 128)) {
+                std::vector<C> w1, w2;
+                stage1_twiddles(w1, w2, h_, h_ / 16);
+                if (!(st = upload_table(&Tw1_, w1)).good()) return st;
+            }
             using L = RowTable<real>;
             std::vector<C> blob((L::bytes(h_) + sizeof(C) - 1) / sizeof(C), C{0, 0});
             unsigned char *b = reinterpret_cast<unsigned char *>(blob.data());
-            std::vector<C> wh(wp.begin(), wp.begin() + h_ / 2 + 1);
+            std::vector<C> wh(wp.begin(), wp.begin() + h_ / 2);
             memcpy(b + L::wp(h_), wh.data(), wh.size() * sizeof(C));
             for (auto &w : wh) {
                 w.x *= real(0.5);
@@ -1801,16 +1805,15 @@ class EngineT : public Engine {
             ra_.spec = specb_;
             ra_.tab = Trow_;
             ra_.err = err_;
-            // The persistent fp32 rows (k*_wr) keep their place where every
-            // SM has at least two rows: their prefetch then pays (1024^2:
-            // K1, K3, K5 72, 40, 123 us against 130, 102, 159), while with
-            // fewer rows most of the chip idles (1024x64: 19, 12, 25
-            // against 14, 12, 15; 512x4: 12, 10, 15 against 10, 10, 10).
-            // Everything else is faster here at every size: 64^2 fp32 31,
-            // 15, 27 -> 9, 10, 10; 384^2 fp32 74, 37, 83 -> 24, 25, 28; 64^2
-            // fp64 88, 35, 75 -> 31, 31, 30; 512^2 fp64 641, 263, 761 -> 488,
-            // 320, 614; 2048^2 fp32 716, 479, 1186 -> 590, 309, 620.
-            rowk_ = !(k1wr_ && k3wr_ && k5wr_ && (long)B_ * ny_ >= 2L * nsm_);
+            // The persistent fp32 rows (k*_wr) take over once there is a row
+            // for half of their resident blocks (1, 2, 4 rows an SM at nx =
+            // 1024, 512, 256): blocks that follow each other on an SM then
+            // overlap copies and arithmetic without a hand-over between
+            // blocks.  A step, persistent against cluster rows: 1024x128 147,
+            // 137 us; 1024x192 220, 223; 1024x256 234, 280; 1024^2 827, 1057;
+            // 512x192 142, 130; 512x256 141, 140; 512x384 199, 221; 512^2 236,
+            // 274; 256x512 161, 154; 256x768 210, 228; 256x1024 258, 290.
+            rowk_ = !(k1wr_ && k3wr_ && k5wr_ && (long)B_ * ny_ * nt_wr_host(h_) >= 256L * nsm_);
         }
         if (cs_.k && (cs_.tw == 0 || h_ % cs_.tw == 0) && cs_.smem <= budget_) {
             rowcol_ = rows_ok;
@@ -1868,8 +1871,8 @@ class EngineT : public Engine {
         return Status::ok();
     }
 
-    // the warp-resident final row kernel where it applies (fp32, nx = 512 or
-    // 1024, and its shared memory fits)
+    // the persistent fp32 row kernels where they apply (nx = 256, 512, 1024, and
+    // their shared memory fits)
     Status configure_wr() {
         if constexpr (wr_ok_) {
             const bool rows = (h_ == 512 || h_ == 256 || h_ == 128) && Tw1_;
@@ -1878,7 +1881,7 @@ class EngineT : public Engine {
             Status st;
             if (rows && k5_wr_smem(h_) <= budget_) {
                 smem5w_ = k5_wr_smem(h_);
-                st = h_ == 512 ? occupancy(k5_wr<512>, nt_k5wr_host(h_), smem5w_, &nb)
+                st = h_ == 512 ? occupancy(k5_wr<512>, NTr, smem5w_, &nb)
                    : h_ == 256 ? occupancy(k5_wr<256>, NTr, smem5w_, &nb)
                                : occupancy(k5_wr<128>, NTr, smem5w_, &nb);
                 if (!st.good()) return st;
@@ -1889,7 +1892,7 @@ class EngineT : public Engine {
             }
             if (rows && k3_wr_smem(h_) <= budget_) {
                 smem3w_ = k3_wr_smem(h_);
-                st = h_ == 512 ? occupancy(k3_wr<512>, nt_k3wr_host(h_), smem3w_, &nb)
+                st = h_ == 512 ? occupancy(k3_wr<512>, NTr, smem3w_, &nb)
                    : h_ == 256 ? occupancy(k3_wr<256>, NTr, smem3w_, &nb)
                                : occupancy(k3_wr<128>, NTr, smem3w_, &nb);
                 if (!st.good()) return st;
@@ -1900,7 +1903,7 @@ class EngineT : public Engine {
             }
             if (rows && k1_wr_smem(h_) <= budget_) {
                 smem1w_ = k1_wr_smem(h_);
-                st = h_ == 512 ? occupancy(k1_wr<512>, nt_k1wr_host(h_), smem1w_, &nb)
+                st = h_ == 512 ? occupancy(k1_wr<512>, NTr, smem1w_, &nb)
                    : h_ == 256 ? occupancy(k1_wr<256>, NTr, smem1w_, &nb)
                                : occupancy(k1_wr<128>, NTr, smem1w_, &nb);
                 if (!st.good()) return st;
@@ -2158,7 +2161,7 @@ class EngineT : public Engine {
         }
         if constexpr (wr_ok_) {
             if (!k1done && k1wr_) {
-                const int nt = nt_k1wr_host(h_);
+                const int nt = nt_wr_host(h_);
                 auto *kern = h_ == 512 ? k1_wr<512> : h_ == 256 ? k1_wr<256> : k1_wr<128>;
                 if (!(st = launch_pdl("k1_wr", kern, grid1w_, nt, smem1w_, cur, specb_, fieldsb_,
                                       (const float2 *)Tw1_, (const float2 *)Trow_, (const float *)kxt_, kp_, err_)).good())
@@ -2190,7 +2193,7 @@ class EngineT : public Engine {
         }
         if constexpr (wr_ok_) {
             if (!k3done && k3wr_) {
-                const int nt = nt_k3wr_host(h_);
+                const int nt = nt_wr_host(h_);
                 auto *kern = h_ == 512 ? k3_wr<512> : h_ == 256 ? k3_wr<256> : k3_wr<128>;
                 if (!(st = launch_pdl("k3_wr", kern, grid3w_, nt, smem3w_, specb_,
                                       (const float2 *)Tw1_, (const float2 *)Wp_, (const float2 *)Trow_, (const float *)kxt_, kp_, err_)).good())
@@ -2215,7 +2218,7 @@ class EngineT : public Engine {
         }
         if constexpr (wr_ok_) {
             if (k5wr_) {
-                const int nt = nt_k5wr_host(h_);
+                const int nt = nt_wr_host(h_);
                 auto *kern = h_ == 512 ? k5_wr<512> : h_ == 256 ? k5_wr<256> : k5_wr<128>;
                 if (!(st = launch_pdl("k5_wr", kern, grid5w_, nt, smem5w_, (const float2 *)specb_,
                                       (const float *)fieldsb_, (const float *)auxb_, cur, base, out, alpha, beta,

@@ -202,19 +202,20 @@ template <int H, typename C, typename Put>
 __device__ __forceinline__ void row_post(const C *z, const C *wh, int j, const Put &put) {
     using R = decltype(z[0].x);
     constexpr int P = Row<R, H>::P;
+    static_assert(H % (2 * P) == 0, "row configuration");
 #pragma unroll
-    for (int k0 = 0; k0 <= H / 2; k0 += P) {
+    for (int k0 = 0; k0 < H / 2; k0 += P) {
         const int k = k0 + j;
-        if (k > H / 2) break;
-        if (k == 0) {
+        if (k == 0) {   // bins 0 and H / 2
             const C z0 = z[0];
             put(0, C{z0.x + z0.y, z0.x - z0.y});
+            put(H / 2, cconj(z[H / 2]));
         } else {
             const C p = z[k], q = z[H - k];
             const C s = cadd(p, cconj(q)), d = csub(p, cconj(q));
             const C w = cmul(wh[k], cmul_mi(d));
             put(k, C{R(0.5) * s.x + w.x, R(0.5) * s.y + w.y});
-            if (H - k != k) put(H - k, C{R(0.5) * s.x - w.x, -(R(0.5) * s.y - w.y)});
+            put(H - k, C{R(0.5) * s.x - w.x, -(R(0.5) * s.y - w.y)});
         }
     }
 }
@@ -877,13 +878,16 @@ template <int H, typename C>
 __device__ __forceinline__ void row_dx(C *z, const C *wh, const C *wp, const decltype(C::x) *kx, int j) {
     using R = decltype(z[0].x);
     constexpr int P = Row<R, H>::P;
+    static_assert(H % (2 * P) == 0, "row configuration");
     const R sx = R(1.0 / (2 * H));
 #pragma unroll
-    for (int k0 = 0; k0 <= H / 2; k0 += P) {
+    for (int k0 = 0; k0 < H / 2; k0 += P) {
         const int k = k0 + j;
-        if (k > H / 2) break;
-        if (k == 0) {
+        if (k == 0) {   // bins 0 and H / 2: Y = i m conj z, Z = 2 conj Y
             z[0] = C{0, 0};
+            const C zh = z[H / 2];
+            const R m = R(2) * (kx[H / 2] * sx);
+            z[H / 2] = C{m * zh.y, -m * zh.x};
         } else {
             const C p = z[k], q = z[H - k];
             const C s = cadd(p, cconj(q)), d = csub(p, cconj(q));
@@ -895,7 +899,7 @@ __device__ __forceinline__ void row_dx(C *z, const C *wh, const C *wp, const dec
             const C a = cadd(yk, yc), e = csub(yk, yc);
             const C t = cmul_i(cmul(e, cconj(wp[k])));
             z[k] = cadd(a, t);
-            if (H - k != k) z[H - k] = cconj(csub(a, t));
+            z[H - k] = cconj(csub(a, t));
         }
     }
 }

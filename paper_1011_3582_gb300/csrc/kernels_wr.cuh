@@ -32,53 +32,15 @@ template <> struct RowCfg<512> { static constexpr int E = 16, P = 32; };
 template <> struct RowCfg<256> { static constexpr int E = 16, P = 16; };
 template <> struct RowCfg<128> { static constexpr int E = 16, P = 8; };
 
-// threads per block of the row kernels: 16 warps, or 8 for H = 128 (four
-// rows per warp: 32 row groups, one per convection row)
-// Threads of the final row kernel at H = 512: 256, i.e. two blocks per SM,
-// each with one head buffer and one-ring chunks (measured at 1024^2: 131 us
-// against 146 us for one 512-thread block with two head buffers; the
-// FFTLB_K5_NT512 build flag selects 512)
-#ifndef FFTLB_K5_NT512
-#define FFTLB_K5_NT512 256
-#endif
-template <int H> __host__ __device__ constexpr int nt_wr() { return H >= 256 ? 512 : 256; }
-inline int nt_wr_host(int H) { return H >= 256 ? 512 : 256; }
-// Threads of the forward row kernel at H = 512: 256, i.e. two blocks per
-// SM, each with 8-row chunks (measured at 1024^2: 68.7 us against 83.3 us
-// for one 512-thread block with 16-row chunks; FFTLB_K1_NT512 selects 512)
-#ifndef FFTLB_K1_NT512
-#define FFTLB_K1_NT512 256
-#endif
-template <int H> __host__ __device__ constexpr int nt_k1wr() { return H == 512 ? FFTLB_K1_NT512 : nt_wr<H>(); }
-inline int nt_k1wr_host(int H) { return H == 512 ? FFTLB_K1_NT512 : nt_wr_host(H); }
-// Threads of the level-1 row kernel at H = 512: 256 with one row buffer,
-// i.e. two blocks per SM (measured at 1024^2: 39.3 us against 46.4 us for
-// one 512-thread block with two row buffers; FFTLB_K3_NT512 selects 512)
-#ifndef FFTLB_K3_NT512
-#define FFTLB_K3_NT512 256
-#endif
-template <int H> __host__ __device__ constexpr int nt_k3wr() { return H == 512 ? FFTLB_K3_NT512 : nt_wr<H>(); }
-inline int nt_k3wr_host(int H) { return H == 512 ? FFTLB_K3_NT512 : nt_wr_host(H); }
-template <int H> __host__ __device__ constexpr int nb_k3wr() { return nt_k3wr<H>() == 512 || H < 256 ? 2 : 1; }
-inline int nb_k3wr_host(int H) { return nt_k3wr_host(H) == 512 || H < 256 ? 2 : 1; }
-template <int H> __host__ __device__ constexpr int nt_k5wr() { return H == 512 ? FFTLB_K5_NT512 : nt_wr<H>(); }
-inline int nt_k5wr_host(int H) { return H == 512 ? FFTLB_K5_NT512 : nt_wr_host(H); }
-// head buffers of the final row kernel: two (the next row's head fetched a
-// row ahead) unless its blocks are half size
-template <int H> __host__ __device__ constexpr int nhb_k5wr() { return nt_k5wr<H>() == 512 || H < 256 ? 2 : 1; }
-// sites per unrolled pass of the final row kernel's epilogue (the loads of
-// the next site's distributions issue before the current site's arithmetic;
-// measured at 1024^2: 132.2 us with 1, 131.1 with 2, 130.5 with 4)
-#ifndef FFTLB_K5_UNROLL
-#define FFTLB_K5_UNROLL 4
-#endif
-constexpr int K5U = FFTLB_K5_UNROLL;
-// FFTLB_K5_VEC > 0: the epilogue with four consecutive sites per thread
-// (where nx is four times the block size) and 16-byte accesses (measured at
-// 1024^2: 130.9 us scalar, 126.7 us with 1, 131.9 us with 2)
-#ifndef FFTLB_K5_VEC
-#define FFTLB_K5_VEC 1
-#endif
+// Threads per block: 4 sites of a row each, i.e. 8 row groups and chunks of one
+// ring of velocities at every length, and as many blocks on an SM as 128
+// registers a thread allow.  Few large blocks with more rows in a chunk wait for
+// their own copies and barriers: 512 threads a block at nx = 512 and 256 at nx =
+// 256 took K1, K3, K5 27, 23, 47 us on 512^2 (here 23, 16, 32) and 45, 35, 77 on
+// 256x2048 (45, 29, 59); 512 threads at nx = 1024 83, 46, 146 on 1024^2 (61, 40,
+// 104).
+template <int H> __host__ __device__ constexpr int nt_wr() { return H / 2; }
+inline int nt_wr_host(int H) { return H / 2; }
 
 // position of stage-1 output (l, k1) in the row buffer.  P >= 16: k1 P +
 // (l ^ (k1 mod P)) (for P = 2E, k1 < E: k1 P + (l ^ k1)); P = 8: the row
@@ -178,23 +140,23 @@ __device__ __forceinline__ void row_fft_wr(C *z, const C *tw, int j, int rsw) {
 // half-length transform of the packed row) -> one-sided spectrum X[0 .. H-1]
 // with the real Nyquist value in the imaginary part of X[0], written to
 // out (global memory, coalesced: lanes take consecutive k and H - k).
-// Wh[k] = exp(-2 pi i k / 2H) / 2, k <= H / 2.
+// Wh[k] = exp(-2 pi i k / 2H) / 2, k < H / 2.
 template <int H, typename C>
 __device__ __forceinline__ void r2c_post_wr(const C *z, C *out, const C *Wh, int j) {
     using R = decltype(z[0].x);
     constexpr int P = RowCfg<H>::P;
 #pragma unroll
-    for (int k0 = 0; k0 <= H / 2; k0 += P) {
+    for (int k0 = 0; k0 < H / 2; k0 += P) {
         const int k = k0 + j;
-        if (k > H / 2) break;
         if (k == 0) {
             const C z0 = z[0];
             out[0] = C{z0.x + z0.y, z0.x - z0.y};
+            out[H / 2] = cconj(z[H / 2]);
         } else {
             const C p = z[k], q = z[H - k];
             const C s = cadd(p, cconj(q)), w = cmul(Wh[k], cmul_mi(csub(p, cconj(q))));
             out[k] = C{R(0.5) * s.x + w.x, R(0.5) * s.y + w.y};
-            if (H - k != k) out[H - k] = C{R(0.5) * s.x - w.x, w.y - R(0.5) * s.y};
+            out[H - k] = C{R(0.5) * s.x - w.x, w.y - R(0.5) * s.y};
         }
     }
 }
@@ -207,16 +169,16 @@ __device__ __forceinline__ void r2c_post_dx(const C *z, C *dst, const float *__r
     using R = decltype(z[0].x);
     constexpr int P = RowCfg<H>::P;
 #pragma unroll
-    for (int k0 = 0; k0 <= H / 2; k0 += P) {
+    for (int k0 = 0; k0 < H / 2; k0 += P) {
         const int k = k0 + j;
-        if (k > H / 2) break;
         if (k == 0) {
             dst[0] = C{0, 0};
+            dst[H / 2] = imul(kxt[H / 2] * sx, cconj(z[H / 2]));
         } else {
             const C p = z[k], q = z[H - k];
             const C s = cadd(p, cconj(q)), w = cmul(Wh[k], cmul_mi(csub(p, cconj(q))));
             dst[k] = imul(kxt[k] * sx, C{R(0.5) * s.x + w.x, R(0.5) * s.y + w.y});
-            if (H - k != k) dst[H - k] = imul(kxt[H - k] * sx, C{R(0.5) * s.x - w.x, w.y - R(0.5) * s.y});
+            dst[H - k] = imul(kxt[H - k] * sx, C{R(0.5) * s.x - w.x, w.y - R(0.5) * s.y});
         }
     }
 }
@@ -226,21 +188,23 @@ __device__ __forceinline__ void r2c_post_dx(const C *z, C *dst, const float *__r
 // conj X[H - k]; the half-length inverse of Z is the real row.
 template <int H, typename C>
 __device__ __forceinline__ void c2r_pre_wr(C *z, const C *Wp, int j) {
+    using R = decltype(z[0].x);
     constexpr int P = RowCfg<H>::P;
 #pragma unroll
-    for (int k0 = 0; k0 <= H / 2; k0 += P) {
+    for (int k0 = 0; k0 < H / 2; k0 += P) {
         const int k = k0 + j;
-        if (k > H / 2) break;
         if (k == 0) {
             const C x0 = z[0];
             z[0] = C{x0.x + x0.y, x0.x - x0.y};
+            const C xh = z[H / 2];   // Z = 2 conj X
+            z[H / 2] = C{R(2) * xh.x, R(-2) * xh.y};
         } else {
             // with a = p + conj q, e = i (p - conj q) conj w: Z[k] = a + e,
             // Z[H - k] = conj(a - e)
             const C p = z[k], q = z[H - k];
             const C a = cadd(p, cconj(q)), e = cmul_i(cmul(csub(p, cconj(q)), cconj(Wp[k])));
             z[k] = cadd(a, e);
-            if (H - k != k) z[H - k] = cconj(csub(a, e));
+            z[H - k] = cconj(csub(a, e));
         }
     }
 }
@@ -298,16 +262,16 @@ __device__ __forceinline__ void k1w_issue(const float *f, float *dst, uint64_t *
 }
 
 template <int H>
-__global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_wr(const float *__restrict__ f, float2 *spec, float *__restrict__ fields,
+__global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k1_wr(const float *__restrict__ f, float2 *spec, float *__restrict__ fields,
                                                  const float2 *__restrict__ tw_g, const float2 *__restrict__ Wh_g,
                                                  const float *__restrict__ kxt, KP<float> P, int *err) {
     using C = float2;
     using real = float;
-    constexpr int NX = 2 * H, NT = nt_k1wr<H>(), NWARP = NT / 32;
+    constexpr int NX = 2 * H, NT = nt_wr<H>(), NWARP = NT / 32;
     constexpr int PL = RowCfg<H>::P, RPW = 32 / PL;
     constexpr int NG = NWARP * RPW;                // row groups per block
     constexpr int CH = NG + 1, NCH = NMOV / NG;    // rows per chunk buffer, chunks per row
-    constexpr int SMAX = (NX + NT - 1) / NT;
+    constexpr int SMAX = NX / NT;
     static_assert(NMOV % NG == 0 && NG % 8 == 0, "chunking");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar0, bar1;
@@ -317,7 +281,7 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
     const size_t N = (size_t)NX * ny, slot = (size_t)ny * H;
     SmemCursor sc{smem_raw, 0u};
     C *tw = (C *)sc.take(H * sizeof(C));
-    C *Wh = (C *)sc.take((H / 2 + 1) * sizeof(C));
+    C *Wh = (C *)sc.take(H / 2 * sizeof(C));
     real *kxs = (real *)sc.take(H * sizeof(real));   // k_x of the row bins
     real *buf0 = (real *)sc.take((size_t)CH * NX * sizeof(real));
     real *buf1 = (real *)sc.take((size_t)CH * NX * sizeof(real));
@@ -334,7 +298,7 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
         if (njobs > 1) k1w_issue(f, buf1, &bar1, 1, NCH, NG, nx, ny, N);
     }
     load_tab4(tw, tw_g, H, NT);
-    load_tab4(Wh, Wh_g, H / 2 + 1, NT);
+    load_tab4(Wh, Wh_g, H / 2, NT);
     load_tab4(kxs, kxt, H, NT);
     grid_dep_wait();
     __syncthreads();
@@ -449,8 +413,8 @@ __global__ void __launch_bounds__(nt_k1wr<H>(), nt_k1wr<H>() >= 512 ? 1 : 2) k1_
 // shared memory of k1_wr<H>
 inline size_t k1_wr_smem(int H) {
     const int P = H == 512 ? 32 : H == 256 ? 16 : 8;
-    const int CH = (nt_k1wr_host(H) / 32) * (32 / P) + 1;
-    return smem_bytes({(size_t)H * 8, (size_t)(H / 2 + 1) * 8, (size_t)H * 4, (size_t)CH * 2 * H * 4,
+    const int CH = nt_wr_host(H) / P + 1;
+    return smem_bytes({(size_t)H * 8, (size_t)H / 2 * 8, (size_t)H * 4, (size_t)CH * 2 * H * 4,
                        (size_t)CH * 2 * H * 4, (size_t)6 * 2 * H * 4});
 }
 
@@ -459,8 +423,8 @@ inline size_t k1_wr_smem(int H) {
 // factor k_x or start from a row spectrum (stage_layout.cuh) -> Lambda (Eq. 19),
 // Phi (Eq. 23), the numerators of C (Eq. 22) and B (Eq. 21) -> d_x of Lambda_xx,
 // Lambda_xy, Phi_x (a forward and an inverse row each) added to the numerators.
-// Persistent over the rows of all runs, one row per pass, one or two buffers
-// (11 transformed rows and 8 real ones).
+// Persistent over the rows of all runs, one row per pass and one buffer (11
+// transformed rows and 8 real ones); the other blocks of the SM cover the copy.
 // ---------------------------------------------------------------------------
 
 template <typename C>
@@ -475,66 +439,50 @@ __device__ __forceinline__ void k3_issue(const C *spec, C *dst, uint64_t *bar, i
 }
 
 template <int H>
-__global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_wr(float2 *spec, const float2 *__restrict__ tw_g,
+__global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k3_wr(float2 *spec, const float2 *__restrict__ tw_g,
                                                  const float2 *__restrict__ Wp_g, const float2 *__restrict__ Wh_g,
                                                  const float *__restrict__ kxt,
                                                  KP<float> P, int *err) {
     using C = float2;
     using real = float;
-    constexpr int NX = 2 * H, NT = nt_k3wr<H>(), NB = nb_k3wr<H>();
+    constexpr int NX = 2 * H, NT = nt_wr<H>();
     constexpr int PL = RowCfg<H>::P, RPW = 32 / PL, NG = (NT / 32) * RPW;   // row groups
-    constexpr int SMAX = (NX + NT - 1) / NT;
+    constexpr int SMAX = NX / NT;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bar0, bar1;
+    __shared__ __align__(8) uint64_t bar;
     const int ny = P.ny, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int grp = warp * RPW + lane / PL, j = lane & (PL - 1);
     const int rsw = PL == 8 ? ((lane / PL) & 1) : 0;
     const size_t slot = (size_t)ny * H;
     SmemCursor sc{smem_raw, 0u};
     C *tw = (C *)sc.take(H * sizeof(C));
-    C *Wp = (C *)sc.take((H / 2 + 1) * sizeof(C));
-    C *Wh = (C *)sc.take((H / 2 + 1) * sizeof(C));
+    C *Wp = (C *)sc.take(H / 2 * sizeof(C));
+    C *Wh = (C *)sc.take(H / 2 * sizeof(C));
     real *kxs = (real *)sc.take(H * sizeof(real));   // k_x of the row bins
-    C *buf0 = (C *)sc.take((size_t)NK3 * H * sizeof(C));
-    C *buf1 = NB > 1 ? (C *)sc.take((size_t)NK3 * H * sizeof(C)) : buf0;
+    C *dc = (C *)sc.take((size_t)NK3 * H * sizeof(C));
+    real *d = reinterpret_cast<real *>(dc);
     const int NY = P.nrun * ny;
     const int nrows = (int)blockIdx.x < NY ? (NY - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     if (tid == 0) {   // (the first copies start before the tables load)
-        mbar_init(&bar0, 1);
-        mbar_init(&bar1, 1);
+        mbar_init(&bar, 1);
         mbar_init_fence();
         grid_dep_wait();
-        if (nrows > 0) k3_issue(spec, buf0, &bar0, 0, ny, slot, H);
-        if (NB > 1 && nrows > 1) k3_issue(spec, buf1, &bar1, 1, ny, slot, H);
+        if (nrows > 0) k3_issue(spec, dc, &bar, 0, ny, slot, H);
     }
     load_tab4(tw, tw_g, H, NT);
-    load_tab4(Wp, Wp_g, H / 2 + 1, NT);
-    load_tab4(Wh, Wh_g, H / 2 + 1, NT);
+    load_tab4(Wp, Wp_g, H / 2, NT);
+    load_tab4(Wh, Wh_g, H / 2, NT);
     load_tab4(kxs, kxt, H, NT);
     grid_dep_wait();
     __syncthreads();
-    uint32_t par0 = 0, par1 = 0;
-    bool pend0 = nrows > 0, pend1 = NB > 1 && nrows > 1;
     for (int ri = 0; ri < nrows; ++ri) {
-        const bool odd = NB > 1 && (ri & 1);
-        uint64_t *bar = odd ? &bar1 : &bar0;
         const int yg = (int)blockIdx.x + ri * (int)gridDim.x;
         const int run = yg / ny, y = yg - run * ny;
         C *spec_r = spec + (size_t)run * NSLOT * slot + (size_t)y * H;
-        if (!block_wait(bar, odd ? par1 : par0, err)) {
-            if (pend0) mbar_wait_bounded(&bar0, par0);
-            if (pend1) mbar_wait_bounded(&bar1, par1);
+        if (!block_wait(&bar, ri & 1, err)) {
+            mbar_wait_bounded(&bar, ri & 1);
             return;
         }
-        if (odd) {
-            par1 ^= 1;
-            pend1 = false;
-        } else {
-            par0 ^= 1;
-            pend0 = false;
-        }
-        C *dc = odd ? buf1 : buf0;
-        real *d = reinterpret_cast<real *>(dc);
         for (int k = tid; k < H; k += NT) k3_form_x<real>(dc, H, k, kxs[k], P.scale_x);
         __syncthreads();
         for (int r = grp; r < NSP; r += NG) {   // (uniform over each row group)
@@ -579,18 +527,13 @@ __global__ void __launch_bounds__(nt_k3wr<H>(), nt_k3wr<H>() >= 512 ? 1 : 2) k3_
         }
         fence_proxy_async();
         __syncthreads();
-        if (tid == 0 && ri + NB < nrows) {   // row ri + NB reuses this buffer
-            k3_issue(spec, dc, bar, ri + NB, ny, slot, H);
-            if (odd) pend1 = true;
-            else pend0 = true;
-        }
+        if (tid == 0 && ri + 1 < nrows) k3_issue(spec, dc, &bar, ri + 1, ny, slot, H);
     }
 }
 
 // shared memory of k3_wr<H>
 inline size_t k3_wr_smem(int H) {
-    return smem_bytes({(size_t)H * 8, (size_t)(H / 2 + 1) * 8, (size_t)(H / 2 + 1) * 8, (size_t)H * 4, (size_t)NK3 * 2 * H * 4,
-                       nb_k3wr_host(H) > 1 ? (size_t)NK3 * 2 * H * 4 : 0});
+    return smem_bytes({(size_t)H * 8, (size_t)H / 2 * 8, (size_t)H / 2 * 8, (size_t)H * 4, (size_t)NK3 * 2 * H * 4});
 }
 
 // ---------------------------------------------------------------------------
@@ -598,37 +541,32 @@ inline size_t k3_wr_smem(int H) {
 // A, B, C, C_q (Eqs. 20-23), f^eq (Eq. 3), I (Eq. 11), BGK and the RK
 // combination (Eq. 10), as k5_pipe, with warp-resident row transforms.
 // Persistent over the rows of all runs; per row: the head (3 level-2
-// spectra, rho, u_x, u_y, T, the 3 aux numerators; two buffers, prefetched
-// a row ahead) and 32 / CH chunks of CH convection rows (two buffers), each
-// chunk one row per row group (CH = 16 warps x rows per warp: two rings for
-// H = 512, all four for H = 256).
+// spectra, rho, u_x, u_y, T, the 3 aux numerators) and 4 chunks of 8 convection
+// rows, one ring each (two buffers), one row per row group.
 // ---------------------------------------------------------------------------
 
 template <int H>
-__global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_wr(const float2 *spec, const float *__restrict__ fields,
+__global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k5_wr(const float2 *spec, const float *__restrict__ fields,
                                                  const float *__restrict__ aux, const float *fcur, const float *fbase,
                                                  float *fout, float alpha, float beta,
                                                  const float2 *__restrict__ tw_g, const float2 *__restrict__ Wp_g,
                                                  KP<float> P, int *err) {
     using C = float2;
     using real = float;
-    constexpr int NX = 2 * H, NT = nt_k5wr<H>(), NWARP = NT / 32, NHB = nhb_k5wr<H>();
+    constexpr int NX = 2 * H, NT = nt_wr<H>();
     constexpr int PL = RowCfg<H>::P, RPW = 32 / PL;          // lanes per row, rows per warp
-    constexpr int CH = NWARP * RPW, NCH = NMOV / CH;           // rows per chunk, chunks per row
-    constexpr int NRING = CH / 8;                              // rings per chunk
-    constexpr int SMAX = (NX + NT - 1) / NT;
-    static_assert(NMOV % CH == 0 && CH % 8 == 0, "chunking");
+    constexpr int CH = 8, NCH = NMOV / CH;                     // rows (one ring) per chunk, chunks per row
+    static_assert(NX == 4 * NT && NT == CH * PL, "four sites a thread, one row a group");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bar0, bar1, hbar0, hbar1;
+    __shared__ __align__(8) uint64_t bar0, bar1, hbar;
     const int nx = NX, ny = P.ny, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int grow = warp * RPW + lane / PL, j = lane & (PL - 1);   // row within the chunk, lane within the row
     const int rsw = PL == 8 ? ((lane / PL) & 1) : 0;
     const size_t N = (size_t)NX * ny, slot = (size_t)ny * H;
     SmemCursor sc{smem_raw, 0u};
     C *tw = (C *)sc.take(H * sizeof(C));
-    C *Wp = (C *)sc.take((H / 2 + 1) * sizeof(C));
-    real *head0 = (real *)sc.take((size_t)NHEAD * NX * sizeof(real));
-    real *head1 = NHB > 1 ? (real *)sc.take((size_t)NHEAD * NX * sizeof(real)) : head0;
+    C *Wp = (C *)sc.take(H / 2 * sizeof(C));
+    real *Hd = (real *)sc.take((size_t)NHEAD * NX * sizeof(real));
     real *buf0 = (real *)sc.take((size_t)CH * NX * sizeof(real));
     real *buf1 = (real *)sc.take((size_t)CH * NX * sizeof(real));
     const int NY = P.nrun * ny;
@@ -637,8 +575,7 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
     if (tid == 0) {   // (the first copies start before the tables load)
         mbar_init(&bar0, 1);
         mbar_init(&bar1, 1);
-        mbar_init(&hbar0, 1);
-        mbar_init(&hbar1, 1);
+        mbar_init(&hbar, 1);
         mbar_init_fence();
         // Only the head's level-2 rows come from the launch just before this
         // one (the level-2 columns); the convection spectra, fields, aux rows
@@ -648,29 +585,25 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
         if (njobs > 0) k5_issue_chunk<real>(spec, buf0, &bar0, 0, NCH, CH, nx, ny, slot, H);
         if (njobs > 1) k5_issue_chunk<real>(spec, buf1, &bar1, 1, NCH, CH, nx, ny, slot, H);
         grid_dep_wait();
-        if (nrows > 0) k5_issue_head<real>(spec, fields, aux, head0, &hbar0, 0, nx, ny, N, slot, H);
-        if (NHB > 1 && nrows > 1) k5_issue_head<real>(spec, fields, aux, head1, &hbar1, 1, nx, ny, N, slot, H);
+        if (nrows > 0) k5_issue_head<real>(spec, fields, aux, Hd, &hbar, 0, nx, ny, N, slot, H);
     }
     load_tab4(tw, tw_g, H, NT);
-    load_tab4(Wp, Wp_g, H / 2 + 1, NT);
+    load_tab4(Wp, Wp_g, H / 2, NT);
     __syncthreads();
-    uint32_t par0 = 0, par1 = 0, hpar0 = 0, hpar1 = 0;
-    bool pend0 = njobs > 0, pend1 = njobs > 1, hpend0 = nrows > 0, hpend1 = NHB > 1 && nrows > 1;
+    uint32_t par0 = 0, par1 = 0;
+    bool pend0 = njobs > 0, pend1 = njobs > 1, hpend = nrows > 0;
     const real dt = P.dt, itau = real(1) / P.tau;
     const bool with_base = alpha != real(0);
     for (int jb = 0; jb < njobs; ++jb) {
         const bool odd = jb & 1;
         const int ri = jb / NCH, c = jb - ri * NCH;
-        const bool hodd = NHB > 1 && (ri & 1);
         const int yg = (int)blockIdx.x + ri * (int)gridDim.x;
         const int run = yg / ny, y = yg - run * ny;
         const size_t fo = (size_t)run * Q * N;
-        real *Hd = hodd ? head1 : head0;
         if (!block_wait(odd ? &bar1 : &bar0, odd ? par1 : par0, err)) {
             if (pend0) mbar_wait_bounded(&bar0, par0);
             if (pend1) mbar_wait_bounded(&bar1, par1);
-            if (hpend0) mbar_wait_bounded(&hbar0, hpar0);
-            if (hpend1) mbar_wait_bounded(&hbar1, hpar1);
+            if (hpend) mbar_wait_bounded(&hbar, ri & 1);
             return;
         }
         if (odd) {
@@ -692,20 +625,13 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
                 row_fft_wr<H, +1>(zr, tw, j, rsw);
             }
             if (c == 0) {
-                if (!block_wait(hodd ? &hbar1 : &hbar0, hodd ? hpar1 : hpar0, err)) {
+                if (!block_wait(&hbar, ri & 1, err)) {
                     if (pend0) mbar_wait_bounded(&bar0, par0);
                     if (pend1) mbar_wait_bounded(&bar1, par1);
-                    if (hpend0) mbar_wait_bounded(&hbar0, hpar0);
-                    if (hpend1) mbar_wait_bounded(&hbar1, hpar1);
+                    mbar_wait_bounded(&hbar, ri & 1);
                     return;
                 }
-                if (hodd) {
-                    hpar1 ^= 1;
-                    hpend1 = false;
-                } else {
-                    hpar0 ^= 1;
-                    hpend0 = false;
-                }
+                hpend = false;
             }
         }
         __syncthreads();
@@ -713,194 +639,124 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
             // per-site coefficients over the head rows (same site, same
             // thread): row 0 <- e0, 1 <- e1x, 2 <- e1y, 7 <- C + C_q, 8 <- 1/T;
             // the rest velocity's update
-            if constexpr (NX == 4 * NT && FFTLB_K5_VEC > 0) {   // four consecutive sites per thread
-                const int x0 = 4 * tid;
-                const size_t o = fo + (size_t)y * nx + x0;
-                real rho[4], ux[4], uy[4], T[4], dLx[4], dLy[4], dPh[4], a7[4], a8[4], a9[4], fc[4], fb[4];
-                ld4(rho, Hd + 3 * nx + x0);
-                ld4(ux, Hd + 4 * nx + x0);
-                ld4(uy, Hd + 5 * nx + x0);
-                ld4(T, Hd + 6 * nx + x0);
-                ld4(dLx, Hd + x0);
-                ld4(dLy, Hd + nx + x0);
-                ld4(dPh, Hd + 2 * nx + x0);
-                ld4(a7, Hd + 7 * nx + x0);
-                ld4(a8, Hd + 8 * nx + x0);
-                ld4(a9, Hd + 9 * nx + x0);
-                ld4(fc, fcur + o);
-                if (with_base) ld4(fb, fbase + o);
-                real e0[4], e1x[4], e1y[4], CC[4], iT[4], fn[4];
+            const int x0 = 4 * tid;
+            const size_t o = fo + (size_t)y * nx + x0;
+            real rho[4], ux[4], uy[4], T[4], dLx[4], dLy[4], dPh[4], a7[4], a8[4], a9[4], fc[4], fb[4];
+            ld4(rho, Hd + 3 * nx + x0);
+            ld4(ux, Hd + 4 * nx + x0);
+            ld4(uy, Hd + 5 * nx + x0);
+            ld4(T, Hd + 6 * nx + x0);
+            ld4(dLx, Hd + x0);
+            ld4(dLy, Hd + nx + x0);
+            ld4(dPh, Hd + 2 * nx + x0);
+            ld4(a7, Hd + 7 * nx + x0);
+            ld4(a8, Hd + 8 * nx + x0);
+            ld4(a9, Hd + 9 * nx + x0);
+            ld4(fc, fcur + o);
+            if (with_base) ld4(fb, fbase + o);
+            real e0[4], e1x[4], e1y[4], CC[4], iT[4], fn[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const real rT = rho[q] * T[q];
-                    const real inv2 = real(1) / (real(2) * rho[q] * T[q] * T[q]);
-                    const real Bx = (a8[q] + dLx[q]) / rT;      // Eq. 21
-                    const real By = (a9[q] + dLy[q]) / rT;
-                    CC[q] = (a7[q] + dPh[q]) * inv2;            // C + C_q, Eqs. 22-23
-                    const real A = real(-2) * CC[q] * T[q];      // Eq. 20
-                    const real u2 = ux[q] * ux[q] + uy[q] * uy[q];
-                    e0[q] = A - (Bx * ux[q] + By * uy[q]) + CC[q] * u2;
-                    e1x[q] = Bx - real(2) * CC[q] * ux[q];
-                    e1y[q] = By - real(2) * CC[q] * uy[q];
-                    iT[q] = real(1) / T[q];
-                    real F[5];
-                    weights_Fk<real>(T[q], F);
-                    const real qq = real(0.5) * u2 / T[q], om = real(1) - qq;
-                    const real fe = rho[q] * F[0] * (om + real(0.5) * qq * qq);
-                    fn[q] = rk_combine(with_base, beta, dt, fc[q], fb[q], -(fc[q] - fe) * itau - e0[q] * fe);
-                }
-                st4(Hd + x0, e0);
-                st4(Hd + nx + x0, e1x);
-                st4(Hd + 2 * nx + x0, e1y);
-                st4(Hd + 7 * nx + x0, CC);
-                st4(Hd + 8 * nx + x0, iT);
-                st4(fout + o, fn);
-            } else
-#pragma unroll 1
-            for (int s = 0; s < SMAX; ++s) {
-                const int x = tid + s * NT;
-                if (x < nx) {
-                    const real rho = Hd[3 * nx + x], ux = Hd[4 * nx + x], uy = Hd[5 * nx + x], T = Hd[6 * nx + x];
-                    const real dLx = Hd[x], dLy = Hd[nx + x], dPh = Hd[2 * nx + x];
-                    const real rT = rho * T;
-                    const real inv2 = real(1) / (real(2) * rho * T * T);
-                    const real Bx = (Hd[8 * nx + x] + dLx) / rT;      // Eq. 21
-                    const real By = (Hd[9 * nx + x] + dLy) / rT;
-                    const real CC = (Hd[7 * nx + x] + dPh) * inv2;    // C + C_q, Eqs. 22-23
-                    const real A = real(-2) * CC * T;                 // Eq. 20
-                    const real u2 = ux * ux + uy * uy;
-                    const real e0 = A - (Bx * ux + By * uy) + CC * u2;
-                    Hd[x] = e0;
-                    Hd[nx + x] = Bx - real(2) * CC * ux;
-                    Hd[2 * nx + x] = By - real(2) * CC * uy;
-                    Hd[7 * nx + x] = CC;
-                    Hd[8 * nx + x] = real(1) / T;
-                    real F[5];
-                    weights_Fk<real>(T, F);
-                    const real qq = real(0.5) * u2 / T, om = real(1) - qq;
-                    const real fe = rho * F[0] * (om + real(0.5) * qq * qq);
-                    const size_t o = fo + (size_t)y * nx + x;
-                    const real fc = fcur[o];
-                    fout[o] = rk_combine(with_base, beta, dt, fc, with_base ? fbase[o] : real(0), -(fc - fe) * itau - e0 * fe);
-                }
+            for (int q = 0; q < 4; ++q) {
+                const real rT = rho[q] * T[q];
+                const real inv2 = real(1) / (real(2) * rho[q] * T[q] * T[q]);
+                const real Bx = (a8[q] + dLx[q]) / rT;      // Eq. 21
+                const real By = (a9[q] + dLy[q]) / rT;
+                CC[q] = (a7[q] + dPh[q]) * inv2;            // C + C_q, Eqs. 22-23
+                const real A = real(-2) * CC[q] * T[q];      // Eq. 20
+                const real u2 = ux[q] * ux[q] + uy[q] * uy[q];
+                e0[q] = A - (Bx * ux[q] + By * uy[q]) + CC[q] * u2;
+                e1x[q] = Bx - real(2) * CC[q] * ux[q];
+                e1y[q] = By - real(2) * CC[q] * uy[q];
+                iT[q] = real(1) / T[q];
+                real F[5];
+                weights_Fk<real>(T[q], F);
+                const real qq = real(0.5) * u2 / T[q], om = real(1) - qq;
+                const real fe = rho[q] * F[0] * (om + real(0.5) * qq * qq);
+                fn[q] = rk_combine(with_base, beta, dt, fc[q], fb[q], -(fc[q] - fe) * itau - e0[q] * fe);
             }
+            st4(Hd + x0, e0);
+            st4(Hd + nx + x0, e1x);
+            st4(Hd + 2 * nx + x0, e1y);
+            st4(Hd + 7 * nx + x0, CC);
+            st4(Hd + 8 * nx + x0, iT);
+            st4(fout + o, fn);
             __syncthreads();
         }
-        // epilogue: the NRING rings of the chunk (ring k = c NRING + rr:
-        // velocities 1 + 8k .. 8 + 8k of Eq. 1, one speed, one weight, the
-        // eight directions known at compile time)
-#pragma unroll 1
-        for (int rr = 0; rr < NRING; ++rr) {
-            const int k = c * NRING + rr;
-            const int v0 = 8 * k;
+        // epilogue: ring c (velocities 1 + 8c .. 8 + 8c of Eq. 1, one speed, one
+        // weight, the eight directions known at compile time), four consecutive
+        // sites per thread: 16-byte loads and stores (1024^2: 126.7 us against
+        // 130.9 site by site)
+        {
+            const int v0 = 8 * c;
             const real sk = VX<real>(1 + v0), sk2 = V2<real>(1 + v0);
-            const real *cres = B + (size_t)rr * 8 * NX;
-            if constexpr (NX == 4 * NT && FFTLB_K5_VEC > 0) {
-                // four consecutive sites per thread: 16-byte loads and stores
-                const int x0 = 4 * tid;
-                const size_t o0 = fo + (size_t)(1 + v0) * N + (size_t)y * nx + x0;
-                real rho[4], ux[4], uy[4], T[4], iT[4], e0[4], e1x[4], e1y[4], CC[4];
-                ld4(rho, Hd + 3 * nx + x0);
-                ld4(ux, Hd + 4 * nx + x0);
-                ld4(uy, Hd + 5 * nx + x0);
-                ld4(T, Hd + 6 * nx + x0);
-                ld4(iT, Hd + 8 * nx + x0);
-                ld4(e0, Hd + x0);
-                ld4(e1x, Hd + nx + x0);
-                ld4(e1y, Hd + 2 * nx + x0);
-                ld4(CC, Hd + 7 * nx + x0);
-                real p0[4], p1[4], p2[4], p3[4], p4[4], h0[4], uxk[4], uyk[4], exk[4], eyk[4];
+            const real *cres = B;
+            const int x0 = 4 * tid;
+            const size_t o0 = fo + (size_t)(1 + v0) * N + (size_t)y * nx + x0;
+            real rho[4], ux[4], uy[4], T[4], iT[4], e0[4], e1x[4], e1y[4], CC[4];
+            ld4(rho, Hd + 3 * nx + x0);
+            ld4(ux, Hd + 4 * nx + x0);
+            ld4(uy, Hd + 5 * nx + x0);
+            ld4(T, Hd + 6 * nx + x0);
+            ld4(iT, Hd + 8 * nx + x0);
+            ld4(e0, Hd + x0);
+            ld4(e1x, Hd + nx + x0);
+            ld4(e1y, Hd + 2 * nx + x0);
+            ld4(CC, Hd + 7 * nx + x0);
+            real p0[4], p1[4], p2[4], p3[4], p4[4], h0[4], uxk[4], uyk[4], exk[4], eyk[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const real qq = real(0.5) * (ux[q] * ux[q] + uy[q] * uy[q]) * iT[q], om = real(1) - qq;
-                    const real rF = rho[q] * weight_Fk<real>(k, T[q]);   // Eq. 4
-                    const real r1 = rF * iT[q], r2 = r1 * iT[q], r3 = r2 * iT[q];
-                    p0[q] = rF * (om + real(0.5) * qq * qq);   // rho F_k times the factors of Eq. 3
-                    p1[q] = r1 * om;
-                    p2[q] = real(0.5) * r2 * om;
-                    p3[q] = r3 * (real(1) / real(6));
-                    p4[q] = r3 * iT[q] * (real(1) / real(24));
-                    h0[q] = itau - (e0[q] + CC[q] * sk2);
-                    uxk[q] = sk * ux[q];
-                    uyk[q] = sk * uy[q];
-                    exk[q] = sk * e1x[q];
-                    eyk[q] = sk * e1y[q];
-                }
-                // directions r and r + 4 together: f^eq = even +- odd in v.u;
-                // rhs = (1 / tau - g) f^eq - f / tau - convection with g = -I /
-                // f^eq (Eqs. 10, 11).  The distributions of two such pairs are
-                // loaded before any of their stores, as fout may alias fcur or
-                // fbase.
-                const real *__restrict__ pc = fcur + o0;
-                const real *__restrict__ pb = fbase + o0;
-                real *__restrict__ po = fout + o0;
-#pragma unroll
-                for (int r0 = 0; r0 < 4; r0 += 2) {
-                    real fc[4][4], fb[4][4];
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const int d = r0 + (r >> 1) + 4 * (r & 1);
-                        ld4(fc[r], pc + (size_t)d * N);
-                        if (with_base) ld4_once(fb[r], pb + (size_t)d * N);
-                    }
-#pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        real cv[2][4], fn[2][4];
-                        ld4(cv[0], cres + (size_t)(r0 + r) * NX + x0);
-                        ld4(cv[1], cres + (size_t)(r0 + r + 4) * NX + x0);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const real vu = dir_dot<real>(r0 + r, uxk[q], uyk[q]), w2 = vu * vu;
-                            const real ev = p0[q] + w2 * (p2[q] + w2 * p4[q]), od = vu * (p1[q] + w2 * p3[q]);   // Eq. 3
-                            const real ed = dir_dot<real>(r0 + r, exk[q], eyk[q]);
-#pragma unroll
-                            for (int s = 0; s < 2; ++s) {
-                                const real fe = s ? ev - od : ev + od, hd = s ? h0[q] + ed : h0[q] - ed;
-                                const real f = fc[2 * r + s][q];
-                                const real rhs = hd * fe - cv[s][q] - f * itau;
-                                fn[s][q] = rk_combine(with_base, beta, dt, f, fb[2 * r + s][q], rhs);
-                            }
-                        }
-                        st4_once(po + (size_t)(r0 + r) * N, fn[0]);
-                        st4_once(po + (size_t)(r0 + r + 4) * N, fn[1]);
-                    }
-                }
-            } else {
-#pragma unroll(K5U)
-            for (int s = 0; s < SMAX; ++s) {
-                const int x = tid + s * NT;
-                if (x >= nx) continue;
-                real fc[8], fb[8];
-                const size_t o0 = fo + (size_t)(1 + v0) * N + (size_t)y * nx + x;
-                const real *pc = fcur + o0;
-                const real *pb = fbase + o0;
-#pragma unroll
-                for (int r = 0; r < 8; ++r) {
-                    fc[r] = pc[r * N];
-                    fb[r] = with_base ? pb[r * N] : real(0);
-                }
-                real *po = fout + o0;
-                const real rho = Hd[3 * nx + x], ux = Hd[4 * nx + x], uy = Hd[5 * nx + x], T = Hd[6 * nx + x];
-                const real iT = Hd[8 * nx + x];
-                const real e0 = Hd[x], e1x = Hd[nx + x], e1y = Hd[2 * nx + x], CC = Hd[7 * nx + x];
-                const real Fk = weight_Fk<real>(k, T);   // Eq. 4
-                const real qq = real(0.5) * (ux * ux + uy * uy) * iT, om = real(1) - qq;
-                const real p0 = om + real(0.5) * qq * qq, p1 = om * iT, p2 = real(0.5) * om * iT * iT;
-                const real p3 = iT * iT * iT * (real(1) / real(6)), p4 = iT * iT * iT * iT * (real(1) / real(24));
-                const real rF = rho * Fk;
-                const real g0 = e0 + CC * sk2;
-                const real uxk = sk * ux, uyk = sk * uy, exk = sk * e1x, eyk = sk * e1y;
-#pragma unroll
-                for (int r = 0; r < 8; ++r) {
-                    const real vu = dir_dot<real>(r, uxk, uyk);
-                    const real br = p0 + vu * (p1 + vu * (p2 + vu * (p3 + vu * p4)));
-                    const real fe = rF * br;                                                 // Eq. 3
-                    const real I = -(g0 + dir_dot<real>(r, exk, eyk)) * fe;                   // Eq. 11
-                    const real conv = cres[(size_t)r * NX + x];
-                    const real rhs = -conv - (fc[r] - fe) * itau + I;                        // Eq. 10
-                    po[r * N] = rk_combine(with_base, beta, dt, fc[r], fb[r], rhs);
-                }
+            for (int q = 0; q < 4; ++q) {
+                const real qq = real(0.5) * (ux[q] * ux[q] + uy[q] * uy[q]) * iT[q], om = real(1) - qq;
+                const real rF = rho[q] * weight_Fk<real>(c, T[q]);   // Eq. 4
+                const real r1 = rF * iT[q], r2 = r1 * iT[q], r3 = r2 * iT[q];
+                p0[q] = rF * (om + real(0.5) * qq * qq);   // rho F_k times the factors of Eq. 3
+                p1[q] = r1 * om;
+                p2[q] = real(0.5) * r2 * om;
+                p3[q] = r3 * (real(1) / real(6));
+                p4[q] = r3 * iT[q] * (real(1) / real(24));
+                h0[q] = itau - (e0[q] + CC[q] * sk2);
+                uxk[q] = sk * ux[q];
+                uyk[q] = sk * uy[q];
+                exk[q] = sk * e1x[q];
+                eyk[q] = sk * e1y[q];
             }
+            // directions r and r + 4 together: f^eq = even +- odd in v.u;
+            // rhs = (1 / tau - g) f^eq - f / tau - convection with g = -I /
+            // f^eq (Eqs. 10, 11).  The distributions of two such pairs are
+            // loaded before any of their stores, as fout may alias fcur or
+            // fbase.
+            const real *__restrict__ pc = fcur + o0;
+            const real *__restrict__ pb = fbase + o0;
+            real *__restrict__ po = fout + o0;
+#pragma unroll
+            for (int r0 = 0; r0 < 4; r0 += 2) {
+                real fc[4][4], fb[4][4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int d = r0 + (r >> 1) + 4 * (r & 1);
+                    ld4(fc[r], pc + (size_t)d * N);
+                    if (with_base) ld4_once(fb[r], pb + (size_t)d * N);
+                }
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    real cv[2][4], fn[2][4];
+                    ld4(cv[0], cres + (size_t)(r0 + r) * NX + x0);
+                    ld4(cv[1], cres + (size_t)(r0 + r + 4) * NX + x0);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const real vu = dir_dot<real>(r0 + r, uxk[q], uyk[q]), w2 = vu * vu;
+                        const real ev = p0[q] + w2 * (p2[q] + w2 * p4[q]), od = vu * (p1[q] + w2 * p3[q]);   // Eq. 3
+                        const real ed = dir_dot<real>(r0 + r, exk[q], eyk[q]);
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) {
+                            const real fe = s ? ev - od : ev + od, hd = s ? h0[q] + ed : h0[q] - ed;
+                            const real f = fc[2 * r + s][q];
+                            const real rhs = hd * fe - cv[s][q] - f * itau;
+                            fn[s][q] = rk_combine(with_base, beta, dt, f, fb[2 * r + s][q], rhs);
+                        }
+                    }
+                    st4_once(po + (size_t)(r0 + r) * N, fn[0]);
+                    st4_once(po + (size_t)(r0 + r + 4) * N, fn[1]);
+                }
             }
         }
         fence_proxy_async();
@@ -924,10 +780,9 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
                 if (nodd) pend1 = true;
                 else pend0 = true;
             }
-            if (c == NCH - 1 && ri + NHB < nrows) {   // the row's head buffer is free
-                k5_issue_head<real>(spec, fields, aux, Hd, hodd ? &hbar1 : &hbar0, ri + NHB, nx, ny, N, slot, H);
-                if (hodd) hpend1 = true;
-                else hpend0 = true;
+            if (c == NCH - 1 && ri + 1 < nrows) {   // the row's head buffer is free
+                k5_issue_head<real>(spec, fields, aux, Hd, &hbar, ri + 1, nx, ny, N, slot, H);
+                hpend = true;
             }
         }
     }
@@ -935,11 +790,7 @@ __global__ void __launch_bounds__(nt_k5wr<H>(), nt_k5wr<H>() >= 512 ? 1 : 2) k5_
 
 // shared memory of k5_wr<H>
 inline size_t k5_wr_smem(int H) {
-    const int P = H == 512 ? 32 : H == 256 ? 16 : 8;
-    const int NT = nt_k5wr_host(H), CH = (NT / 32) * (32 / P);
-    const int NHB = NT == 512 || H < 256 ? 2 : 1;
-    return smem_bytes({(size_t)H * 8, (size_t)(H / 2 + 1) * 8, (size_t)NHEAD * 2 * H * 4,
-                       NHB > 1 ? (size_t)NHEAD * 2 * H * 4 : 0, (size_t)CH * 2 * H * 4, (size_t)CH * 2 * H * 4});
+    return smem_bytes({(size_t)H * 8, (size_t)H / 2 * 8, (size_t)NHEAD * 2 * H * 4, (size_t)8 * 2 * H * 4, (size_t)8 * 2 * H * 4});
 }
 
 }  // namespace fftlb

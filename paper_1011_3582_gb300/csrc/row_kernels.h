@@ -39,12 +39,12 @@ __host__ __device__ constexpr int row_stride(int size, int H) {
 }
 
 // The tables of the row kernels as one block of bytes: wh[k] = exp(-2 pi i k /
-// 2H) / 2 (k <= H / 2), kx[k] (k < H), the stage-1 twiddles tw[k1 P + l] = exp(-2
-// pi i l k1 / H), wp[k] = exp(-2 pi i k / 2H) (k <= H / 2); offsets of its parts,
+// 2H) / 2 (k < H / 2), kx[k] (k < H), the stage-1 twiddles tw[k1 P + l] = exp(-2
+// pi i l k1 / H), wp[k] = exp(-2 pi i k / 2H) (k < H / 2); offsets of its parts,
 // each a multiple of 16 bytes
 template <typename real> struct RowTable {
     static __host__ __device__ constexpr unsigned up(unsigned b) { return (b + 15u) & ~15u; }
-    static __host__ __device__ constexpr unsigned half(int H) { return up((H / 2 + 1) * 2 * sizeof(real)); }
+    static __host__ __device__ constexpr unsigned half(int H) { return up(H / 2 * 2 * sizeof(real)); }
     static __host__ __device__ constexpr unsigned kx(int H) { return half(H); }
     static __host__ __device__ constexpr unsigned tw(int H) { return kx(H) + up(H * sizeof(real)); }
     static __host__ __device__ constexpr unsigned wp(int H) { return tw(H) + H * 2 * sizeof(real); }

@@ -23,6 +23,11 @@ COLS = [4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024,
 SHAPES = [(n, 6) for n in ROWS] + [(32, n) for n in COLS] + [(36, 64), (64, 54), (12, 96), (8, 16)]
 
 
+# rows just above the line where the persistent fp32 rows take over (one row a
+# block) and a few more than their resident blocks (a second row in some)
+PERSISTENT = [(256, 648), (256, 1296), (512, 324), (512, 648), (1024, 162), (1024, 324)]
+
+
 @pytest.fixture(scope="module")
 def fl():
     return lib()
@@ -32,8 +37,8 @@ def fields_of(nx, ny, seed):
     return W.smooth_random(nx, ny, seed=seed, rho0=1.3, T0=0.9, amp=0.05, umax=0.02)
 
 
-@pytest.mark.parametrize("precision", [64, 32])
-@pytest.mark.parametrize("nx,ny", SHAPES)
+@pytest.mark.parametrize("nx,ny,precision", [(nx, ny, p) for nx, ny in SHAPES for p in (64, 32)] +
+                         [(nx, ny, 32) for nx, ny in PERSISTENT])
 def test_one_step_matches_oracle(fl, nx, ny, precision):
     if precision == 64 and max(nx, ny) > 1024:
         pytest.skip("fp64 grids end at 1024")
