@@ -11,17 +11,16 @@ namespace fftlb {
 // per thread)
 __host__ __device__ constexpr int col_p(int size, int NY) {
     return NY == 2048 || NY == 1536 ? 64
-         : NY == 1024 || NY == 768 ? 32
-         : NY == 512 ? (size == 8 ? 32 : 16)
+         : NY == 1024 || NY == 768 || NY == 512 ? 32
          : NY == 384 || NY == 256 ? 16
          : NY == 192 || NY == 128 || NY == 96 || NY == 64 ? 8
          : NY == 48 || NY == 32 || NY == 24 || NY == 16 ? 4 : 0;
 }
-// stage 2 with two threads per P-point DFT (64 points do not fit one thread's
-// registers; nor, in fp64 at two blocks per SM, do 32 of 512)
-__host__ __device__ constexpr bool col_pair(int size, int NY) {
-    return NY == 2048 || NY == 1536 || (NY == 512 && size == 8);
-}
+// stage 2 with two threads per P-point DFT: 64 points do not fit one thread's
+// registers; nor, in fp64 at two blocks per SM, do 32 of 512; and 16 values a
+// thread instead of 32 leave the fp32 columns of 512 24 warps an SM instead of
+// 16 (2048x512: convection 74 -> 69.5 us)
+__host__ __device__ constexpr bool col_pair(int size, int NY) { return NY == 2048 || NY == 1536 || NY == 512; }
 // columns per tile: 64 bytes of every row, 32 where a tile of 64 would leave
 // one block per SM
 __host__ __device__ constexpr int col_tw(int size, int NY) {

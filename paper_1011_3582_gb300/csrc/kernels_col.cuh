@@ -64,9 +64,14 @@ template <typename real, int NY> __device__ __forceinline__ int cp(int c, int l,
 
 template <typename real, int NY> constexpr int col_minb() {
     using G = Col<real, NY>;
-    // 128 registers a thread where a thread holds up to 32 fp32 or 16 fp64
-    // complex values, 255 beyond
-    return sizeof(real) == 4 || (G::E <= 16 && G::PH <= 16) ? (512 / G::NT > 16 ? 16 : 512 / G::NT) : (256 / G::NT > 16 ? 16 : 256 / G::NT);
+    // threads an SM: 255 registers for more than 16 fp64 complex values a
+    // thread, 128 up to there and for 32 fp32 ones, 85 for 16 of those on columns
+    // of 256 and 512 (2048x256: convection 34.7 us with 128, 30.6 with 85, 30.7
+    // with 64; 2048x512: 74, 69.5, 75.7; shorter columns are small grids, where
+    // 128 are the faster code: 128^2 59.4 us a step against 62.1)
+    constexpr bool half = G::E <= 16 && G::PH <= 16;
+    constexpr int nt = sizeof(real) == 4 ? (half && NY >= 256 ? 768 : 512) : half ? 512 : 256;
+    return nt / G::NT > 16 ? 16 : nt / G::NT;
 }
 
 // The tables of kcol_reg's length in shared memory behind the tile (copied by
