@@ -423,23 +423,28 @@ inline size_t k1_wr_smem(int H) {
 // factor k_x or start from a row spectrum (stage_layout.cuh) -> Lambda (Eq. 19),
 // Phi (Eq. 23), the numerators of C (Eq. 22) and B (Eq. 21) -> d_x of Lambda_xx,
 // Lambda_xy, Phi_x (a forward and an inverse row each) added to the numerators.
-// Persistent over the rows of all runs, one row per pass and one buffer (11
-// transformed rows and 8 real ones); the other blocks of the SM cover the copy.
+// Persistent over the rows of all runs, one row per pass and one buffer of the 11
+// transformed rows; the 8 real rows are read where they are used, from the L2
+// they were sent to with the row's copies, which leaves room and registers for a
+// third block on the SM (all 19 rows staged, two blocks: 39.6 us on 1024^2, 73.6
+// on 1024x2048; so 36.8 and 65.5).
 // ---------------------------------------------------------------------------
 
+// the row's spectra into dst, its real rows into L2
 template <typename C>
 __device__ __forceinline__ void k3_issue(const C *spec, C *dst, uint64_t *bar, int ri, int ny, size_t slot, int h) {
     const int yg = (int)blockIdx.x + ri * (int)gridDim.x;
     const int run = yg / ny, y = yg - run * ny;
     spec += (size_t)run * NSLOT * slot + (size_t)y * h;
     const uint32_t rowbytes = (uint32_t)(h * sizeof(C));
-    mbar_expect_tx(bar, (uint32_t)(NK3 - 3) * rowbytes);   // D_LAP, D_DIVX, D_DIVY are formed in K3
-    for (int o = 0; o < NK3; ++o)
+    mbar_expect_tx(bar, (uint32_t)(NSP - 3) * rowbytes);   // D_LAP, D_DIVX, D_DIVY are formed in K3
+    for (int o = 0; o < NSP; ++o)
         if (k3_src_slot(o) >= 0) bulk_g2s(dst + (size_t)o * h, spec + (size_t)k3_src_slot(o) * slot, rowbytes, bar);
+    for (int o = NSP; o < NK3; ++o) bulk_prefetch_l2(spec + (size_t)k3_src_slot(o) * slot, rowbytes);
 }
 
 template <int H>
-__global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k3_wr(float2 *spec, const float2 *__restrict__ tw_g,
+__global__ void __launch_bounds__(nt_wr<H>(), 768 / nt_wr<H>()) k3_wr(float2 *spec, const float2 *__restrict__ tw_g,
                                                  const float2 *__restrict__ Wp_g, const float2 *__restrict__ Wh_g,
                                                  const float *__restrict__ kxt,
                                                  KP<float> P, int *err) {
@@ -459,8 +464,7 @@ __global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k3_wr(float2 *sp
     C *Wp = (C *)sc.take(H / 2 * sizeof(C));
     C *Wh = (C *)sc.take(H / 2 * sizeof(C));
     real *kxs = (real *)sc.take(H * sizeof(real));   // k_x of the row bins
-    C *dc = (C *)sc.take((size_t)NK3 * H * sizeof(C));
-    real *d = reinterpret_cast<real *>(dc);
+    C *dc = (C *)sc.take((size_t)NSP * H * sizeof(C));
     const int NY = P.nrun * ny;
     const int nrows = (int)blockIdx.x < NY ? (NY - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     if (tid == 0) {   // (the first copies start before the tables load)
@@ -494,20 +498,29 @@ __global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k3_wr(float2 *sp
         __syncthreads();
         auto out = [&](int s) { return reinterpret_cast<real *>(spec_r + (size_t)s * slot); };
 #pragma unroll 1
-        for (int s = 0; s < SMAX; ++s) {
-            const int x = tid + s * NT;
-            const Level2<real> l = level2_site<real>([&](int o) { return d[o * NX + x]; }, P);
-            out(SLOT_L2)[x] = l.Lxy;
-            out(SLOT_L2 + 1)[x] = l.Lyy;
-            out(SLOT_L2 + 2)[x] = l.Phy;
+        for (int s = 0; s < SMAX; s += 2) {   // two consecutive sites
+            const int x = 2 * tid + s * NT;
+            float2 v[NK3];
+#pragma unroll
+            for (int o = NSP; o < NK3; ++o)
+                v[o] = *reinterpret_cast<const float2 *>(out(k3_src_slot(o)) + x);
+#pragma unroll
+            for (int o = 0; o < NSP; ++o) v[o] = dc[o * H + (x >> 1)];
+            const Level2<real> l = level2_site<real>([&](int o) { return v[o].x; }, P);
+            const Level2<real> m = level2_site<real>([&](int o) { return v[o].y; }, P);
+            auto st = [&](int q, real a, real b) { *reinterpret_cast<float2 *>(out(q) + x) = make_float2(a, b); };
+            st(SLOT_L2, l.Lxy, m.Lxy);
+            st(SLOT_L2 + 1, l.Lyy, m.Lyy);
+            st(SLOT_L2 + 2, l.Phy, m.Phy);
             // rows 0..2: transformed next; 3..5: the numerators their d_x
-            // joins (same site, same thread)
-            d[x] = l.Phx;
-            d[NX + x] = l.Lxx;
-            d[2 * NX + x] = l.Lxy;
-            d[3 * NX + x] = l.Cn;
-            d[4 * NX + x] = l.Bx;
-            d[5 * NX + x] = l.By;
+            // joins (same sites, same thread)
+            auto keep = [&](int r, real a, real b) { dc[r * H + (x >> 1)] = make_float2(a, b); };
+            keep(0, l.Phx, m.Phx);
+            keep(1, l.Lxx, m.Lxx);
+            keep(2, l.Lxy, m.Lxy);
+            keep(3, l.Cn, m.Cn);
+            keep(4, l.Bx, m.Bx);
+            keep(5, l.By, m.By);
         }
         __syncthreads();
         for (int r = grp; r < 3; r += NG) {
@@ -520,10 +533,12 @@ __global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k3_wr(float2 *sp
             row_fft_wr<H, +1>(zr, tw, j, rsw);
         }
         __syncthreads();
-        for (int s = 0; s < SMAX; ++s) {
-            const int x = tid + s * NT;
 #pragma unroll
-            for (int r = 0; r < 3; ++r) out(SLOT_A + r)[x] = d[(3 + r) * NX + x] + d[r * NX + x];
+        for (int s = 0; s < SMAX; s += 2) {
+            const int x = 2 * tid + s * NT;
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+                *reinterpret_cast<float2 *>(out(SLOT_A + r) + x) = cadd(dc[(3 + r) * H + (x >> 1)], dc[r * H + (x >> 1)]);
         }
         fence_proxy_async();
         __syncthreads();
@@ -533,7 +548,7 @@ __global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k3_wr(float2 *sp
 
 // shared memory of k3_wr<H>
 inline size_t k3_wr_smem(int H) {
-    return smem_bytes({(size_t)H * 8, (size_t)H / 2 * 8, (size_t)H / 2 * 8, (size_t)H * 4, (size_t)NK3 * 2 * H * 4});
+    return smem_bytes({(size_t)H * 8, (size_t)H / 2 * 8, (size_t)H / 2 * 8, (size_t)H * 4, (size_t)NSP * 2 * H * 4});
 }
 
 // ---------------------------------------------------------------------------
