@@ -91,6 +91,12 @@ template <int DIR, typename C> struct SmallDFT<32, DIR, C> {
         for (int k = 0; k < 16; ++k) {
             R c, s;
             w32<DIR, R>(k, c, s);
+            if (sizeof(R) == 8 && k > 0 && k != 8) {
+                butterfly(e[k], o[k], c, s);
+                v[k] = e[k];
+                v[k + 16] = o[k];
+                continue;
+            }
             const C t = k == 0 ? o[k] : C{o[k].x * c - o[k].y * s, o[k].x * s + o[k].y * c};
             v[k] = cadd(e[k], t);
             v[k + 16] = csub(e[k], t);
