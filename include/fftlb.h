@@ -163,7 +163,7 @@ const char *fftlb_kernel_name(int kind);
 
 /* Launch-parameter tuning of the pipelined stage kernels.  The runtime
  * parameters are tuning[5] = {column tile width of the convection pass,
- * column tile width of the level-1/2 passes, distribution rows per chunk of
+ * column tile width of the level-2 pass, distribution rows per chunk of
  * the forward row kernel, convection rows per chunk of the final row kernel,
  * head buffers of the final row kernel (1 or 2)}.  fftlb_tuning reads them
  * (set = 0) or applies them (set = 1; 0 entries keep the current value;

@@ -5,7 +5,7 @@
 // arenas store the group's runs back to back: each pipelined kernel of a
 // stage is one persistent launch over the rows or column tiles of all runs
 // of the group.  One time step of every group is captured once into a CUDA
-// graph on one internal stream (18 kernel nodes per group for SSP-RK3),
+// graph on one internal stream (15 kernel nodes per group for SSP-RK3),
 // and every fftlb_batch_step replays the graph on the caller's stream.
 // Declarations and contracts: include/fftlb.h.
 #include <map>

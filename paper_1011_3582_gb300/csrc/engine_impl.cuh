@@ -42,6 +42,8 @@
 #include <string>
 #include <vector>
 
+#include "async_copy.cuh"
+#include "block_sum.cuh"
 #include "col_kernels.h"
 #include "engine.h"
 #include "fft_device.cuh"
@@ -535,12 +537,14 @@ __global__ void __launch_bounds__(NT) k_inv_grad_y(const typename cplx_of<real>:
 template <typename real>
 __global__ void __launch_bounds__(256) k_inv_sites(const real *__restrict__ f, real *__restrict__ fields, double *partial,
                                                    size_t N, real pa, real pb) {
-    __shared__ double red[6][8];
+    __shared__ double buf[6][256];
     struct __align__(16) V4 {
         real v[4];
     };
-    double m = 0, px = 0, py = 0, e = 0, bad = 0;
+    grid_dep_wait();
+    double m = 0, px = 0, py = 0, e = 0;
     real um = 0;
+    int bad = 0;
     for (size_t g = blockIdx.x * (size_t)256 + threadIdx.x; g < N / 4; g += (size_t)gridDim.x * 256) {
         real m0[4] = {0, 0, 0, 0}, m1[4] = {0, 0, 0, 0}, m2[4] = {0, 0, 0, 0}, m3[4] = {0, 0, 0, 0};
 #pragma unroll 11
@@ -570,56 +574,35 @@ __global__ void __launch_bounds__(256) k_inv_sites(const real *__restrict__ f, r
             um = um > sqrt(u2) ? um : sqrt(u2);
             const bool ok = isfinite(rho) && isfinite(ux) && isfinite(uy) && isfinite(T) && rho > real(0) && T > real(0) &&
                             pb * rho < real(1);
-            bad += ok ? 0.0 : 1.0;
+            bad += ok ? 0 : 1;
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) *reinterpret_cast<V4 *>(fields + (size_t)q * N + 4 * g) = o[q];
     }
-    double v[6] = {m, px, py, e, (double)um, bad};
-#pragma unroll
-    for (int q = 0; q < 6; ++q)
-        for (int w = 16; w > 0; w >>= 1) {
-            const double o = __shfl_down_sync(0xffffffffu, v[q], w);
-            v[q] = q == 4 ? fmax(v[q], o) : v[q] + o;
-        }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0)
-        for (int q = 0; q < 6; ++q) red[q][warp] = v[q];
-    __syncthreads();
-    if (threadIdx.x < 6) {
-        double acc = red[threadIdx.x][0];
-        for (int w = 1; w < 8; ++w) acc = threadIdx.x == 4 ? fmax(acc, red[threadIdx.x][w]) : acc + red[threadIdx.x][w];
-        partial[(size_t)blockIdx.x * 6 + threadIdx.x] = acc;
-    }
+    const double v[6] = {m, px, py, e, (double)um, (double)bad};
+    block_totals<6, 256, 4>(v, buf, [&](int q, double s) { partial[(size_t)blockIdx.x * 6 + q] = s; });
 }
 
 // The invariants from n blocks' six partial sums and the ng gradient-energy
 // partials after them: out[0..5] = mass, px, py, e_T (with K / 2 times the
 // gradient energy), max |u|, count; out[6] = the device error word.
-static __global__ void k_reduce_partials(const double *partial, int n, int ng, double K, double *out, const int *err) {
-    __shared__ double red[7][NT / 32];
+static __global__ void __launch_bounds__(NT) k_reduce_partials(const double *partial, int n, int ng, double K, double *out,
+                                                               const int *err) {
+    __shared__ double buf[7][NT], tot[7];
     const int tid = threadIdx.x;
+    grid_dep_wait();
     double acc[7] = {0, 0, 0, 0, 0, 0, 0};
     for (int b = tid; b < n; b += NT)
+#pragma unroll
         for (int q = 0; q < 6; ++q) {
             const double v = partial[(size_t)b * 6 + q];
             acc[q] = (q == 4) ? fmax(acc[q], v) : acc[q] + v;
         }
     for (int b = tid; b < ng; b += NT) acc[6] += partial[(size_t)6 * n + b];
-    for (int q = 0; q < 7; ++q)
-        for (int w = 16; w > 0; w >>= 1) {
-            const double o = __shfl_down_sync(0xffffffffu, acc[q], w);
-            acc[q] = q == 4 ? fmax(acc[q], o) : acc[q] + o;
-        }
-    if ((tid & 31) == 0)
-        for (int q = 0; q < 7; ++q) red[q][tid >> 5] = acc[q];
+    block_totals<7, NT, 4>(acc, buf, [&](int q, double s) { tot[q] = s; });
     __syncthreads();
-    if (tid == 0) {
-        for (int q = 0; q < 7; ++q)
-            for (int w = 1; w < NT / 32; ++w) red[q][0] = q == 4 ? fmax(red[q][0], red[q][w]) : red[q][0] + red[q][w];
-        for (int q = 0; q < 6; ++q) out[q] = q == 3 ? red[3][0] + 0.5 * K * red[6][0] : red[q][0];
-        out[6] = (double)*err;
-    }
+    if (tid < 6) out[tid] = tid == 3 ? tot[3] + 0.5 * K * tot[6] : tot[tid];
+    else if (tid == 6) out[6] = (double)*err;
 }
 
 }  // namespace fftlb
@@ -2256,8 +2239,9 @@ class EngineT : public Engine {
         int n0 = 0, nx0 = 0, ny0 = 0;   // blocks of the site sums and of the two energies
         if (rowcol_) {
             n0 = inv_blocks();
-            k_inv_sites<real><<<n0, 256, 0, stream_>>>(f0_, fields_, partial_, N_, kp_.a, kp_.b);
-            FFTLB_LAUNCHED("k_inv_sites");
+            Status st = launch_pdl("k_inv_sites", k_inv_sites<real>, n0, 256, 0, (const real *)f0_, fields_, partial_, N_,
+                                   kp_.a, kp_.b);
+            if (!st.good()) return st;
             if (with_grad) {
                 EnergyArgs<real> a{};
                 a.rho = reinterpret_cast<const C *>(fields_);
@@ -2271,9 +2255,9 @@ class EngineT : public Engine {
                 ny0 = (int)col_tiles();
                 a.partial_x = partial_ + (size_t)n0 * 6;
                 a.partial_y = a.partial_x + nx0;
-                void *args[1] = {&a};
-                FFTLB_CU(cudaLaunchKernel(rs_.energy, dim3(nx0), dim3(rs_.nt), args, rs_.smem_rows, stream_));
-                FFTLB_CU(cudaLaunchKernel(cs_.energy, dim3(ny0), dim3(cs_.nt), args, cs_.smem, stream_));
+                using Energy = void (*)(const EnergyArgs<real>);
+                if (!(st = launch_pdl("energy_row", (Energy)rs_.energy, nx0, rs_.nt, rs_.smem_rows, a)).good()) return st;
+                if (!(st = launch_pdl("energy_col", (Energy)cs_.energy, ny0, cs_.nt, cs_.smem, a)).good()) return st;
             }
         } else {
             n0 = ny_;
@@ -2288,8 +2272,9 @@ class EngineT : public Engine {
                 nx0 = ny0 = ny_;
             }
         }
-        k_reduce_partials<<<1, NT, 0, stream_>>>(partial_, n0, nx0 + ny0, (double)p_.K, red_, err_);
-        FFTLB_LAUNCHED("k_reduce_partials");
+        Status st = launch_pdl("k_reduce_partials", k_reduce_partials, 1, NT, 0, (const double *)partial_, n0, nx0 + ny0,
+                               (double)p_.K, red_, (const int *)err_);
+        if (!st.good()) return st;
         FFTLB_CU(cudaMemcpyAsync(host_red_, red_, 8 * sizeof(double), cudaMemcpyDeviceToHost, stream_));
         FFTLB_CU(cudaStreamSynchronize(stream_));
         for (int q = 0; q < 6; ++q) out[q] = host_red_[q];

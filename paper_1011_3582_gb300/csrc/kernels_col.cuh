@@ -16,9 +16,11 @@
 // one tile, and several blocks on an SM overlap loads and transforms.  A
 // persistent kernel that staged tiles by tensor copies (two buffers, L2
 // prefetch) took 77.7 us for the convection launch of 1024^2 fp32 and 17.9 for
-// level 2 (one job's latency), 24.5 and 11.8 at 512^2; this one 79.2 and 14.6,
-// 20.9 and 10.2.  Both are held by the FMA pipe and the loads' latency at 16
-// warps per SM (44% of the issue slots, 3.4 TB/s).
+// level 2 (one job's latency), 24.5 and 11.8 at 512^2; this one 78 and 14.5,
+// 22.5 and 8.2.  Both are held by the latency of shared memory and of the loads
+// at 16 warps per SM (44% of the issue slots, 3.9 TB/s at 1024^2, 3.0 with the
+// 32-byte rows of 2048); 24 warps, which 16 values a thread allow, gain 6% (see
+// col_minb).
 // The packed column 0 of the tile at k_x = 0 (DC real, row-Nyquist imaginary)
 // needs no pairing of (k_y, -k_y): both columns it carries take the multiplier
 // at k_x = 0, because the Nyquist bin of k_x is zero.
@@ -304,6 +306,7 @@ __global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) energ
     const int h = A.h, c = threadIdx.x % TW, jl = threadIdx.x / TW;
     const C *__restrict__ in = A.rho + (size_t)blockIdx.x * TW + c;
     ColTab<real, NY>::issue(T, A.ctab, &bar);
+    grid_dep_wait();
     C v[E];
 #pragma unroll
     for (int q = 0; q < E; ++q) v[q] = in[(size_t)(jl + P * q) * h];
@@ -321,6 +324,7 @@ __global__ void __launch_bounds__(128) energy_line(const __grid_constant__ Energ
     using C = typename cplx_of<real>::type;
     const int h = A.h, kx = (int)blockIdx.x * 128 + (int)threadIdx.x;
     double e = 0;
+    grid_dep_wait();
     if (kx < h) {
         C v[NY];
 #pragma unroll

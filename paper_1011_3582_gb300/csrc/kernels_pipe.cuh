@@ -13,7 +13,7 @@
 //              column tiles fetched by 2-D tensor copies into one or two
 //              buffers; the spectral multiply is fused with the last
 //              forward pass and its adjoint (fft_device.cuh).
-//   k3_pipe    one row per block: 15 derivative rows + rho, T.
+//   k3_pipe    one row per block: 11 derivative rows + 8 real rows.
 //   k5_pipe    persistent over rows; the per-row head (level-2 spectra,
 //              fields, aux) and CH-row chunks of convection spectra are
 //              prefetched (one or two chunk buffers).
@@ -28,8 +28,8 @@
 // per SM (its 8-row chunks give one radix-16 butterfly per thread; 229 ->
 // 171 us); the column kernels two 256-thread blocks, each with a single
 // staged tile, so that one block's barrier waits and tile loads overlap the
-// other's passes (convection 227 -> 212 us, level 1 144 -> 129 us against
-// one double-buffered 512-thread block); the final row kernel one 512-thread
+// other's passes (convection 227 -> 212 us against one double-buffered
+// 512-thread block); the final row kernel one 512-thread
 // block (its per-site epilogue needs the registers).
 #ifndef FFTLB_NT32_K1
 #define FFTLB_NT32_K1 256

@@ -11,9 +11,9 @@
 // spread over all SMs in units smaller than a row.  So here a row is shared by
 // a thread-block cluster of CS blocks: each takes 32 / CS of the distribution
 // rows (or its share of the derivative rows), and what a site needs from all
-// of them (partial moments, derivatives, coefficients) is exchanged through
-// distributed shared memory, every block taking a slice of the sites.  No
-// block is persistent: the overlap of one row's loads with another's
+// of them (partial moments, derivatives, coefficients) goes through distributed
+// shared memory, every block taking a slice of the sites.  No block is
+// persistent: the overlap of one row's loads with another's
 // transforms comes from several resident blocks per SM.
 //
 // A half row of H = E P complex values is transformed by P lanes of one warp
@@ -972,6 +972,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) energy_
     const int tid = threadIdx.x, j = tid & (P - 1), grp = tid / P, y = (int)blockIdx.x * G::NG + grp;
     const bool mine = y < A.ny;
     C *z = B + grp * G::RC;
+    grid_dep_wait();
     if (mine) {
         const C *__restrict__ in = A.rho + (size_t)y * H;
 #pragma unroll
