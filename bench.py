@@ -121,15 +121,15 @@ def write_ncu_traffic(csv_path, precision, n, note, out_path=None):
     out, single = {}, 0
     for i in sorted(per):
         name, by = per[i]
-        if "k1_pipe" in name or "k1_wr" in name:
+        if "k1_pipe" in name or "k1_wr" in name or "k1_row" in name:
             k = "row_forward_moments"
-        elif "k3_pipe" in name or "k3_wr" in name:
+        elif "k3_pipe" in name or "k3_wr" in name or "k3_row" in name:
             k = "row_level1"
-        elif "k5_pipe" in name or "k5_wr" in name:
+        elif "k5_pipe" in name or "k5_wr" in name or "k5_row" in name:
             k = "row_final"
         elif "kcolm_wr" in name:
             k = "col_level1"
-        elif "kcol_wr" in name or "kcol_pipe" in name:
+        elif "kcol_wr" in name or "kcol_pipe" in name or "kcol_reg" in name or "kcol_line" in name:
             # (logs with a separate level-1 launch: the second of three template arguments)
             m = re.search(r"kcol_pipe<\s*\w+\s*,\s*(\w+)\s*,", name)
             if m and m.group(1) not in ("false", "0"):
