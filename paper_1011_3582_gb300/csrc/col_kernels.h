@@ -8,12 +8,15 @@
 namespace fftlb {
 
 // Threads per column of NY = E P values (0: no configuration, or a column
-// per thread)
+// per thread).  fp64 at 24, 32 and 48: 8, so that the 4 columns of a tile fill a
+// warp, which takes as long half empty; with 4 threads a column the two launches
+// took 22.5 and 22.0 us on 96x48 (16.3, 15.6 so), 131 and 22.5 on 1024x48 (82,
+// 16.2), 43 and 14.6 on 512x32 (37, 13.7), 39.5 and 14.5 on 512x24 (35.4, 13.1).
 __host__ __device__ constexpr int col_p(int size, int NY) {
     return NY == 2048 || NY == 1536 ? 64
          : NY == 1024 || NY == 768 || NY == 512 ? 32
          : NY == 384 || NY == 256 ? 16
-         : NY == 192 || NY == 128 || NY == 96 || NY == 64 ? 8
+         : NY == 192 || NY == 128 || NY == 96 || NY == 64 || (size == 8 && (NY == 48 || NY == 32 || NY == 24)) ? 8
          : NY == 48 || NY == 32 || NY == 24 || NY == 16 ? 4 : 0;
 }
 // stage 2 with two threads per P-point DFT: 64 points do not fit one thread's
