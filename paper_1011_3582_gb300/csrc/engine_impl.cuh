@@ -1180,26 +1180,29 @@ class EngineT : public Engine {
         const long double pi = 3.141592653589793238462643383279502884L;
         w.resize(len);
         for (int m = 0; m < len; ++m) {
+            if (n % 2 == 0 && m >= n / 2) {   // half a turn on
+                w[m] = C{-w[m - n / 2].x, -w[m - n / 2].y};
+                continue;
+            }
             const long double a = 2.0L * pi * (long double)m / (long double)n;
             w[m].x = (real)cosl(a);
             w[m].y = (real)(-sinl(a));
         }
     }
 
+    // The tables below are read off w[m] = exp(-2 pi i m / n), m < n: a long
+    // double sine or cosine takes a microsecond where long double is emulated
+    // (a handle of 512^2 fp64 3.0 ms to create with one each, 1.8 so).
+
     // a[k1 P + l] = b[l E + k1] = exp(-2 pi i l k1 / n), n = E P
-    static void stage1_twiddles(std::vector<C> &a, std::vector<C> &b, int n, int P) {
-        const long double pi = 3.141592653589793238462643383279502884L;
+    static void stage1_twiddles(std::vector<C> &a, std::vector<C> &b, int n, int P, const std::vector<C> &w) {
         const int E = n / P;
         a.resize(n);
         b.resize(n);
         for (int k1 = 0; k1 < E; ++k1)
             for (int l = 0; l < P; ++l) {
-                const long double t = 2.0L * pi * (long double)(l * k1) / (long double)n;
-                C w;
-                w.x = (real)cosl(t);
-                w.y = (real)(-sinl(t));
-                a[(size_t)k1 * P + l] = w;
-                b[(size_t)l * E + k1] = w;
+                a[(size_t)k1 * P + l] = w[l * k1];
+                b[(size_t)l * E + k1] = w[l * k1];
             }
     }
     Status upload_table(C **dst, const std::vector<C> &t) {
@@ -1211,10 +1214,9 @@ class EngineT : public Engine {
 
     // per-pass twiddle tables of the power-of-two passes (see
     // pass_twiddle_len): T[t Ns + k] = exp(-2 pi i t k / (Ns R))
-    static void pass_twiddles(std::vector<C> &T, int n, int maxlr) {
+    static void pass_twiddles(std::vector<C> &T, int n, int maxlr, const std::vector<C> &w) {
         T.clear();
         if (!is_pow2(n)) return;
-        const long double pi = 3.141592653589793238462643383279502884L;
         int logn = 0;
         while ((1 << logn) < n) ++logn;
         int logNs = 0, rem = logn;
@@ -1223,13 +1225,7 @@ class EngineT : public Engine {
             if (logNs > 0) {
                 const int Ns = 1 << logNs, R = 1 << lr;
                 for (int t = 0; t < R; ++t)
-                    for (int k = 0; k < Ns; ++k) {
-                        const long double a = 2.0L * pi * (long double)(t * k) / (long double)(Ns * R);
-                        C w;
-                        w.x = (real)cosl(a);
-                        w.y = (real)(-sinl(a));
-                        T.push_back(w);
-                    }
+                    for (int k = 0; k < Ns; ++k) T.push_back(w[t * k * (n / (Ns * R))]);
             }
             logNs += lr;
             rem -= lr;
@@ -1239,7 +1235,8 @@ class EngineT : public Engine {
     Status build_tables() {
         std::vector<real> kx(h_ + 1), ky(ny_);
         for (int j = 0; j <= h_; ++j) kx[j] = (real)kappa(j, nx_);   // j = h is the Nyquist bin
-        for (int j = 0; j < ny_; ++j) ky[j] = (real)kappa(j < ny_ / 2 ? j : j - ny_, ny_);
+        for (int j = 0; j <= ny_ / 2; ++j) ky[j] = (real)kappa(j, ny_);   // (odd; zero at the Nyquist bin)
+        for (int j = ny_ / 2 + 1; j < ny_; ++j) ky[j] = -ky[ny_ - j];
         std::vector<C> wr, wp, wc;
         twiddles(wr, h_, h_);
         twiddles(wp, nx_, h_);
@@ -1250,9 +1247,9 @@ class EngineT : public Engine {
         FFTLB_CU(cudaMemcpy(Wp_, wp.data(), wp.size() * sizeof(C), cudaMemcpyHostToDevice));
         FFTLB_CU(cudaMemcpy(Wc_, wc.data(), wc.size() * sizeof(C), cudaMemcpyHostToDevice));
         std::vector<C> tr, tr8, tc;
-        pass_twiddles(tr, h_, 4);
-        pass_twiddles(tr8, h_, 3);
-        pass_twiddles(tc, ny_, 4);
+        pass_twiddles(tr, h_, 4, wr);
+        pass_twiddles(tr8, h_, 3, wr);
+        pass_twiddles(tc, ny_, 4, wc);
         ntr_ = (int)tr.size();
         ntr8_ = (int)tr8.size();
         ntc_ = (int)tc.size();
@@ -1266,10 +1263,10 @@ class EngineT : public Engine {
         const int rp = row_p((int)sizeof(real), h_);
         if (own_len(h_) && rp > 0) {
             std::vector<C> t1, t2;
-            stage1_twiddles(t1, t2, h_, rp);
-            if (wr_ok_ && (h_ == 512 || h_ == 256 || h_ == 128)) {
+            stage1_twiddles(t1, t2, h_, rp, wr);
+            if (wr_ok_ && (h_ == 512 || h_ == 256 || h_ == 128)) {   // (E = 16 there)
                 std::vector<C> w1, w2;
-                stage1_twiddles(w1, w2, h_, h_ / 16);
+                stage1_twiddles(w1, w2, h_, h_ / 16, wr);
                 if (!(st = upload_table(&Tw1_, w1)).good()) return st;
             }
             using L = RowTable<real>;
@@ -1288,11 +1285,10 @@ class EngineT : public Engine {
         }
         const int cp = col_p((int)sizeof(real), ny_);
         if (own_len(ny_) && cp > 0) {
-            std::vector<C> t1, t2, w;
-            stage1_twiddles(t1, t2, ny_, cp);
+            std::vector<C> t1, t2;
+            stage1_twiddles(t1, t2, ny_, cp, wc);
             t1.insert(t1.end(), t2.begin(), t2.end());
-            twiddles(w, cp, cp);
-            t1.insert(t1.end(), w.begin(), w.end());
+            for (int k = 0; k < cp; ++k) t1.push_back(wc[k * (ny_ / cp)]);   // exp(-2 pi i k / P)
             const size_t n = t1.size();
             t1.resize(n + ny_ / 2);   // ny reals
             memcpy(t1.data() + n, ky.data(), ny_ * sizeof(real));
