@@ -1,0 +1,49 @@
+"""What the C ABI promises about its buffers, its batches, its rounding and its
+tuning, where a fast route could break it."""
+import numpy as np
+import pytest
+
+from gpu_common import lib
+from paper_1011_3582_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def fl():
+    return lib()
+
+
+def gradient_of(h, g, n, shape):
+    """The gradient of n fields between disjoint, aligned buffers."""
+    out = torch.empty((2 * n,) + shape, dtype=torch.float64, device="cuda")
+    h.gradient(g, out, n)
+    torch.cuda.synchronize()
+    return out
+
+
+# two routes, each within 1e-12 (fp64) or 2e-5 (fp32) of the largest derivative
+# from the true one (test_gpu_spectral.py)
+GRADIENT_TOL = {64: 2e-12, 32: 4e-5}
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("nx,ny", [(64, 64), (32, 12), (96, 24), (36, 16)])
+@pytest.mark.parametrize("n,at", [(1, 0), (1, 1), (3, 0), (3, 2), (2, 0.5)])
+def test_gradient_output_may_overlap_its_input(fl, nx, ny, precision, n, at):
+    """g lies in out's range, from plane `at` of it on (the last case: half a
+    plane in); every derivative is that of the g handed over."""
+    rng = np.random.default_rng(nx + ny + n)
+    src = torch.from_numpy(rng.standard_normal((n, ny, nx))).cuda()
+    with fl.Handle(fl.params(nx=nx, ny=ny, precision=precision)) as h:
+        ref = gradient_of(h, src, n, (ny, nx))
+        buf = torch.empty(2 * n * ny * nx, dtype=torch.float64, device="cuda")
+        first = int(at * ny * nx)
+        g = buf[first:first + n * ny * nx].view(n, ny, nx)
+        g.copy_(src)
+        torch.cuda.synchronize()
+        h.gradient(g, buf, n)
+        torch.cuda.synchronize()
+    err = (buf.view(2 * n, ny, nx) - ref).abs().amax(dim=(1, 2))
+    assert (err <= GRADIENT_TOL[precision] * ref.abs().amax(dim=(1, 2))).all()
