@@ -131,8 +131,8 @@ fftlb_status fftlb_invariants(fftlb_t h, double out[6]);
  * nfields real device fields g[nfields][ny][nx] (fp64) writes
  *   out[2*i]   = D_x g_i,   out[2*i+1] = D_y g_i   (device, fp64).
  * The handle's state f is untouched; its scratch buffers may be used.  out may
- * overlap g (every derivative is that of the g handed over; disjoint buffers
- * are faster).  1 <= nfields <= 16. */
+ * overlap g (every derivative is that of the g handed over); disjoint buffers
+ * on 16-byte boundaries are faster.  1 <= nfields <= 16. */
 fftlb_status fftlb_gradient(fftlb_t h, const double *g, double *out, int nfields);
 
 /* Checkpoint: write / read f, the step count and the parameters (binary,

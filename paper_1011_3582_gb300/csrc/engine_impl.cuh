@@ -819,11 +819,13 @@ class EngineT : public Engine {
             return Status::err(FFTLB_ERR_ARG, "gradient: need device pointers and 1 <= nfields <= 16");
         // D_x by rows, D_y by columns, straight between the caller's buffers;
         // where out overlaps g, whose rows would be overwritten before the
-        // columns are read, through the slots instead (all of g is read first)
+        // columns are read, or where a buffer is not aligned for the 16-byte
+        // accesses of those kernels, through the slots instead (all of g is
+        // read first, one double at a time)
         const uintptr_t g0 = reinterpret_cast<uintptr_t>(g), o0 = reinterpret_cast<uintptr_t>(out);
         const uintptr_t gb = (uintptr_t)nfields * N_ * sizeof(double);
         const bool apart = g0 + gb <= o0 || o0 + 2 * gb <= g0;
-        if (rowcol_ && apart) {
+        if (rowcol_ && apart && aligned16(g) && aligned16(out)) {
             GradArgs<real> a{};
             a.g = reinterpret_cast<const double2 *>(g);
             a.out = reinterpret_cast<double2 *>(out);

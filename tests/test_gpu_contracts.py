@@ -47,3 +47,25 @@ def test_gradient_output_may_overlap_its_input(fl, nx, ny, precision, n, at):
         torch.cuda.synchronize()
     err = (buf.view(2 * n, ny, nx) - ref).abs().amax(dim=(1, 2))
     assert (err <= GRADIENT_TOL[precision] * ref.abs().amax(dim=(1, 2))).all()
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("nx,ny", [(64, 64), (32, 12), (48, 16), (36, 16)])
+@pytest.mark.parametrize("goff,ooff", [(1, 0), (0, 1), (1, 1)])
+def test_gradient_takes_buffers_on_any_double(fl, nx, ny, precision, goff, ooff):
+    """g and out one double off a 16-byte boundary."""
+    n, N = 2, nx * ny
+    rng = np.random.default_rng(nx * ny + goff)
+    src = torch.from_numpy(rng.standard_normal((n, ny, nx))).cuda()
+    with fl.Handle(fl.params(nx=nx, ny=ny, precision=precision)) as h:
+        ref = gradient_of(h, src, n, (ny, nx))
+        g = torch.empty(n * N + 1, dtype=torch.float64, device="cuda")[goff:goff + n * N].view(n, ny, nx)
+        buf = torch.full((2 * n * N + 2,), 7.0, dtype=torch.float64, device="cuda")
+        out = buf[ooff:ooff + 2 * n * N].view(2 * n, ny, nx)
+        g.copy_(src)
+        torch.cuda.synchronize()
+        h.gradient(g, out, n)
+        torch.cuda.synchronize()
+    err = (out - ref).abs().amax(dim=(1, 2))
+    assert (err <= GRADIENT_TOL[precision] * ref.abs().amax(dim=(1, 2))).all()
+    assert (buf[:ooff] == 7.0).all() and (buf[ooff + 2 * n * N:] == 7.0).all()
