@@ -5,10 +5,15 @@
 
 namespace fftlb {
 
-__device__ __forceinline__ void block_sum_store(double v, double *out) {
-    __shared__ double red[32];
-    const int nw = (int)((blockDim.x + 31) >> 5), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int w = 16; w > 0; w >>= 1) v += __shfl_down_sync(0xffffffffu, v, w);
+// The sum over the block's NT threads into *out: whole warps, or one part of a
+// warp (16 threads: fp64 columns of 16), whose shuffles name its own lanes alone.
+template <int NT> __device__ __forceinline__ void block_sum_store(double v, double *out) {
+    static_assert(NT % 32 == 0 || NT == 16 || NT == 8, "whole warps, or a power of two of lanes");
+    constexpr int nl = NT < 32 ? NT : 32, nw = (NT + 31) / 32;
+    constexpr unsigned lanes = nl == 32 ? 0xffffffffu : (1u << nl) - 1u;
+    __shared__ double red[nw];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int w = nl / 2; w > 0; w >>= 1) v += __shfl_down_sync(lanes, v, w);
     if (lane == 0) red[warp] = v;
     __syncthreads();
     if (threadIdx.x == 0) {

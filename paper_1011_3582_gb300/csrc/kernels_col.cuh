@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(Col<real, NY>::NT, col_minb<real, NY>()) energ
         return u;
     });
     if (!ok) return;
-    block_sum_store(e * (1.0 / NY), A.partial_y + blockIdx.x);
+    block_sum_store<Col<real, NY>::NT>(e * (1.0 / NY), A.partial_y + blockIdx.x);
 }
 template <typename real, int NY>
 __global__ void __launch_bounds__(128) energy_line(const __grid_constant__ EnergyArgs<real> A) {
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(128) energy_line(const __grid_constant__ Energ
             e += (double)(m * m * (v[k].x * v[k].x + v[k].y * v[k].y));
         }
     }
-    block_sum_store(e * (1.0 / NY), A.partial_y + blockIdx.x);
+    block_sum_store<128>(e * (1.0 / NY), A.partial_y + blockIdx.x);
 }
 
 // One column of a short grid per thread.

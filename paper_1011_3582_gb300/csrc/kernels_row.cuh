@@ -989,7 +989,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) energy_
             }
         });
     }
-    block_sum_store(e * (1.0 / (2 * H)), A.partial_x + blockIdx.x);
+    block_sum_store<G::NT>(e * (1.0 / (2 * H)), A.partial_x + blockIdx.x);
 }
 
 template <typename real, int H> RowSet row_set() {
