@@ -1799,8 +1799,11 @@ class EngineT : public Engine {
             // blocks.  A step, persistent against cluster rows: 1024x128 147,
             // 137 us; 1024x192 220, 223; 1024x256 234, 280; 1024^2 827, 1057;
             // 512x192 142, 130; 512x256 141, 140; 512x384 199, 221; 512^2 236,
-            // 274; 256x512 161, 154; 256x768 210, 228; 256x1024 258, 290.
-            rowk_ = !(k1wr_ && k3wr_ && k5wr_ && (long)B_ * ny_ * nt_wr_host(h_) >= 256L * nsm_);
+            // 274; 256x512 161, 154; 256x768 210, 228; 256x1024 258, 290.  The
+            // rows of one run count, not those of its group: the two families
+            // round differently, and a run's bits are those of a single handle
+            // (four 256^2 runs in one group take the cluster rows' 290 us).
+            rowk_ = !(k1wr_ && k3wr_ && k5wr_ && (long)ny_ * nt_wr_host(h_) >= 256L * nsm_);
         }
         if (cs_.k && (cs_.tw == 0 || h_ % cs_.tw == 0) && cs_.smem <= budget_) {
             rowcol_ = rows_ok;

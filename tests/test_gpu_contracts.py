@@ -69,3 +69,23 @@ def test_gradient_takes_buffers_on_any_double(fl, nx, ny, precision, goff, ooff)
     err = (out - ref).abs().amax(dim=(1, 2))
     assert (err <= GRADIENT_TOL[precision] * ref.abs().amax(dim=(1, 2))).all()
     assert (buf[:ooff] == 7.0).all() and (buf[ooff + 2 * n * N:] == 7.0).all()
+
+
+@pytest.mark.parametrize("nx,ny,runs", [(256, 256, 4), (512, 162, 2), (1024, 96, 2), (256, 648, 2), (512, 324, 2), (1024, 162, 2)])
+def test_fp32_batch_runs_equal_single_handles_at_any_group_size(fl, nx, ny, runs):
+    """A run's bits do not depend on how many runs share its group: three shapes that
+    alone have too few rows for the persistent row kernels, and three that have
+    enough."""
+    prm = fl.params(nx=nx, ny=ny, integrator=3, precision=32)
+    starts = [W.smooth_random(nx, ny, seed=s, rho0=1.3, T0=0.9, amp=0.05, umax=0.02) for s in range(runs)]
+    with fl.Batch([prm] * runs, autotune=False) as b:
+        for i, f in enumerate(starts):
+            b.set_fields(i, *f)
+        b.step(2)
+        got = [(b.get_f(i), b.invariants(i)) for i in range(runs)]
+    for f, (g, inv) in zip(starts, got):
+        with fl.Handle(prm) as h:
+            h.set_fields(*f)
+            h.step(2)
+            assert np.array_equal(h.get_f(), g)
+            assert h.invariants() == inv
