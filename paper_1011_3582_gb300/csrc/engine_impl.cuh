@@ -535,7 +535,7 @@ __global__ void __launch_bounds__(NT) k_inv_grad_y(const typename cplx_of<real>:
 // bytes a load; bound by the 33 values a site it reads.  Per-site values in
 // the working precision, sums in fp64.
 template <typename real>
-__global__ void __launch_bounds__(256) k_inv_sites(const real *__restrict__ f, real *__restrict__ fields, double *partial,
+__global__ void __launch_bounds__(256) k_inv_sites(const real *f, real *__restrict__ fields, double *partial,
                                                    size_t N, real pa, real pb) {
     __shared__ double buf[6][256];
     struct __align__(16) V4 {

@@ -32,6 +32,9 @@
 // stage writes.  A step on 64^2 fp32 83 -> 50 us, on 64^2 fp64 241 -> 204, on
 // 2048^2 fp32 4618 -> 4547.  Triggered early instead, the waiting blocks fill the
 // SMs that are idle first and then run crowded there (64^2 fp64 389 us).
+// What the stage writes is read by ordinary loads: read-only ones are for memory
+// that nothing writes while the kernel runs, and these kernels run from before
+// their wait on.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -93,8 +96,6 @@ template <int P> __device__ __forceinline__ unsigned lanes_of_row() {
     if constexpr (P >= 32) return 0xffffffffu;
     else return ((1u << P) - 1u) << ((threadIdx.x & 31) & ~(P - 1));
 }
-
-template <typename T> __device__ __forceinline__ T ldro(const T *p) { return __ldg(p); }
 
 // The table block [wh][kx][tw][wp] (row_table): K1 takes its first three
 // parts, K5 the last two, K3 all.
@@ -239,11 +240,11 @@ __device__ __forceinline__ void row_pre(C *z, const C *wp, int j, const C *__res
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int k = j + P * (i0 + u), kc = k == 0 ? H / 2 : H - k;   // (lane 0's first pair: bins 0 and H / 2)
-            pa[u] = ldro(a + k);
-            qa[u] = ldro(a + kc);
+            pa[u] = a[k];
+            qa[u] = a[kc];
             if constexpr (NS > 1) {
-                pb[u] = ldro(b + k);
-                qb[u] = ldro(b + kc);
+                pb[u] = b[k];
+                qb[u] = b[kc];
             }
         }
         if (i0 == 0) ready();

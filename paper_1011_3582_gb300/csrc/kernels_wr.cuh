@@ -262,7 +262,7 @@ __device__ __forceinline__ void k1w_issue(const float *f, float *dst, uint64_t *
 }
 
 template <int H>
-__global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k1_wr(const float *__restrict__ f, float2 *spec, float *__restrict__ fields,
+__global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k1_wr(const float *f, float2 *spec, float *__restrict__ fields,
                                                  const float2 *__restrict__ tw_g, const float2 *__restrict__ Wh_g,
                                                  const float *__restrict__ kxt, KP<float> P, int *err) {
     using C = float2;
@@ -561,8 +561,8 @@ inline size_t k3_wr_smem(int H) {
 // ---------------------------------------------------------------------------
 
 template <int H>
-__global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k5_wr(const float2 *spec, const float *__restrict__ fields,
-                                                 const float *__restrict__ aux, const float *fcur, const float *fbase,
+__global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k5_wr(const float2 *spec, const float *fields,
+                                                 const float *aux, const float *fcur, const float *fbase,
                                                  float *fout, float alpha, float beta,
                                                  const float2 *__restrict__ tw_g, const float2 *__restrict__ Wp_g,
                                                  KP<float> P, int *err) {
