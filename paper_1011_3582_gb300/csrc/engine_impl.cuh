@@ -2085,9 +2085,10 @@ class EngineT : public Engine {
     }
 
   private:
-    // Launch of a warp-resident kernel with programmatic stream serialization
-    // (kernels_row.cuh says what it gives; each kernel calls grid_dep_wait
-    // before it touches memory that earlier kernels wrote or read)
+    // Launch of a kernel with programmatic stream serialization (kernels_row.cuh
+    // says what it gives): before it touches memory that earlier kernels wrote or
+    // read, every thread of the kernel has called grid_dep_wait, or a thread of
+    // its block has and handed over by a barrier
     template <typename... KArgs, typename... Args>
     Status launch_pdl(const char *name, void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
                       Args &&...args) {

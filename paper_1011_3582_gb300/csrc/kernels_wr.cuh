@@ -592,14 +592,9 @@ __global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k5_wr(const floa
         mbar_init(&bar1, 1);
         mbar_init(&hbar, 1);
         mbar_init_fence();
-        // Only the head's level-2 rows come from the launch just before this
-        // one (the level-2 columns); the convection spectra, fields, aux rows
-        // and distributions were complete before that launch began, and that
-        // launch touches none of what this kernel writes.  So under a
-        // programmatic dependent launch only the head copies wait.
+        grid_dep_wait();
         if (njobs > 0) k5_issue_chunk<real>(spec, buf0, &bar0, 0, NCH, CH, nx, ny, slot, H);
         if (njobs > 1) k5_issue_chunk<real>(spec, buf1, &bar1, 1, NCH, CH, nx, ny, slot, H);
-        grid_dep_wait();
         if (nrows > 0) k5_issue_head<real>(spec, fields, aux, Hd, &hbar, 0, nx, ny, N, slot, H);
     }
     load_tab4(tw, tw_g, H, NT);

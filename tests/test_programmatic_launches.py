@@ -58,3 +58,11 @@ def test_read_only_loads_are_of_tables():
     for f in ("kernels_row.cuh", "kernels_wr.cuh", "kernels_col.cuh"):
         for arg in re.findall(r"__ldg\(([\w.]+)", source(f)):
             assert arg in TABLES or arg == "p" and f == "kernels_col.cuh", (f, arg)   # p: tab(), a table value
+
+
+def test_copies_of_the_stage_follow_the_wait():
+    """Only tables are copied to shared memory before grid_dep_wait."""
+    for name, _, body in waiting():
+        before = body[:body.index("grid_dep_wait")]
+        for call in re.findall(r"\b(\w*(?:issue\w*|bulk_\w+|prefetch\w*|tma_\w+))(?:<[\w, ]+>)?\(", before):
+            assert call in ("table_issue", "issue"), (name, call)   # issue: ColTab's
