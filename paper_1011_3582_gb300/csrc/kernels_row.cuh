@@ -810,7 +810,7 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
             p2[q] = real(0.5) * r2 * om;
             p3[q] = r3 * (real(1) / real(6));
             p4[q] = r3 * iT[q] * (real(1) / real(24));
-            h0[q] = itau - (e0[q] + CC[q] * sk2);
+            h0[q] = e0[q] + CC[q] * sk2;
             ux[q] *= sk;
             uy[q] *= sk;
             ex[q] *= sk;
@@ -847,10 +847,12 @@ __global__ void __launch_bounds__(Row<real, H>::NT, row_minb<real, H>()) k5_row(
 #pragma unroll
                     for (int s = 0; s < 2; ++s) {
                         const real fe = s ? ev - od : ev + od;
-                        // (1 / tau - g) f^eq - f / tau - convection, g = -I / f^eq (Eqs. 10, 11)
-                        const real hd = s ? h0[q] + ed : h0[q] - ed;
+                        // -(f - f^eq) / tau - g f^eq - convection, g = -I / f^eq (Eqs. 10, 11);
+                        // the difference before its product with 1 / tau: as (1 / tau - g)
+                        // f^eq - f / tau it is an operation less and rounds f dt / tau twice
+                        const real g = s ? h0[q] - ed : h0[q] + ed;
                         const real f = fc[2 * h + s][q];
-                        const real rhs = hd * fe - cv[2 * h + s][q] - f * itau;
+                        const real rhs = -(f - fe) * itau - cv[2 * h + s][q] - g * fe;
                         fn[s][q] = rk_combine(with_base, beta, dt, f, fb[2 * h + s][q], rhs);
                     }
                 }

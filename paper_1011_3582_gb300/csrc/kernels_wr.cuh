@@ -723,15 +723,15 @@ __global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k5_wr(const floa
                 p2[q] = real(0.5) * r2 * om;
                 p3[q] = r3 * (real(1) / real(6));
                 p4[q] = r3 * iT[q] * (real(1) / real(24));
-                h0[q] = itau - (e0[q] + CC[q] * sk2);
+                h0[q] = e0[q] + CC[q] * sk2;
                 uxk[q] = sk * ux[q];
                 uyk[q] = sk * uy[q];
                 exk[q] = sk * e1x[q];
                 eyk[q] = sk * e1y[q];
             }
             // directions r and r + 4 together: f^eq = even +- odd in v.u;
-            // rhs = (1 / tau - g) f^eq - f / tau - convection with g = -I /
-            // f^eq (Eqs. 10, 11).  The distributions of two such pairs are
+            // rhs = -(f - f^eq) / tau - g f^eq - convection with g = -I / f^eq
+            // (Eqs. 10, 11).  The distributions of two such pairs are
             // loaded before any of their stores, as fout may alias fcur or
             // fbase.
             const real *__restrict__ pc = fcur + o0;
@@ -758,9 +758,9 @@ __global__ void __launch_bounds__(nt_wr<H>(), 512 / nt_wr<H>()) k5_wr(const floa
                         const real ed = dir_dot<real>(r0 + r, exk[q], eyk[q]);
 #pragma unroll
                         for (int s = 0; s < 2; ++s) {
-                            const real fe = s ? ev - od : ev + od, hd = s ? h0[q] + ed : h0[q] - ed;
+                            const real fe = s ? ev - od : ev + od, g = s ? h0[q] - ed : h0[q] + ed;
                             const real f = fc[2 * r + s][q];
-                            const real rhs = hd * fe - cv[s][q] - f * itau;
+                            const real rhs = -(f - fe) * itau - cv[s][q] - g * fe;
                             fn[s][q] = rk_combine(with_base, beta, dt, f, fb[2 * r + s][q], rhs);
                         }
                     }

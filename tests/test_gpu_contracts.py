@@ -89,3 +89,36 @@ def test_fp32_batch_runs_equal_single_handles_at_any_group_size(fl, nx, ny, runs
             h.step(2)
             assert np.array_equal(h.get_f(), g)
             assert h.invariants() == inv
+
+
+@pytest.mark.parametrize("nx,ny,nstates", [(64, 32, 24), (256, 16, 12), (1024, 96, 12), (36, 16, 12)])
+def test_fp32_relaxation_is_rounded_after_the_difference(fl, nx, ny, nstates):
+    """One Euler step of a uniform state: no derivative term, so f' = f - (dt /
+    tau) (f - f^eq).  A handle with dt = tau = 1 returns the kernel's own f^eq
+    (f - (f - f^eq) is exact for neighbouring numbers).  With dt = tau = 0.01
+    the result is the same sum with 1 / tau and dt rounded: (f - f^eq), below
+    2^-16 of f here, is exact or rounded once, the products after it carry three
+    roundings of that small number, and the last addition rounds f' itself, by
+    at most u = 2^-24 of it: together below (1 + 2^-10) u.  Two products of the
+    size of f / tau, subtracted, would each leave a rounding of their own."""
+    rng = np.random.default_rng(nx + ny)
+    one = np.ones((ny, nx))
+    worst = 0.0
+    with fl.Handle(fl.params(nx=nx, ny=ny, integrator=1, precision=32, dt=1.0, tau=1.0)) as h1, \
+            fl.Handle(fl.params(nx=nx, ny=ny, integrator=1, precision=32, dt=0.01, tau=0.01)) as h:
+        for _ in range(nstates):
+            rho, T = rng.uniform(0.4, 1.6), rng.uniform(0.85, 1.0)
+            ux, uy = rng.uniform(-0.05, 0.05, 2)
+            h1.set_fields(rho * one, ux * one, uy * one, T * one)
+            f = h1.get_f()[:, 0, 0]
+            h1.step(1)
+            feq = h1.get_f()[:, 0, 0]
+            assert (np.abs(f - feq) < 2.0 ** -16 * np.abs(f)).all()
+            h.set_fields(rho * one, ux * one, uy * one, T * one)
+            h.step(1)
+            got = h.get_f()
+            assert (got == got[:, :1, :1]).all()
+            r = float(np.float32(0.01)) / float(np.float32(0.01))
+            want = f + r * (feq - f)
+            worst = max(worst, (np.abs(got[:, 0, 0] - want) / np.abs(want)).max())
+    assert worst <= (1 + 2.0 ** -10) * 2.0 ** -24
