@@ -169,10 +169,12 @@ const char *fftlb_kernel_name(int kind);
  * head buffers of the final row kernel (1 or 2)}.  fftlb_tuning reads them
  * (set = 0) or applies them (set = 1; 0 entries keep the current value;
  * FFTLB_ERR_ARG if a value is invalid or does not fit in shared memory).
- * fftlb_autotune times candidate values on the handle's current state
- * (saved and restored, so the state is unchanged) one parameter at a time,
- * keeps the fastest, and returns the best stage time in *stage_ms (may be
- * NULL).  Neither changes results: only the order of independent work. */
+ * fftlb_autotune times candidate values on the handle's current state (which
+ * it leaves as it is) one parameter at a time, keeps the fastest, and returns
+ * the best stage time in *stage_ms (may be NULL).  It leaves out the parameters
+ * of kernels that the grid's stage does not launch (most lengths take kernels
+ * without any): where none is left, it times one set of stages and changes
+ * nothing.  Neither call changes results: only the order of independent work. */
 fftlb_status fftlb_autotune(fftlb_t h, double *stage_ms);
 fftlb_status fftlb_tuning(fftlb_t h, int tuning[5], int set);
 

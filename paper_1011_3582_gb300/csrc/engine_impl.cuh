@@ -2059,7 +2059,11 @@ class EngineT : public Engine {
         double best_ms = 0;
         Status st = time_stage(&best_ms);
         const int cand[NTUNE][4] = {{8, 4, 2, 1}, {8, 4, 2, 1}, {8, 7, 6, 0}, {8, 6, 4, 2}, {2, 1, 0, 0}};
+        // (the parameters of kernels that this grid's stage launches)
+        const bool cols = !colk_, k1 = !rowk_ && !k1wr_, k5 = !rowk_ && !k5wr_;
+        const bool takes[NTUNE] = {cols, cols, k1, k5, k5};
         for (int p = 0; p < NTUNE && st.good(); ++p) {
+            if (!takes[p]) continue;
             for (int c = 0; c < 4 && cand[p][c]; ++c) {
                 int t[NTUNE];
                 for (int q = 0; q < NTUNE; ++q) t[q] = best[q];

@@ -122,3 +122,22 @@ def test_fp32_relaxation_is_rounded_after_the_difference(fl, nx, ny, nstates):
             want = f + r * (feq - f)
             worst = max(worst, (np.abs(got[:, 0, 0] - want) / np.abs(want)).max())
     assert worst <= (1 + 2.0 ** -10) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("nx,ny,tuned", [(128, 64, ()), (36, 64, (2, 3, 4)), (64, 54, (0, 1)), (36, 54, (0, 1, 2, 3, 4))])
+def test_autotune_times_only_what_the_stage_launches(fl, nx, ny, tuned):
+    """A grid whose rows and columns take no runtime parameter is timed once (two
+    warm-up stages and three timed ones) and keeps its parameters; with one axis
+    on the pipelined kernels only that axis's parameters move."""
+    f = W.smooth_random(nx, ny, seed=3, rho0=1.3, T0=0.9, amp=0.05, umax=0.02)
+    with fl.Handle(fl.params(nx=nx, ny=ny, precision=32)) as h:
+        h.set_fields(*f)
+        before, f0 = h.tuning(), h.get_f()
+        h.profile(True)
+        ms = h.autotune()
+        stages = h.profile_read()["row_forward_moments"][1]
+        h.profile(False)
+        after = h.tuning()
+        assert ms > 0 and np.array_equal(h.get_f(), f0)
+    assert (stages == 5) == (not tuned)
+    assert all(a == b for i, (a, b) in enumerate(zip(before, after)) if i not in tuned)
