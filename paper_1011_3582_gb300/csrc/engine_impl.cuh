@@ -297,44 +297,29 @@ struct FieldPtrs {
     double *p[4];
 };
 
-// Moments rho, u_x, u_y, T (Eqs. 7-9) of the state straight into fp64 fields, V
-// consecutive sites per thread (4 with 16-byte accesses, where the fields are so
-// aligned, or 1).  Bound by the 33 values a site it reads.
-template <typename real, int V>
+// Moments rho, u_x, u_y, T (Eqs. 7-9) of the state straight into fp64 fields, one
+// site per thread.  Large grids are bound by the 33 values a site they read,
+// small ones by one thread's chain of loads and divisions: with four sites a
+// thread and 16-byte accesses fp64 took 56 us at 64^2 and 128^2 (27 so; 51 with
+// the fields converted by a second launch), fp32 18 (15), 1024^2 fp32 53 (43) and
+// only 512^2 fp32 less (20; 23).
+template <typename real>
 __global__ void __launch_bounds__(256) k_fields_out(const real *__restrict__ f, FieldPtrs out, size_t N) {
-    struct __align__(V == 4 ? 16 : sizeof(real)) VR {
-        real v[V];
-    };
-    struct __align__(V == 4 ? 16 : 8) VD {
-        double v[V];
-    };
-    for (size_t g = blockIdx.x * (size_t)256 + threadIdx.x; g < N / V; g += (size_t)gridDim.x * 256) {
-        real m0[V], m1[V], m2[V], m3[V];
-#pragma unroll
-        for (int s = 0; s < V; ++s) m0[s] = m1[s] = m2[s] = m3[s] = real(0);
+    for (size_t s = blockIdx.x * (size_t)256 + threadIdx.x; s < N; s += (size_t)gridDim.x * 256) {
+        real m0 = 0, m1 = 0, m2 = 0, m3 = 0;
 #pragma unroll 11
         for (int i = 0; i < Q; ++i) {
-            const VR w = *reinterpret_cast<const VR *>(f + (size_t)i * N + V * g);
-#pragma unroll
-            for (int s = 0; s < V; ++s) {
-                m0[s] += w.v[s];
-                m1[s] += VX<real>(i) * w.v[s];
-                m2[s] += VY<real>(i) * w.v[s];
-                m3[s] += V2<real>(i) * w.v[s];
-            }
+            const real v = f[(size_t)i * N + s];
+            m0 += v;
+            m1 += VX<real>(i) * v;
+            m2 += VY<real>(i) * v;
+            m3 += V2<real>(i) * v;
         }
-        VD o[4];
-#pragma unroll
-        for (int s = 0; s < V; ++s) {
-            const real ux = m1[s] / m0[s], uy = m2[s] / m0[s];
-            o[0].v[s] = (double)m0[s];
-            o[1].v[s] = (double)ux;
-            o[2].v[s] = (double)uy;
-            o[3].v[s] = (double)(real(0.5) * (m3[s] / m0[s] - (ux * ux + uy * uy)));
-        }
+        const real ux = m1 / m0, uy = m2 / m0;
+        const double o[4] = {(double)m0, (double)ux, (double)uy, (double)(real(0.5) * (m3 / m0 - (ux * ux + uy * uy)))};
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if (out.p[q]) *reinterpret_cast<VD *>(out.p[q] + V * g) = o[q];
+            if (out.p[q]) out.p[q][s] = o[q];
     }
 }
 
@@ -750,10 +735,7 @@ class EngineT : public Engine {
         double *tmp = reinterpret_cast<double *>(scratch_d_);
         FieldPtrs o;
         for (int i = 0; i < 4; ++i) o.p[i] = on_device ? dst[i] : dst[i] ? tmp + i * N_ : nullptr;
-        if (aligned16(o.p[0]) && aligned16(o.p[1]) && aligned16(o.p[2]) && aligned16(o.p[3]))
-            k_fields_out<real, 4><<<grid1d(4), 256, 0, stream_>>>(f0_, o, N_);
-        else
-            k_fields_out<real, 1><<<grid1d(), 256, 0, stream_>>>(f0_, o, N_);
+        k_fields_out<real><<<grid1d(), 256, 0, stream_>>>(f0_, o, N_);
         FFTLB_LAUNCHED("k_fields_out");
         if (on_device) return Status::ok();
         for (int i = 0; i < 4; ++i)
@@ -1027,8 +1009,8 @@ class EngineT : public Engine {
         fields_ = fieldsb_ + r * NSLOT * N_;
     }
 
-    unsigned grid1d(int per = 1) const {   // per: sites per thread
-        size_t b = (N_ / per + 255) / 256;
+    unsigned grid1d() const {
+        size_t b = (N_ + 255) / 256;
         return (unsigned)(b > 4096 ? 4096 : b);
     }
     static bool aligned16(const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
