@@ -515,37 +515,40 @@ __global__ void __launch_bounds__(NT) k_inv_grad_y(const typename cplx_of<real>:
 
 // Invariant sums without transforms: the moments (Eqs. 7-9) into fields and per
 // block mass, px, py, e_T of Eq. 17 without its gradient part, max |u| and the
-// count of non-finite or unphysical sites, partial[6 block + ..].  Four
-// consecutive sites per thread (N is a multiple of 4: both axes are even), 16
-// bytes a load; bound by the 33 values a site it reads.  Per-site values in
-// the working precision, sums in fp64.
-template <typename real>
+// count of non-finite or unphysical sites, partial[6 block + ..].  V consecutive
+// sites per thread (N is a multiple of 4: both axes are even).  Four, with
+// 16-byte loads, where that leaves a block for three quarters of the SMs: there
+// the 33 values a site bound it (a call at 1024^2 fp32 81 us, 88 with one; 384^2
+// fp64 132, 140).  One on smaller grids, where a thread's chain of loads and
+// divisions does (256^2 fp64 82, 106 with four; 128^2 58, 95; 64^2 49, 84).
+// Per-site values in the working precision, sums in fp64.
+template <typename real, int V>
 __global__ void __launch_bounds__(256) k_inv_sites(const real *f, real *__restrict__ fields, double *partial,
                                                    size_t N, real pa, real pb) {
     __shared__ double buf[6][256];
-    struct __align__(16) V4 {
-        real v[4];
+    struct __align__(V == 4 ? 16 : sizeof(real)) VR {
+        real v[V];
     };
     grid_dep_wait();
     double m = 0, px = 0, py = 0, e = 0;
     real um = 0;
     int bad = 0;
-    for (size_t g = blockIdx.x * (size_t)256 + threadIdx.x; g < N / 4; g += (size_t)gridDim.x * 256) {
-        real m0[4] = {0, 0, 0, 0}, m1[4] = {0, 0, 0, 0}, m2[4] = {0, 0, 0, 0}, m3[4] = {0, 0, 0, 0};
+    for (size_t g = blockIdx.x * (size_t)256 + threadIdx.x; g < N / V; g += (size_t)gridDim.x * 256) {
+        real m0[V] = {}, m1[V] = {}, m2[V] = {}, m3[V] = {};
 #pragma unroll 11
         for (int i = 0; i < Q; ++i) {
-            const V4 w = *reinterpret_cast<const V4 *>(f + (size_t)i * N + 4 * g);
+            const VR w = *reinterpret_cast<const VR *>(f + (size_t)i * N + V * g);
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
+            for (int s = 0; s < V; ++s) {
                 m0[s] += w.v[s];
                 m1[s] += VX<real>(i) * w.v[s];
                 m2[s] += VY<real>(i) * w.v[s];
                 m3[s] += V2<real>(i) * w.v[s];
             }
         }
-        V4 o[4];
+        VR o[4];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
+        for (int s = 0; s < V; ++s) {
             const real rho = m0[s], ux = m1[s] / rho, uy = m2[s] / rho, u2 = ux * ux + uy * uy;
             const real T = real(0.5) * (m3[s] / rho - u2);
             o[0].v[s] = rho;
@@ -562,7 +565,7 @@ __global__ void __launch_bounds__(256) k_inv_sites(const real *f, real *__restri
             bad += ok ? 0 : 1;
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) *reinterpret_cast<V4 *>(fields + (size_t)q * N + 4 * g) = o[q];
+        for (int q = 0; q < 4; ++q) *reinterpret_cast<VR *>(fields + (size_t)q * N + V * g) = o[q];
     }
     const double v[6] = {m, px, py, e, (double)um, (double)bad};
     block_totals<6, 256, 4>(v, buf, [&](int q, double s) { partial[(size_t)blockIdx.x * 6 + q] = s; });
@@ -2233,8 +2236,8 @@ class EngineT : public Engine {
         int n0 = 0, nx0 = 0, ny0 = 0;   // blocks of the site sums and of the two energies
         if (rowcol_) {
             n0 = inv_blocks();
-            Status st = launch_pdl("k_inv_sites", k_inv_sites<real>, n0, 256, 0, (const real *)f0_, fields_, partial_, N_,
-                                   kp_.a, kp_.b);
+            auto *sites = inv_wide() ? k_inv_sites<real, 4> : k_inv_sites<real, 1>;
+            Status st = launch_pdl("k_inv_sites", sites, n0, 256, 0, (const real *)f0_, fields_, partial_, N_, kp_.a, kp_.b);
             if (!st.good()) return st;
             if (with_grad) {
                 EnergyArgs<real> a{};
@@ -2276,8 +2279,9 @@ class EngineT : public Engine {
         if (e) return Status::err(FFTLB_ERR_TIMEOUT, "a bounded device wait ran out (error word " + std::to_string(e) + ")");
         return Status::ok();
     }
-    // blocks of k_inv_sites: enough for every SM, each with whole vectors of sites
-    int inv_blocks() const { return (int)std::min<size_t>((N_ / 4 + 255) / 256, (size_t)4 * nsm_); }
+    // sites per thread (see k_inv_sites) and blocks of k_inv_sites
+    bool inv_wide() const { return N_ >= (size_t)768 * nsm_; }
+    int inv_blocks() const { return (int)std::min<size_t>((N_ / (inv_wide() ? 4 : 1) + 255) / 256, (size_t)4 * nsm_); }
 };
 
 }  // namespace fftlb

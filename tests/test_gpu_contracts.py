@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 from gpu_common import lib
+from oracle import fftlb_oracle as O
 from paper_1011_3582_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -141,3 +142,25 @@ def test_autotune_times_only_what_the_stage_launches(fl, nx, ny, tuned):
         assert ms > 0 and np.array_equal(h.get_f(), f0)
     assert (stages == 5) == (not tuned)
     assert all(a == b for i, (a, b) in enumerate(zip(before, after)) if i not in tuned)
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("nx,ny", [(36, 18), (96, 48), (384, 288), (384, 324)])
+def test_invariants_on_both_sides_of_the_wide_site_sums(fl, nx, ny, precision):
+    """The conservation sums with one and with four sites a thread (the last
+    grid), measured against the sums of the parts' absolute values: every
+    per-site value carries at most 16 roundings, summed in fp64."""
+    f = W.smooth_random(nx, ny, seed=nx + ny, rho0=1.3, T0=0.9, amp=0.05, umax=0.02)
+    p = O.Params(nx=nx, ny=ny)
+    with fl.Handle(fl.params(nx=nx, ny=ny, precision=precision)) as h:
+        h.set_fields(*f)
+        inv = h.invariants()
+    f0 = O.init_equilibrium(*f, p)
+    ref = O.invariants(f0, p)
+    rho, ux, uy, T = O.moments(f0)
+    area = p.dx ** 2
+    grad2 = O.D(rho, "x", p.dx, 4) ** 2 + O.D(rho, "y", p.dx, 4) ** 2
+    scale = dict(mass=rho.sum() * area, px=(4.3 * rho).sum() * area, py=(4.3 * rho).sum() * area, umax=4.3,
+                 eT=(rho * T + p.a * rho ** 2 + p.K * grad2 / 2 + rho).sum() * area)
+    for k, s in scale.items():
+        assert abs(inv[k] - ref[k]) <= (1e-13 if precision == 64 else 2e-6) * s
