@@ -892,11 +892,11 @@ class EngineT : public Engine {
     int conv_groups_ = 0, l2_groups_ = 0, grad_groups_ = 0, inv_groups_ = 0;
     int nconv_ = NMOV;   // convection groups (velocities with v_y != 0)
     int nconvl_ = NMOV;  // ... and the level-1 groups after them
-    // warp-resident fp32 row kernels (kernels_wr.cuh) for nx = 512, 1024:
-    // their stage-1 twiddle table and launch shape
+    // persistent fp32 row kernels (kernels_wr.cuh) for nx = 256, 512, 1024: their
+    // stage-1 twiddle table (that of the cluster rows) and launch shape
     static constexpr bool wr_ok_ = std::is_same<real, float>::value && !SPLIT;
     bool k5wr_ = false, k1wr_ = false, k3wr_ = false;
-    C *Tw1_ = nullptr;
+    const C *Tw1_ = nullptr;   // in Trow_
     size_t smem5w_ = 0, smem1w_ = 0, smem3w_ = 0;
     int grid5w_ = 1, grid1w_ = 1, grid3w_ = 1;
     // row and column kernels of kernels_row.cuh / kernels_col.cuh, the
@@ -914,8 +914,7 @@ class EngineT : public Engine {
     // test hook: nonzero = every stage starts with k_wait_selftest (ns)
     unsigned long long wait_test_ns_ = 0;
     // launch configuration
-    int TW_ = 1;
-    size_t smem_col1_ = 0, smem_col2_ = 0, smem_rows1_ = 0, smem_inv_ = 0;
+    size_t smem_rows1_ = 0;   // k_inv_rows
     // pipelined kernels
     int *err_ = nullptr;
     int nsm_ = 1;
@@ -1251,11 +1250,6 @@ class EngineT : public Engine {
         if (own_len(h_) && rp > 0) {
             std::vector<C> t1, t2;
             stage1_twiddles(t1, t2, h_, rp, wr);
-            if (wr_ok_ && (h_ == 512 || h_ == 256 || h_ == 128)) {   // (E = 16 there)
-                std::vector<C> w1, w2;
-                stage1_twiddles(w1, w2, h_, h_ / 16, wr);
-                if (!(st = upload_table(&Tw1_, w1)).good()) return st;
-            }
             using L = RowTable<real>;
             std::vector<C> blob((L::bytes(h_) + sizeof(C) - 1) / sizeof(C), C{0, 0});
             unsigned char *b = reinterpret_cast<unsigned char *>(blob.data());
@@ -1269,6 +1263,7 @@ class EngineT : public Engine {
             memcpy(b + L::kx(h_), kx.data(), h_ * sizeof(real));
             memcpy(b + L::tw(h_), t1.data(), t1.size() * sizeof(C));
             if (!(st = upload_table(&Trow_, blob)).good()) return st;
+            Tw1_ = Trow_ + L::tw(h_) / sizeof(C);
         }
         const int cp = col_p((int)sizeof(real), ny_);
         if (own_len(ny_) && cp > 0) {
@@ -1446,24 +1441,7 @@ class EngineT : public Engine {
         FFTLB_CU(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
         const size_t budget = (size_t)maxsm - 2048;   // static shared memory headroom
         optin_ = (size_t)maxsm;
-        // column tile width: largest of 8, 4, 2, 1 dividing h with the
-        // batched column FFT fitting the registers (TW ny <= 16 NT) and
-        // 3 tiles in shared memory
-        TW_ = 1;
-        for (int tw = 8; tw >= 1; tw >>= 1) {
-            if (h_ % tw) continue;
-            if ((size_t)tw * ny_ > 16 * NT) continue;
-            if ((size_t)(ny_ + 3 * tw * ny_) * cs > budget) continue;
-            TW_ = tw;
-            break;
-        }
-        smem_col1_ = (size_t)(ny_ + 2 * TW_ * ny_) * cs;
-        smem_col2_ = (size_t)(ny_ + 3 * TW_ * ny_) * cs;
         smem_rows1_ = (size_t)3 * h_ * cs;
-        smem_inv_ = (size_t)4 * h_ * cs;
-        if (smem_col2_ > budget || smem_inv_ > budget)
-            return Status::err(FFTLB_ERR_ARG, "grid too large for shared-memory tiles");
-        FFTLB_CU(cudaFuncSetAttribute(k_col<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
         FFTLB_CU(cudaFuncSetAttribute(k_inv_rows<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
         kp_.nx = nx_;
         kp_.ny = ny_;

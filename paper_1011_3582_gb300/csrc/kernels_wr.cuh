@@ -23,6 +23,7 @@
 
 #include "fft_small.cuh"
 #include "kernels_pipe.cuh"
+#include "row_kernels.h"
 
 namespace fftlb {
 
@@ -31,6 +32,8 @@ template <int H> struct RowCfg;
 template <> struct RowCfg<512> { static constexpr int E = 16, P = 32; };
 template <> struct RowCfg<256> { static constexpr int E = 16, P = 16; };
 template <> struct RowCfg<128> { static constexpr int E = 16, P = 8; };
+// (the cluster rows' lanes: both families read one table of stage-1 twiddles)
+static_assert(RowCfg<512>::P == row_p(4, 512) && RowCfg<256>::P == row_p(4, 256) && RowCfg<128>::P == row_p(4, 128), "lanes a row");
 
 // Threads per block: 4 sites of a row each, i.e. 8 row groups and chunks of one
 // ring of velocities at every length, and as many blocks on an SM as 128
