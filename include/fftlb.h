@@ -91,7 +91,8 @@ typedef struct {
 
 /* Create a handle for problem *p on the current CUDA device.  velset may be
  * NULL (paper's set).  cuda_stream is a cudaStream_t (may be NULL).
- * Allocates ~ (2*33 + 38 + 15 + 5 + 7) nx ny values of the chosen precision.
+ * Allocates ~ (2*33 + 61) nx ny values of the chosen precision (states and
+ * spectra; 33 fewer with integrator 1) and 33 nx ny doubles of staging.
  * Errors: FFTLB_ERR_ARG (sizes, tau <= 0, window, integrator, precision,
  * a velocity set other than that of live handles of the same precision),
  * FFTLB_ERR_OOM, FFTLB_ERR_CUDA.  On error *h is set to NULL. */
@@ -196,16 +197,17 @@ fftlb_status fftlb_debug_wait_test(fftlb_t h, long long ns);
 /* Batched sweep: nruns independent problems (each its own grid, parameters
  * and state; the same velocity set) advanced together.  Runs with identical
  * fftlb_params (check_every aside) form a group whose states are stored
- * back to back; every kernel of a stage is one persistent launch over the
- * rows / column tiles of all runs of the group.  One time step of every
+ * back to back; every kernel of a stage is one launch over the rows / column
+ * tiles of all runs of the group.  One time step of every
  * group, the groups one after another on one internal stream, is captured
  * once into a CUDA graph; fftlb_batch_step(b, n) replays it n times on
  * cuda_stream (borrowed; NULL = legacy default stream).  With autotune != 0,
- * fftlb_batch_create tunes each group's launch parameters on a uniform
- * state.  check_every is ignored (no host checks inside replays); call
+ * fftlb_batch_create tunes each group's launch parameters (as fftlb_autotune)
+ * on a uniform state.  check_every is ignored (no host checks inside replays); call
  * fftlb_batch_invariants to inspect a run.  Per-run calls take the run
  * index; they are ordered after the steps already launched.  Results of a
- * run are identical to those of a single handle with the same parameters.
+ * run are identical to those of a single handle with the same parameters,
+ * however many runs share its group.
  * Memory: as nruns single handles. */
 typedef struct fftlb_batch_s *fftlb_batch_t;
 fftlb_status fftlb_batch_create(fftlb_batch_t *b, int nruns, const fftlb_params *params,

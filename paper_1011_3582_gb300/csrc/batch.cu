@@ -2,9 +2,8 @@
 // grids and temperatures, arXiv:1011.3582 Sec. 4.1) advanced together.
 // Runs that share every parameter (grid, dx, dt, tau, EOS, K, H, q, zeta,
 // window, integrator, precision) form one group, held by one engine whose
-// arenas store the group's runs back to back: each pipelined kernel of a
-// stage is one persistent launch over the rows or column tiles of all runs
-// of the group.  One time step of every group is captured once into a CUDA
+// arenas store the group's runs back to back: each kernel of a stage is one
+// launch over the rows or column tiles of all runs of the group.  One time step of every group is captured once into a CUDA
 // graph on one internal stream (15 kernel nodes per group for SSP-RK3),
 // and every fftlb_batch_step replays the graph on the caller's stream.
 // Declarations and contracts: include/fftlb.h.

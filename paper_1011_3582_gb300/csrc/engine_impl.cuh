@@ -86,9 +86,10 @@ template <> __device__ __forceinline__ double FKC<double>(int k, int j) { return
 template <> __device__ __forceinline__ float FKC<float>(int k, int j) { return c_Fkf[k][j]; }
 
 // nrun: independent runs of this grid stored back to back (f [run][33][ny][nx],
-// spectra [run][58][ny][nx/2], fields [run][4][ny][nx], aux [run][3][ny][nx]);
-// the pipelined kernels treat the nrun * ny rows (or column tiles) of all
-// runs as one job list
+// slots [run][NSLOT][ny][nx/2], see stage_layout.cuh; the fields and aux pointers
+// the kernels take are slots SLOT_F and SLOT_A of run 0, NSLOT slots from run to
+// run); the kernels treat the nrun * ny rows (or column tiles) of all runs as one
+// job list
 // tc16: the A fragments of the split-BF16 tensor-core first pass
 // (tc_dft16_pass), or nullptr for the plain radix-16 first pass
 template <typename real> struct KP {
@@ -175,8 +176,8 @@ __device__ __forceinline__ void weights_Fk(real T, real F[5]) {
 }
 
 // ---------------------------------------------------------------------------
-// column pass for the gradient and the invariants (one tile per block):
-// forward -> multiplier -> inverse
+// column pass of fftlb_gradient_static (noalloc.cu), one tile per block: forward
+// -> multiplier -> inverse
 // ---------------------------------------------------------------------------
 
 template <typename real>

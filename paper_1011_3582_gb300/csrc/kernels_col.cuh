@@ -69,8 +69,9 @@ template <typename real, int NY> constexpr int col_minb() {
     // threads an SM: 255 registers for more than 16 fp64 complex values a
     // thread, 128 up to there and for 32 fp32 ones, 85 for 16 of those on columns
     // of 256 and 512 (2048x256: convection 34.7 us with 128, 30.6 with 85, 30.7
-    // with 64; 2048x512: 74, 69.5, 75.7; shorter columns are small grids, where
-    // 128 are the faster code: 128^2 59.4 us a step against 62.1)
+    // with 64; 2048x512: 74, 69.5, 75.7).  Shorter columns keep 128: with 85 those
+    // of 128 spill (2048x128: 18.6 us with 128, 20.8 with 85; 1024x128 12.4, 14.4;
+    // 16 runs of 128^2 309, 317 a step), 192, 96 and 64 take as long either way
     constexpr bool half = G::E <= 16 && G::PH <= 16;
     constexpr int nt = sizeof(real) == 4 ? (half && NY >= 256 ? 768 : 512) : half ? 512 : 256;
     return nt / G::NT > 16 ? 16 : nt / G::NT;

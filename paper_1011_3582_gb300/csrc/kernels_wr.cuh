@@ -239,7 +239,7 @@ __device__ __forceinline__ void st4_once(float *p, const float (&a)[4]) {
 // ---------------------------------------------------------------------------
 // K1 (fp32, nx = 2H): moments rho, u, T (Eqs. 7-9), the level-1 fields
 // Pi = P^w - rho T (Eq. 18) and g = M/T, and the forward row transforms of
-// the 32 moving f_i and of rho, u_x, u_y, T, Pi, g, as k1_pipe, with
+// the 24 f_i with v_x != 0 and of rho, u_x, u_y, T, Pi, g, as k1_pipe, with
 // warp-resident row transforms.  Persistent over the rows of all runs;
 // per row, 32 / NG chunks of distribution rows (the first also holds the
 // rest velocity's row, which only enters the moments), NG = rows per block
